@@ -134,6 +134,7 @@ __global__ void __launch_bounds__(kThreadsStream) decode_attn_stream(const __gri
         uint8_t* sV = sK + TILE;
         if (pages == 0) {
           mbar_arrive(&full[st]);  // only the row's own key here: nothing to copy
+          armed[st] = -1;          // and nothing in flight (the stage's previous copies were consumed)
         } else {
           mbar_arrive_expect_tx(&full[st], 2 * pages * HALVES * kPage * 128);
           for (int pg = 0; pg < pages; ++pg) {

@@ -131,3 +131,29 @@ def test_decode_step_rejects_bad_arguments():
     ctx.decode_step(dm.crf, ad.crf, pool, [20], [pt], tok[:1], nxt[:1], ws, logits=logits[:1])
     ctx.check()
     assert not torch.all(logits[0] == 7.0) and int(nxt[0]) >= 0
+
+
+def test_chunk_boundary_positions_do_not_stall():
+    """Rows whose position opens a new 128-key chunk (it holds only the row's own key), each streamed
+    by blocks of three chunks: the empty chunk reuses a stage whose copies are long consumed, and no
+    wait is left for them (a wait for a passed phase runs into the 2 s limit at every layer)."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import time
+    import paper_2609_30884_gb300 as crf
+    cfg, lc = synth.TINY, synth.LORA_TINY
+    rows, pos = 32, 640
+    dm, ad = DeviceModel(cfg), DeviceAdapter(cfg, lc, 1)
+    P = rows * pages_needed(pos + 1) + 3
+    pts = split_page_tables([pos + 1] * rows, P, seed=8)
+    pool = make_pool(cfg, P, fill="random", seed=4)
+    ctx = crf.Context(0)
+    tok = synth.token_ids(cfg, rows, device="cuda")
+    nxt = torch.empty(rows, dtype=torch.int32, device="cuda")
+    ws = ctx.decode_workspace(dm.crf, ad.crf, [pos] * rows, pts, tok)
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    ctx.decode_step(dm.crf, ad.crf, pool, [pos] * rows, pts, tok, nxt, ws)
+    ctx.check()
+    assert time.perf_counter() - t0 < 1.5
+    ctx.close()
