@@ -170,13 +170,18 @@ struct Plan {
   size_t off_g0, off_g1, off_x1, off_xn, off_q, off_o, off_mlp, off_xa, off_bx, off_rope;
   size_t off_dx0, off_dec;  // decode: bf16 starting rows, fp32 scratch
   size_t off_abort, off_ptab;  // the call's abort word; the page-check table (ptab_slots ints)
-  // the projections' XA ready words (4 launches x ceil(M / 256) row blocks per layer) and the
-  // decode-row norms' per-row counters (kMaxReq), laid out after the abort word so one clear at
-  // the start of the call covers them all
-  size_t flag_words = kMaxReq;
+  // the projections' XA ready words (4 launches x ceil(M / 256) row blocks per layer), laid out
+  // after the abort word so one clear at the start of the call covers them all
+  size_t flag_words = 0;
   uint32_t ptab_slots = 2;
-  size_t dec_bytes;
   size_t total;
+};
+
+// Scratch of the decode rows (byte offsets from its start, 256-byte aligned): the fp32 rows, their
+// slices' sums of squares, the bf16 terms entering the four passes, one pass's partial sums and the
+// attention partials.
+struct DecodeScratch {
+  size_t x, nss, xs, os, ms, y, part, total;
 };
 
 // output rows of module m (q, k, v, o, gate, up, down) and their sum
@@ -190,6 +195,49 @@ int module_rows_total(const Dims& D) {
   return t;
 }
 
+// The four weight passes of a decode layer: q|k|v, o, gate|up, down.
+struct DecodePasses {
+  RowsPlan qkv, o, gu, down;
+};
+DecodePasses decode_passes(const Dims& D, uint32_t mask, int num_sms) {
+  auto any = [&](std::initializer_list<int> mods) {
+    bool a = false;
+    for (int m : mods) a |= ((mask >> m) & 1u) != 0;
+    return a;
+  };
+  const int qkv[3] = {D.qd, D.kvd, D.kvd}, gu[2] = {D.f, D.f};
+  DecodePasses p;
+  p.qkv = rows_plan(3, qkv, any({CRF_MOD_Q, CRF_MOD_K, CRF_MOD_V}), D.h, num_sms);
+  p.o = rows_plan(1, &D.h, any({CRF_MOD_O}), D.qd, num_sms);
+  p.gu = rows_plan(2, gu, any({CRF_MOD_GATE, CRF_MOD_UP}), D.h, num_sms);
+  p.down = rows_plan(1, &D.h, any({CRF_MOD_DOWN}), D.f, num_sms);
+  return p;
+}
+
+DecodeScratch decode_scratch(const Dims& D, uint32_t mask, int rows, int attn_splits, int num_sms) {
+  DecodeScratch s;
+  size_t o = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = o;
+    o = align256(o + bytes);
+    return at;
+  };
+  const size_t R = static_cast<size_t>(rows), T = static_cast<size_t>(rows_terms(rows));
+  const DecodePasses p = decode_passes(D, mask, num_sms);
+  size_t y = 0;
+  for (const RowsPlan* q : {&p.qkv, &p.o, &p.gu, &p.down})
+    y = std::max(y, R * static_cast<size_t>(q->splits) * q->ncols * sizeof(float));
+  s.x = take(R * D.h * sizeof(float));
+  s.nss = take(R * norm_slices(D.h) * sizeof(float));
+  s.xs = take(R * T * D.h * 2);
+  s.os = take(R * T * D.qd * 2);
+  s.ms = take(R * T * D.f * 2);
+  s.y = take(y);
+  s.part = take(R * D.hq * static_cast<size_t>(attn_splits) * (D.d + 2) * sizeof(float));
+  s.total = o;
+  return s;
+}
+
 // decode attention partials: one per chunk of the longest prefix
 int dec_splits(int max_n) { return decode_attention_splits(max_n); }
 
@@ -200,7 +248,7 @@ uint32_t ptab_slots_for(long ids) {
   return s;
 }
 
-Plan make_plan(const Dims& D, const crf_request* reqs, int n_req) {
+Plan make_plan(const Dims& D, const crf_request* reqs, int n_req, uint32_t mask, int num_sms) {
   Plan p;
   for (int l = 0; l < D.N; ++l) {
     int m = 0;
@@ -239,16 +287,11 @@ Plan make_plan(const Dims& D, const crf_request* reqs, int n_req) {
     for (int i = 0; i < n_req; ++i) any |= reqs[i].s <= l && l < reqs[i].e;
     layers += any ? 1 : 0;
   }
-  p.flag_words = static_cast<size_t>(layers) * 4 * ((p.M + 255) / 256) + kMaxReq;
+  p.flag_words = static_cast<size_t>(layers) * 4 * ((p.M + 255) / 256);
   p.off_abort = take((1 + p.flag_words) * sizeof(int));
   p.off_ptab = take(static_cast<size_t>(p.ptab_slots) * sizeof(int));
   p.splits = dec_splits(p.max_n);
-  // decode scratch per row, fp32: x, xn, x1, q, k, v, o, xa (7 slots), gu, m, norm partials,
-  // attention partials
-  const size_t dec_row = static_cast<size_t>(3 * D.h + 2 * D.qd + 2 * D.kvd + 7 * kRankPad + 3 * D.f + norm_up_slices(D.h)) * 4 +
-                         static_cast<size_t>(D.hq) * p.splits * (D.d + 2) * 4;
-  p.dec_bytes = align256(dec_row * std::max(1, p.dec_rows));
-  p.off_dec = take(p.dec_rows ? p.dec_bytes : 0);
+  p.off_dec = take(p.dec_rows ? decode_scratch(D, mask, p.dec_rows, p.splits, num_sms).total : 0);
   p.total = o;
   return p;
 }
@@ -507,22 +550,24 @@ crf_status run_layer(const LayerCtx& c, int l, const __nv_bfloat16* X_in, __nv_b
 // Carry the last prefix row of every listed request through layers [e_i, N) against each
 // layer's cached K/V at positions < n_i - 1 (fp32 rows). Rows are ordered by window end, so
 // the rows active at a layer are a prefix of the batch and each layer's weights are read once
-// for all of them (GEMV launches of up to 8 rows).
+// for all of them.
 struct DecodeRow {
   int e;            // first layer to run
   int pos;          // position of the row (= n - 1)
   const int32_t* page_table;
   const __nv_bfloat16* start;  // bf16 [h], or null when the row starts from `token`'s embedding
-  void* out;        // bf16 [h], or null (the final fp32 rows stay in the decode scratch)
+  void* out;        // bf16 [h], or null (the rows stay in the decode scratch)
   const int32_t* token = nullptr;  // device, the row's input token (generation steps)
 };
 
-// Generation steps (crf_decode_step) write each layer's k, v of the row into its page slot and
-// take RoPE angles from a table of the rows' own positions; the first-step rows of a window do
-// neither (their positions are in the window's full table, and the historical cache stays).
+// Generation steps (crf_decode_step) write each layer's k, v of the row into its page slot, take
+// RoPE angles from a table of the rows' own positions and end in the final norm, as the LM head's
+// input; the first-step rows of a window do neither (their positions are in the window's full
+// table, the historical cache stays, and the rows leave as bf16).
 struct DecodeOpts {
   bool write_kv = false;
   const float2* rope_by_row = nullptr;
+  const __nv_bfloat16* final_norm = nullptr;
 };
 
 crf_status decode_rows(const LayerCtx& c, std::vector<DecodeRow> rows, const DecodeOpts& opt = DecodeOpts()) {
@@ -532,172 +577,128 @@ crf_status decode_rows(const LayerCtx& c, std::vector<DecodeRow> rows, const Dec
   if (R == 0) return CRF_OK;
   std::stable_sort(rows.begin(), rows.end(), [](const DecodeRow& a, const DecodeRow& b) { return a.e < b.e; });
   const int l0 = rows[0].e;
-  const size_t Rs = static_cast<size_t>(R);
-  const int rank = c.ad->dims.rank;
-  float* x = reinterpret_cast<float*>(c.ws + p.off_dec);
-  float* xn = x + Rs * D.h;
-  float* x1 = xn + Rs * D.h;
-  float* q = x1 + Rs * D.h;
-  float* k = q + Rs * D.qd;
-  float* v = k + Rs * D.kvd;
-  float* o = v + Rs * D.kvd;
-  float* xa = o + Rs * D.qd;  // one [R, rank] slot per module: q, k, v, o, gate, up, down
-  float* gu = xa + 7 * Rs * kRankPad;
-  float* m = gu + Rs * 2 * D.f;
-  float* npart = m + Rs * D.f;  // [R, slices] partial sums of squares of the norms
-  float* part = npart + Rs * norm_up_slices(D.h);
-  int* ncount = reinterpret_cast<int*>(c.ws + p.off_abort) + 1 + (p.flag_words - kMaxReq);
-  auto xa_of = [&](int mod) { return xa + static_cast<size_t>(mod) * Rs * kRankPad; };
-  auto up_of = [&](int l, int mod) {
+  const int sms = c.ctx->num_sms;
+  const uint32_t mask = c.ad->dims.module_mask;
+  const DecodePasses passes = decode_passes(D, mask, sms);
+  // the scratch was sized for p.dec_rows >= R rows: both use the term count of the rows that run
+  const DecodeScratch ds = decode_scratch(D, mask, R, p.splits, sms);
+  const int terms = rows_terms(R);
+  uint8_t* base = c.ws + p.off_dec;
+  float* x = reinterpret_cast<float*>(base + ds.x);
+  float* nss = reinterpret_cast<float*>(base + ds.nss);
+  auto* xs = reinterpret_cast<__nv_bfloat16*>(base + ds.xs);
+  auto* os = reinterpret_cast<__nv_bfloat16*>(base + ds.os);
+  auto* ms = reinterpret_cast<__nv_bfloat16*>(base + ds.ms);
+  float* y = reinterpret_cast<float*>(base + ds.y);
+  float* part = reinterpret_cast<float*>(base + ds.part);
+  const RowLora lora{c.ad->dims.rank, c.scale};
+  // the up product of module m of layer l, the `i`-th module of a pass whose modules start at `m0`
+  auto up_of = [&](int l, int m, int m0, const RowsPlan& pl, int nseg) {
     RowUp u{};
-    if (adapted(c.ad, mod)) {
-      u.B = static_cast<const __nv_bfloat16*>(c.ad->B[l * 7 + mod]);
-      u.xa = xa_of(mod);
-    }
+    if (!adapted(c.ad, m)) return u;
+    int slot = 0;
+    for (int k = m0; k < m; ++k) slot += adapted(c.ad, k) ? 1 : 0;
+    u.B = static_cast<const __nv_bfloat16*>(c.ad->B[l * 7 + m]);
+    u.xa_col = pl.tile0[nseg] * 128 + 16 * slot;
     return u;
   };
-  // kernels per layer: 2 norms (with the pending up products), 4 GEMV passes per 8 rows, RoPE
-  // (with the q|k|v up products), 2 attention, SwiGLU (with the gate|up up products), the K/V
-  // write of a generation step; then the last layer's down up product and a conversion per row
-  int launches = 0;
-  for (const auto& r : rows) launches += (r.start ? 1 : 0) + (r.out ? 1 : 0);
-  bool any_token = false;
-  for (const auto& r : rows) any_token |= r.token != nullptr;
-  launches += any_token ? 1 : 0;
-  for (int l = l0; l < D.N; ++l) {
-    int nr = 0;
-    for (const auto& r : rows) nr += r.e <= l;
-    launches += 6 + (opt.write_kv ? 1 : 0) + 4 * ((nr + 7) / 8);
-  }
-  if (l0 < D.N && adapted(c.ad, CRF_MOD_DOWN)) ++launches;
-  ProfScope ps(c.ctx, kPDecode, c.st, launches);
-  TokenRows tr{};
-  for (int i = 0; i < R; ++i) {
-    if (rows[i].token) {
-      tr.token[i] = rows[i].token;
-    } else {
-      CRF_CUDA(launch_bf16_to_f32(rows[i].start, x + i * static_cast<size_t>(D.h), D.h, c.st));
+  auto part_of = [&](const RowsPlan& pl, int nr) { return RowPart{y, pl.splits, nr, pl.ncols}; };
+  // one weight pass over modules [m0, m0 + nm) of layer l and their LoRA A rows (Eq. S3)
+  auto pass = [&](int l, int nr, int m0, int nm, const RowsPlan& pl, const __nv_bfloat16* in, int in_dim,
+                  bool normed) -> cudaError_t {
+    RowsGemmDesc g{};
+    g.nseg = nm;
+    for (int s = 0; s < nm; ++s) {
+      const int m = m0 + s;
+      g.W[s] = static_cast<const __nv_bfloat16*>(c.model->layers[l].W[m]);
+      g.out[s] = module_rows(D, m);
+      if (adapted(c.ad, m)) g.LA[g.n_lora++] = static_cast<const __nv_bfloat16*>(c.ad->A[l * 7 + m]);
     }
-  }
-  if (any_token) {
-    // token rows are the whole batch (a generation step), so one launch covers them
-    for (int i = 0; i < R; ++i)
-      if (!rows[i].token) return fail(CRF_EINVAL, "decode rows mix token and hidden starts");
-    CRF_CUDA(launch_embed_rows_f32(static_cast<const __nv_bfloat16*>(c.model->embed), tr, R, x, D.h, D.V,
-                                   c.ctx->status_dev, c.st));
-  }
-  // one weight pass per group of up to 8 rows: the modules' base rows (y = W in + bias + resid)
-  // and, as segments of their own, their LoRA A rows (xa = (alpha/r) A in, Eq. S3)
-  auto proj = [&](int l, int nr, const int* mods, int nm, const float* in, int in_dim, float* const* ys,
-                  const int* outs, const float* resid, int resid_ld) -> cudaError_t {
-    for (int r0 = 0; r0 < nr; r0 += 8) {
-      GemvDesc g{};
-      g.abort = c.abort;
-      g.in_dim = in_dim;
-      g.x = in + static_cast<size_t>(r0) * in_dim;
-      g.rows = std::min(8, nr - r0);
-      for (int s = 0; s < nm; ++s) {
-        const int mod = mods[s];
-        GemvSeg& sg = g.seg[g.nseg++];
-        sg.W = static_cast<const __nv_bfloat16*>(c.model->layers[l].W[mod]);
-        sg.out_dim = outs[s];
-        sg.scale = 1.f;
-        sg.bias = (mod < 3 && D.bias) ? static_cast<const __nv_bfloat16*>(c.model->layers[l].bias[mod])
-                                      : nullptr;
-        sg.y = ys[s] + static_cast<size_t>(r0) * outs[s];
-        sg.resid = resid ? resid + static_cast<size_t>(r0) * resid_ld : nullptr;
-      }
-      for (int s = 0; s < nm; ++s) {
-        const int mod = mods[s];
-        if (!adapted(c.ad, mod)) continue;
-        GemvSeg& sg = g.seg[g.nseg++];
-        sg.W = static_cast<const __nv_bfloat16*>(c.ad->A[l * 7 + mod]);
-        sg.out_dim = rank;
-        sg.scale = c.scale;
-        sg.y = xa_of(mod) + static_cast<size_t>(r0) * rank;
-      }
-      cudaError_t e = launch_gemv(g, c.ctx->num_sms, c.st, nr);
-      if (e != cudaSuccess) return e;
+    g.rank = lora.rank;
+    g.in_dim = in_dim;
+    g.x = in;
+    g.rows = nr;
+    g.terms = terms;
+    g.y = y;
+    if (normed) {
+      g.nss = nss;
+      g.slices = norm_slices(in_dim);
+      g.eps = D.eps;
     }
-    return cudaSuccess;
+    g.status = c.ctx->status_dev;
+    g.abort = c.abort;
+    return launch_rows_gemm(g, pl, sms, c.st);
   };
-  const int m_qkv[3] = {CRF_MOD_Q, CRF_MOD_K, CRF_MOD_V};
-  const int o_qkv[3] = {D.qd, D.kvd, D.kvd};
-  float* const y_qkv[3] = {q, k, v};
-  const int m_o[1] = {CRF_MOD_O}, o_o[1] = {D.h};
-  float* const y_o[1] = {x1};
-  const int m_gu[2] = {CRF_MOD_GATE, CRF_MOD_UP}, o_gu[2] = {D.f, D.f};
-  float* const y_gu[2] = {gu, gu + Rs * D.f};
-  const int m_d[1] = {CRF_MOD_DOWN}, o_d[1] = {D.h};
-  float* const y_d[1] = {x};
-  RowPositions rp{};
-  for (int i = 0; i < R; ++i) rp.pos[i] = rows[i].pos;
-  int nr_prev = 0;  // rows that carry the previous layer's pending down up product
-  {
-    // the layer loop is a chain of short kernels only: each may become resident and prefetch its
-    // weights while the one before it finishes
-    PdlScope pdl;
-    for (int l = l0; l < D.N; ++l) {
-      int nr = 0;
-      while (nr < R && rows[nr].e <= l) ++nr;
-      const crf_layer_weights& w = c.model->layers[l];
-      // x += the previous layer's down up product (rows active there), xn = RMSNorm(x)
-      CRF_CUDA(launch_norm_up_rows(x, D.h, nr, l > l0 ? up_of(l - 1, CRF_MOD_DOWN) : RowUp{}, nr_prev, rank,
-                                   static_cast<const __nv_bfloat16*>(w.ln1), D.eps, xn, npart, ncount, c.st));
-      CRF_CUDA(proj(l, nr, m_qkv, 3, xn, D.h, y_qkv, o_qkv, nullptr, 0));
-      const RowUp up_qkv[3] = {up_of(l, CRF_MOD_Q), up_of(l, CRF_MOD_K), up_of(l, CRF_MOD_V)};
-      CRF_CUDA(launch_rope_up_rows(q, D.hq, k, D.hkv, v, nr, D.d, up_qkv, rank,
-                                   opt.rope_by_row ? opt.rope_by_row
-                                                   : reinterpret_cast<const float2*>(c.ws + p.off_rope),
-                                   rp, opt.rope_by_row != nullptr, c.st));
-      DecodeAttnDesc a;
-      std::memset(&a, 0, sizeof(a));
-      a.q = q;
-      a.k_self = k;
-      a.v_self = v;
-      a.kpages = static_cast<const __nv_bfloat16*>(c.pool->k_pages[l]);
-      a.vpages = static_cast<const __nv_bfloat16*>(c.pool->v_pages[l]);
-      for (int i = 0; i < nr; ++i) {
-        a.page_table[i] = rows[i].page_table;
-        a.pos[i] = rows[i].pos;
-      }
-      a.out = o;
-      a.part = part;
-      a.rows = nr;
-      a.n_q_heads = D.hq;
-      a.n_kv_heads = D.hkv;
-      a.head_dim = D.d;
-      a.splits = p.splits;
-      a.abort = c.abort;
-      CRF_CUDA(launch_decode_attention(a, c.pool->num_pages, c.ctx->num_sms, c.ctx->status_dev, c.st));
-      if (opt.write_kv) {
-        RowPages pg{};
-        for (int i = 0; i < nr; ++i) {
-          pg.page_table[i] = rows[i].page_table;
-          pg.pos[i] = rows[i].pos;
-        }
-        pg.num_pages = c.pool->num_pages;
-        CRF_CUDA(launch_kv_write_rows(k, v, c.pool->k_pages[l], c.pool->v_pages[l], pg, nr, D.hkv, D.d,
-                                      c.ctx->status_dev, c.abort, c.st));
-      }
-      // x1 = x + o W_o^T, then x1 += the o up product and xn = RMSNorm(x1)
-      CRF_CUDA(proj(l, nr, m_o, 1, o, D.qd, y_o, o_o, x, D.h));
-      CRF_CUDA(launch_norm_up_rows(x1, D.h, nr, up_of(l, CRF_MOD_O), nr, rank,
-                                   static_cast<const __nv_bfloat16*>(w.ln2), D.eps, xn, npart, ncount, c.st));
-      CRF_CUDA(proj(l, nr, m_gu, 2, xn, D.h, y_gu, o_gu, nullptr, 0));
-      // gate rows then up rows: SwiGLU over [nr, f] with the up half Rs * f further on
-      CRF_CUDA(launch_swiglu_up_rows(gu, gu + Rs * D.f, m, nr, D.f, up_of(l, CRF_MOD_GATE), up_of(l, CRF_MOD_UP),
-                                     rank, c.st));
-      // x = x1 + m W_d^T; its up product is added by the next layer's norm (or below)
-      CRF_CUDA(proj(l, nr, m_d, 1, m, D.f, y_d, o_d, x1, D.h));
-      nr_prev = nr;
+  // kernels per layer: 2 norms, 4 weight passes, 2 attention, SwiGLU; then the rows' way out
+  ProfScope ps(c.ctx, kPDecode, c.st, 9 * (D.N - l0) + 1);
+  int nr_prev = 0;  // rows that carry the previous layer's pending down product
+  // a chain of short kernels only: each may become resident, and a weight pass request its first
+  // weights, while the ones before it finish
+  PdlScope pdl;
+  for (int l = l0; l < D.N; ++l) {
+    int nr = nr_prev;
+    RowStart start{};
+    start.embed = static_cast<const __nv_bfloat16*>(c.model->embed);
+    start.vocab = D.V;
+    for (; nr < R && rows[nr].e <= l; ++nr) {
+      start.row[nr] = rows[nr].start;
+      start.token[nr] = rows[nr].token;
     }
-    if (l0 < D.N) CRF_CUDA(launch_rows_up(x, D.h, nr_prev, up_of(D.N - 1, CRF_MOD_DOWN), rank, c.st));
+    const crf_layer_weights& w = c.model->layers[l];
+    CRF_CUDA(launch_add_norm_rows(x, D.h, nr, part_of(passes.down, nr_prev),
+                                  l > l0 ? up_of(l - 1, CRF_MOD_DOWN, CRF_MOD_DOWN, passes.down, 1) : RowUp{}, lora,
+                                  nr_prev, nr > nr_prev ? &start : nullptr, static_cast<const __nv_bfloat16*>(w.ln1), xs,
+                                  terms, nss, c.ctx->status_dev, c.st));
+    CRF_CUDA(pass(l, nr, CRF_MOD_Q, 3, passes.qkv, xs, D.h, true));
+    DecodeAttnDesc a;
+    std::memset(&a, 0, sizeof(a));
+    a.qkv = part_of(passes.qkv, nr);
+    for (int m = 0; m < 3; ++m) {
+      a.col[m] = passes.qkv.tile0[m] * 128;
+      a.up[m] = up_of(l, m, CRF_MOD_Q, passes.qkv, 3);
+      a.bias[m] = D.bias ? static_cast<const __nv_bfloat16*>(w.bias[m]) : nullptr;
+    }
+    a.lora = lora;
+    a.rope = opt.rope_by_row ? opt.rope_by_row : reinterpret_cast<const float2*>(c.ws + p.off_rope);
+    a.rope_by_row = opt.rope_by_row != nullptr;
+    a.kpages = static_cast<__nv_bfloat16*>(c.pool->k_pages[l]);
+    a.vpages = static_cast<__nv_bfloat16*>(c.pool->v_pages[l]);
+    a.write_kv = opt.write_kv;
+    for (int i = 0; i < nr; ++i) {
+      a.page_table[i] = rows[i].page_table;
+      a.pos[i] = rows[i].pos;
+    }
+    a.out = os;
+    a.terms = terms;
+    a.part = part;
+    a.rows = nr;
+    a.n_q_heads = D.hq;
+    a.n_kv_heads = D.hkv;
+    a.head_dim = D.d;
+    a.splits = p.splits;
+    a.abort = c.abort;
+    CRF_CUDA(launch_decode_attention(a, c.pool->num_pages, sms, c.ctx->status_dev, c.st));
+    CRF_CUDA(pass(l, nr, CRF_MOD_O, 1, passes.o, os, D.qd, false));
+    CRF_CUDA(launch_add_norm_rows(x, D.h, nr, part_of(passes.o, nr), up_of(l, CRF_MOD_O, CRF_MOD_O, passes.o, 1), lora, nr,
+                                  nullptr, static_cast<const __nv_bfloat16*>(w.ln2), xs, terms, nss, c.ctx->status_dev,
+                                  c.st));
+    CRF_CUDA(pass(l, nr, CRF_MOD_GATE, 2, passes.gu, xs, D.h, true));
+    CRF_CUDA(launch_swiglu_rows(part_of(passes.gu, nr), passes.gu.tile0[1] * 128, D.f,
+                                up_of(l, CRF_MOD_GATE, CRF_MOD_GATE, passes.gu, 2),
+                                up_of(l, CRF_MOD_UP, CRF_MOD_GATE, passes.gu, 2), lora, ms, terms, c.st));
+    CRF_CUDA(pass(l, nr, CRF_MOD_DOWN, 1, passes.down, ms, D.f, false));
+    nr_prev = nr;
   }
-  for (int i = 0; i < R; ++i)
-    if (rows[i].out)
-      CRF_CUDA(launch_f32_to_bf16(x + i * static_cast<size_t>(D.h),
-                                  static_cast<__nv_bfloat16*>(rows[i].out), D.h, c.st, c.abort));
+  const RowPart last = part_of(passes.down, R);
+  const RowUp up = up_of(D.N - 1, CRF_MOD_DOWN, CRF_MOD_DOWN, passes.down, 1);
+  if (opt.final_norm) {
+    CRF_CUDA(launch_add_norm_rows(x, D.h, R, last, up, lora, R, nullptr, opt.final_norm, xs, terms, nss,
+                                  c.ctx->status_dev, c.st));
+  } else {
+    RowOuts outs{};
+    for (int i = 0; i < R; ++i) outs.out[i] = static_cast<__nv_bfloat16*>(rows[i].out);
+    CRF_CUDA(launch_finish_rows(x, D.h, R, last, up, lora, outs, c.abort, c.st));
+  }
   return CRF_OK;
 }
 
@@ -762,33 +763,29 @@ crf_status validate_requests(const crf_ctx* ctx, const crf_model* model, const c
   return CRF_OK;
 }
 
-// Workspace of one generation step: the decode-row scratch, the rows' RoPE angles, the final
-// normalised rows and (when the caller passes no buffer) the logits.
+// Workspace of one generation step: the decode-row scratch, the rows' RoPE angles and (when the
+// caller passes no buffer) the logits.
 struct StepPlan {
   Plan p;
-  size_t off_angles, off_norm, off_logits, total;
+  size_t off_angles, off_logits, total;
 };  // p.off_abort / p.off_ptab / p.ptab_slots: the page check of the rows' tables
 
-StepPlan make_step_plan(const Dims& D, const crf_decode_row* rows, int n) {
+StepPlan make_step_plan(const Dims& D, const crf_decode_row* rows, int n, uint32_t mask, int num_sms) {
   StepPlan sp;
   Plan& p = sp.p;
   p.dec_rows = n;
   p.max_n = 1;
   for (int i = 0; i < n; ++i) p.max_n = std::max(p.max_n, rows[i].pos + 1);
   p.splits = dec_splits(p.max_n);
-  const size_t dec_row = static_cast<size_t>(3 * D.h + 2 * D.qd + 2 * D.kvd + 7 * kRankPad + 3 * D.f + norm_up_slices(D.h)) * 4 +
-                         static_cast<size_t>(D.hq) * p.splits * (D.d + 2) * 4;
-  p.dec_bytes = align256(dec_row * std::max(1, n));
   size_t o = 0;
   auto take = [&](size_t bytes) {
     const size_t at = o;
     o = align256(o + bytes);
     return at;
   };
-  p.off_dec = take(p.dec_bytes);
+  p.off_dec = take(decode_scratch(D, mask, n, p.splits, num_sms).total);
   p.off_rope = 0;
   sp.off_angles = take(static_cast<size_t>(n) * (D.d / 2) * sizeof(float2));
-  sp.off_norm = take(static_cast<size_t>(n) * D.h * 4);
   sp.off_logits = take(static_cast<size_t>(n) * D.V * 4);
   long ids = 0;
   for (int i = 0; i < n; ++i) ids += rows[i].pos / kPage + 1;
@@ -895,7 +892,7 @@ crf_status crf_workspace_size(crf_ctx* ctx, const crf_model* model, const crf_lo
   for (int i = 0; i < n_req; ++i)
     if (reqs[i].n_tokens < 1 || reqs[i].s < 0 || reqs[i].s > reqs[i].e || reqs[i].e > D.N)
       return fail(CRF_EINVAL, "request %d malformed", i);
-  *bytes = make_plan(D, reqs, n_req).total;
+  *bytes = make_plan(D, reqs, n_req, lora->module_mask, ctx->num_sms).total;
   return CRF_OK;
 }
 
@@ -914,7 +911,7 @@ crf_status crf_recompute_window(crf_ctx* ctx, const crf_model* model, const crf_
   const Dims D = dims_of(model->dims);
   s = validate_requests(ctx, model, cur, pool, reqs, n_req, D);
   if (s != CRF_OK) return s;
-  const Plan plan = make_plan(D, reqs, n_req);
+  const Plan plan = make_plan(D, reqs, n_req, cur->dims.module_mask, ctx->num_sms);
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255))
     return fail(CRF_EINVAL, "workspace null or not 256-byte aligned");
   if (ws_bytes < plan.total)
@@ -1091,7 +1088,7 @@ crf_status crf_decode_workspace_size(crf_ctx* ctx, const crf_model* model, const
   if (n_rows < 1 || n_rows > CRF_MAX_REQUESTS) return fail(CRF_EINVAL, "n_rows out of range");
   for (int i = 0; i < n_rows; ++i)
     if (rows[i].pos < 0) return fail(CRF_EINVAL, "row %d: negative position", i);
-  *bytes = make_step_plan(dims_of(model->dims), rows, n_rows).total;
+  *bytes = make_step_plan(dims_of(model->dims), rows, n_rows, lora->module_mask, ctx->num_sms).total;
   return CRF_OK;
 }
 
@@ -1121,7 +1118,7 @@ crf_status crf_decode_step(crf_ctx* ctx, const crf_model* model, const crf_adapt
       return fail(CRF_EINVAL, "kv pool layer %d null or misaligned", l);
   s = validate_decode_rows(pool, rows, n_rows);
   if (s != CRF_OK) return s;
-  const StepPlan sp = make_step_plan(D, rows, n_rows);
+  const StepPlan sp = make_step_plan(D, rows, n_rows, cur->dims.module_mask, ctx->num_sms);
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255))
     return fail(CRF_EINVAL, "workspace null or not 256-byte aligned");
   if (ws_bytes < sp.total) return fail(CRF_ENOMEM, "workspace %zu bytes, %zu needed", ws_bytes, sp.total);
@@ -1169,17 +1166,19 @@ crf_status crf_decode_step(crf_ctx* ctx, const crf_model* model, const crf_adapt
   DecodeOpts opt;
   opt.write_kv = true;
   opt.rope_by_row = angles;
+  opt.final_norm = static_cast<const __nv_bfloat16*>(model->final_norm);
   s = decode_rows(c, dec, opt);
   if (s != CRF_OK) return s;
-  // final norm, LM head, greedy token: the fp32 rows are the head of the decode scratch
-  float* x = reinterpret_cast<float*>(ws + sp.p.off_dec);
-  float* hn = reinterpret_cast<float*>(ws + sp.off_norm);
+  // LM head over the final rows' terms, greedy token
+  const DecodeScratch ds = decode_scratch(D, cur->dims.module_mask, n_rows, sp.p.splits, ctx->num_sms);
+  const uint8_t* base = ws + sp.p.off_dec;
   float* z = logits ? logits : reinterpret_cast<float*>(ws + sp.off_logits);
   {
-    ProfScope ps(ctx, kPLmHead, st, 3);
-    CRF_CUDA(launch_rmsnorm_f32(x, static_cast<const __nv_bfloat16*>(model->final_norm), hn, n_rows, D.h, D.eps, st));
-    CRF_CUDA(launch_lm_head(static_cast<const __nv_bfloat16*>(model->lm_head), hn, n_rows, D.V, D.h, z,
-                            ctx->num_sms, st, c.abort));
+    ProfScope ps(ctx, kPLmHead, st, 2);
+    CRF_CUDA(launch_lm_head(static_cast<const __nv_bfloat16*>(model->lm_head),
+                            reinterpret_cast<const __nv_bfloat16*>(base + ds.xs), rows_terms(n_rows),
+                            reinterpret_cast<const float*>(base + ds.nss), n_rows, D.V, D.h, D.eps, z, ctx->num_sms,
+                            ctx->status_dev, st, c.abort));
     CRF_CUDA(launch_argmax_rows(z, n_rows, D.V, next_tokens, st, c.abort));
   }
   return CRF_OK;
@@ -1259,7 +1258,8 @@ crf_status crf_kl_workspace_size(crf_ctx* ctx, int n_rows, int vocab, int hidden
   const int sp = kl_splits(ctx, n_rows, vocab);
   size_t o = align256(static_cast<size_t>(n_rows) * sp * 5 * sizeof(float));
   if (hidden > 0) {
-    o += align256(static_cast<size_t>(2 * n_rows) * hidden * sizeof(float)) * 2;
+    o += align256(static_cast<size_t>(2 * n_rows) * rows_terms(2 * n_rows) * hidden * 2);
+    o += align256(static_cast<size_t>(2 * n_rows) * norm_slices(hidden) * sizeof(float));
     o += align256(static_cast<size_t>(2 * n_rows) * vocab * sizeof(float));
   }
   *bytes = o;
@@ -1291,19 +1291,17 @@ crf_status crf_kl(crf_ctx* ctx, const crf_model* model, const void* ref, const v
   const float* zr = static_cast<const float*>(ref);
   const float* zc = static_cast<const float*>(cur);
   if (model) {
-    float* hf = reinterpret_cast<float*>(ws + o);
-    o += align256(static_cast<size_t>(2 * n_rows) * hidden * sizeof(float));
-    float* hn = reinterpret_cast<float*>(ws + o);
-    o += align256(static_cast<size_t>(2 * n_rows) * hidden * sizeof(float));
+    const int terms = rows_terms(2 * n_rows);
+    auto* xs = reinterpret_cast<__nv_bfloat16*>(ws + o);
+    o += align256(static_cast<size_t>(2 * n_rows) * terms * hidden * 2);
+    float* nss = reinterpret_cast<float*>(ws + o);
+    o += align256(static_cast<size_t>(2 * n_rows) * norm_slices(hidden) * sizeof(float));
     float* logits = logits_out ? logits_out : reinterpret_cast<float*>(ws + o);
-    ProfScope ps(ctx, kPLmHead, st, 4);
-    CRF_CUDA(launch_bf16_to_f32(static_cast<const __nv_bfloat16*>(ref), hf, n_rows * hidden, st));
-    CRF_CUDA(launch_bf16_to_f32(static_cast<const __nv_bfloat16*>(cur), hf + static_cast<size_t>(n_rows) * hidden,
-                                n_rows * hidden, st));
-    CRF_CUDA(launch_rmsnorm_f32(hf, static_cast<const __nv_bfloat16*>(model->final_norm), hn, 2 * n_rows,
-                                hidden, model->dims.rms_eps, st));
-    CRF_CUDA(launch_lm_head(static_cast<const __nv_bfloat16*>(model->lm_head), hn, 2 * n_rows, vocab,
-                            hidden, logits, ctx->num_sms, st));
+    ProfScope ps(ctx, kPLmHead, st, 1 + (2 * n_rows + kRowsMax - 1) / kRowsMax);
+    CRF_CUDA(launch_head_rows(static_cast<const __nv_bfloat16*>(ref), static_cast<const __nv_bfloat16*>(cur), n_rows,
+                              hidden, static_cast<const __nv_bfloat16*>(model->final_norm), xs, terms, nss, st));
+    CRF_CUDA(launch_lm_head(static_cast<const __nv_bfloat16*>(model->lm_head), xs, terms, nss, 2 * n_rows, vocab, hidden,
+                            model->dims.rms_eps, logits, ctx->num_sms, ctx->status_dev, st));
     zr = logits;
     zc = logits + static_cast<size_t>(n_rows) * vocab;
   }

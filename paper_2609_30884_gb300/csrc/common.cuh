@@ -145,24 +145,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 // while the kernel before it in the stream is still running. griddep_wait() returns once that
 // kernel has completed and its writes are visible (at once for a kernel launched without the
 // attribute), so a kernel touches nothing that an earlier kernel of the stream may write before
-// it: only weights, which no kernel writes. griddep_launch_dependents() then lets the next kernel
-// of the stream start its own prologue; issuing it after the wait keeps at most one kernel ahead.
+// it: only weights, which no kernel writes. griddep_launch_dependents() lets the next kernel of the
+// stream become resident; every kernel of a chain issues it first and waits before it ends, so a
+// kernel's wait covers every kernel before it however far the chain runs ahead.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-__device__ __forceinline__ void griddep_begin() {
-  griddep_wait();
-  griddep_launch_dependents();
-}
-
-// Ask L2 for bytes [p, p + n), n < 4 GB (128-byte lines; the block's threads share the lines in turn).
-static __device__ __noinline__ void prefetch_l2_range(const void* p, size_t n) {
-  const char* c = static_cast<const char*>(p);
-  const uint32_t lines = static_cast<uint32_t>((n + 127) / 128);
-#pragma unroll 1
-  for (uint32_t i = threadIdx.x; i < lines; i += blockDim.x)
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(c + static_cast<size_t>(i) * 128));
 }
 
 // ---------------------------------------------------------------- clusters
@@ -351,6 +339,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
         "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
         "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+}
+// Each thread of the warp reads 16 consecutive fp32 columns of its TMEM lane.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32"
+      " {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_ld_wait() {

@@ -6,7 +6,11 @@
 //   row's own fresh (k, v) at position pos.
 // The work is memory-bound (K and V of every cached position are read once): the positions
 // are cut into chunks of 128 and streamed.
-//   decode_attn_stream  one block per SM, walking a run of consecutive chunks of one (row,
+//   decode_attn_stream  finishes q (and, where the row's own position falls, k and v) from the
+//                       q|k|v pass's partial sums: K splits, bias, up products, rotate-half RoPE, the
+//                       row's K/V into its page slot in a generation step; a block needs only its
+//                       group's heads, so this costs it less than a kernel of its own would. Then
+//                       one block per SM, walking a run of consecutive chunks of one (row,
 //                       kv head) through a two- or three-stage ring: a copy warp gathers the next
 //                       chunk's K and V pages with TMA (128-byte swizzle) while four compute
 //                       warps score the current one. The group's query heads (padded to 16 rows)
@@ -20,9 +24,9 @@
 //                       The chunks per block are the fewest that keep all blocks in one wave;
 //   decode_attn_merge   one block per (query head, row, 32-column slice): rescales the blocks'
 //                       partials to the common max and normalises, every partial's loads
-//                       independent of the others.
-#include "common.cuh"
-#include "kernels.h"
+//                       independent of the others; o leaves as the o pass's bf16 terms.
+#include "rows.cuh"
+#include "tma_map.h"
 
 #include <algorithm>
 #include <cfloat>
@@ -71,9 +75,9 @@ __global__ void __launch_bounds__(kThreadsStream) decode_attn_stream(const __gri
   constexpr int HALF = kChunk * 128;     // bytes of one 64-column half of a K (or V) tile
   constexpr int TILE = HALVES * HALF;
   constexpr int QHALF = 16 * 128;        // one 64-column half of the 16-row Q tile
+  constexpr int HALF_D = D / 2;
   const DecodeAttnDesc& p = a.d;
-  griddep_begin();  // q, k, v of the rows come from the kernel before
-  if (call_aborted(p.abort)) return;
+  griddep_launch_dependents();
   // block -> (row, kv head, its chunks c_beg .. c_end - 1, partial slot)
   int r = -1, g = 0, slot = 0, c_beg = 0, c_end = 0;
   {
@@ -105,6 +109,8 @@ __global__ void __launch_bounds__(kThreadsStream) decode_attn_stream(const __gri
   uint8_t* sQl = sQ + HALVES * QHALF;                       // lo, same layout
   __shared__ float red_m[4][16], red_l[4][16];
   __shared__ float s_self[16];  // the row's own key, scored in fp32
+  __shared__ float s_xa[3][kRankPad];           // the row's scaled down products of q, k, v
+  __shared__ float s_q[kMaxGroup][D], s_k[D], s_v[D];  // finished q (log2 units), own k and v
   __shared__ __align__(8) uint64_t full[kStages], empty[kStages];
   __shared__ volatile int abort_flag;
 
@@ -121,7 +127,8 @@ __global__ void __launch_bounds__(kThreadsStream) decode_attn_stream(const __gri
 
   if (warp == 4) {
     // ---------------------------------------------------------------- producer
-    if (lane == 0) {
+    griddep_wait();  // the page-table check has passed judgement
+    if (lane == 0 && !call_aborted(p.abort)) {
       const int32_t* pt = p.page_table[r];
       int armed[kStages];
       for (int st = 0; st < kStages; ++st) armed[st] = -1;
@@ -158,16 +165,49 @@ __global__ void __launch_bounds__(kThreadsStream) decode_attn_stream(const __gri
   }
 
   // -------------------------------------------------------------------- compute warps 0..3
-  // q of the group's heads (rows >= grp zero) as bf16 hi + lo, pre-scaled so scores are in
-  // log2 units
+  griddep_wait();  // the q|k|v pass's output
+  if (call_aborted(p.abort)) return;
+  // q pre-scaled so scores are in log2 units
   const float qscale = 1.4426950408889634f * rsqrtf(static_cast<float>(D));
-  const float* qrow0 = p.q + (size_t)r * p.n_q_heads * D + (size_t)(g * grp) * D;
+  if (tid < 3 * kRankPad) {
+    const int m = tid / kRankPad, k = tid % kRankPad;
+    float v = 0.f;
+    if ((m == 0 || self_here) && p.up[m].B && k < p.lora.rank)
+      v = part_sum(p.qkv, r, p.up[m].xa_col + k) * p.lora.scale;
+    s_xa[m][k] = v;
+  }
+  named_bar_sync_dec(1, 128);
+  const float2* angles = p.rope + static_cast<size_t>(p.rope_by_row ? r : pos) * HALF_D;
+  auto element = [&](int m, int j) {  // projection m's output j of the row
+    float v = part_sum(p.qkv, r, p.col[m] + j);
+    if (p.bias[m]) v += __bfloat162float(p.bias[m][j]);
+    if (p.up[m].B) v += up_dot(up_row(p.up[m].B, j, p.lora.rank), s_xa[m]);
+    return v;
+  };
+  // rotation pairs of the group's q heads, then of the own k
+  const int n_pairs = (grp + (self_here ? 1 : 0)) * HALF_D;
+  for (int i = tid; i < n_pairs; i += 128) {
+    const int h = i / HALF_D, e = i % HALF_D;
+    const int m = h < grp ? 0 : 1;
+    const int j = (m == 0 ? g * grp + h : g) * D + e;
+    const float x1 = element(m, j), x2 = element(m, j + HALF_D);
+    const float2 cs = angles[e];
+    const float y1 = x1 * cs.x - x2 * cs.y, y2 = x2 * cs.x + x1 * cs.y;
+    float* dst = m == 0 ? s_q[h] : s_k;
+    const float f = m == 0 ? qscale : 1.f;
+    dst[e] = y1 * f;
+    dst[e + HALF_D] = y2 * f;
+  }
+  if (self_here)
+    for (int e = tid; e < D; e += 128) s_v[e] = element(2, g * D + e);
+  named_bar_sync_dec(1, 128);
+  // the MMA operand: q of the group's heads (rows >= grp zero) as bf16 hi + lo
   for (int i = tid; i < 16 * (D / 2); i += 128) {
     const int row = i / (D / 2), d = 2 * (i % (D / 2));
     float v0 = 0.f, v1 = 0.f;
     if (row < grp) {
-      v0 = qrow0[(size_t)row * D + d] * qscale;
-      v1 = qrow0[(size_t)row * D + d + 1] * qscale;
+      v0 = s_q[row][d];
+      v1 = s_q[row][d + 1];
     }
     const float h0 = __bfloat162float(__float2bfloat16_rn(v0));
     const float h1 = __bfloat162float(__float2bfloat16_rn(v1));
@@ -178,12 +218,20 @@ __global__ void __launch_bounds__(kThreadsStream) decode_attn_stream(const __gri
   }
   if (self_here) {
     // the row's own key, scored in fp32 (warp w takes heads w, w + 4)
-    const float* ks = p.k_self + (size_t)r * p.n_kv_heads * D + g * D;
     for (int h = warp; h < grp; h += 4) {
       float dot = 0.f;
-      for (int d = lane; d < D; d += 32) dot += qrow0[(size_t)h * D + d] * ks[d];
+      for (int d = lane; d < D; d += 32) dot += s_q[h][d] * s_k[d];
       dot = warp_sum(dot);
-      if (lane == 0) s_self[h] = dot * qscale;
+      if (lane == 0) s_self[h] = dot;
+    }
+    if (p.write_kv) {
+      // this layer's copies may read the slot meanwhile: its score is masked and its V row zeroed
+      const int page = checked_page(p.page_table[r][pos / kPage], a.num_pages, tid == 0 ? a.status : nullptr);
+      const size_t dst = ((static_cast<size_t>(page) * p.n_kv_heads + g) * kPage + pos % kPage) * D;
+      for (int e = tid; e < D; e += 128) {
+        p.kpages[dst + e] = __float2bfloat16_rn(s_k[e]);
+        p.vpages[dst + e] = __float2bfloat16_rn(s_v[e]);
+      }
     }
   }
   named_bar_sync_dec(1, 128);
@@ -366,7 +414,6 @@ __global__ void __launch_bounds__(kThreadsStream) decode_attn_stream(const __gri
     named_bar_sync_dec(1, 128);
   }
   if (!ok) return;
-  const float* vs = p.v_self + (size_t)r * p.n_kv_heads * D + g * D;
   for (int q = tid; q < grp * D; q += 128) {
     const int h = q / D, d = q % D;
     float M = red_m[0][h];
@@ -378,7 +425,7 @@ __global__ void __launch_bounds__(kThreadsStream) decode_attn_stream(const __gri
       ps = ex2_approx(s_self[h] - M);
     }
     float* out = p.part + (((size_t)r * p.n_q_heads + g * grp + h) * p.splits + slot) * (D + 2);
-    out[d] = o_red[h][d] + ps * vs[d];
+    out[d] = o_red[h][d] + (self_here ? ps * s_v[d] : 0.f);
     if (d == 0) {
       float L = ps;
 #pragma unroll
@@ -393,8 +440,9 @@ __global__ void __launch_bounds__(kThreadsStream) decode_attn_stream(const __gri
 // (each chunk's loads independent of the others), lane = one output column; the warps'
 // sums meet in a fixed order.
 template <int D>
-__global__ void __launch_bounds__(128) decode_attn_merge(const DecodeAttnDesc p) {
-  griddep_begin();  // the partials come from decode_attn_stream
+__global__ void __launch_bounds__(128) decode_attn_merge(const __grid_constant__ DecodeAttnDesc p) {
+  griddep_launch_dependents();
+  griddep_wait();  // the partials come from decode_attn_stream
   const int h = blockIdx.x, r = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int col = blockIdx.z * 32 + lane;
   const int n_chunks = (p.pos[r] / kChunk + p.chunks_per_block) / p.chunks_per_block;  // partials
@@ -420,38 +468,13 @@ __global__ void __launch_bounds__(128) decode_attn_merge(const DecodeAttnDesc p)
   if (warp == 0) {
     const float o = (red_o[0][lane] + red_o[1][lane]) + (red_o[2][lane] + red_o[3][lane]);
     const float L = (red_l[0] + red_l[1]) + (red_l[2] + red_l[3]);
-    p.out[(size_t)r * p.n_q_heads * D + h * D + col] = o / L;
+    const int qd = p.n_q_heads * D;
+    __nv_bfloat16* dst = p.out + static_cast<size_t>(r) * p.terms * qd + h * D + col;
+    if (p.terms == 2)
+      store_terms<2>(dst, qd, o / L);
+    else
+      store_terms<3>(dst, qd, o / L);
   }
-}
-
-using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn_dec() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* ptr = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000, cudaEnableDefault,
-                                         &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(ptr);
-  }
-  return fn;
-}
-
-bool pool_map(CUtensorMap* m, const void* base, long rows, int cols) {
-  EncodeTiledFn fn = encode_fn_dec();
-  if (!fn) return false;
-  cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
-  cuuint64_t strides[1] = {static_cast<cuuint64_t>(cols) * 2};
-  cuuint32_t box[2] = {64, static_cast<cuuint32_t>(kPage)};
-  cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
-            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <int D, int kStages>
@@ -501,8 +524,9 @@ cudaError_t launch_decode_attention(const DecodeAttnDesc& d, int num_pages, int 
   DecodeArgs a;
   std::memset(&a, 0, sizeof(a));
   const long pool_rows = static_cast<long>(num_pages) * d.n_kv_heads * kPage;
-  if (!pool_map(&a.tmK, d.kpages, pool_rows, d.head_dim)) return cudaErrorInvalidValue;
-  if (!pool_map(&a.tmV, d.vpages, pool_rows, d.head_dim)) return cudaErrorInvalidValue;
+  if (!tensor_map_rows(&a.tmK, d.kpages, pool_rows, d.head_dim, kPage) ||
+      !tensor_map_rows(&a.tmV, d.vpages, pool_rows, d.head_dim, kPage))
+    return cudaErrorInvalidValue;
   a.d = d;
   a.d.chunks_per_block = cpb;
   a.num_pages = num_pages;

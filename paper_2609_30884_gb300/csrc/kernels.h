@@ -172,115 +172,132 @@ struct AttnDesc {
 cudaError_t launch_attention_tc(const AttnDesc& d, int num_pages, int total_rows,
                                 cudaStream_t stream);
 
-// Small-M decode path (the last prefix row through the layers after the window).
-// Up to three row-stacked weight segments share one launch and one input x:
-// y_s[r, j] = sum_i W_s[j, i] x[r, i] (+ bias_s[j]) (+ sum_k BL_s[j, k] xa_s[r, k]) (+ resid_s[r, j])
-// y = scale * (W x) + bias + resid for each segment of weight rows sharing the input rows x: the
-// projections' base rows and, as segments of their own, the LoRA A rows (y = the scaled down
-// product xa, [rows, rank]).
-struct GemvSeg {
-  const __nv_bfloat16* W;  // [out_dim, in_dim]
-  int out_dim;
-  float scale;
-  const __nv_bfloat16* bias;  // [out_dim] or null
-  const float* resid;         // [rows, out_dim] fp32 or null
-  float* y;                   // [rows, out_dim] fp32
+// ------------------------------------------------------------------ decode rows
+// The last prefix row of each request through the layers after its window, and the rows of a
+// generation step: fp32 rows, one weight pass (rows GEMM) for all of them, short kernels between.
+constexpr int kRowsMax = 64;         // rows of one weight pass
+constexpr int kRowsMaxSeg = 3;       // projections that share an input
+constexpr int kRowsMaxSplits = 16;   // K splits of a weight tile
+constexpr int kRowsRing = 76 * 1024;      // shared-memory ring of a pass inside a dependent chain
+constexpr int kRowsRingMax = 200 * 1024;  // and of one alone on its SMs
+// fp32 rows enter a weight pass as bf16 terms: three (exact) for one or two rows, two (about 16
+// mantissa bits) from three rows on. Chosen by the rows of the whole call, so that equal rows in
+// different passes stay equal.
+inline int rows_terms(int total_rows) { return total_rows <= 2 ? 3 : 2; }
+
+// How a weight pass over `nseg` projections is cut: 128-row weight tiles (tile0[s]: first of
+// segment s; tile0[nseg]: the tile of the adapter's A rows, module i at its rows 16 i, if any) and
+// K splits. Its output has `ncols` = 128 x tiles columns: output j of segment s is column
+// 128 tile0[s] + j.
+struct RowsPlan {
+  int tile0[kRowsMaxSeg + 1];
+  int tiles, kb, splits, ncols;
 };
-constexpr int kGemvMaxSeg = 6;
-struct GemvDesc {
-  GemvSeg seg[kGemvMaxSeg];
+RowsPlan rows_plan(int nseg, const int* outs, bool lora, int in_dim, int num_sms, bool split = true);
+struct RowsGemmDesc {
+  const __nv_bfloat16* W[kRowsMaxSeg];  // [out, in_dim]
+  int out[kRowsMaxSeg];
   int nseg;
+  const __nv_bfloat16* LA[kRowsMaxSeg];  // LoRA A rows [rank, in_dim] of the adapted modules
+  int n_lora, rank;
   int in_dim;
-  const float* x;  // [rows, in_dim] fp32
-  int rows;        // 1..8
-  int prefetch;    // set by the launcher: prefetch the block's weight rows into L2 before the wait
-  const int* abort;  // per-call abort word, or null
+  const __nv_bfloat16* x;  // [rows * terms, in_dim]: term t of row r at r * terms + t
+  int rows, terms;
+  float* y;                // [splits][rows][ncols] partial sums
+  int ncols;               // 0: the plan's
+  // when given: row r is scaled by rsqrt(sum_i nss[r][i] / in_dim + eps) (RMSNorm, rows enter as x * g)
+  const float* nss;        // [rows, slices]
+  int slices;
+  float eps;
+  int* status;
+  const int* abort;        // per-call abort word, or null: a rejected call stores nothing
 };
-// Tensor-core GEMV (mma.sync, rows as a bf16 hi/lo pair); launch_gemv uses it when the call's
-// rows (total_rows, the rows of all chunks one caller splits into launches of <= 8; 0 = d.rows)
-// number three or more (one or two rows run faster on the CUDA-core kernel). One kernel per call
-// keeps equal rows equal across chunks.
-cudaError_t launch_gemv(const GemvDesc& d, int num_sms, cudaStream_t stream, int total_rows = 0);
-cudaError_t launch_gemv_tc(const GemvDesc& d, int num_sms, cudaStream_t stream);
+cudaError_t launch_rows_gemm(const RowsGemmDesc& d, const RowsPlan& plan, int num_sms, cudaStream_t stream);
+
+// A weight pass's output as its consumer reads it: element (r, col) is the sum over s of
+// p[(s * rows + r) * ncols + col].
+struct RowPart {
+  const float* p;
+  int splits, rows, ncols;
+};
 // The adapter's up product for decode rows, added where the projection's output is consumed:
-// up[r, j] = sum_k B[j, k] xa[r, k] (B [out_dim, rank] bf16, xa [rows, rank] fp32 already scaled
-// by alpha / r); a null B adds nothing.
+// up[r, j] = sum_k B[j, k] (alpha / r) xa[r, k] with B [out_dim, rank] bf16 and xa the columns
+// xa_col.. of the pass's output; a null B adds nothing.
 struct RowUp {
   const __nv_bfloat16* B;
-  const float* xa;
+  int xa_col;
 };
-// x[r] += up(r) for r < up_rows (the rows that carry a pending product), then for every row
-// xn[r] = rmsnorm(x[r]) * g (eps): the residual stream's update and the next RMSNorm in one launch,
-// over norm_up_slices(dim) blocks per row. part: [rows, slices] fp32 scratch; counter: [rows] ints,
-// zero before the first launch and left zero by every launch.
-int norm_up_slices(int dim);
-cudaError_t launch_norm_up_rows(float* x, int dim, int rows, RowUp up, int up_rows, int rank,
-                                const __nv_bfloat16* g, float eps, float* xn, float* part, int* counter,
-                                cudaStream_t stream);
-// x[r] += up(r) for every row (the last projection's product, before the rows leave).
-cudaError_t launch_rows_up(float* x, int dim, int rows, RowUp up, int rank, cudaStream_t stream);
-cudaError_t launch_rmsnorm_f32(const float* x, const __nv_bfloat16* g, float* y, int rows,
-                               int hidden, float eps, cudaStream_t stream);
+struct RowLora {
+  int rank;
+  float scale;  // alpha / r
+};
+// Where rows that join at this layer start: a bf16 row, or a token's embedding.
+struct RowStart {
+  const __nv_bfloat16* row[kMaxReq];
+  const int32_t* token[kMaxReq];
+  const __nv_bfloat16* embed;
+  int vocab;
+};
+// The residual stream before a norm: x[r] = its start (rows >= up_rows), else x[r] + the pending
+// pass's output (from column 0) + up product; then xs[r] = the terms of x[r] * g and nss[r][slice] =
+// the slice's sum of squares, for the pass that applies 1 / rms. Token ids outside [0, vocab) read
+// row 0 and set kStatusBounds.
+int norm_slices(int dim);
+cudaError_t launch_add_norm_rows(float* x, int dim, int rows, const RowPart& part, const RowUp& up, const RowLora& lora,
+                                 int up_rows, const RowStart* start, const __nv_bfloat16* g, __nv_bfloat16* xs,
+                                 int terms, float* nss, int* status, cudaStream_t stream);
+// out[r] = bf16(x[r] + the last pass's output + up product) for every row with a non-null out.
+struct RowOuts {
+  __nv_bfloat16* out[kMaxReq];
+};
+cudaError_t launch_finish_rows(const float* x, int dim, int rows, const RowPart& part, const RowUp& up,
+                               const RowLora& lora, const RowOuts& outs, const int* abort, cudaStream_t stream);
+// ms[r] = the terms of silu(g) * u, g and u the pass's columns 0.. and up_col.. plus their up products.
+cudaError_t launch_swiglu_rows(const RowPart& part, int up_col, int f, const RowUp& up_g, const RowUp& up_u,
+                               const RowLora& lora, __nv_bfloat16* ms, int terms, cudaStream_t stream);
+// LM-head inputs: rows [0, n_ref) of ref, then of cur (bf16): xs = the terms of h * g, nss as above.
+cudaError_t launch_head_rows(const __nv_bfloat16* ref, const __nv_bfloat16* cur, int n_ref, int hidden,
+                             const __nv_bfloat16* g, __nv_bfloat16* xs, int terms, float* nss, cudaStream_t stream);
 // Single-query attention of `rows` decode rows (one per request) over pages [0, pos) plus own k/v.
-struct DecodeAttnDesc {
-  const float* q;          // [rows, Hq*d] fp32 post-RoPE
-  const float* k_self;     // [rows, Hkv*d]
-  const float* v_self;
-  const __nv_bfloat16* kpages;
-  const __nv_bfloat16* vpages;
-  const int32_t* page_table[kMaxReq];  // per decode row
-  int pos[kMaxReq];        // position of the decode row (= number of cached keys before it)
-  float* out;              // [rows, Hq*d]
-  float* part;             // scratch [rows, Hq, splits, d + 2]
-  int rows, n_q_heads, n_kv_heads, head_dim, splits, max_pos;
-  int chunks_per_block;    // set by launch_decode_attention
-  const int* abort;        // per-call abort word, or null
-};
-// Decode attention streamed in 128-position chunks (TMA-staged pages, one block per SM walking
-// a run of chunks of one row and kv head) + merge of the blocks' partials. `splits` in the
-// descriptor must be at least decode_attention_splits(max position + 1).
-cudaError_t launch_decode_attention(const DecodeAttnDesc& d, int num_pages, int num_sms, int* status,
-                                    cudaStream_t stream);
-int decode_attention_splits(int max_positions);
 struct RowPositions {
   int pos[kMaxReq];
 };
-// q, k, v of decode rows: the up products added (up[0..2] for q, k, v), then rotate-half RoPE on
-// q [rows, hq, head_dim] and k [rows, hkv, head_dim], row r at position pos.pos[r]; (cos, sin)
-// from `table` [positions][head_dim / 2], or with table_by_row from row r of a
-// [rows][head_dim / 2] table of the rows' own positions.
-cudaError_t launch_rope_up_rows(float* q, int hq, float* k, int hkv, float* v, int rows, int head_dim,
-                                const RowUp* up, int rank, const float2* table, const RowPositions& pos,
-                                bool table_by_row, cudaStream_t stream);
+struct DecodeAttnDesc {
+  RowPart qkv;             // the q|k|v pass's output
+  int col[3];              // its first columns of q, k, v
+  RowUp up[3];
+  RowLora lora;
+  const __nv_bfloat16* bias[3];
+  const float2* rope;      // (cos, sin) [positions][head_dim / 2], or [rows][head_dim / 2] with rope_by_row
+  int rope_by_row;
+  __nv_bfloat16* kpages;
+  __nv_bfloat16* vpages;
+  int write_kv;            // the row's own k, v go into slot pos % 16 of page page_table[pos / 16]
+  const int32_t* page_table[kMaxReq];  // per decode row
+  int pos[kMaxReq];        // position of the decode row (= number of cached keys before it)
+  __nv_bfloat16* out;      // the terms of o: [rows * terms, Hq*d]
+  int terms;
+  float* part;             // scratch [rows, Hq, splits, d + 2]
+  int rows, n_q_heads, n_kv_heads, head_dim, splits;
+  int chunks_per_block;    // set by launch_decode_attention
+  const int* abort;        // per-call abort word, or null
+};
+// Decode attention: q, k, v finished from the pass's output (bias, up products, rotate-half RoPE),
+// streamed over 128-position chunks (TMA-staged pages, one block per SM walking a run of chunks of
+// one row and kv head) + merge of the blocks' partials. `splits` in the descriptor must be at
+// least decode_attention_splits(max position + 1).
+cudaError_t launch_decode_attention(const DecodeAttnDesc& d, int num_pages, int num_sms, int* status,
+                                    cudaStream_t stream);
+int decode_attention_splits(int max_positions);
 // (cos, sin) of the rows' positions: table [rows][head_dim / 2].
 cudaError_t launch_rope_table_rows(float2* table, const RowPositions& pos, int rows, int head_dim,
                                    double theta, cudaStream_t stream);
-struct TokenRows {
-  const int32_t* token[kMaxReq];  // device pointer to each row's input token id
-};
-// x [rows, hidden] fp32 = embed[token_r].
-cudaError_t launch_embed_rows_f32(const __nv_bfloat16* embed, const TokenRows& t, int rows, float* x,
-                                  int hidden, int vocab, int* status, cudaStream_t stream);
-struct RowPages {
-  const int32_t* page_table[kMaxReq];
-  int pos[kMaxReq];
-  int num_pages;
-};
-// Rows' fp32 k, v [rows, hkv * head_dim] into their page slot (page_table[pos / 16], pos % 16).
-cudaError_t launch_kv_write_rows(const float* k, const float* v, void* kpages, void* vpages,
-                                 const RowPages& rp, int rows, int hkv, int head_dim, int* status,
-                                 const int* abort, cudaStream_t stream);
 // out[r] = argmax of logits row r (lowest index among equal maxima).
 // One block whose wait on an mbarrier nothing arrives on runs out after the bounded-wait limit
 // and raises kStatusTimeout in *status (the failure path, exercised without a fault).
 cudaError_t launch_wait_selftest(int* status, cudaStream_t stream);
 cudaError_t launch_argmax_rows(const float* logits, int rows, int vocab, int32_t* out,
                                cudaStream_t stream, const int* abort = nullptr);
-// m[r, j] = silu(g[r, j] + up_g) * (u[r, j] + up_u) over [rows, f] (gate and up in separate buffers).
-cudaError_t launch_swiglu_up_rows(const float* g, const float* u, float* m, int rows, int f, RowUp up_g,
-                                  RowUp up_u, int rank, cudaStream_t stream);
-cudaError_t launch_f32_to_bf16(const float* x, __nv_bfloat16* y, int n, cudaStream_t stream,
-                               const int* abort = nullptr);
 // dst[0 .. n) = src[0 .. n) (bf16), unless the call's abort word is set.
 cudaError_t launch_copy_bf16(__nv_bfloat16* dst, const __nv_bfloat16* src, size_t n, const int* abort,
                              cudaStream_t stream);
@@ -295,11 +312,11 @@ struct PageCheck {
 };
 cudaError_t launch_validate_pages(const PageCheck& pc, int num_pages, int* table, uint32_t mask, int* abort,
                                   int* status, cudaStream_t stream);
-cudaError_t launch_bf16_to_f32(const __nv_bfloat16* x, float* y, int n, cudaStream_t stream);
 
-// LM head + KL: logits [2*rows, V] (ref rows first) from final-normed hidden rows.
-cudaError_t launch_lm_head(const __nv_bfloat16* W, const float* h, int rows, int vocab, int hidden,
-                           float* logits, int num_sms, cudaStream_t stream, const int* abort = nullptr);
+// Logits [rows, V] fp32 of rows given as terms and sums of squares (launch_head_rows, launch_add_norm_rows).
+cudaError_t launch_lm_head(const __nv_bfloat16* W, const __nv_bfloat16* xs, int terms, const float* nss, int rows,
+                           int vocab, int hidden, float eps, float* logits, int num_sms, int* status,
+                           cudaStream_t stream, const int* abort = nullptr);
 // KL per row from fp32 logits; part: scratch [rows][splits][5].
 cudaError_t launch_kl(const float* zref, const float* zcur, int rows, int vocab, float* out,
                       float* part, int splits, cudaStream_t stream);

@@ -1,0 +1,333 @@
+// Weight passes of the decode rows (the first-step rows of a window, the rows of a generation
+// step, the LM head): y[r, j] = sum_i W[j, i] x[r, i] for up to 64 fp32 rows x, every weight read
+// once for all of them. Adapted projections of Eq. S3 for single rows (Section 3.1, Section S2.1).
+//
+// The work is bound by the weight bytes. tcgen05.mma takes the weights as the 128-row A operand,
+// straight from the shared-memory ring that TMA fills, so no thread touches a weight. The rows are
+// the B operand: each fp32 row enters as bf16 terms in rows of their own (kTerms per row, 2: about
+// 16 mantissa bits, 3: the whole fp32 value), and the epilogue adds a row's term columns; products
+// of bf16 values are exact in fp32, accumulation is fp32.
+//
+// Units of work: (128-row weight tile, K split); a tile's `splits` units are spread over CTAs so
+// that a narrow projection still fills the chip, and each writes its own partial sums
+// [split][row][column]. The consumer of the output adds them in split order (part_sum), which it
+// does while it adds the adapter's up product anyway: no reduction pass, no atomics. The adapter's
+// A rows (up to three modules, 16 rows each) are one more tile of the pass, so the down products
+// come out of it too. An RMSNorm's 1 / rms is a factor of the whole row: the rows enter as x * g
+// and the epilogue multiplies by it (nss: the sums of squares by slice).
+//
+// One CTA per SM (a ring of at most ~74 KB) and dependent launch: the ring's first weights are
+// requested before the wait for the kernel that makes x, so the copies run through the short
+// kernels between two passes.
+#include "common.cuh"
+#include "kernels.h"
+#include "tma_map.h"
+
+#include <algorithm>
+#include <cstring>
+
+namespace crf {
+
+namespace {
+
+constexpr int kTile = 128;
+constexpr int kBlockK = 64;
+constexpr int kRgThreads = 192;  // producer, MMA and four epilogue warps
+constexpr int kMaxStages = 12;
+constexpr int kWBytes = kTile * kBlockK * 2;
+
+struct RowsGemmArgs {
+  CUtensorMap tmW[kRowsMaxSeg];
+  CUtensorMap tmA[kRowsMaxSeg];  // LoRA A rows, box of 16
+  CUtensorMap tmX;               // the rows' terms, box of n
+  RowsPlan plan;
+  int nseg, n_lora, units;
+  int rows, n, stages, acc_cols;
+  uint32_t tmem_cols;
+  float* y;
+  const float* nss;
+  int slices;
+  float inv_dim, eps;
+  int* status;
+  const int* abort;
+};
+
+// The steps (K blocks) of this CTA's units, in order.
+struct Steps {
+  int u, tile, kb, end;
+  __device__ __forceinline__ void at(const RowsGemmArgs& a, int unit) {
+    u = unit;
+    tile = unit / a.plan.splits;
+    const int p = unit - tile * a.plan.splits;
+    kb = p * a.plan.kb / a.plan.splits;
+    end = (p + 1) * a.plan.kb / a.plan.splits;
+  }
+  __device__ __forceinline__ void next(const RowsGemmArgs& a) {
+    if (++kb == end) at(a, u + gridDim.x);
+  }
+  __device__ __forceinline__ bool more(const RowsGemmArgs& a) const { return u < a.units; }
+};
+
+template <int kTerms>
+__global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_constant__ RowsGemmArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages];
+  __shared__ __align__(8) uint64_t tfull[2], tempty[2], drain_bar;
+  __shared__ uint32_t tmem_base_sh;
+  __shared__ float s_inv[kRowsMax];
+  __shared__ volatile int abort_flag;
+
+  griddep_launch_dependents();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int stage_bytes = kWBytes + a.n * kBlockK * 2;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < a.stages; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&tfull[i], 1);
+      mbar_init(&tempty[i], 4);
+    }
+    mbar_init(&drain_bar, 1);
+    abort_flag = 0;
+    fence_barrier_init();
+  }
+  if (warp == 1) {
+    tmem_alloc(&tmem_base_sh, a.tmem_cols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_base_sh;
+
+  if (warp == 0) {
+    // ---------------------------------------------------------------- producer
+    if (lane == 0) {
+      int armed[kMaxStages];
+      for (int i = 0; i < a.stages; ++i) armed[i] = -1;
+      auto load_w = [&](const Steps& s, int st, int parity) {
+        uint8_t* dst = smem + st * stage_bytes;
+        const bool lora = s.tile == a.plan.tile0[a.nseg];
+        mbar_arrive_expect_tx(&full[st], (lora ? a.n_lora * 16 * kBlockK * 2 : kWBytes) + a.n * kBlockK * 2);
+        armed[st] = parity;
+        if (lora) {
+          for (int i = 0; i < a.n_lora; ++i)
+            tma_load_2d(dst + i * 16 * kBlockK * 2, &a.tmA[i], &full[st], s.kb * kBlockK, 0);
+        } else {
+          int seg = 0;
+          while (seg + 1 < a.nseg && s.tile >= a.plan.tile0[seg + 1]) ++seg;
+          tma_load_2d(dst, &a.tmW[seg], &full[st], s.kb * kBlockK, (s.tile - a.plan.tile0[seg]) * kTile);
+        }
+      };
+      auto load_x = [&](const Steps& s, int st) {
+        tma_load_2d(smem + st * stage_bytes + kWBytes, &a.tmX, &full[st], s.kb * kBlockK, 0);
+      };
+      Steps w, x;
+      w.at(a, blockIdx.x);
+      x.at(a, blockIdx.x);
+      // weights of the first stages before the wait, their rows after it
+      int pre = 0;
+      for (; pre < a.stages && w.more(a); ++pre, w.next(a)) load_w(w, pre, 0);
+      griddep_wait();
+      asm volatile("fence.proxy.async.global;" ::: "memory");
+      for (int i = 0; i < pre; ++i, x.next(a)) load_x(x, i);
+      bool ok = true;
+      int st = 0;
+      uint32_t ph = 1;
+      for (; ok && w.more(a); w.next(a)) {
+        ok = mbar_wait(&empty[st], ph ^ 1, &abort_flag, a.status);
+        if (!ok) break;
+        load_w(w, st, static_cast<int>(ph));
+        load_x(w, st);
+        if (++st == a.stages) {
+          st = 0;
+          ph ^= 1;
+        }
+      }
+      if (!ok) {
+        volatile int never = 0;
+        for (int i = 0; i < a.stages; ++i)
+          if (armed[i] >= 0) mbar_wait(&full[i], static_cast<uint32_t>(armed[i]), &never, nullptr);
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------------------------------------------------------- MMA issuer
+    if (lane == 0) {
+      const uint32_t idesc = idesc_bf16_f32(kTile, a.n);
+      bool ok = true, issued = false;
+      int st = 0, it = 0;
+      uint32_t ph = 0;
+      Steps s;
+      for (s.at(a, blockIdx.x); ok && s.more(a); ++it) {
+        const int acc = it & 1;
+        if (!mbar_wait(&tempty[acc], ((it >> 1) & 1) ^ 1, &abort_flag, a.status)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t d = tmem + acc * a.acc_cols;
+        const int unit = s.u;
+        for (bool first = true; s.u == unit; s.next(a), first = false) {
+          if (!mbar_wait(&full[st], ph, &abort_flag, a.status)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t base = smem_u32(smem + st * stage_bytes);
+          const uint64_t wd = smem_desc(base, 16, 1024, kSwizzle128B);
+          const uint64_t xd = smem_desc(base + kWBytes, 16, 1024, kSwizzle128B);
+#pragma unroll
+          for (int k = 0; k < kBlockK / 16; ++k)
+            mma_bf16_ss(d, wd + 2 * k, xd + 2 * k, idesc, (!first || k > 0) ? 1u : 0u);
+          issued = true;
+          mma_commit(&empty[st]);
+          if (++st == a.stages) {
+            st = 0;
+            ph ^= 1;
+          }
+        }
+        if (ok) mma_commit(&tfull[acc]);
+      }
+      if (!ok && issued) {
+        mma_commit(&drain_bar);
+        volatile int never = 0;
+        mbar_wait(&drain_bar, 0, &never, nullptr);
+      }
+    }
+  } else {
+    // ---------------------------------------------------------------- epilogue (warps 2..5)
+    griddep_wait();  // nss comes from the kernel before, and earlier kernels read y
+    const int et = threadIdx.x - 64;
+    if (et < a.rows) {
+      float ss = 0.f;
+      for (int i = 0; a.nss && i < a.slices; ++i) ss += __ldcg(a.nss + et * a.slices + i);
+      s_inv[et] = a.nss ? rsqrtf(ss * a.inv_dim + a.eps) : 1.f;
+    }
+    const bool skip = call_aborted(a.abort);
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    const int quarter = warp & 3;
+    const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
+    int it = 0;
+    for (int u = blockIdx.x; u < a.units; u += gridDim.x, ++it) {
+      const int acc = it & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(&tfull[acc], (it >> 1) & 1, &abort_flag, a.status))) break;
+      tc_fence_after();
+      const int tile = u / a.plan.splits;
+      const int col = tile * kTile + quarter * 32 + lane;
+      float* y = a.y + static_cast<size_t>(u - tile * a.plan.splits) * a.rows * a.plan.ncols + col;
+      const bool store = !skip && col < a.plan.ncols;
+      for (int c = 0; c < a.n; c += 16) {
+        uint32_t v[16];
+        tmem_ld16(tmem + lane_off + acc * a.acc_cols + c, v);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 16 / kTerms; ++i) {
+          const int r = c / kTerms + i;
+          float s = __uint_as_float(v[kTerms * i]);
+#pragma unroll
+          for (int t = 1; t < kTerms; ++t) s += __uint_as_float(v[kTerms * i + t]);
+          if (store && r < a.rows) y[static_cast<size_t>(r) * a.plan.ncols] = s * s_inv[r];
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tempty[acc]);
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, a.tmem_cols);
+  }
+}
+
+template <int kTerms>
+cudaError_t launch_terms(const RowsGemmArgs& a, int grid, int smem, cudaStream_t stream) {
+  static PerDevice once;
+  int dev = 0;
+  if (once.pending(&dev)) {
+    cudaError_t e = cudaFuncSetAttribute(rows_gemm_kernel<kTerms>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kRowsRingMax + 1024);
+    if (e != cudaSuccess) return e;
+    once.done(dev);
+  }
+  return launch_kernel(rows_gemm_kernel<kTerms>, dim3(grid), dim3(kRgThreads), smem, stream, a);
+}
+
+}  // namespace
+
+RowsPlan rows_plan(int nseg, const int* outs, bool lora, int in_dim, int num_sms, bool split) {
+  RowsPlan p;
+  std::memset(&p, 0, sizeof(p));
+  p.kb = (in_dim + kBlockK - 1) / kBlockK;
+  for (int s = 0; s < nseg; ++s) {
+    p.tile0[s] = p.tiles;
+    p.tiles += (outs[s] + kTile - 1) / kTile;
+  }
+  p.tile0[nseg] = p.tiles;
+  if (lora) ++p.tiles;
+  p.ncols = p.tiles * kTile;
+  // splits: the fewest K blocks on the busiest CTA, a unit's fixed cost counted as three blocks
+  // and each split's share of the consumer's sum as a quarter
+  p.splits = 1;
+  double best = 0;
+  for (int s = 1; s <= (split ? std::min(kRowsMaxSplits, p.kb) : 1); ++s) {
+    const double waves = (static_cast<long>(p.tiles) * s + num_sms - 1) / num_sms;
+    const double cost = waves * ((p.kb + s - 1) / s + 3) + 0.25 * s;
+    if (s == 1 || cost < best) {
+      best = cost;
+      p.splits = s;
+    }
+  }
+  return p;
+}
+
+cudaError_t launch_rows_gemm(const RowsGemmDesc& d, const RowsPlan& plan, int num_sms, cudaStream_t stream) {
+  RowsGemmArgs a;
+  std::memset(&a, 0, sizeof(a));
+  if (d.rows < 1 || d.rows > kRowsMax || d.nseg < 1 || d.nseg > kRowsMaxSeg || d.n_lora < 0 || d.n_lora > kRowsMaxSeg ||
+      (d.terms != 2 && d.terms != 3) || (d.terms == 3 && d.rows > 5) || d.in_dim % 8 != 0)
+    return cudaErrorInvalidValue;
+  for (int s = 0; s < kRowsMaxSeg; ++s) {
+    const int src = s < d.nseg ? s : 0;  // unused maps alias a valid one
+    if (!tensor_map_rows(&a.tmW[s], d.W[src], d.out[src], d.in_dim, kTile)) return cudaErrorInvalidValue;
+    if (s < d.n_lora) {
+      if (!tensor_map_rows(&a.tmA[s], d.LA[s], d.rank, d.in_dim, 16)) return cudaErrorInvalidValue;
+    } else {
+      a.tmA[s] = a.tmW[0];
+    }
+  }
+  a.n = (d.rows * d.terms + 15) / 16 * 16;
+  if (!tensor_map_rows(&a.tmX, d.x, static_cast<long>(d.rows) * d.terms, d.in_dim, a.n)) return cudaErrorInvalidValue;
+  a.plan = plan;
+  if (d.ncols > 0) a.plan.ncols = d.ncols;
+  a.nseg = d.nseg;
+  a.n_lora = d.n_lora;
+  a.units = plan.tiles * plan.splits;
+  a.rows = d.rows;
+  a.acc_cols = 16;
+  while (a.acc_cols < a.n) a.acc_cols *= 2;
+  a.tmem_cols = std::max(32, 2 * a.acc_cols);
+  const int stage = kWBytes + a.n * kBlockK * 2;
+  const int ring = pdl_active() ? kRowsRing : kRowsRingMax;
+  a.stages = std::min(kMaxStages, ring / stage);
+  a.y = d.y;
+  a.nss = d.nss;
+  a.slices = d.slices;
+  a.inv_dim = 1.f / d.in_dim;
+  a.eps = d.eps;
+  a.status = d.status;
+  a.abort = d.abort;
+  const int grid = std::min(num_sms, a.units);
+  if (grid < 1) return cudaSuccess;
+  const int smem = a.stages * stage + 1024;
+  return d.terms == 2 ? launch_terms<2>(a, grid, smem, stream) : launch_terms<3>(a, grid, smem, stream);
+}
+
+}  // namespace crf
