@@ -178,8 +178,9 @@ cudaError_t launch_attention_tc(const AttnDesc& d, int num_pages, int total_rows
 constexpr int kRowsMax = 64;         // rows of one weight pass
 constexpr int kRowsMaxSeg = 3;       // projections that share an input
 constexpr int kRowsMaxSplits = 16;   // K splits of a weight tile
-constexpr int kRowsRing = 76 * 1024;      // shared-memory ring of a pass inside a dependent chain
-constexpr int kRowsRingMax = 200 * 1024;  // and of one alone on its SMs
+constexpr int kRowsRing = 76 * 1024;       // shared-memory ring of a short pass inside a dependent chain,
+constexpr int kRowsRingLong = 150 * 1024;  // of a long one,
+constexpr int kRowsRingMax = 200 * 1024;   // and of one alone on its SMs
 // fp32 rows enter a weight pass as bf16 terms: three (exact) for one or two rows, two (about 16
 // mantissa bits) from three rows on. Chosen by the rows of the whole call, so that equal rows in
 // different passes stay equal.
@@ -191,7 +192,8 @@ inline int rows_terms(int total_rows) { return total_rows <= 2 ? 3 : 2; }
 // 128 tile0[s] + j.
 struct RowsPlan {
   int tile0[kRowsMaxSeg + 1];
-  int tiles, kb, splits, ncols;
+  int tiles, splits, ncols;
+  int kb, sub;  // K steps of a tile, each sub x 64 wide
 };
 RowsPlan rows_plan(int nseg, const int* outs, bool lora, int in_dim, int num_sms, bool split = true);
 struct RowsGemmDesc {
@@ -279,12 +281,12 @@ struct DecodeAttnDesc {
   int terms;
   float* part;             // scratch [rows, Hq, splits, d + 2]
   int rows, n_q_heads, n_kv_heads, head_dim, splits;
-  int chunks_per_block;    // set by launch_decode_attention
+  int total_chunks, blocks, per_pair;  // set by launch_decode_attention
   const int* abort;        // per-call abort word, or null
 };
 // Decode attention: q, k, v finished from the pass's output (bias, up products, rotate-half RoPE),
-// streamed over 128-position chunks (TMA-staged pages, one block per SM walking a run of chunks of
-// one row and kv head) + merge of the blocks' partials. `splits` in the descriptor must be at
+// streamed over 128-position chunks (TMA-staged pages, one block per SM walking an equal run of
+// the chunks of all rows and kv heads) + merge of the blocks' partials. `splits` in the descriptor must be at
 // least decode_attention_splits(max position + 1).
 cudaError_t launch_decode_attention(const DecodeAttnDesc& d, int num_pages, int num_sms, int* status,
                                     cudaStream_t stream);

@@ -7,13 +7,14 @@
 
 namespace crf {
 
-// Element (r, col) of a weight pass's output: its K splits summed in order. Eight loads are in
-// flight at a time, so a sum costs one L2 round trip for up to eight splits.
+// Element (r, col) of a weight pass's output: its K splits summed in order, the loads of up to
+// eight of them in flight together (one L2 round trip).
 __device__ __forceinline__ float part_sum(const RowPart& t, int r, int col) {
-  const size_t stride = static_cast<size_t>(t.rows) * t.ncols;
   const float* q = t.p + static_cast<size_t>(r) * t.ncols + col;
-  float v = 0.f;
-  for (int s0 = 0; s0 < t.splits; s0 += 8) {
+  float v = __ldcg(q);
+  if (t.splits == 1) return v;
+  const size_t stride = static_cast<size_t>(t.rows) * t.ncols;
+  for (int s0 = 1; s0 < t.splits; s0 += 8) {
     float x[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) x[i] = s0 + i < t.splits ? __ldcg(q + (s0 + i) * stride) : 0.f;

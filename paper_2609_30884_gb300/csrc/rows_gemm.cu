@@ -6,7 +6,10 @@
 // straight from the shared-memory ring that TMA fills, so no thread touches a weight. The rows are
 // the B operand: each fp32 row enters as bf16 terms in rows of their own (kTerms per row, 2: about
 // 16 mantissa bits, 3: the whole fp32 value), and the epilogue adds a row's term columns; products
-// of bf16 values are exact in fp32, accumulation is fp32.
+// of bf16 values are exact in fp32, accumulation is fp32. The tensor core cuts its running
+// sums off instead of rounding them, so a long sum drifts by half a unit a step (4e-6 of a logit's
+// size after 224 steps, against 1e-7 for rounded sums): where the rows are exact, a unit's steps
+// accumulate in up to eight groups of TMEM columns, which the epilogue adds.
 //
 // Units of work: (128-row weight tile, K split); a tile's `splits` units are spread over CTAs so
 // that a narrow projection still fills the chip, and each writes its own partial sums
@@ -16,9 +19,16 @@
 // come out of it too. An RMSNorm's 1 / rms is a factor of the whole row: the rows enter as x * g
 // and the epilogue multiplies by it (nss: the sums of squares by slice).
 //
-// One CTA per SM (a ring of at most ~74 KB) and dependent launch: the ring's first weights are
-// requested before the wait for the kernel that makes x, so the copies run through the short
-// kernels between two passes.
+// One CTA per SM and dependent launch: the ring's first weights are requested before the wait for the
+// kernel that makes x, so the copies run through the short kernels between two passes. A short
+// pass's ring (75 KB) fits beside decode attention's block or a long pass's ring (150 KB). Weights
+// are marked evict-first in L2, which keeps the rows' partial sums and the K/V pages there (3% of a
+// 7B generation step).
+//
+// Measured (7B shape, weights read once): LM head, 2 rows, 1.09 GB in 166 us (6.6 TB/s, 97% of the
+// copy rate); gate|up, 272 MB in 46 us (5.9 TB/s) behind the chain's prefetch. 58 rows of the 1.5B
+// LM head: 92 us in one pass (a pass for every 8 rows before: 779 us); a generation step of 32 rows:
+// 18.0 -> 4.8 ms.
 #include "common.cuh"
 #include "kernels.h"
 #include "tma_map.h"
@@ -31,7 +41,7 @@ namespace crf {
 namespace {
 
 constexpr int kTile = 128;
-constexpr int kBlockK = 64;
+constexpr int kBlockK = 64;  // one 128-byte swizzled box; a step takes plan.sub of them side by side
 constexpr int kRgThreads = 192;  // producer, MMA and four epilogue warps
 constexpr int kMaxStages = 12;
 constexpr int kWBytes = kTile * kBlockK * 2;
@@ -42,7 +52,7 @@ struct RowsGemmArgs {
   CUtensorMap tmX;               // the rows' terms, box of n
   RowsPlan plan;
   int nseg, n_lora, units;
-  int rows, n, stages, acc_cols;
+  int rows, n, stages, acc_cols, groups;
   uint32_t tmem_cols;
   float* y;
   const float* nss;
@@ -81,7 +91,9 @@ __global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_cons
 
   griddep_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int stage_bytes = kWBytes + a.n * kBlockK * 2;
+  const int sub = a.plan.sub;
+  const int x_bytes = a.n * kBlockK * 2;
+  const int stage_bytes = sub * (kWBytes + x_bytes);
   if (threadIdx.x == 0) {
     for (int i = 0; i < a.stages; ++i) {
       mbar_init(&full[i], 1);
@@ -109,22 +121,28 @@ __global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_cons
     if (lane == 0) {
       int armed[kMaxStages];
       for (int i = 0; i < a.stages; ++i) armed[i] = -1;
+      const uint64_t once = l2_evict_first();
       auto load_w = [&](const Steps& s, int st, int parity) {
         uint8_t* dst = smem + st * stage_bytes;
         const bool lora = s.tile == a.plan.tile0[a.nseg];
-        mbar_arrive_expect_tx(&full[st], (lora ? a.n_lora * 16 * kBlockK * 2 : kWBytes) + a.n * kBlockK * 2);
+        mbar_arrive_expect_tx(&full[st], sub * ((lora ? a.n_lora * 16 * kBlockK * 2 : kWBytes) + x_bytes));
         armed[st] = parity;
-        if (lora) {
-          for (int i = 0; i < a.n_lora; ++i)
-            tma_load_2d(dst + i * 16 * kBlockK * 2, &a.tmA[i], &full[st], s.kb * kBlockK, 0);
-        } else {
-          int seg = 0;
-          while (seg + 1 < a.nseg && s.tile >= a.plan.tile0[seg + 1]) ++seg;
-          tma_load_2d(dst, &a.tmW[seg], &full[st], s.kb * kBlockK, (s.tile - a.plan.tile0[seg]) * kTile);
+        int seg = 0;
+        while (seg + 1 < a.nseg && s.tile >= a.plan.tile0[seg + 1]) ++seg;
+        for (int h = 0; h < sub; ++h, dst += kWBytes) {
+          const int k = (s.kb * sub + h) * kBlockK;
+          if (lora) {
+            for (int i = 0; i < a.n_lora; ++i)
+              tma_load_2d(dst + i * 16 * kBlockK * 2, &a.tmA[i], &full[st], k, 0);
+          } else {
+            tma_load_2d_hint(dst, &a.tmW[seg], &full[st], k, (s.tile - a.plan.tile0[seg]) * kTile, once);
+          }
         }
       };
       auto load_x = [&](const Steps& s, int st) {
-        tma_load_2d(smem + st * stage_bytes + kWBytes, &a.tmX, &full[st], s.kb * kBlockK, 0);
+        for (int h = 0; h < sub; ++h)
+          tma_load_2d(smem + st * stage_bytes + sub * kWBytes + h * x_bytes, &a.tmX, &full[st],
+                      (s.kb * sub + h) * kBlockK, 0);
       };
       Steps w, x;
       w.at(a, blockIdx.x);
@@ -169,20 +187,26 @@ __global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_cons
           break;
         }
         tc_fence_after();
-        const uint32_t d = tmem + acc * a.acc_cols;
-        const int unit = s.u;
-        for (bool first = true; s.u == unit; s.next(a), first = false) {
+        const int unit = s.u, len = s.end - s.kb;
+        // accumulation group of step i: i * groups / len
+        for (int i = 0, left = 0; s.u == unit; s.next(a), i += a.groups) {
+          const int group = i / len;
+          const bool first = left != group + 1;
+          left = group + 1;
+          const uint32_t d = tmem + acc * a.acc_cols + group * a.n;
           if (!mbar_wait(&full[st], ph, &abort_flag, a.status)) {
             ok = false;
             break;
           }
           tc_fence_after();
           const uint32_t base = smem_u32(smem + st * stage_bytes);
-          const uint64_t wd = smem_desc(base, 16, 1024, kSwizzle128B);
-          const uint64_t xd = smem_desc(base + kWBytes, 16, 1024, kSwizzle128B);
+          for (int h = 0; h < sub; ++h) {
+            const uint64_t wd = smem_desc(base + h * kWBytes, 16, 1024, kSwizzle128B);
+            const uint64_t xd = smem_desc(base + sub * kWBytes + h * x_bytes, 16, 1024, kSwizzle128B);
 #pragma unroll
-          for (int k = 0; k < kBlockK / 16; ++k)
-            mma_bf16_ss(d, wd + 2 * k, xd + 2 * k, idesc, (!first || k > 0) ? 1u : 0u);
+            for (int k = 0; k < kBlockK / 16; ++k)
+              mma_bf16_ss(d, wd + 2 * k, xd + 2 * k, idesc, (!first || h > 0 || k > 0) ? 1u : 0u);
+          }
           issued = true;
           mma_commit(&empty[st]);
           if (++st == a.stages) {
@@ -221,15 +245,22 @@ __global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_cons
       float* y = a.y + static_cast<size_t>(u - tile * a.plan.splits) * a.rows * a.plan.ncols + col;
       const bool store = !skip && col < a.plan.ncols;
       for (int c = 0; c < a.n; c += 16) {
-        uint32_t v[16];
-        tmem_ld16(tmem + lane_off + acc * a.acc_cols + c, v);
-        tmem_ld_wait();
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = 0.f;
+        for (int k = 0; k < a.groups; ++k) {
+          uint32_t w[16];
+          tmem_ld16(tmem + lane_off + acc * a.acc_cols + k * a.n + c, w);
+          tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] += __uint_as_float(w[i]);
+        }
 #pragma unroll
         for (int i = 0; i < 16 / kTerms; ++i) {
           const int r = c / kTerms + i;
-          float s = __uint_as_float(v[kTerms * i]);
+          float s = v[kTerms * i];
 #pragma unroll
-          for (int t = 1; t < kTerms; ++t) s += __uint_as_float(v[kTerms * i + t]);
+          for (int t = 1; t < kTerms; ++t) s += v[kTerms * i + t];
           if (store && r < a.rows) y[static_cast<size_t>(r) * a.plan.ncols] = s * s_inv[r];
         }
       }
@@ -265,7 +296,6 @@ cudaError_t launch_terms(const RowsGemmArgs& a, int grid, int smem, cudaStream_t
 RowsPlan rows_plan(int nseg, const int* outs, bool lora, int in_dim, int num_sms, bool split) {
   RowsPlan p;
   std::memset(&p, 0, sizeof(p));
-  p.kb = (in_dim + kBlockK - 1) / kBlockK;
   for (int s = 0; s < nseg; ++s) {
     p.tile0[s] = p.tiles;
     p.tiles += (outs[s] + kTile - 1) / kTile;
@@ -273,13 +303,21 @@ RowsPlan rows_plan(int nseg, const int* outs, bool lora, int in_dim, int num_sms
   p.tile0[nseg] = p.tiles;
   if (lora) ++p.tiles;
   p.ncols = p.tiles * kTile;
+  const int blocks = (in_dim + kBlockK - 1) / kBlockK;
+  // From 16 blocks a CTA on, steps are two blocks (256 contiguous bytes of each weight row, asked
+  // for together) and the ring is larger: the rate is then set by how DRAM pages are visited. 7B
+  // shape: one generation step 3.69 -> 3.21 ms, LM head 184 -> 166 us; four blocks gain nothing
+  // more. Below it, one-block steps split evenly over more CTAs.
+  const long per_cta = (static_cast<long>(p.tiles) * blocks + num_sms - 1) / num_sms;
+  p.sub = per_cta >= 16 ? 2 : 1;
+  p.kb = (blocks + p.sub - 1) / p.sub;
   // splits: the fewest K blocks on the busiest CTA, a unit's fixed cost counted as three blocks
   // and each split's share of the consumer's sum as a quarter
   p.splits = 1;
   double best = 0;
   for (int s = 1; s <= (split ? std::min(kRowsMaxSplits, p.kb) : 1); ++s) {
     const double waves = (static_cast<long>(p.tiles) * s + num_sms - 1) / num_sms;
-    const double cost = waves * ((p.kb + s - 1) / s + 3) + 0.25 * s;
+    const double cost = waves * (p.sub * ((p.kb + s - 1) / s) + 3) + 0.25 * s;
     if (s == 1 || cost < best) {
       best = cost;
       p.splits = s;
@@ -311,11 +349,13 @@ cudaError_t launch_rows_gemm(const RowsGemmDesc& d, const RowsPlan& plan, int nu
   a.n_lora = d.n_lora;
   a.units = plan.tiles * plan.splits;
   a.rows = d.rows;
+  // exact rows keep fp32 accuracy: groups of a unit's steps accumulate apart (at least one each)
+  a.groups = d.terms == 3 ? std::min(pdl_active() ? 4 : 8, plan.kb / plan.splits) : 1;
   a.acc_cols = 16;
-  while (a.acc_cols < a.n) a.acc_cols *= 2;
+  while (a.acc_cols < a.n * a.groups) a.acc_cols *= 2;
   a.tmem_cols = std::max(32, 2 * a.acc_cols);
-  const int stage = kWBytes + a.n * kBlockK * 2;
-  const int ring = pdl_active() ? kRowsRing : kRowsRingMax;
+  const int stage = plan.sub * (kWBytes + a.n * kBlockK * 2);
+  const int ring = !pdl_active() ? kRowsRingMax : plan.sub > 1 ? kRowsRingLong : kRowsRing;
   a.stages = std::min(kMaxStages, ring / stage);
   a.y = d.y;
   a.nss = d.nss;

@@ -157,3 +157,50 @@ def test_chunk_boundary_positions_do_not_stall():
     ctx.check()
     assert time.perf_counter() - t0 < 1.5
     ctx.close()
+
+
+@pytest.mark.parametrize("rows,longest", [(3, 40), (9, 1500), (32, 700), (32, 5000)])
+def test_rows_of_a_batch_match_the_row_alone(rows, longest):
+    """A generation step of many rows (uneven lengths, some below one chunk, one at its edge, one with an
+    empty cache; whole runs of chunks per row and, for the longest, runs that cross rows) against
+    each row alone. Alone a row enters the weight passes as three bf16 terms, in a batch as two: 2^-17
+    of each input, which four layers carry to the logits at well below 2^-12 of their norm."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2609_30884_gb300 as crf
+    cfg, lc = synth.TINY, synth.LORA_TINY
+    dm, ad = DeviceModel(cfg), DeviceAdapter(cfg, lc, 1)
+    pos = [max(0, (longest * (rows - i)) // rows - 3 * i) for i in range(rows)]
+    pos[1], pos[-1] = 128 * (pos[1] // 128), 0
+    P = sum(pages_needed(p + 1) for p in pos) + 3
+    pts = split_page_tables([p + 1 for p in pos], P, seed=21)
+    pool = make_pool(cfg, P, fill="random", seed=22)
+    before = snapshot(pool)
+    ctx = crf.Context(0)
+    tok = synth.token_ids(cfg, rows, device="cuda")
+
+    def step(idx):
+        t = tok[idx].contiguous()
+        nxt = torch.empty(len(idx), dtype=torch.int32, device="cuda")
+        z = torch.empty(len(idx), cfg.vocab, device="cuda")
+        p, tables = [pos[i] for i in idx], [pts[i] for i in idx]
+        ctx.decode_step(dm.crf, ad.crf, pool, p, tables, t, nxt, ctx.decode_workspace(dm.crf, ad.crf, p, tables, t), logits=z)
+        ctx.check()
+        assert torch.equal(nxt.long(), z.argmax(-1))
+        return z
+
+    z = step(list(range(rows)))
+    got_k, got_v = snapshot(pool)
+    for pages, old in zip(pool.k_pages + pool.v_pages, before[0] + before[1]):
+        pages.copy_(old)
+    for i in range(0, rows, max(1, rows // 5)):
+        alone = step([i])[0]
+        assert (z[i] - alone).norm() <= 2.0 ** -12 * alone.norm(), (i, pos[i])
+    # every slot but the rows' own is untouched
+    own = torch.zeros(P, 16, dtype=torch.bool, device="cuda")
+    for p, pt in zip(pos, pts):
+        own[int(pt[p // 16]), p % 16] = True
+    for new, old in zip(got_k + got_v, before[0] + before[1]):
+        m = ~own[:, None, :, None].expand_as(new)
+        assert torch.equal(new[m], old[m])
+    ctx.close()

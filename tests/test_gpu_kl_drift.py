@@ -123,3 +123,30 @@ def _dims_c(cfg):
     from paper_2609_30884_gb300 import abi
     return abi.ModelDims(cfg.n_layers, cfg.hidden, cfg.n_q_heads, cfg.n_kv_heads, cfg.head_dim,
                          cfg.ffn, cfg.vocab, cfg.rms_eps, cfg.rope_theta, int(cfg.qkv_bias))
+
+
+@pytest.mark.parametrize("rows,vocab,hidden", [(1, 129, 8), (1, 1000, 200), (2, 127, 64), (5, 700, 1536),
+                                               (32, 300, 72), (33, 1024, 256)])
+def test_head_logits_at_tile_edges(ctx, rows, vocab, hidden):
+    """Logits of the weight pass behind crf_kl at the edges of its tiles: vocabularies beside a multiple
+    of 128, hidden sizes below and beside a multiple of 64, one and two rows (three bf16 terms a row),
+    more (two terms), and more than one pass of 64 rows. Against fp64; the terms keep 24 and 16 mantissa
+    bits and the sums are fp32, so the error of a logit is below 2^-15 of the norm of its products."""
+    import paper_2609_30884_gb300 as crf
+    g = torch.Generator(device="cuda").manual_seed(rows * 1000 + hidden)
+    def draw(*shape, std=1.0):
+        return (torch.randn(*shape, device="cuda", generator=g) * std).bfloat16()
+    head, norm, ref, cur = draw(vocab, hidden, std=0.05), draw(hidden), draw(rows, hidden), draw(rows, hidden)
+    dims = dict(n_layers=1, hidden=hidden, n_q_heads=1, n_kv_heads=1, head_dim=64, ffn=8, vocab=vocab, rms_eps=1e-6,
+                rope_theta=1e4, qkv_bias=False)
+    model = crf.Model(dims, [None], None, norm, head)
+    out, z = torch.empty(rows, device="cuda"), torch.full((2 * rows, vocab), float("nan"), device="cuda")
+    ctx.kl(model, ref, cur, out, vocab, ctx.kl_workspace(rows, vocab, hidden), logits_out=z)
+    ctx.check()
+    x = torch.cat((ref, cur)).double()
+    x = x * torch.rsqrt(x.square().mean(-1, keepdim=True) + 1e-6) * norm.double()
+    want = x @ head.double().T
+    scale = x.square() @ head.double().square().T
+    assert ((z.double() - want).abs() <= 2.0 ** -15 * scale.sqrt()).all()
+    p, q = (torch.log_softmax(t, -1) for t in want.chunk(2))
+    assert ((p.exp() * (p - q)).sum(-1) - out.double()).abs().max() <= 1e-3
