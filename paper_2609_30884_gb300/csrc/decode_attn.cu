@@ -12,14 +12,15 @@
 //                       start and end in some blocks (the launcher weighs the two). A copy warp
 //                       gathers K and V pages with TMA (128-byte swizzle) into a two-stage ring and
 //                       does not wait for the kernel before: no kernel of the call writes the
-//                       cached positions of the layer. Eight compute warps take 16 keys of a
-//                       chunk each. For each pair that its run meets, a block first finishes q
+//                       cached positions of the layer. Compute warps w and w + 4 take keys
+//                       32 w .. 32 w + 31 of each chunk: both score them, each multiplies its half of
+//                       V's columns. For each pair that its run meets, a block first finishes q
 //                       (and, where the row's own position falls, k and v) from the q|k|v pass's
 //                       partial sums: K splits, bias, up products, rotate-half RoPE, the row's K/V
 //                       into its page slot in a generation step. The group's query heads (at most
 //                       8) are rows 0..7 of the mma.sync m16n8k16 A operand as bf16(q) and rows
 //                       8..15 as bf16(q - bf16(q)), so one product gives the score at fp32
-//                       accuracy (K is exact in bf16); P enters P V the same way. Every warp keeps
+//                       accuracy (K is exact in bf16); P enters P V as bf16. Every warp keeps
 //                       an online-softmax state (max, sum and unnormalised o in registers) over
 //                       its keys; at the pair's end the warps and the row's own key and value
 //                       (scored and added in fp32) meet at the common max in a fixed order and
@@ -44,7 +45,7 @@ constexpr int kComputeWarps = 8;
 constexpr int kCompute = 32 * kComputeWarps;
 constexpr int kThreadsStream = kCompute + 32;  // + one copy warp
 constexpr int kMaxGroup = 8;
-constexpr int kRedSlots = 4;  // warps whose o meet in shared memory at a time
+constexpr int kRedSlots = 4;  // 32-key slices of a chunk, whose o meet in shared memory
 
 __device__ __forceinline__ void named_bar_sync_dec() {
   asm volatile("bar.sync 1, %0;" ::"n"(kCompute) : "memory");
@@ -116,8 +117,8 @@ struct ChunkAt {
     }
     g = b / per;
     b -= g * per;
-    c = b * n / per;
-    x1 = x0 + g * n + (b + 1) * n / per;
+    c = b * p.per_pair;
+    x1 = x0 + g * n + min(n, c + p.per_pair);
     x0 += g * n + c;
   }
   __device__ __forceinline__ void next(const DecodeAttnDesc& p) {
@@ -134,7 +135,7 @@ struct StreamSmem {
   static constexpr int HALVES = D / 64;
   static constexpr int HALF = kChunk * 128;   // bytes of one 64-column half of a K (or V) tile
   static constexpr int TILE = HALVES * HALF;
-  // o of kRedSlots warps at the pair's end; before it the finished q in fp32 and the A operand
+  // o of the kRedSlots slices at the pair's end; before it the finished q in fp32 and the A operand
   static constexpr int RED = kRedSlots * kMaxGroup * D * 4;
   static constexpr int QF = kMaxGroup * D * 4;
   static constexpr int QHALF = 16 * 128;      // one 64-column half of the 16-row A operand
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(kThreadsStream, 1) decode_attn_stream(const __
   uint8_t* sQ = smem + 2 * kStages * TILE;                   // A operand: [HALVES][16 rows][128 B], swizzled
   float (*s_q)[D] = reinterpret_cast<float (*)[D]>(sQ + HALVES * S::QHALF);
   float (*o_red)[kMaxGroup][D] = reinterpret_cast<float (*)[kMaxGroup][D]>(sQ);
-  __shared__ float red_m[kComputeWarps][kMaxGroup], red_l[kComputeWarps][kMaxGroup];
+  __shared__ float red_m[kRedSlots][kMaxGroup], red_l[kRedSlots][kMaxGroup];
   __shared__ float s_self[kMaxGroup];           // the row's own key, scored in fp32
   __shared__ float s_xa[3][kRankPad];           // the row's scaled down products of q, k, v
   __shared__ float s_k[D], s_v[D];              // own k and v
@@ -258,7 +259,7 @@ __global__ void __launch_bounds__(kThreadsStream, 1) decode_attn_stream(const __
     const int n_run = min(x1 - x, k.n - k.c);       // chunks of this pair in the block's run
     const bool self_here = k.c + n_run == k.n;      // the run's last chunk holds the row's own position
     // partial slot: blocks of the pair before this one
-    const int slot = p.per_pair ? (k.c * pair_blocks(p, r) + k.n - 1) / k.n
+    const int slot = p.per_pair ? k.c / p.per_pair
                                 : static_cast<int>(blockIdx.x) - block_of_chunk(p, x - k.c);
 
     // 1. the elements' K splits (those of every turn in flight together), and meanwhile the down
@@ -365,54 +366,57 @@ __global__ void __launch_bounds__(kThreadsStream, 1) decode_attn_stream(const __
       }
     }
 
-    // 3. the run's chunks. This warp's state over its 16 keys of every chunk: max and partial sum
-    // of head r0 (log2 units), and its share of the unnormalised o (columns cq, cq + 1 of every 8;
-    // elements 2 and 3 are the share of P's low part)
+    // 3. the run's chunks. This warp's state over its 32 keys of every chunk: max and partial sum
+    // of head r0 (log2 units), and its half of the unnormalised o's columns (cq, cq + 1 of every 8)
     float m0 = -INFINITY, l0 = 0.f;
-    float O[D / 8][4];
+    float O[D / 16][4];
 #pragma unroll
-    for (int dn = 0; dn < D / 8; ++dn)
+    for (int dn = 0; dn < D / 16; ++dn)
 #pragma unroll
       for (int e = 0; e < 4; ++e) O[dn][e] = 0.f;
+    const int key0 = (warp & 3) * 32;
+    const int u0 = (warp >> 2) * (D / 16);  // first 16-byte unit (8 columns) of this warp's half of V
     for (int q = 0; q < n_run; ++q, ++x, k.next(p)) {
       const int i = x - x0, st = i % kStages;
       const int n_cached = min(kChunk, pos - k.c * kChunk);  // cached keys of this chunk
       if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&full[st], (i / kStages) & 1, &abort_flag, a.status));
       const uint32_t k_base = smem_u32(sKV + st * 2 * TILE), v_base = k_base + TILE;
-      const int key0 = warp * 16;
-      if (ok && key0 < n_cached && n_cached < key0 + 16) {
+      if (ok && key0 < n_cached && n_cached < key0 + 32) {
         // V rows from the row's own slot on are zeroed (its value is added in fp32 at the end, and
-        // 0 * stale data must not produce NaN in P V); each warp reads its own 16 rows only
-        for (int w = lane; w < 16 * HALVES * 8; w += 32) {
-          const int t2 = key0 + w / (HALVES * 8), hf = (w / 8) % HALVES, cc = w % 8;
+        // 0 * stale data must not produce NaN in P V); each warp reads its own rows and half only
+        for (int w = lane; w < 32 * (D / 16); w += 32) {
+          const int t2 = key0 + w / (D / 16), u = u0 + w % (D / 16);
           if (t2 >= n_cached)
-            *reinterpret_cast<uint4*>(sKV + st * 2 * TILE + TILE + hf * HALF + t2 * 128 + (cc << 4)) =
-                make_uint4(0, 0, 0, 0);
+            *reinterpret_cast<uint4*>(sKV + st * 2 * TILE + TILE + (u / 8) * HALF + t2 * 128 +
+                                      (((u % 8) ^ (t2 & 7)) << 4)) = make_uint4(0, 0, 0, 0);
         }
         fence_proxy_async_smem();  // before the stage's next copies
         __syncwarp();
       }
       if (ok && key0 < n_cached) {
-        // S = Q K^T for this warp's 16 keys: 2 n-tiles of 8 keys
-        float sc[2][4];
+        // S = Q K^T for this warp's 32 keys: 4 n-tiles of 8 keys
+        float sc[4][4];
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
+        for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
           for (int e = 0; e < 4; ++e) sc[nt][e] = 0.f;
-        const int key = key0 + (mi >> 1) * 8 + li;
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks) {
           const int cc = 2 * (ks % 4) + (mi & 1);
-          uint32_t b0, b1, b2, b3;
-          ldsm_x4(k_base + (ks / 4) * HALF + key * 128 + ((cc ^ (key & 7)) << 4), b0, b1, b2, b3);
-          mma16816(sc[0], qf[ks], b0, b1);
-          mma16816(sc[1], qf[ks], b2, b3);
+#pragma unroll
+          for (int np = 0; np < 2; ++np) {
+            const int key = key0 + (2 * np + (mi >> 1)) * 8 + li;
+            uint32_t b0, b1, b2, b3;
+            ldsm_x4(k_base + (ks / 4) * HALF + key * 128 + ((cc ^ (key & 7)) << 4), b0, b1, b2, b3);
+            mma16816(sc[2 * np], qf[ks], b0, b1);
+            mma16816(sc[2 * np + 1], qf[ks], b2, b3);
+          }
         }
         // high + low part, mask past this chunk's cached keys, online max / sum update
-        float s[4];
+        float s[8];
         float c0 = -INFINITY;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
+        for (int e = 0; e < 8; ++e) {
           s[e] = sc[e >> 1][e & 1] + sc[e >> 1][2 + (e & 1)];
           if (key0 + (e >> 1) * 8 + cq + (e & 1) >= n_cached) s[e] = -INFINITY;
           c0 = fmaxf(c0, s[e]);
@@ -426,68 +430,55 @@ __global__ void __launch_bounds__(kThreadsStream, 1) decode_attn_stream(const __
           m0 = n0;
           l0 *= a0;
 #pragma unroll
-          for (int dn = 0; dn < D / 8; ++dn)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) O[dn][e] *= a0;
+          for (int dn = 0; dn < D / 16; ++dn) {
+            O[dn][0] *= a0;
+            O[dn][1] *= a0;
+          }
         }
         const float z0 = m0 == -INFINITY ? 0.f : m0;
-        uint32_t pa[4];
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-          const float p0 = ex2_approx(s[2 * nt] - z0), p1 = ex2_approx(s[2 * nt + 1] - z0);
-          l0 += p0 + p1;
-          const float h0 = __bfloat162float(__float2bfloat16_rn(p0)), h1 = __bfloat162float(__float2bfloat16_rn(p1));
-          pa[2 * nt] = pack_bf16(h0, h1);
-          pa[2 * nt + 1] = pack_bf16(p0 - h0, p1 - h1);
+        for (int e = 0; e < 8; ++e) {
+          s[e] = ex2_approx(s[e] - z0);
+          l0 += s[e];
         }
         // O += P V: P from the score fragments, V by transposing loads
-        const int vkey = key0 + (mi & 1) * 8 + li;
 #pragma unroll
-        for (int dp = 0; dp < D / 16; ++dp) {
-          const int gc = 2 * dp + (mi >> 1);  // 16-byte chunk of the row (8 dims)
-          const int hf = gc / 8, cc = gc % 8;
-          uint32_t b0, b1, b2, b3;
-          ldsm_x4_t(v_base + hf * HALF + vkey * 128 + ((cc ^ (vkey & 7)) << 4), b0, b1, b2, b3);
-          mma16816(O[2 * dp], pa, b0, b1);
-          mma16816(O[2 * dp + 1], pa, b2, b3);
+        for (int j = 0; j < 2; ++j) {
+          const uint32_t pa[4] = {pack_bf16(s[4 * j], s[4 * j + 1]), 0u, pack_bf16(s[4 * j + 2], s[4 * j + 3]), 0u};
+          const int vkey = key0 + 16 * j + (mi & 1) * 8 + li;
+#pragma unroll
+          for (int dp = 0; dp < D / 32; ++dp) {
+            const int u = u0 + 2 * dp + (mi >> 1);  // 16-byte unit of the row (8 dims)
+            uint32_t b0, b1, b2, b3;
+            ldsm_x4_t(v_base + (u / 8) * HALF + vkey * 128 + (((u % 8) ^ (vkey & 7)) << 4), b0, b1, b2, b3);
+            mma16816(O[2 * dp], pa, b0, b1);
+            mma16816(O[2 * dp + 1], pa, b2, b3);
+          }
         }
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[st]);  // this warp is done with the stage
     }
 
-    // 4. the warps' states (and the row's own key) meet at the common max, in a fixed order
+    // 4. the slices' states (and the row's own key) meet at the common max, in a fixed order
 #pragma unroll
     for (int o = 1; o <= 2; o <<= 1) l0 += __shfl_xor_sync(0xffffffffu, l0, o);
-    if ((lane & 3) == 0) red_m[warp][r0] = m0;
+    if (warp < kRedSlots && (lane & 3) == 0) red_m[warp][r0] = m0;
     ok = named_bar_and_dec(ok);
     float M = self_here && r0 < grp ? s_self[r0] : -INFINITY;
 #pragma unroll
-    for (int w = 0; w < kComputeWarps; ++w) M = fmaxf(M, red_m[w][r0]);
+    for (int w = 0; w < kRedSlots; ++w) M = fmaxf(M, red_m[w][r0]);
     const float f0 = m0 == -INFINITY ? 0.f : ex2_approx(m0 - M);
-    if ((lane & 3) == 0) red_l[warp][r0] = l0 * f0;
+    if (warp < kRedSlots && (lane & 3) == 0) red_l[warp][r0] = l0 * f0;
 #pragma unroll
-    for (int round = 0; round < kComputeWarps / kRedSlots; ++round) {
-      if (warp / kRedSlots == round) {
-        float* dst = &o_red[warp % kRedSlots][r0][cq];
-#pragma unroll
-        for (int dn = 0; dn < D / 8; ++dn) {
-          float2 v = make_float2((O[dn][0] + O[dn][2]) * f0, (O[dn][1] + O[dn][3]) * f0);
-          if (round > 0) {
-            const float2 w = *reinterpret_cast<const float2*>(dst + dn * 8);
-            v.x += w.x;
-            v.y += w.y;
-          }
-          *reinterpret_cast<float2*>(dst + dn * 8) = v;
-        }
-      }
-      named_bar_sync_dec();
-    }
+    for (int dn = 0; dn < D / 16; ++dn)
+      *reinterpret_cast<float2*>(&o_red[warp & 3][r0][8 * (u0 + dn) + cq]) = make_float2(O[dn][0] * f0, O[dn][1] * f0);
+    named_bar_sync_dec();
     if (ok && tid < grp * (D / 4)) {  // four columns of one head per thread
       const int h = tid / (D / 4), d = 4 * (tid % (D / 4));
       float mx = self_here ? s_self[h] : -INFINITY, L = 0.f;
 #pragma unroll
-      for (int w = 0; w < kComputeWarps; ++w) {
+      for (int w = 0; w < kRedSlots; ++w) {
         mx = fmaxf(mx, red_m[w][h]);
         L += red_l[w][h];
       }

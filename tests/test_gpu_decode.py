@@ -163,8 +163,11 @@ def test_chunk_boundary_positions_do_not_stall():
 def test_rows_of_a_batch_match_the_row_alone(rows, longest):
     """A generation step of many rows (uneven lengths, some below one chunk, one at its edge, one with an
     empty cache; whole runs of chunks per row and, for the longest, runs that cross rows) against
-    each row alone. Alone a row enters the weight passes as three bf16 terms, in a batch as two: 2^-17
-    of each input, which four layers carry to the logits at well below 2^-12 of their norm."""
+    each row alone. Two roundings part them: a row alone enters the weight passes as three bf16 terms, in
+    a batch as two (2^-17 of each input), and its softmax weights are rounded to bf16 relative to running
+    maxima that depend on how its chunks are dealt out, so two runs' weights differ by at most 2 x 2^-9
+    of themselves and an attention output by at most 2^-8 of its weighted |v|: 2^-6 of the logits'
+    norm over four layers if every rounding went the same way."""
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     import paper_2609_30884_gb300 as crf
@@ -195,7 +198,7 @@ def test_rows_of_a_batch_match_the_row_alone(rows, longest):
         pages.copy_(old)
     for i in range(0, rows, max(1, rows // 5)):
         alone = step([i])[0]
-        assert (z[i] - alone).norm() <= 2.0 ** -12 * alone.norm(), (i, pos[i])
+        assert (z[i] - alone).norm() <= 2.0 ** -6 * alone.norm(), (i, pos[i])
     # every slot but the rows' own is untouched
     own = torch.zeros(P, 16, dtype=torch.bool, device="cuda")
     for p, pt in zip(pos, pts):
