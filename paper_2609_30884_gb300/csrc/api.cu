@@ -170,8 +170,8 @@ struct Plan {
   size_t off_g0, off_g1, off_x1, off_xn, off_q, off_o, off_mlp, off_xa, off_bx, off_rope;
   size_t off_dx0, off_dec;  // decode: bf16 starting rows, fp32 scratch
   size_t off_abort, off_ptab;  // the call's abort word; the page-check table (ptab_slots ints)
-  // the projections' XA ready words (4 launches x ceil(M / 256) row blocks per layer), laid out
-  // after the abort word so one clear at the start of the call covers them all
+  // the projections' XA ready words (4 launches x ceil(M / 256) row blocks per layer),
+  // laid out after the abort word so one clear at the start of the call covers them all
   size_t flag_words = 0;
   uint32_t ptab_slots = 2;
   size_t total;
@@ -433,6 +433,7 @@ crf_status run_layer(const LayerCtx& c, int l, const __nv_bfloat16* X_in, __nv_b
     }
     g.epi = kEpiQkv;
     g.rope = rope;
+    g.rope_positions = p.max_n;
     g.head_dim = D.d;
     g.n_kv_heads = D.hkv;
     g.qbuf = Q;
@@ -661,6 +662,7 @@ crf_status decode_rows(const LayerCtx& c, std::vector<DecodeRow> rows, const Dec
     a.lora = lora;
     a.rope = opt.rope_by_row ? opt.rope_by_row : reinterpret_cast<const float2*>(c.ws + p.off_rope);
     a.rope_by_row = opt.rope_by_row != nullptr;
+    a.rope_positions = p.max_n;
     a.kpages = static_cast<__nv_bfloat16*>(c.pool->k_pages[l]);
     a.vpages = static_cast<__nv_bfloat16*>(c.pool->v_pages[l]);
     a.write_kv = opt.write_kv;

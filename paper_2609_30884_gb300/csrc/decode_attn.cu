@@ -308,12 +308,15 @@ __global__ void __launch_bounds__(kThreadsStream, 1) decode_attn_stream(const __
       named_bar_sync_dec();
     }
     // 2. rotation; q scaled, kept in fp32 for the own key's score and split into the A operand
-    const float2* angles = p.rope + static_cast<size_t>(p.rope_by_row ? r : pos) * HALF_D;
+    auto angle = [&](int e) {
+      return __ldg(p.rope + (p.rope_by_row ? static_cast<size_t>(r) * HALF_D + e
+                                           : (static_cast<size_t>(e / 2) * p.rope_positions + pos) * 2 + e % 2));
+    };
     for (int i = tid; i < kMaxGroup * HALF_D / 2; i += kCompute) {
       const int h = i / (HALF_D / 2), e = 2 * (i % (HALF_D / 2));
       float2 lo = make_float2(0.f, 0.f), hi = lo;  // elements e, e + 1 and their rotation partners
       if (h < grp) {
-        const float2 c0 = __ldg(angles + e), c1 = __ldg(angles + e + 1);
+        const float2 c0 = angle(e), c1 = angle(e + 1);
         const float2 a0 = *reinterpret_cast<const float2*>(&s_q[h][e]);
         const float2 a1 = *reinterpret_cast<const float2*>(&s_q[h][e + HALF_D]);
         lo = make_float2((a0.x * c0.x - a1.x * c0.y) * qscale, (a0.y * c1.x - a1.y * c1.y) * qscale);
@@ -334,7 +337,7 @@ __global__ void __launch_bounds__(kThreadsStream, 1) decode_attn_stream(const __
     }
     if (self_here)
       for (int e = tid; e < HALF_D; e += kCompute) {
-        const float2 cs = __ldg(angles + e);
+        const float2 cs = angle(e);
         const float a0 = s_k[e], a1 = s_k[e + HALF_D];
         s_k[e] = a0 * cs.x - a1 * cs.y;
         s_k[e + HALF_D] = a1 * cs.x + a0 * cs.y;

@@ -1,8 +1,8 @@
 // Persistent tcgen05 GEMM for sm_103a with the unmerged LoRA product and fused epilogues.
 //
-//   D[256 x 256] = A[256 x K] * B[256 x K]^T  (+ XA[256 x 64] * BL^T)
+//   D[256 x BN] = A[256 x K] * B[BN x K]^T  (+ XA[256 x 64] * BL^T),  BN = 256 or 128
 //
-// A cluster of two CTAs on one TPC works on a 256 x 256 tile with cta_group::2 MMAs. Each CTA
+// A cluster of two CTAs on one TPC works on a 256 x BN tile with cta_group::2 MMAs. Each CTA
 // stages its own 128 rows of A and its own half of the B rows, so the operand bytes each SM
 // pulls through L2 per FLOP are two thirds of the single-CTA 128 x 256 tile's. The even CTA
 // issues the MMAs; both CTAs hold 128 accumulator lanes in their own TMEM and drain them through
@@ -15,22 +15,26 @@
 // are bf16, K-major, staged with 128-byte swizzle; accumulation is fp32 in TMEM.
 //
 // The adapter term (alpha/r) (x A^T) B^T of every adapted projection (Eq. S3, W = W0 + (alpha/r)
-// B A kept unmerged) is computed in the same launch, on the operand tiles already staged:
-//  - the first output tile of each 256-row block (its XA tile) also accumulates x A^T for the
-//    GEMM's adapted modules (N = 16 per module, B operand = the LoRA A rows, staged beside the W
-//    rows) into the other accumulator's first columns, which the epilogue of the previous tile has
-//    drained by then. Its epilogue warps store that product, scaled, as a bf16 pair [hi | lo] per
-//    module (16 + 16 columns of the XA buffer) and count themselves done in the row block's ready
-//    word;
+// B A kept unmerged) is computed in the same launch:
+//  - XA items come first in the order of work: one per row block, an MMA of N = 16 per module over
+//    the x rows against the LoRA A rows, whose epilogue warps store the product, scaled, as a bf16
+//    pair [hi | lo] per module (16 + 16 columns of the XA buffer) and count themselves into the row
+//    block's ready word;
 //  - every output tile of an adapted module adds one 64-wide K block: A side = the XA columns of
-//    its row block (the XA tile writes them into its own stage; the others copy them once the
-//    ready word shows both CTAs done), B side = BX, the module's B rows twice over ([B | B],
-//    against [hi | lo]) under the K steps of its slot and zeros under the other slot, so one K
-//    block serves two stacked modules and the two halves of a pair alike. The RMSNorm launch
-//    before the layer's projections builds the BX rows.
-// XA tiles run first, one per unit, ahead of the other tiles of their row block, so those rarely
-// wait; the wait is bounded like every other. x is read once: the XA product needs no pass of its
-// own.
+//    its row block (copied once the ready word shows all its warps), B side = BX, the module's B
+//    rows twice over ([B | B], against [hi | lo]) under the K steps of its slot and zeros under the
+//    other slot, so one K block serves two stacked modules and the two halves of a pair alike. The
+//    RMSNorm launch before the layer's projections builds the BX rows.
+// An item takes about as long as a tile's main loop and starts with the first wave, so that wave
+// hardly waits. Formed by each row block's first tile, in the other accumulator, the product took
+// that tile 1.4 to 1.8 times a plain one's time and every other tile of the first wave waited for it
+// (1.5B shape, 2003 rows: 7 of the 28 us of q|k|v, 19 of the 77 us of down). Items over a quarter of K
+// each were slower: their sums met through memory.
+//
+// Measured (us a launch: items, epilogue through shared memory and tile width together, before ->
+// now): 1.5B shape, 2003 rows: q|k|v 34 -> 28, o 33 -> 24, gate|up 99 -> 88, down 84 -> 60; 4096 rows:
+// 45 -> 39, 48 -> 35, 164 -> 150, 131 -> 108; 7B, 16384 rows: 370 -> 358, 282 -> 283, 2582 -> 2546,
+// 1288 -> 1356 (K = 18944 makes its 64 items long).
 #include "common.cuh"
 #include "kernels.h"
 
@@ -47,6 +51,7 @@ constexpr int BM = 128;
 constexpr int BK = 64;
 constexpr int kRasterGroup = 8;
 constexpr int kThreads = 192;
+constexpr int kXaGroups = 8;     // epilogue warps of a pair: each stores 32 of a row block's XA rows
 
 struct GemmArgs {
   CUtensorMap tmA;
@@ -61,10 +66,11 @@ struct GemmArgs {
   int ext_on[3];      // per group: tile has the LoRA K block
   int ext_steps[3];   // per group: K = 16 steps of that block that carry data
   int xa_base[3];     // per group: first XA column of that block
-  int row_tiles, total_n, total_tiles;
+  int row_tiles, total_n;
   int n_slots;        // adapted modules (XA slots); 0: no XA product
   int xa_n;           // N of the XA product: 16 per slot, two CTA halves of 16 x slots_per_cta
-  int xa_lead;        // XA tiles placed before every other tile (the rest follow their row block)
+  int xa_items;        // XA items (row_tiles or none), before the tiles in the order
+  int total_items;     // XA items and tiles
   int rank;
   __nv_bfloat16* xa;
   int* xa_flags;
@@ -76,6 +82,7 @@ struct GemmArgs {
   int ld_resid;
   const __nv_bfloat16* bias[3];
   const float2* rope;
+  int rope_positions;
   int head_dim, n_kv_heads;
   __nv_bfloat16* qbuf;
   int ldq;
@@ -88,33 +95,20 @@ struct GemmArgs {
 
 struct Tile {
   int m_blk, g, n_loc;
-  bool xa;  // the row block's first output tile, which also forms its XA product
+  bool xa;  // an XA item
 };
 
-// Output tiles run in bands of kRasterGroup column tiles over every row block (the band's B
-// rows stay in L2). With an adapter, band 0 is reordered so that each row block's first tile
-// (its XA tile) runs ahead of the block's other band-0 tiles: the first `lead` XA tiles, then
-// per row block m the XA tile of m + lead followed by m's other band-0 tiles (lead = all row
-// blocks puts every XA tile first).
+// XA items first, row block by row block; then the output tiles in bands of kRasterGroup column
+// tiles over every row block (the band's B rows stay in L2).
 __device__ __forceinline__ Tile decode_tile(int t, const GemmArgs& a) {
   Tile r;
-  r.xa = false;
-  if (a.n_slots > 0) {
-    const int w0 = min(kRasterGroup, a.total_n);
-    const int lead = min(a.xa_lead, a.row_tiles);
-    const int g1 = a.row_tiles - lead;  // row blocks whose other tiles follow an XA tile
-    if (t < lead) {
-      t = t * w0;  // the plain order's index of tile (t, 0)
-    } else if (t - lead < g1 * w0) {
-      const int u = t - lead;
-      const int m = u / w0, i = u - m * w0;
-      t = i == 0 ? (m + lead) * w0 : m * w0 + i;
-    } else if (t - lead - g1 * w0 < lead * (w0 - 1)) {
-      const int v = t - lead - g1 * w0;
-      const int m = g1 + v / (w0 - 1);
-      t = m * w0 + 1 + v % (w0 - 1);
-    }  // else: the later bands keep their plain index
+  r.xa = t < a.xa_items;
+  if (r.xa) {
+    r.m_blk = t;
+    r.g = r.n_loc = 0;
+    return r;
   }
+  t -= a.xa_items;
   const int band_tiles = a.row_tiles * kRasterGroup;
   const int band = t / band_tiles;
   const int idx = t - band * band_tiles;
@@ -122,7 +116,6 @@ __device__ __forceinline__ Tile decode_tile(int t, const GemmArgs& a) {
   const int width = min(kRasterGroup, a.total_n - n0);
   r.m_blk = idx / width;
   int n = n0 + (idx - r.m_blk * width);
-  r.xa = a.n_slots > 0 && n == 0;
   int g = 0;
   while (g < a.ngroups - 1 && n >= a.group_tiles[g]) {
     n -= a.group_tiles[g];
@@ -147,28 +140,6 @@ __device__ __forceinline__ void store16_bf16(__nv_bfloat16* dst, const float (&v
   reinterpret_cast<uint4*>(dst)[1] = w1;
 }
 
-// Store the first `n` (<= 16) values; n == 16 takes the vector path.
-__device__ __forceinline__ void store_bf16_n(__nv_bfloat16* dst, const float (&v)[16], int n) {
-  if (n >= 16) {
-    store16_bf16(dst, v);
-  } else {
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-      if (j < n) dst[j] = __float2bfloat16_rn(v[j]);
-  }
-}
-
-__device__ __forceinline__ void load16_bf16(const __nv_bfloat16* src, float (&v)[16]) {
-  const uint4 w0 = reinterpret_cast<const uint4*>(src)[0];
-  const uint4 w1 = reinterpret_cast<const uint4*>(src)[1];
-  const uint32_t w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    v[2 * j] = bf16_lo(w[j]);
-    v[2 * j + 1] = bf16_hi(w[j]);
-  }
-}
-
 // Find the request and position of batched row `row`; returns false if none.
 __device__ __forceinline__ bool row_lookup(const ReqTable& rt, int row, int& pos,
                                            const int32_t*& pt) {
@@ -183,44 +154,74 @@ __device__ __forceinline__ bool row_lookup(const ReqTable& rt, int row, int& pos
   return false;
 }
 
+// Epilogue rows move through shared memory, 32 rows x 64 columns of a warp at a time: a thread owns a
+// row of the accumulator, but 32 threads on 32 rows of a matrix cost 32 wavefronts an access, eight
+// threads on 128 contiguous bytes of a row cost one. Slot (row, 16-byte unit u) of a warp's 4 KB scratch
+// is at row * 128 + ((u ^ (row & 7)) << 4): no bank conflicts either way.
+constexpr int kScratchBytes = 4 * 4096;
+__device__ __forceinline__ uint4* scratch_at(uint8_t* s, int row, int u) {
+  return reinterpret_cast<uint4*>(s + row * 128 + ((u ^ (row & 7)) << 4));
+}
+// Rows' 64 columns from scratch to the rows' own destinations (`dst`: this lane's row, null: none);
+// units from `units` on are outside the matrix.
+__device__ __forceinline__ void scratch_store(uint8_t* s, int lane, __nv_bfloat16* dst, int units) {
+  __syncwarp();
+  const unsigned long long p = reinterpret_cast<unsigned long long>(dst);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = 4 * i + (lane >> 3), u = lane & 7;
+    uint4* q = reinterpret_cast<uint4*>(__shfl_sync(0xffffffffu, p, r));
+    const uint4 v = *scratch_at(s, r, u);
+    if (q != nullptr && u < units) q[u] = v;
+  }
+  __syncwarp();
+}
+
+// One row's share of a tile, 64 accumulator columns at a time, so that their TMEM loads and the
+// residual's or rotation table's are in flight together (16 at a time and straight to memory, the
+// epilogue of a 256-column tile took 8-10 us). Twice the epilogue warps instead was slower: they
+// compete with the producer and the MMA thread.
 template <int BN, int EPI>
-__device__ __forceinline__ void epilogue_tile(const GemmArgs& a, const Tile& tl, uint32_t tacc,
-                                              int row) {
+__device__ __forceinline__ void epilogue_tile(const GemmArgs& a, const Tile& tl, uint32_t tacc, int row, int lane,
+                                              uint8_t* scr) {
   const bool row_ok = row < a.M;
-  uint32_t r0[16], r1[16];
-  float v[16], w[16];
 
   if constexpr (EPI == kEpiResid) {
     const int col0 = tl.n_loc * BN;
-    const int ncols = a.group_cols[tl.g];
-    // residual chunk c + 16 is requested while chunk c is drained: its load latency overlaps
-    auto load_resid = [&](int col, float (&dst)[16]) {
-      const int n = min(16, ncols - col);
-      if (n >= 16) {
-        load16_bf16(a.resid + (size_t)row * a.ld_resid + col, dst);
-      } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-          dst[j] = j < n ? __bfloat162float(a.resid[(size_t)row * a.ld_resid + col + j]) : 0.f;
-      }
-    };
-    float wn[16];
-    if (row_ok && col0 < ncols) load_resid(col0, w);
+    const int ncols = a.group_cols[tl.g];  // a multiple of 8
+    __nv_bfloat16* out = row_ok ? a.out + (size_t)row * a.ldo : nullptr;
+    const int row_w = row - lane;  // the warp's first row
 #pragma unroll 1
-    for (int c = 0; c < BN; c += 16) {
-      tmem_ld16(tacc + c, r0);
-      const bool more = row_ok && c + 16 < BN && col0 + c + 16 < ncols;
-      if (more) load_resid(col0 + c + 16, wn);
-      tmem_ld_wait();
+    for (int c = 0; c < BN; c += 64) {
       const int col = col0 + c;
-      if (!row_ok || col >= ncols) continue;
+      uint32_t r[2][32];
+      tmem_ld32(tacc + c, r[0]);
+      tmem_ld32(tacc + c + 32, r[1]);
+      const int units = (ncols - col) / 8;
+      uint4 w[8];
 #pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = w[j] + __uint_as_float(r0[j]);
-      store_bf16_n(a.out + (size_t)row * a.ldo + col, v, min(16, ncols - col));
-      if (more) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) w[j] = wn[j];
+      for (int i = 0; i < 8; ++i) {
+        const int rr = row_w + 4 * i + (lane >> 3), u = lane & 7;
+        w[i] = rr < a.M && u < units
+                   ? *(reinterpret_cast<const uint4*>(a.resid + (size_t)rr * a.ld_resid + col) + u)
+                   : make_uint4(0, 0, 0, 0);
       }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) *scratch_at(scr, 4 * i + (lane >> 3), lane & 7) = w[i];
+      __syncwarp();
+      tmem_ld_wait();
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const uint4 x = *scratch_at(scr, lane, k);
+        const uint32_t u[4] = {x.x, x.y, x.z, x.w};
+        uint32_t p[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          p[e] = pack_bf16(bf16_lo(u[e]) + __uint_as_float(r[k >> 2][(8 * k + 2 * e) & 31]),
+                           bf16_hi(u[e]) + __uint_as_float(r[k >> 2][(8 * k + 2 * e + 1) & 31]));
+        *scratch_at(scr, lane, k) = make_uint4(p[0], p[1], p[2], p[3]);
+      }
+      scratch_store(scr, lane, out ? out + col : nullptr, units);
     }
     return;
   }
@@ -228,27 +229,39 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs& a, const Tile& tl,
   if constexpr (EPI == kEpiSwiGLU) {
     constexpr int HALF = BN / 2;
     const int f0 = tl.n_loc * HALF;
-    const int ffn = a.group_cols[0];
+    const int ffn = a.group_cols[0];  // a multiple of 8
 #pragma unroll 1
-    for (int c = 0; c < HALF; c += 16) {
-      tmem_ld16(tacc + c, r0);
-      tmem_ld16(tacc + HALF + c, r1);
-      tmem_ld_wait();
-      const int col = f0 + c;
-      if (!row_ok || col >= ffn) continue;
+    for (int c = 0; c < HALF; c += 64) {
+#pragma unroll 1
+      for (int h2 = 0; h2 < 64; h2 += 32) {
+        uint32_t gt[32], up[32];
+        tmem_ld32(tacc + c + h2, gt);
+        tmem_ld32(tacc + HALF + c + h2, up);
+        tmem_ld_wait();
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float gt = __uint_as_float(r0[j]);
-        const float up = __uint_as_float(r1[j]);
-        v[j] = gt / (1.0f + __expf(-gt)) * up;
+        for (int k = 0; k < 4; ++k) {
+          uint32_t p[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            float v[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const float x = __uint_as_float(gt[8 * k + 2 * e + h]);
+              v[h] = __fdividef(x, 1.0f + __expf(-x)) * __uint_as_float(up[8 * k + 2 * e + h]);
+            }
+            p[e] = pack_bf16(v[0], v[1]);
+          }
+          *scratch_at(scr, lane, h2 / 8 + k) = make_uint4(p[0], p[1], p[2], p[3]);
+        }
       }
-      store_bf16_n(a.out + (size_t)row * a.ldo + col, v, min(16, ffn - col));
+      scratch_store(scr, lane, row_ok ? a.out + (size_t)row * a.ldo + f0 + c : nullptr, (ffn - f0 - c) / 8);
     }
     return;
   }
 
   if constexpr (EPI == kEpiQkv) {
-    // kEpiQkv: group 0 = q, 1 = k, 2 = v; tiles are head-aligned (BN % head_dim == 0).
+    // kEpiQkv: group 0 = q, 1 = k, 2 = v; tiles are head-aligned (BN % head_dim == 0). Per head 32
+    // rotation pairs at a time: 32 columns from its first half and 32 from its second.
     const int d = a.head_dim;
     const int half = d >> 1;
     int pos = 0;
@@ -269,63 +282,71 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs& a, const Tile& tl,
         head_stride = (size_t)kPage * d;
       }
     }
-    // Chunks of 16 rotation pairs outermost: a chunk's cos/sin (one row of the angle table,
-    // shared by every head of the tile) is loaded once, and the next chunk's is requested
-    // while this one is applied, so the table's load latency overlaps the TMEM drain.
     const bool rot = have && g < 2;
-    const float4* rope4 = reinterpret_cast<const float4*>(a.rope + (size_t)pos * half);
-    float4 cs[8], csn[8];
-    if (rot) {
-  #pragma unroll
-      for (int k = 0; k < 8; ++k) cs[k] = rope4[k];
-    }
-  #pragma unroll 1
-    for (int i0 = 0; i0 < half; i0 += 16) {
-      const bool more = rot && i0 + 16 < half;
-      if (more) {
-  #pragma unroll
-        for (int k = 0; k < 8; ++k) csn[k] = rope4[(i0 + 16) / 2 + k];
+    const float4* rope4 = reinterpret_cast<const float4*>(a.rope) + pos;
+#pragma unroll 1
+    for (int i0 = 0; i0 < half; i0 += 32) {
+      float4 cs[16];  // (cos, sin) of two pairs each: consecutive positions are neighbours
+      if (rot) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) cs[k] = rope4[(size_t)(i0 / 2 + k) * a.rope_positions];
       }
-  #pragma unroll 1
+#pragma unroll 1
       for (int hh = 0; hh < BN / d; ++hh) {
         const int head = (tl.n_loc * BN) / d + hh;
         const int gcol = head * d;
-        tmem_ld16(tacc + hh * d + i0, r0);
-        tmem_ld16(tacc + hh * d + half + i0, r1);
+        if (gcol >= a.group_cols[g]) break;
+        uint32_t r0[32], r1[32];
+        tmem_ld32(tacc + hh * d + i0, r0);
+        tmem_ld32(tacc + hh * d + half + i0, r1);
         tmem_ld_wait();
-        if (!have || gcol >= a.group_cols[g]) continue;
-  #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          v[j] = __uint_as_float(r0[j]);
-          w[j] = __uint_as_float(r1[j]);
-        }
-        if (bias) {
-          float b0[16], b1[16];
-          load16_bf16(bias + gcol + i0, b0);
-          load16_bf16(bias + gcol + half + i0, b1);
-  #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            v[j] += b0[j];
-            w[j] += b1[j];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {  // 8 pairs
+          float v[8], w[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            v[j] = __uint_as_float(r0[8 * k + j]);
+            w[j] = __uint_as_float(r1[8 * k + j]);
           }
-        }
-        if (g < 2) {
-  #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const float c = (j & 1) ? cs[j >> 1].z : cs[j >> 1].x;
-            const float sn = (j & 1) ? cs[j >> 1].w : cs[j >> 1].y;
-            const float x1 = v[j], x2 = w[j];
-            v[j] = x1 * c - x2 * sn;
-            w[j] = x2 * c + x1 * sn;
+          if (bias) {
+            const uint4 b0 = *reinterpret_cast<const uint4*>(bias + gcol + i0 + 8 * k);
+            const uint4 b1 = *reinterpret_cast<const uint4*>(bias + gcol + half + i0 + 8 * k);
+            const uint32_t u0[4] = {b0.x, b0.y, b0.z, b0.w}, u1[4] = {b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              v[2 * j] += bf16_lo(u0[j]);
+              v[2 * j + 1] += bf16_hi(u0[j]);
+              w[2 * j] += bf16_lo(u1[j]);
+              w[2 * j + 1] += bf16_hi(u1[j]);
+            }
           }
+          if (g < 2) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const float4 q = cs[4 * k + (j >> 1)];
+              const float c = (j & 1) ? q.z : q.x, sn = (j & 1) ? q.w : q.y;
+              const float x1 = v[j], x2 = w[j];
+              v[j] = x1 * c - x2 * sn;
+              w[j] = x2 * c + x1 * sn;
+            }
+          }
+          *scratch_at(scr, lane, k) = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
+                                                 pack_bf16(v[6], v[7]));
+          *scratch_at(scr, lane, 4 + k) = make_uint4(pack_bf16(w[0], w[1]), pack_bf16(w[2], w[3]),
+                                                     pack_bf16(w[4], w[5]), pack_bf16(w[6], w[7]));
         }
-        __nv_bfloat16* dst = dst_row + head * head_stride;
-        store16_bf16(dst + i0, v);
-        store16_bf16(dst + half + i0, w);
-      }
-      if (more) {
-  #pragma unroll
-        for (int k = 0; k < 8; ++k) cs[k] = csn[k];
+        // units 0..3: pairs' first elements, units 4..7: the second ones, half a head further on
+        __nv_bfloat16* dst = dst_row ? dst_row + head * head_stride + i0 : nullptr;
+        __syncwarp();
+        const unsigned long long p = reinterpret_cast<unsigned long long>(dst);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int r = 4 * i + (lane >> 3), u = lane & 7;
+          __nv_bfloat16* q = reinterpret_cast<__nv_bfloat16*>(__shfl_sync(0xffffffffu, p, r));
+          const uint4 x = *scratch_at(scr, r, u);
+          if (q != nullptr) *reinterpret_cast<uint4*>(q + (u & 3) * 8 + (u >= 4 ? half : 0)) = x;
+        }
+        __syncwarp();
       }
     }
   }
@@ -357,13 +378,14 @@ __device__ __forceinline__ void fence_proxy_async_global() {
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
-// Stage layout: the A tile (this CTA's 128 rows x 64), the B tile (its 128 rows x 64) and, for XA
-// tiles, the LoRA A rows of its half of the XA product (up to 32 rows x 64); 128-byte swizzle.
-constexpr int kABytes = BM * BK * 2;
-constexpr int kBBytes = 128 * BK * 2;
-constexpr int kLaBytes = 32 * BK * 2;
-constexpr int kStageBytes = kABytes + kBBytes + kLaBytes;
+// Stage layout: the A tile (this CTA's 128 rows x 64) and the B tile (its BN / 2 rows x 64; in an XA
+// item the LoRA A rows of its half of the XA product, up to 32); 128-byte swizzle.
 constexpr int kPair = 2;
+constexpr int kABytes = BM * BK * 2;
+template <int BN>
+constexpr int kBBytes = BN / kPair * BK * 2;
+template <int BN>
+constexpr int kStageBytes = kABytes + kBBytes<BN>;
 
 // Producer ring position (stage, phase) and whether every wait so far succeeded.
 struct Ring {
@@ -394,57 +416,37 @@ __device__ __forceinline__ void tile_b_rows(const GemmArgs& a, const Tile& tl, u
   b_step = nseg == 1 ? 0 : seg_rows * BK * 2;
 }
 
-// Copies of an XA tile: per K block the tile's x and W rows, as for any output tile, and the LoRA
-// A rows of this CTA's half of the XA product (16 rows per XA slot; CTA r takes slots
-// [r * spc, r * spc + spc)). Its LoRA stage, if it has one, gets the BX rows only: the epilogue
-// warps write the A side from the XA product.
+// Copies of an XA item: per K block the row block's x rows and the LoRA A rows of this
+// CTA's half of the XA product (16 rows per XA slot; CTA r takes slots [r * spc, r * spc + spc)).
 template <int BN, int STAGES>
-__device__ __noinline__ Ring load_xa_tile(const GemmArgs& a, const Tile& tl, int m0, uint32_t rank, bool leader,
+__device__ __noinline__ Ring load_xa_item(const GemmArgs& a, int m0, uint32_t rank, bool leader,
                                           uint8_t* smem, uint64_t* full_bar, uint64_t* empty_bar,
                                           int* armed_parity, volatile int* abort_flag, Ring ring) {
-  int g0, nb, yb, b_step;
-  tile_b_rows<BN>(a, tl, rank, g0, nb, yb, b_step);
   const int spc = a.xa_n / (16 * kPair);
   const int s0 = static_cast<int>(rank) * spc, s1 = min(a.n_slots, s0 + spc);
-  const uint32_t bytes = kPair * (kABytes + kBBytes) + a.n_slots * 16 * BK * 2;
+  const uint32_t bytes = kPair * kABytes + a.n_slots * 16 * BK * 2;
   for (int kb = 0; kb < a.num_kb; ++kb) {
     if (!mbar_wait(&empty_bar[ring.stage], ring.phase ^ 1, abort_flag, a.status)) {
       ring.ok = 0;
       return ring;
     }
-    uint8_t* sa = smem + ring.stage * kStageBytes;
-    uint8_t* sb = sa + kABytes;
-    uint8_t* sl = sb + kBBytes;
+    uint8_t* sa = smem + ring.stage * kStageBytes<BN>;
+    uint8_t* sl = sa + kABytes;
     if (leader) {
       mbar_arrive_expect_tx(&full_bar[ring.stage], bytes);
       armed_parity[ring.stage] = ring.phase;
     }
     const uint32_t bar = mapa_shared(&full_bar[ring.stage], 0);
     tma_load_2d_pair(sa, &a.tmA, bar, kb * BK, m0);
-    for (int j = 0; j < nb; ++j) tma_load_2d_pair(sb + j * b_step, &a.tmB[g0 + j], bar, kb * BK, yb);
     for (int j = s0; j < s1; ++j) tma_load_2d_pair(sl + (j - s0) * 16 * BK * 2, &a.tmLA[j], bar, kb * BK, 0);
-    ring_next<STAGES>(ring);
-  }
-  if (a.ext_on[tl.g]) {
-    if (!mbar_wait(&empty_bar[ring.stage], ring.phase ^ 1, abort_flag, a.status)) {
-      ring.ok = 0;
-      return ring;
-    }
-    uint8_t* sb = smem + ring.stage * kStageBytes + kABytes;
-    if (leader) {
-      mbar_arrive_expect_tx(&full_bar[ring.stage], kPair * kBBytes);
-      armed_parity[ring.stage] = ring.phase;
-    }
-    const uint32_t bar = mapa_shared(&full_bar[ring.stage], 0);
-    for (int j = 0; j < nb; ++j) tma_load_2d_pair(sb + j * b_step, &a.tmBX[g0 + j], bar, 0, yb);
     ring_next<STAGES>(ring);
   }
   return ring;
 }
 
-// The LoRA stage of any other output tile: once the stage is free, wait (unless seen already)
-// until both CTAs of the row block's XA tile have stored its XA rows, and copy those rows (the A
-// side of the K block) and the tile's BX rows (the B side).
+// The LoRA stage of an output tile: once the stage is free, wait (unless seen already) until the row
+// block's XA rows are stored, and copy those rows (the A side of the K block) and the tile's BX rows
+// (the B side).
 template <int BN, int STAGES>
 __device__ __noinline__ Ring load_lora_stage(const GemmArgs& a, const Tile& tl, int m0, uint32_t rank, bool xa_ready,
                                              bool leader, uint8_t* smem, uint64_t* full_bar, uint64_t* empty_bar,
@@ -453,16 +455,16 @@ __device__ __noinline__ Ring load_lora_stage(const GemmArgs& a, const Tile& tl, 
     ring.ok = 0;
     return ring;
   }
-  if (!xa_ready && !flag_wait(a.xa_flags + tl.m_blk, 4 * kPair, abort_flag, a.status)) {
+  if (!xa_ready && !flag_wait(a.xa_flags + tl.m_blk, kXaGroups, abort_flag, a.status)) {
     ring.ok = 0;
     return ring;
   }
-  fence_proxy_async_global();  // the TMA copy below reads what the XA tile's stores wrote
+  fence_proxy_async_global();  // the TMA copy below reads what the XA items' stores wrote
   int g0, nb, yb, b_step;
   tile_b_rows<BN>(a, tl, rank, g0, nb, yb, b_step);
-  uint8_t* sa = smem + ring.stage * kStageBytes;
+  uint8_t* sa = smem + ring.stage * kStageBytes<BN>;
   if (leader) {
-    mbar_arrive_expect_tx(&full_bar[ring.stage], kPair * (kABytes + kBBytes));
+    mbar_arrive_expect_tx(&full_bar[ring.stage], kPair * kStageBytes<BN>);
     armed_parity[ring.stage] = ring.phase;
   }
   const uint32_t bar = mapa_shared(&full_bar[ring.stage], 0);
@@ -472,117 +474,62 @@ __device__ __noinline__ Ring load_lora_stage(const GemmArgs& a, const Tile& tl, 
   return ring;
 }
 
-// MMAs of an XA tile: per K block the tile's product into d_tmem and the XA product x A^T into
-// the other accumulator's first xa_n columns (x_tmem); then xa_full for the epilogue warps, which
-// drain the XA product (xa_done, having written it into the tile's LoRA stage) before the LoRA
-// stage, or the next tile, may use those columns.
+// MMAs of an XA item into d_tmem's first xa_n columns. One this narrow still takes about 115 cycles (a
+// full tile's 128), the latency of the sum it adds to; spread over two or four accumulators they took
+// longer (1.5B down, 2003 rows: 60 -> 76 us).
 template <int BN, int STAGES>
-__device__ __noinline__ Ring mma_xa_tile(const GemmArgs& a, const Tile& tl, uint32_t d_tmem, uint32_t x_tmem,
-                                         uint32_t idesc, uint32_t idesc_xa, uint8_t* smem, uint64_t* full_bar,
-                                         uint64_t* empty_bar, uint64_t* xa_full, uint64_t* xa_done,
-                                         uint32_t xa_parity, volatile int* abort_flag, Ring ring) {
+__device__ __noinline__ Ring mma_xa_item(const GemmArgs& a, uint32_t d_tmem, uint32_t idesc_xa,
+                                         uint8_t* smem, uint64_t* full_bar, uint64_t* empty_bar,
+                                         volatile int* abort_flag, Ring ring) {
   for (int kb = 0; kb < a.num_kb; ++kb) {
     if (!mbar_wait(&full_bar[ring.stage], ring.phase, abort_flag, a.status)) {
       ring.ok = 0;
       return ring;
     }
     tc_fence_after();
-    const uint32_t sa = smem_u32(smem + ring.stage * kStageBytes);
+    const uint32_t sa = smem_u32(smem + ring.stage * kStageBytes<BN>);
     const uint64_t ad = smem_desc(sa, 16, 1024, kSwizzle128B);
-    const uint64_t bd = smem_desc(sa + kABytes, 16, 1024, kSwizzle128B);
-    const uint64_t ld = smem_desc(sa + kABytes + kBBytes, 16, 1024, kSwizzle128B);
+    const uint64_t ld = smem_desc(sa + kABytes, 16, 1024, kSwizzle128B);
 #pragma unroll
-    for (int k = 0; k < BK / 16; ++k) {
-      const uint32_t acc = (kb > 0 || k > 0) ? 1u : 0u;
-      mma_bf16_ss_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, acc);
-      mma_bf16_ss_pair(x_tmem, ad + 2 * k, ld + 2 * k, idesc_xa, acc);
-    }
-    mma_commit_pair(&empty_bar[ring.stage], 0x3);
-    ring_next<STAGES>(ring);
-  }
-  mma_commit_pair(xa_full, 0x3);
-  if (!mbar_wait<true>(xa_done, xa_parity, abort_flag, a.status)) {
-    ring.ok = 0;
-    return ring;
-  }
-  tc_fence_after();
-  if (a.ext_on[tl.g]) {
-    // BX copies landed; the A side (the XA product) came with xa_done
-    if (!mbar_wait(&full_bar[ring.stage], ring.phase, abort_flag, a.status)) {
-      ring.ok = 0;
-      return ring;
-    }
-    tc_fence_after();
-    const uint32_t sa = smem_u32(smem + ring.stage * kStageBytes);
-    const uint64_t ad = smem_desc(sa, 16, 1024, kSwizzle128B);
-    const uint64_t bd = smem_desc(sa + kABytes, 16, 1024, kSwizzle128B);
-    for (int k = 0; k < a.ext_steps[tl.g]; ++k) mma_bf16_ss_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, 1u);
+    for (int k = 0; k < BK / 16; ++k)
+      mma_bf16_ss_pair(d_tmem, ad + 2 * k, ld + 2 * k, idesc_xa, (kb > 0 || k > 0) ? 1u : 0u);
     mma_commit_pair(&empty_bar[ring.stage], 0x3);
     ring_next<STAGES>(ring);
   }
   return ring;
 }
 
-// XA tile, after its main loop: slot j of the XA product (columns 16j .. 16j + 15 of x_tmem) is
-// x A_j^T for this thread's row. Scaled by alpha / r it is stored as hi = bf16(v) at XA columns
-// 32j.. and lo = bf16(v - hi) at 32j + 16.. (the pair carries about 16 mantissa bits): to the XA
-// buffer for the row block's other tiles, and into the tile's own LoRA stage `st` (A side, the 64
-// columns from xa_base) when it has one. Then xa_done for the MMAs and the row block's ready word.
-template <int BN>
-__device__ __noinline__ bool drain_xa(const GemmArgs& a, const Tile& tl, uint32_t x_tmem, int row, int row_in_cta,
-                                      int st, int lane, uint8_t* smem, uint64_t* xa_full, uint64_t* xa_done,
-                                      uint32_t xa_parity, volatile int* abort_flag) {
-  if (!__all_sync(0xffffffffu, mbar_wait(xa_full, xa_parity, abort_flag, a.status))) return false;
-  tc_fence_after();
-  const bool ext = a.ext_on[tl.g] != 0;
-  const int xb = a.xa_base[tl.g];
-  uint8_t* arow = smem + st * kStageBytes + row_in_cta * 128;
-  uint32_t r0[16];
-  float v[16], w[16];
-#pragma unroll 1
-  for (int j = 0; j < a.n_slots; ++j) {
-    tmem_ld16(x_tmem + 16 * j, r0);
-    tmem_ld_wait();
+// XA item, after its MMAs: slot j (columns 16j .. 16j + 15 of tacc) is x A_j^T for this thread's row.
+// Scaled by alpha / r it is stored as hi = bf16(v) at XA columns 32j.. and lo = bf16(v - hi) at
+// 32j + 16.. (the pair carries about 16 mantissa bits); then the warp counts into the ready word.
+__device__ __noinline__ void drain_xa(const GemmArgs& a, int m_blk, uint32_t tacc, int row, int lane) {
+  uint32_t r[3][16];
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+    if (j < a.n_slots) tmem_ld16(tacc + 16 * j, r[j]);
+  tmem_ld_wait();
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    if (j >= a.n_slots || row >= a.M) continue;
+    float v[16], w[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-      v[i] = __uint_as_float(r0[i]) * a.scale;
+      v[i] = __uint_as_float(r[j][i]) * a.scale;
       w[i] = v[i] - __bfloat162float(__float2bfloat16_rn(v[i]));
     }
-    if (row < a.M) {
-      store16_bf16(a.xa + (size_t)row * kXaCols + 32 * j, v);
-      store16_bf16(a.xa + (size_t)row * kXaCols + 32 * j + 16, w);
-    }
-    const int c0 = (32 * j - xb) / 8;  // 16-byte unit of hi within the stage's 64 columns
-    if (ext && 32 * j >= xb && 32 * j < xb + BK) {
-      uint4 q[4];
-      q[0] = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
-      q[1] = make_uint4(pack_bf16(v[8], v[9]), pack_bf16(v[10], v[11]), pack_bf16(v[12], v[13]),
-                        pack_bf16(v[14], v[15]));
-      q[2] = make_uint4(pack_bf16(w[0], w[1]), pack_bf16(w[2], w[3]), pack_bf16(w[4], w[5]), pack_bf16(w[6], w[7]));
-      q[3] = make_uint4(pack_bf16(w[8], w[9]), pack_bf16(w[10], w[11]), pack_bf16(w[12], w[13]),
-                        pack_bf16(w[14], w[15]));
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        *reinterpret_cast<uint4*>(arow + (((c0 + u) ^ (row_in_cta & 7)) << 4)) = q[u];
-    }
+    store16_bf16(a.xa + (size_t)row * kXaCols + 32 * j, v);
+    store16_bf16(a.xa + (size_t)row * kXaCols + 32 * j + 16, w);
   }
-  // TMEM columns read (tcgen05.wait::ld above); XA rows visible to the tensor core of this CTA
-  // (shared) and to the other tiles' copies (global, GPU scope)
-  tc_fence_before();
-  fence_proxy_async_smem();
+  // XA rows visible to the tiles' copies (global, GPU scope)
   __threadfence();
   fence_proxy_async_global();
   __syncwarp();
-  if (lane == 0) {
-    mbar_arrive_cluster(mapa_shared(xa_done, 0));
-    atomicAdd(a.xa_flags + tl.m_blk, 1);
-  }
-  return true;
+  if (lane == 0) atomicAdd(a.xa_flags + m_blk, 1);
 }
 
 template <int BN, int STAGES, int EPI>
 __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_constant__ GemmArgs a) {
-  static_assert(BN == 256 && kBBytes == (BN / kPair) * BK * 2, "CTA-pair tiles of 256 columns");
+  static_assert(BN == 256 || BN == 128, "CTA-pair tiles of 256 or 128 columns");
   constexpr uint32_t TMEM_COLS = 2 * BN;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -592,8 +539,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   __shared__ __align__(8) uint64_t tfull_bar[2];
   __shared__ __align__(8) uint64_t tempty_bar[2];
   __shared__ __align__(8) uint64_t drain_bar;
-  __shared__ __align__(8) uint64_t xa_full;         // an XA tile's MMAs done (MMA commit)
-  __shared__ __align__(8) uint64_t xa_done;         // its XA product drained (each epilogue warp of both CTAs)
   __shared__ uint32_t tmem_base_sh;
   __shared__ volatile int abort_flag;
   // a rejected call: every CTA of every cluster sees the same word and leaves before any set-up
@@ -616,8 +561,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       mbar_init(&tempty_bar[i], 4 * kPair);
     }
     mbar_init(&drain_bar, 1);
-    mbar_init(&xa_full, 1);
-    mbar_init(&xa_done, 4 * kPair);
     abort_flag = 0;
     fence_barrier_init();
   }
@@ -642,28 +585,28 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (every CTA)
     // The per-stage loop of the output tiles stays minimal (one thread, on the critical path of
-    // every stage); XA tiles and the LoRA stage go through out-of-line helpers.
+    // every stage); XA items and the LoRA stage go through out-of-line helpers.
     if (lane == 0) {
       Ring ring{0, 0u, 1};
       int armed_parity[STAGES];
       for (int s = 0; s < STAGES; ++s) armed_parity[s] = -1;
-      for (int t = unit; t < a.total_tiles && ring.ok; t += n_units) {
+      for (int t = unit; t < a.total_items && ring.ok; t += n_units) {
         const Tile tl = decode_tile(t, a);
         const int m0 = tl.m_blk * (BM * kPair) + static_cast<int>(rank) * BM;
         if (tl.xa) {
-          ring = load_xa_tile<BN, STAGES>(a, tl, m0, rank, leader, smem, full_bar, empty_bar, armed_parity,
+          ring = load_xa_item<BN, STAGES>(a, m0, rank, leader, smem, full_bar, empty_bar, armed_parity,
                                           &abort_flag, ring);
           continue;
         }
         int g0, nb, yb, b_step;
         tile_b_rows<BN>(a, tl, rank, g0, nb, yb, b_step);
         // Whether the row block's XA rows are stored, asked (acquire) while the stages already
-        // copied still feed the MMAs; only a tile whose XA tile has not finished by then waits at
-        // its LoRA stage.
+        // copied still feed the MMAs; only a tile whose row block's XA items have not finished by
+        // then waits at its LoRA stage.
         int xa_ready = 0;
         if (a.ext_on[tl.g]) {
           asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(xa_ready) : "l"(a.xa_flags + tl.m_blk) : "memory");
-          xa_ready = xa_ready >= 4 * kPair;
+          xa_ready = xa_ready >= kXaGroups;
         }
         int stage = ring.stage;
         uint32_t phase = ring.phase;
@@ -672,11 +615,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             ring.ok = 0;
             break;
           }
-          uint8_t* sa = smem + stage * kStageBytes;
+          uint8_t* sa = smem + stage * kStageBytes<BN>;
           uint8_t* sb = sa + kABytes;
           // the MMA-issuing CTA's full barrier counts the bytes of both CTAs
           if (leader) {
-            mbar_arrive_expect_tx(&full_bar[stage], kPair * (kABytes + kBBytes));
+            mbar_arrive_expect_tx(&full_bar[stage], kPair * kStageBytes<BN>);
             armed_parity[stage] = phase;
           }
           const CUtensorMap* mB = &a.tmB[g0];
@@ -718,8 +661,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       bool issued = false;
       const uint32_t idesc = idesc_bf16_f32(BM * kPair, BN);
       const uint32_t idesc_xa = idesc_bf16_f32(BM * kPair, a.n_slots > 0 ? a.xa_n : 32);
-      uint32_t xa_it = 0;      // XA tiles so far (phase of xa_done)
-      for (int t = unit; t < a.total_tiles && ring.ok; t += n_units, ++it) {
+      for (int t = unit; t < a.total_items && ring.ok; t += n_units, ++it) {
         const Tile tl = decode_tile(t, a);
         const int acc = it & 1;
         const uint32_t acc_phase = (it >> 1) & 1;
@@ -730,16 +672,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * BN;
         if (tl.xa) {
-          // the XA product takes the other accumulator's first columns: its previous tile's
-          // epilogue must have drained them
-          if (!mbar_wait<true>(&tempty_bar[acc ^ 1], (((it + 1) >> 1) & 1) ^ 1, &abort_flag, a.status)) {
-            ring.ok = 0;
-            break;
-          }
-          tc_fence_after();
-          ring = mma_xa_tile<BN, STAGES>(a, tl, d_tmem, tmem_base + (acc ^ 1) * BN, idesc, idesc_xa, smem, full_bar,
-                                         empty_bar, &xa_full, &xa_done, xa_it & 1u, &abort_flag, ring);
-          ++xa_it;
+          ring = mma_xa_item<BN, STAGES>(a, d_tmem, idesc_xa, smem, full_bar, empty_bar, &abort_flag, ring);
           issued = true;
           if (!ring.ok) break;
           mma_commit_pair(&tfull_bar[acc], 0x3);
@@ -753,7 +686,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             break;
           }
           tc_fence_after();
-          const uint32_t sa = smem_u32(smem + stage * kStageBytes);
+          const uint32_t sa = smem_u32(smem + stage * kStageBytes<BN>);
           const uint64_t ad = smem_desc(sa, 16, 1024, kSwizzle128B);
           const uint64_t bd = smem_desc(sa + kABytes, 16, 1024, kSwizzle128B);
           // K = 16 steps advance 32 bytes = 2 units of the descriptor's start-address field
@@ -775,7 +708,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             ring.ok = 0;
           } else {
             tc_fence_after();
-            const uint32_t sa = smem_u32(smem + ring.stage * kStageBytes);
+            const uint32_t sa = smem_u32(smem + ring.stage * kStageBytes<BN>);
             const uint64_t ad = smem_desc(sa, 16, 1024, kSwizzle128B);
             const uint64_t bd = smem_desc(sa + kABytes, 16, 1024, kSwizzle128B);
             for (int k = 0; k < a.ext_steps[tl.g]; ++k) mma_bf16_ss_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, 1u);
@@ -798,30 +731,21 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     const int row_in_cta = quarter * 32 + lane;
     uint32_t tempty_addr[2];
     for (int i = 0; i < 2; ++i) tempty_addr[i] = mapa_shared(&tempty_bar[i], 0);
-    int pos = 0;             // producer stages used by the tiles before this one
-    uint32_t xa_it = 0;      // XA tiles so far (phase of xa_full)
     int it = 0;
-    for (int t = unit; t < a.total_tiles; t += n_units, ++it) {
+    for (int t = unit; t < a.total_items; t += n_units, ++it) {
       const Tile tl = decode_tile(t, a);
       const int acc = it & 1;
       const uint32_t acc_phase = (it >> 1) & 1;
-      const bool ext_tile = a.ext_on[tl.g] != 0;
-      const int st = (pos + a.num_kb) % STAGES;  // the tile's LoRA stage
       const int row = tl.m_blk * (BM * kPair) + static_cast<int>(rank) * BM + row_in_cta;
-      if (tl.xa) {
-        const uint32_t x_tmem = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + (acc ^ 1) * BN;
-        if (!drain_xa<BN>(a, tl, x_tmem, row, row_in_cta, st, lane, smem, &xa_full, &xa_done, xa_it & 1u,
-                          &abort_flag))
-          break;
-        ++xa_it;
-      }
-      pos += a.num_kb + (ext_tile ? 1 : 0);
       // warp-uniform outcome: the TMEM loads of the epilogue are warp-collective
       if (!__all_sync(0xffffffffu, mbar_wait(&tfull_bar[acc], acc_phase, &abort_flag, a.status)))
         break;
       tc_fence_after();
       const uint32_t tacc = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BN;
-      epilogue_tile<BN, EPI>(a, tl, tacc, row);
+      if (tl.xa)
+        drain_xa(a, tl.m_blk, tacc, row, lane);
+      else
+        epilogue_tile<BN, EPI>(a, tl, tacc, row, lane, smem + STAGES * kStageBytes<BN> + quarter * 4096);
       // the accumulator is free once this warp's TMEM loads have completed (tcgen05.wait::ld in
       // the epilogue); the tile's global stores need not be visible first, so the arrival on
       // the MMA-issuing CTA's barrier is relaxed
@@ -876,7 +800,7 @@ bool make_map(CUtensorMap* m, const void* base, int rows, int cols, int ld, int 
 template <int BN, int STAGES, int EPI>
 cudaError_t launch_impl(GemmArgs& args, int num_sms, cudaStream_t stream) {
   constexpr int PAIR = kPair;
-  constexpr int smem = STAGES * kStageBytes + 1024;
+  constexpr int smem = STAGES * kStageBytes<BN> + kScratchBytes + 1024;
   auto kern = gemm_tc_kernel<BN, STAGES, EPI>;
   // the attributes and the co-resident cluster count are per device
   static PerDevice once;
@@ -908,11 +832,9 @@ cudaError_t launch_impl(GemmArgs& args, int num_sms, cudaStream_t stream) {
     once.done(dev);
   }
   // every unit of the grid is resident at once (one CTA per SM): a tile that waits for its row
-  // block's XA tile never waits on a unit that has not started
-  const int units = std::max(1, std::min(max_units, args.total_tiles));
-  // every XA tile first: consecutive tiles go to consecutive units, so the XA products (and the
-  // extra MMAs they cost) spread over the units instead of piling on a few
-  args.xa_lead = args.row_tiles;
+  // block's XA items never waits on a unit that has not started, and every unit runs its XA items
+  // before its tiles
+  const int units = std::max(1, std::min(max_units, args.total_items));
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -928,13 +850,40 @@ cudaError_t launch_impl(GemmArgs& args, int num_sms, cudaStream_t stream) {
   return cudaLaunchKernelEx(&cfg, kern, args);
 }
 
+int group_tiles(const GemmDesc& d, int g, int bn) {
+  if (d.nseg > 1 && d.epi != kEpiSwiGLU) return 1;
+  const int cols = d.nseg > 1 ? bn / d.nseg : bn;
+  return (d.group_cols[g] + cols - 1) / cols;
+}
+
+// 256-column tiles run the MMAs at their best rate; 128-column ones leave less of the last wave empty
+// and half the epilogue exposed at its end. Compared in K blocks of a 256-column tile: a tile's
+// hand-over costs about two, the last epilogue 10 and 5. Which one is taken changes no result: an
+// element's K order is the same.
+int tile_columns(const GemmDesc& d, int row_tiles, int num_kb, int units) {
+  // 128-column block 0.8: its operands are half again as many bytes from L2 per FLOP (down of a 7B
+  // batch of 8228 rows: 445 us on 256 columns, 754 on 128)
+  double cost[2];
+  for (int i = 0; i < 2; ++i) {
+    const int bn = i == 0 ? 256 : 128;
+    long tiles = 0;
+    for (int g = 0; g < d.ngroups; ++g) tiles += static_cast<long>(group_tiles(d, g, bn)) * row_tiles;
+    const long waves = (tiles + units - 1) / std::max(1, units);
+    cost[i] = waves * (num_kb * (i == 0 ? 1.0 : 0.8) + 2) + (i == 0 ? 10 : 5);
+  }
+  return cost[1] < cost[0] ? 128 : 256;
+}
+
 }  // namespace
 
 cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t stream) {
-  constexpr int bn = 256, pair = 2;
+  constexpr int pair = kPair;
   GemmArgs a;
   std::memset(&a, 0, sizeof(a));
   if (d.nseg != 1 && d.nseg != 2) return cudaErrorInvalidValue;
+  a.num_kb = (d.K + BK - 1) / BK;
+  a.row_tiles = (d.M + BM * pair - 1) / (BM * pair);
+  const int bn = tile_columns(d, a.row_tiles, a.num_kb, num_sms / pair);
   // rows of one B load: the CTA's share of the tile (plain) or one stacked segment
   const int b_box = d.nseg == 1 ? bn / pair : bn / d.nseg;
   if (!make_map(&a.tmA, d.A, d.M, d.K, d.lda, BM, BK, CU_TENSOR_MAP_SWIZZLE_128B))
@@ -983,29 +932,25 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t stream) {
   }
   a.M = d.M;
   a.K = d.K;
-  a.num_kb = (d.K + BK - 1) / BK;
   a.ngroups = d.ngroups;
   a.nseg = d.nseg;
   a.total_n = 0;
   for (int g = 0; g < d.ngroups; ++g) {
-    const int cols_per_tile = (d.nseg > 1 && d.epi == kEpiSwiGLU) ? bn / d.nseg : bn;
     a.group_cols[g] = d.group_cols[g];
-    a.group_tiles[g] = (d.nseg > 1 && d.epi != kEpiSwiGLU) ? 1
-                                                            : (d.group_cols[g] + cols_per_tile - 1) /
-                                                                  cols_per_tile;
+    a.group_tiles[g] = group_tiles(d, g, bn);
     a.total_n += a.group_tiles[g];
     a.ext_on[g] = d.ext_on[g];
     a.ext_steps[g] = d.ext_steps[g];
     a.xa_base[g] = d.xa_base[g];
   }
-  a.row_tiles = (d.M + BM * pair - 1) / (BM * pair);
   a.n_slots = any_ext ? d.n_slots : 0;
   // two CTA halves of 16 x ceil(n_slots / 2) rows: N = 32 for one or two slots, 64 for three
   a.xa_n = 32 * ((a.n_slots + 1) / 2);
   a.rank = d.rank;
   a.xa = static_cast<__nv_bfloat16*>(d.XA);
   a.xa_flags = d.xa_flags;
-  a.total_tiles = a.row_tiles * a.total_n;
+  a.xa_items = a.n_slots > 0 ? a.row_tiles : 0;
+  a.total_items = a.xa_items + a.row_tiles * a.total_n;
   a.epi = d.epi;
   a.scale = d.scale;
   a.out = static_cast<__nv_bfloat16*>(d.out);
@@ -1014,6 +959,7 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t stream) {
   a.ld_resid = d.ld_resid;
   for (int i = 0; i < 3; ++i) a.bias[i] = static_cast<const __nv_bfloat16*>(d.bias[i]);
   a.rope = d.rope;
+  a.rope_positions = d.rope_positions;
   a.head_dim = d.head_dim;
   a.n_kv_heads = d.n_kv_heads;
   a.qbuf = static_cast<__nv_bfloat16*>(d.qbuf);
@@ -1023,13 +969,19 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t stream) {
   a.req = d.req;
   a.status = d.status;
   a.abort = d.abort;
-  if (a.total_tiles == 0) return cudaSuccess;
+  if (d.M == 0 || a.total_n == 0) return cudaSuccess;
   // one kernel per epilogue: each carries only its own epilogue code, which keeps the hot loops
   // of all its warps inside the SM's instruction cache
+  if (bn == 128) switch (d.epi) {
+      case kEpiQkv: return launch_impl<128, 8, kEpiQkv>(a, num_sms, stream);
+      case kEpiResid: return launch_impl<128, 8, kEpiResid>(a, num_sms, stream);
+      case kEpiSwiGLU: return launch_impl<128, 8, kEpiSwiGLU>(a, num_sms, stream);
+      default: return cudaErrorInvalidValue;
+    }
   switch (d.epi) {
-    case kEpiQkv: return launch_impl<bn, 6, kEpiQkv>(a, num_sms, stream);
-    case kEpiResid: return launch_impl<bn, 6, kEpiResid>(a, num_sms, stream);
-    case kEpiSwiGLU: return launch_impl<bn, 6, kEpiSwiGLU>(a, num_sms, stream);
+    case kEpiQkv: return launch_impl<256, 6, kEpiQkv>(a, num_sms, stream);
+    case kEpiResid: return launch_impl<256, 6, kEpiResid>(a, num_sms, stream);
+    case kEpiSwiGLU: return launch_impl<256, 6, kEpiSwiGLU>(a, num_sms, stream);
     default: return cudaErrorInvalidValue;
   }
 }

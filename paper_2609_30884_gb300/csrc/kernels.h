@@ -99,10 +99,9 @@ struct GemmDesc {
   int B_rows[3];          // rows of each B matrix
   int ldb[3];
   int group_cols[3];      // valid output columns per group (plain) / per segment (stacked)
-  // Unmerged LoRA (Eq. S3), computed inside the same launch. The first output tile of each
-  // 256-row block also forms XA[:, 32j .. 32j + 32) = hi/lo of (alpha/r) x A_j^T for the n_slots
-  // adapted modules (LA[j] = A_j, [rank, K]) and raises xa_flags[row block]; every output tile of
-  // an adapted group then adds one K block: XA[:, xa_base[g] .. + 64] against BX[i] (the module's
+  // Unmerged LoRA (Eq. S3), computed inside the same launch, which first forms XA[:, 32j .. 32j + 32) =
+  // hi/lo of (alpha/r) x A_j^T for the n_slots adapted modules (LA[j] = A_j, [rank, K]) of each
+  // 256-row block and raises xa_flags[row block]; every output tile of an adapted group then adds one K block: XA[:, xa_base[g] .. + 64] against BX[i] (the module's
   // [B | B] rows under its slot, zeros elsewhere; [B_rows[i], kBxCols], map index i like B).
   void* XA;
   int n_slots;
@@ -121,7 +120,8 @@ struct GemmDesc {
   const void* resid;
   int ld_resid;
   const void* bias[3];
-  const float2* rope;     // [positions][head_dim/2] (cos, sin)
+  const float2* rope;     // (cos, sin) of pair i at position p: entry ((i / 2) rope_positions + p) 2 + i % 2
+  int rope_positions;
   int head_dim, n_kv_heads;
   void* qbuf;
   int ldq;
@@ -136,6 +136,8 @@ struct GemmDesc {
 cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t stream);
 
 // ------------------------------------------------------------------ other kernels
+// (cos, sin) of pair i at position p at table[((i / 2) n_pos + p) 2 + i % 2]: neighbouring rows of a
+// projection read neighbouring entries.
 cudaError_t launch_rope_table(float2* table, int n_pos, int head_dim, double theta,
                               cudaStream_t stream);
 // BX rows of up to 4 modules: out[m][r, :] = 0 except columns [col_off[m], col_off[m] + 32) =
@@ -270,8 +272,8 @@ struct DecodeAttnDesc {
   RowUp up[3];
   RowLora lora;
   const __nv_bfloat16* bias[3];
-  const float2* rope;      // (cos, sin) [positions][head_dim / 2], or [rows][head_dim / 2] with rope_by_row
-  int rope_by_row;
+  const float2* rope;      // launch_rope_table's table, or [rows][head_dim / 2] with rope_by_row
+  int rope_by_row, rope_positions;
   __nv_bfloat16* kpages;
   __nv_bfloat16* vpages;
   int write_kv;            // the row's own k, v go into slot pos % 16 of page page_table[pos / 16]

@@ -13,7 +13,7 @@ namespace crf {
 namespace {
 
 // ------------------------------------------------------------------ RoPE table
-// table[p][i] = (cos, sin)(p * theta^(-2i/d)): the angle in turns, p * theta^(-2i/d) / (2 pi),
+// table[((i / 2) n_pos + p) 2 + i % 2] = (cos, sin)(p * theta^(-2i/d)): the angle in turns, p * theta^(-2i/d) / (2 pi),
 // is formed in fp64 (per-frequency factors computed on the host in fp64), reduced to [0, 1)
 // and evaluated with fp32 sincospi.
 struct RopeFreqs {
@@ -23,7 +23,7 @@ struct RopeFreqs {
 __global__ void rope_table_kernel(float2* table, int n_pos, int half, const __grid_constant__ RopeFreqs f) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n_pos * half) return;
-  const int p = idx / half, i = idx % half;
+  const int p = idx / 2 % n_pos, i = idx / 2 / n_pos * 2 + idx % 2;
   double turns = static_cast<double>(p) * f.turns_per_pos[i];
   turns -= floor(turns);
   float s, c;
