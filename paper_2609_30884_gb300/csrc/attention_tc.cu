@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
   const int J0 = ntiles == 2 ? J - 1 : J;  // kv tiles of query tile 0 (its diagonal is tile J0-1)
   const int n_pages = (n + kPage - 1) / kPage;
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);  // uniform
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     mbar_init(&q_full, 1);
@@ -241,44 +241,56 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
   if (warp < 4) {
     // setmaxnreg inside each role's branch: the softmax code is never reachable from here
     regs_dec_ctl();
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
       // ---------------------------------------------------------------- producer
+      // The whole warp runs the loop, one lane issues; a tile's page ids are read by eight lanes
+      // together, the next tile's while this one's copies are issued.
+      const bool issuer = elect_one();
       bool ok = true;
-      int armed[kSlots];
-      for (int i = 0; i < kSlots; ++i) armed[i] = -1;
-      mbar_arrive_expect_tx(&q_full, ntiles * Q_BYTES);
-      for (int t = 0; t < ntiles; ++t)
-        for (int h = 0; h < HALVES; ++h)
-          tma_load_2d(sQ + t * Q_BYTES + h * (kM * 128), &a.tmQ, &q_full, w.head * D + 64 * h,
-                      row0 + q0 + t * kM);
+      int armed = 0;  // ring items issued
+      if (issuer) {
+        mbar_arrive_expect_tx(&q_full, ntiles * Q_BYTES);
+        for (int t = 0; t < ntiles; ++t)
+          for (int h = 0; h < HALVES; ++h)
+            tma_load_2d(sQ + t * Q_BYTES + h * (kM * 128), &a.tmQ, &q_full, w.head * D + 64 * h,
+                        row0 + q0 + t * kM);
+      }
       int slot = 0;
       uint32_t ph = 0;
-      for (int i = 0; i < 2 * J && ok; ++i) {
-        const int j = i >> 1;
-        const int kv = i & 1;
-        if (!mbar_wait(&kv_empty[slot], ph ^ 1, &abort_flag, a.status)) {
-          ok = false;
-          break;
+      // pages past the prefix repeat the last page: finite data, masked below
+      auto page_id = [&](int j) {
+        return checked_page(pt[min(j * kPagesPerTile + (lane & (kPagesPerTile - 1)), n_pages - 1)], a.req.num_pages,
+                            a.status);
+      };
+      int ids = page_id(0);
+      for (int j = 0; j < J && ok; ++j) {
+        const int next_ids = j + 1 < J ? page_id(j + 1) : 0;
+        for (int kv = 0; kv < 2; ++kv) {
+          ok = mbar_wait_warp(&kv_empty[slot], ph ^ 1, &abort_flag, a.status);
+          if (!ok) break;
+          if (issuer) mbar_arrive_expect_tx(&kv_full[slot], KV_BYTES);
+          uint8_t* dst = sKV + slot * KV_BYTES;
+          const CUtensorMap* map = kv == 0 ? &a.tmK : &a.tmV;
+#pragma unroll
+          for (int p = 0; p < kPagesPerTile; ++p) {
+            const int group = (__shfl_sync(0xffffffffu, ids, p) * a.n_kv_heads + w.g) * (kPage / 8);
+            if (issuer) tma_load_4d(dst + p * (kPage / 8) * GROUP_BYTES, map, &kv_full[slot], 0, 0, 0, group);
+          }
+          ++armed;
+          if (++slot == kSlots) {
+            slot = 0;
+            ph ^= 1;
+          }
         }
-        mbar_arrive_expect_tx(&kv_full[slot], KV_BYTES);
-        uint8_t* dst = sKV + slot * KV_BYTES;
-        const CUtensorMap* map = kv == 0 ? &a.tmK : &a.tmV;
-        for (int p = 0; p < kPagesPerTile; ++p) {
-          // pages past the prefix repeat the last page: finite data, masked below
-          const int page = checked_page(pt[min(j * kPagesPerTile + p, n_pages - 1)], a.req.num_pages, a.status);
-          const int group = (page * a.n_kv_heads + w.g) * (kPage / 8);
-          tma_load_4d(dst + p * (kPage / 8) * GROUP_BYTES, map, &kv_full[slot], 0, 0, 0, group);
-        }
-        armed[slot] = ph;
-        if (++slot == kSlots) {
-          slot = 0;
-          ph ^= 1;
-        }
+        ids = next_ids;
       }
       if (!ok) {
+        // every copy issued lands before the CTA can exit: the last use of every slot
         volatile int never = 0;
-        for (int i = 0; i < kSlots; ++i)
-          if (armed[i] >= 0) mbar_wait(&kv_full[i], armed[i], &never, nullptr);
+        for (int i = 0; i < kSlots && i < armed; ++i) {
+          const int u = armed - 1 - i;
+          mbar_wait(&kv_full[u % kSlots], static_cast<uint32_t>((u / kSlots) & 1), &never, nullptr);
+        }
         mbar_wait(&q_full, 0, &never, nullptr);
       }
     } else if (warp == 1) {
@@ -287,18 +299,17 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
       // query tile overlaps the products of the other; query tile 0 stops one kv tile early
       // (its diagonal), after which tile 1 runs alone. tcgen05.mma of one thread execute in
       // issue order, so S_t(j+1) overwrites the S/P columns only after PV_t(j) has read P_t(j).
-      if (lane == 0) {
-        bool ok = mbar_wait(&q_full, 0, &abort_flag, a.status);
-        bool issued = false;
-        const uint32_t idesc_s = idesc_bf16_f32(kM, kN);
-        const uint32_t idesc_o = idesc_bf16_f32(kM, D, false, true);
-        // ring position of sequence item i (K(j): i = 2j, V(j): i = 2j + 1)
-        auto slot_of = [](int i) { return i % kSlots; };
-        auto parity_of = [](int i) { return static_cast<uint32_t>((i / kSlots) & 1); };
-        auto issue_s = [&](int t, int ks) {
-          const uint32_t kb = smem_u32(sKV + ks * KV_BYTES);
-          const uint32_t qb = smem_u32(sQ + t * Q_BYTES);
-  #pragma unroll
+      // The whole warp runs the loop, one lane issues.
+      const bool issuer = elect_one();
+      bool ok = mbar_wait_warp(&q_full, 0, &abort_flag, a.status);
+      bool issued = false;
+      const uint32_t idesc_s = idesc_bf16_f32(kM, kN);
+      const uint32_t idesc_o = idesc_bf16_f32(kM, D, false, true);
+      auto issue_s = [&](int t, int ks) {
+        const uint32_t kb = smem_u32(sKV + ks * KV_BYTES);
+        const uint32_t qb = smem_u32(sQ + t * Q_BYTES);
+        if (issuer) {
+#pragma unroll
           for (int kk = 0; kk < D / 16; ++kk) {
             const uint32_t in_row = (kk & 3) * 32;
             mma_bf16_ss(tmem + t * 128,
@@ -307,40 +318,45 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
                         idesc_s, kk > 0 ? 1u : 0u);
           }
           mma_commit(&s_full[t]);
-        };
-        if (ok) ok = mbar_wait(&kv_full[slot_of(0)], parity_of(0), &abort_flag, a.status);
-        if (ok) {
-          tc_fence_after();
-          for (int t = 0; t < ntiles; ++t) issue_s(t, slot_of(0));
-          issued = true;
         }
-        for (int j = 0; j < J && ok; ++j) {
-          const uint32_t vb = smem_u32(sKV + slot_of(2 * j + 1) * KV_BYTES);
-          const int ks = slot_of(2 * j + 2);
-          for (int t = (j < J0 ? 0 : 1); t < ntiles; ++t) {
-            // phase j of p_full[t]: P_t(j) is in TMEM, and V(j) and K(j + 1) have landed
-            if (!mbar_wait(&p_full[t], j & 1, &abort_flag, a.status)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-  #pragma unroll
+      };
+      if (ok) ok = mbar_wait_warp(&kv_full[0], 0, &abort_flag, a.status);
+      if (ok) {
+        tc_fence_after();
+        for (int t = 0; t < ntiles; ++t) issue_s(t, 0);
+        issued = true;
+      }
+      // ring slot of V(j); K(j + 1) is in the one after it
+      int vs = 1;
+      for (int j = 0; j < J && ok; ++j) {
+        const uint32_t vb = smem_u32(sKV + vs * KV_BYTES);
+        const int ks = vs + 1 == kSlots ? 0 : vs + 1;
+        for (int t = (j < J0 ? 0 : 1); t < ntiles; ++t) {
+          // phase j of p_full[t]: P_t(j) is in TMEM, and V(j) and K(j + 1) have landed
+          if (!mbar_wait_warp(&p_full[t], j & 1, &abort_flag, a.status)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          if (issuer) {
+#pragma unroll
             for (int kk = 0; kk < kN / 16; ++kk) {
               // P: 16 keys = 8 packed bf16x2 columns; V: 16 key rows = two 8-key groups
               mma_bf16_ts(tmem + 256 + t * 128, tmem + t * 128 + kk * 8,
                           smem_desc(vb + kk * 2 * GROUP_BYTES, 1024, GROUP_BYTES, kSwizzle128B), idesc_o,
                           (j > 0 || kk > 0) ? 1u : 0u);
             }
-            if (j + 1 < (t == 0 ? J0 : J)) issue_s(t, ks);
           }
+          if (j + 1 < (t == 0 ? J0 : J)) issue_s(t, ks);
         }
-        if (ok) {
-          mma_commit(&o_full);
-        } else if (issued) {
-          mma_commit(&drain_bar);
-          volatile int never = 0;
-          mbar_wait(&drain_bar, 0, &never, nullptr);
-        }
+        vs = ks + 1 == kSlots ? 0 : ks + 1;
+      }
+      if (ok) {
+        if (issuer) mma_commit(&o_full);
+      } else if (issued && issuer) {
+        mma_commit(&drain_bar);
+        volatile int never = 0;
+        mbar_wait(&drain_bar, 0, &never, nullptr);
       }
     }
   } else {

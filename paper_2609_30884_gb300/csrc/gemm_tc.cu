@@ -387,11 +387,12 @@ constexpr int kBBytes = BN / kPair * BK * 2;
 template <int BN>
 constexpr int kStageBytes = kABytes + kBBytes<BN>;
 
-// Producer ring position (stage, phase) and whether every wait so far succeeded.
+// Ring position (stage, phase) and whether every wait so far succeeded.
 struct Ring {
   int stage;
   uint32_t phase;
   int ok;
+  int used;  // stages the producer has filled so far
 };
 
 template <int STAGES>
@@ -419,26 +420,26 @@ __device__ __forceinline__ void tile_b_rows(const GemmArgs& a, const Tile& tl, u
 // Copies of an XA item: per K block the row block's x rows and the LoRA A rows of this
 // CTA's half of the XA product (16 rows per XA slot; CTA r takes slots [r * spc, r * spc + spc)).
 template <int BN, int STAGES>
-__device__ __noinline__ Ring load_xa_item(const GemmArgs& a, int m0, uint32_t rank, bool leader,
-                                          uint8_t* smem, uint64_t* full_bar, uint64_t* empty_bar,
-                                          int* armed_parity, volatile int* abort_flag, Ring ring) {
+__device__ __forceinline__ Ring load_xa_item(const GemmArgs& a, int m0, uint32_t rank, bool leader, bool issuer,
+                                             uint8_t* smem, uint64_t* full_bar, uint64_t* empty_bar,
+                                             volatile int* abort_flag, Ring ring) {
   const int spc = a.xa_n / (16 * kPair);
   const int s0 = static_cast<int>(rank) * spc, s1 = min(a.n_slots, s0 + spc);
   const uint32_t bytes = kPair * kABytes + a.n_slots * 16 * BK * 2;
   for (int kb = 0; kb < a.num_kb; ++kb) {
-    if (!mbar_wait(&empty_bar[ring.stage], ring.phase ^ 1, abort_flag, a.status)) {
+    if (!mbar_wait_warp(&empty_bar[ring.stage], ring.phase ^ 1, abort_flag, a.status)) {
       ring.ok = 0;
       return ring;
     }
     uint8_t* sa = smem + ring.stage * kStageBytes<BN>;
     uint8_t* sl = sa + kABytes;
-    if (leader) {
-      mbar_arrive_expect_tx(&full_bar[ring.stage], bytes);
-      armed_parity[ring.stage] = ring.phase;
+    if (issuer) {
+      if (leader) mbar_arrive_expect_tx(&full_bar[ring.stage], bytes);
+      const uint32_t bar = mapa_shared(&full_bar[ring.stage], 0);
+      tma_load_2d_pair(sa, &a.tmA, bar, kb * BK, m0);
+      for (int j = s0; j < s1; ++j) tma_load_2d_pair(sl + (j - s0) * 16 * BK * 2, &a.tmLA[j], bar, kb * BK, 0);
     }
-    const uint32_t bar = mapa_shared(&full_bar[ring.stage], 0);
-    tma_load_2d_pair(sa, &a.tmA, bar, kb * BK, m0);
-    for (int j = s0; j < s1; ++j) tma_load_2d_pair(sl + (j - s0) * 16 * BK * 2, &a.tmLA[j], bar, kb * BK, 0);
+    ++ring.used;
     ring_next<STAGES>(ring);
   }
   return ring;
@@ -448,28 +449,28 @@ __device__ __noinline__ Ring load_xa_item(const GemmArgs& a, int m0, uint32_t ra
 // block's XA rows are stored, and copy those rows (the A side of the K block) and the tile's BX rows
 // (the B side).
 template <int BN, int STAGES>
-__device__ __noinline__ Ring load_lora_stage(const GemmArgs& a, const Tile& tl, int m0, uint32_t rank, bool xa_ready,
-                                             bool leader, uint8_t* smem, uint64_t* full_bar, uint64_t* empty_bar,
-                                             int* armed_parity, volatile int* abort_flag, Ring ring) {
-  if (!mbar_wait(&empty_bar[ring.stage], ring.phase ^ 1, abort_flag, a.status)) {
+__device__ __forceinline__ Ring load_lora_stage(const GemmArgs& a, const Tile& tl, int m0, uint32_t rank, bool xa_ready,
+                                                bool leader, bool issuer, uint8_t* smem, uint64_t* full_bar,
+                                                uint64_t* empty_bar, volatile int* abort_flag, Ring ring) {
+  if (!mbar_wait_warp(&empty_bar[ring.stage], ring.phase ^ 1, abort_flag, a.status)) {
     ring.ok = 0;
     return ring;
   }
-  if (!xa_ready && !flag_wait(a.xa_flags + tl.m_blk, kXaGroups, abort_flag, a.status)) {
+  if (!xa_ready && !__all_sync(0xffffffffu, flag_wait(a.xa_flags + tl.m_blk, kXaGroups, abort_flag, a.status))) {
     ring.ok = 0;
     return ring;
   }
-  fence_proxy_async_global();  // the TMA copy below reads what the XA items' stores wrote
   int g0, nb, yb, b_step;
   tile_b_rows<BN>(a, tl, rank, g0, nb, yb, b_step);
   uint8_t* sa = smem + ring.stage * kStageBytes<BN>;
-  if (leader) {
-    mbar_arrive_expect_tx(&full_bar[ring.stage], kPair * kStageBytes<BN>);
-    armed_parity[ring.stage] = ring.phase;
+  if (issuer) {
+    fence_proxy_async_global();  // the TMA copy below reads what the XA items' stores wrote
+    if (leader) mbar_arrive_expect_tx(&full_bar[ring.stage], kPair * kStageBytes<BN>);
+    const uint32_t bar = mapa_shared(&full_bar[ring.stage], 0);
+    tma_load_2d_pair(sa, &a.tmXA, bar, a.xa_base[tl.g], m0);
+    for (int j = 0; j < nb; ++j) tma_load_2d_pair(sa + kABytes + j * b_step, &a.tmBX[g0 + j], bar, 0, yb);
   }
-  const uint32_t bar = mapa_shared(&full_bar[ring.stage], 0);
-  tma_load_2d_pair(sa, &a.tmXA, bar, a.xa_base[tl.g], m0);
-  for (int j = 0; j < nb; ++j) tma_load_2d_pair(sa + kABytes + j * b_step, &a.tmBX[g0 + j], bar, 0, yb);
+  ++ring.used;
   ring_next<STAGES>(ring);
   return ring;
 }
@@ -478,11 +479,11 @@ __device__ __noinline__ Ring load_lora_stage(const GemmArgs& a, const Tile& tl, 
 // full tile's 128), the latency of the sum it adds to; spread over two or four accumulators they took
 // longer (1.5B down, 2003 rows: 60 -> 76 us).
 template <int BN, int STAGES>
-__device__ __noinline__ Ring mma_xa_item(const GemmArgs& a, uint32_t d_tmem, uint32_t idesc_xa,
-                                         uint8_t* smem, uint64_t* full_bar, uint64_t* empty_bar,
-                                         volatile int* abort_flag, Ring ring) {
+__device__ __forceinline__ Ring mma_xa_item(const GemmArgs& a, uint32_t d_tmem, uint32_t idesc_xa, bool issuer,
+                                            uint8_t* smem, uint64_t* full_bar, uint64_t* empty_bar,
+                                            volatile int* abort_flag, Ring ring) {
   for (int kb = 0; kb < a.num_kb; ++kb) {
-    if (!mbar_wait(&full_bar[ring.stage], ring.phase, abort_flag, a.status)) {
+    if (!mbar_wait_warp(&full_bar[ring.stage], ring.phase, abort_flag, a.status)) {
       ring.ok = 0;
       return ring;
     }
@@ -490,10 +491,12 @@ __device__ __noinline__ Ring mma_xa_item(const GemmArgs& a, uint32_t d_tmem, uin
     const uint32_t sa = smem_u32(smem + ring.stage * kStageBytes<BN>);
     const uint64_t ad = smem_desc(sa, 16, 1024, kSwizzle128B);
     const uint64_t ld = smem_desc(sa + kABytes, 16, 1024, kSwizzle128B);
+    if (issuer) {
 #pragma unroll
-    for (int k = 0; k < BK / 16; ++k)
-      mma_bf16_ss_pair(d_tmem, ad + 2 * k, ld + 2 * k, idesc_xa, (kb > 0 || k > 0) ? 1u : 0u);
-    mma_commit_pair(&empty_bar[ring.stage], 0x3);
+      for (int k = 0; k < BK / 16; ++k)
+        mma_bf16_ss_pair(d_tmem, ad + 2 * k, ld + 2 * k, idesc_xa, (kb > 0 || k > 0) ? 1u : 0u);
+      mma_commit_pair(&empty_bar[ring.stage], 0x3);
+    }
     ring_next<STAGES>(ring);
   }
   return ring;
@@ -544,7 +547,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   // a rejected call: every CTA of every cluster sees the same word and leaves before any set-up
   if (call_aborted(a.abort)) return;
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);  // uniform
   const int lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
@@ -584,79 +587,76 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (every CTA)
-    // The per-stage loop of the output tiles stays minimal (one thread, on the critical path of
-    // every stage); XA items and the LoRA stage go through out-of-line helpers.
-    if (lane == 0) {
-      Ring ring{0, 0u, 1};
-      int armed_parity[STAGES];
-      for (int s = 0; s < STAGES; ++s) armed_parity[s] = -1;
-      for (int t = unit; t < a.total_items && ring.ok; t += n_units) {
-        const Tile tl = decode_tile(t, a);
-        const int m0 = tl.m_blk * (BM * kPair) + static_cast<int>(rank) * BM;
-        if (tl.xa) {
-          ring = load_xa_item<BN, STAGES>(a, m0, rank, leader, smem, full_bar, empty_bar, armed_parity,
-                                          &abort_flag, ring);
-          continue;
+    // The whole warp runs the loop, one lane issues.
+    const bool issuer = elect_one();
+    Ring ring{0, 0u, 1, 0};
+    for (int t = unit; t < a.total_items && ring.ok; t += n_units) {
+      const Tile tl = decode_tile(t, a);
+      const int m0 = tl.m_blk * (BM * kPair) + static_cast<int>(rank) * BM;
+      if (tl.xa) {
+        ring = load_xa_item<BN, STAGES>(a, m0, rank, leader, issuer, smem, full_bar, empty_bar, &abort_flag, ring);
+        continue;
+      }
+      int g0, nb, yb, b_step;
+      tile_b_rows<BN>(a, tl, rank, g0, nb, yb, b_step);
+      // Whether the row block's XA rows are stored, asked (acquire) while the stages already
+      // copied still feed the MMAs; only a tile whose row block's XA items have not finished by
+      // then waits at its LoRA stage.
+      int xa_ready = 0;
+      if (a.ext_on[tl.g]) {
+        asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(xa_ready) : "l"(a.xa_flags + tl.m_blk) : "memory");
+        xa_ready = __all_sync(0xffffffffu, xa_ready >= kXaGroups);
+      }
+      int stage = ring.stage;
+      uint32_t phase = ring.phase;
+      const CUtensorMap* mB = &a.tmB[g0];
+      for (int kb = 0; kb < a.num_kb; ++kb) {
+        if (!mbar_wait_warp(&empty_bar[stage], phase ^ 1, &abort_flag, a.status)) {
+          ring.ok = 0;
+          break;
         }
-        int g0, nb, yb, b_step;
-        tile_b_rows<BN>(a, tl, rank, g0, nb, yb, b_step);
-        // Whether the row block's XA rows are stored, asked (acquire) while the stages already
-        // copied still feed the MMAs; only a tile whose row block's XA items have not finished by
-        // then waits at its LoRA stage.
-        int xa_ready = 0;
-        if (a.ext_on[tl.g]) {
-          asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(xa_ready) : "l"(a.xa_flags + tl.m_blk) : "memory");
-          xa_ready = xa_ready >= kXaGroups;
-        }
-        int stage = ring.stage;
-        uint32_t phase = ring.phase;
-        for (int kb = 0; kb < a.num_kb; ++kb) {
-          if (!mbar_wait(&empty_bar[stage], phase ^ 1, &abort_flag, a.status)) {
-            ring.ok = 0;
-            break;
-          }
+        if (issuer) {
           uint8_t* sa = smem + stage * kStageBytes<BN>;
           uint8_t* sb = sa + kABytes;
           // the MMA-issuing CTA's full barrier counts the bytes of both CTAs
-          if (leader) {
-            mbar_arrive_expect_tx(&full_bar[stage], kPair * kStageBytes<BN>);
-            armed_parity[stage] = phase;
-          }
-          const CUtensorMap* mB = &a.tmB[g0];
+          if (leader) mbar_arrive_expect_tx(&full_bar[stage], kPair * kStageBytes<BN>);
           const uint32_t bar = mapa_shared(&full_bar[stage], 0);
           tma_load_2d_pair(sa, &a.tmA, bar, kb * BK, m0);
           for (int j = 0; j < nb; ++j) tma_load_2d_pair(sb + j * b_step, mB + j, bar, kb * BK, yb);
-          if (++stage == STAGES) {
-            stage = 0;
-            phase ^= 1;
-          }
         }
-        ring.stage = stage;
-        ring.phase = phase;
-        if (ring.ok && a.ext_on[tl.g])
-          ring = load_lora_stage<BN, STAGES>(a, tl, m0, rank, xa_ready != 0, leader, smem, full_bar, empty_bar,
-                                             armed_parity, &abort_flag, ring);
+        ++ring.used;
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1;
+        }
       }
-      if (!ring.ok) {
-        if (leader) {
-          // Let every copy already issued land before the CTA can exit.
-          for (int s = 0; s < STAGES; ++s)
-            if (armed_parity[s] >= 0) {
-              volatile int never = 0;
-              mbar_wait(&full_bar[s], static_cast<uint32_t>(armed_parity[s]), &never, nullptr);
-            }
-        } else {
-          // The peer's copies complete on the other CTA's barriers: give them time to land.
-          const unsigned long long t0 = globaltimer_ns();
-          while (globaltimer_ns() - t0 < 200000ull) {
-          }
+      ring.stage = stage;
+      ring.phase = phase;
+      if (ring.ok && a.ext_on[tl.g])
+        ring = load_lora_stage<BN, STAGES>(a, tl, m0, rank, xa_ready != 0, leader, issuer, smem, full_bar, empty_bar,
+                                           &abort_flag, ring);
+    }
+    if (!ring.ok) {
+      if (leader) {
+        // Let every copy already issued land before the CTA can exit: the last use of every stage.
+        for (int s = 0; s < STAGES && s < ring.used; ++s) {
+          const int u = ring.used - 1 - s;
+          volatile int never = 0;
+          mbar_wait(&full_bar[u % STAGES], static_cast<uint32_t>((u / STAGES) & 1), &never, nullptr);
+        }
+      } else {
+        // The peer's copies complete on the other CTA's barriers: give them time to land.
+        const unsigned long long t0 = globaltimer_ns();
+        while (globaltimer_ns() - t0 < 200000ull) {
         }
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (even CTA)
-    if (lane == 0 && leader) {
-      Ring ring{0, 0u, 1};
+    // The whole warp runs the loop, one lane issues.
+    if (leader) {
+      const bool issuer = elect_one();
+      Ring ring{0, 0u, 1, 0};
       int it = 0;
       bool issued = false;
       const uint32_t idesc = idesc_bf16_f32(BM * kPair, BN);
@@ -665,23 +665,23 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         const Tile tl = decode_tile(t, a);
         const int acc = it & 1;
         const uint32_t acc_phase = (it >> 1) & 1;
-        if (!mbar_wait<true>(&tempty_bar[acc], acc_phase ^ 1, &abort_flag, a.status)) {
+        if (!mbar_wait_warp<true>(&tempty_bar[acc], acc_phase ^ 1, &abort_flag, a.status)) {
           ring.ok = 0;
           break;
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * BN;
+        issued = true;
         if (tl.xa) {
-          ring = mma_xa_item<BN, STAGES>(a, d_tmem, idesc_xa, smem, full_bar, empty_bar, &abort_flag, ring);
-          issued = true;
+          ring = mma_xa_item<BN, STAGES>(a, d_tmem, idesc_xa, issuer, smem, full_bar, empty_bar, &abort_flag, ring);
           if (!ring.ok) break;
-          mma_commit_pair(&tfull_bar[acc], 0x3);
+          if (issuer) mma_commit_pair(&tfull_bar[acc], 0x3);
           continue;
         }
         int stage = ring.stage;
         uint32_t phase = ring.phase;
         for (int kb = 0; kb < a.num_kb; ++kb) {
-          if (!mbar_wait(&full_bar[stage], phase, &abort_flag, a.status)) {
+          if (!mbar_wait_warp(&full_bar[stage], phase, &abort_flag, a.status)) {
             ring.ok = 0;
             break;
           }
@@ -689,12 +689,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           const uint32_t sa = smem_u32(smem + stage * kStageBytes<BN>);
           const uint64_t ad = smem_desc(sa, 16, 1024, kSwizzle128B);
           const uint64_t bd = smem_desc(sa + kABytes, 16, 1024, kSwizzle128B);
-          // K = 16 steps advance 32 bytes = 2 units of the descriptor's start-address field
+          if (issuer) {
+            // K = 16 steps advance 32 bytes = 2 units of the descriptor's start-address field
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k)
-            mma_bf16_ss_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-          issued = true;
-          mma_commit_pair(&empty_bar[stage], 0x3);
+            for (int k = 0; k < BK / 16; ++k)
+              mma_bf16_ss_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+            mma_commit_pair(&empty_bar[stage], 0x3);
+          }
           if (++stage == STAGES) {
             stage = 0;
             phase ^= 1;
@@ -704,22 +705,24 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         ring.phase = phase;
         if (ring.ok && a.ext_on[tl.g]) {
           // the XA and BX copies have landed
-          if (!mbar_wait(&full_bar[ring.stage], ring.phase, &abort_flag, a.status)) {
+          if (!mbar_wait_warp(&full_bar[ring.stage], ring.phase, &abort_flag, a.status)) {
             ring.ok = 0;
           } else {
             tc_fence_after();
             const uint32_t sa = smem_u32(smem + ring.stage * kStageBytes<BN>);
             const uint64_t ad = smem_desc(sa, 16, 1024, kSwizzle128B);
             const uint64_t bd = smem_desc(sa + kABytes, 16, 1024, kSwizzle128B);
-            for (int k = 0; k < a.ext_steps[tl.g]; ++k) mma_bf16_ss_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, 1u);
-            mma_commit_pair(&empty_bar[ring.stage], 0x3);
+            if (issuer) {
+              for (int k = 0; k < a.ext_steps[tl.g]; ++k) mma_bf16_ss_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, 1u);
+              mma_commit_pair(&empty_bar[ring.stage], 0x3);
+            }
             ring_next<STAGES>(ring);
           }
         }
         if (!ring.ok) break;
-        mma_commit_pair(&tfull_bar[acc], 0x3);
+        if (issuer) mma_commit_pair(&tfull_bar[acc], 0x3);
       }
-      if (!ring.ok && issued) {
+      if (!ring.ok && issued && issuer) {
         mma_commit_pair(&drain_bar, 0x1);
         volatile int never = 0;
         mbar_wait(&drain_bar, 0, &never, nullptr);

@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_cons
   __shared__ volatile int abort_flag;
 
   griddep_launch_dependents();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int sub = a.plan.sub;
   const int x_bytes = a.n * kBlockK * 2;
   const int stage_bytes = sub * (kWBytes + x_bytes);
@@ -118,88 +118,93 @@ __global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_cons
 
   if (warp == 0) {
     // ---------------------------------------------------------------- producer
-    if (lane == 0) {
-      int armed[kMaxStages];
-      for (int i = 0; i < a.stages; ++i) armed[i] = -1;
-      const uint64_t once = l2_evict_first();
-      auto load_w = [&](const Steps& s, int st, int parity) {
-        uint8_t* dst = smem + st * stage_bytes;
-        const bool lora = s.tile == a.plan.tile0[a.nseg];
+    // The whole warp runs the loop, one lane issues.
+    const bool issuer = elect_one();
+    const uint64_t once = l2_evict_first();
+    auto load_w = [&](const Steps& s, int st) {
+      uint8_t* dst = smem + st * stage_bytes;
+      const bool lora = s.tile == a.plan.tile0[a.nseg];
+      if (issuer)
         mbar_arrive_expect_tx(&full[st], sub * ((lora ? a.n_lora * 16 * kBlockK * 2 : kWBytes) + x_bytes));
-        armed[st] = parity;
-        int seg = 0;
-        while (seg + 1 < a.nseg && s.tile >= a.plan.tile0[seg + 1]) ++seg;
-        for (int h = 0; h < sub; ++h, dst += kWBytes) {
-          const int k = (s.kb * sub + h) * kBlockK;
-          if (lora) {
-            for (int i = 0; i < a.n_lora; ++i)
-              tma_load_2d(dst + i * 16 * kBlockK * 2, &a.tmA[i], &full[st], k, 0);
-          } else {
-            tma_load_2d_hint(dst, &a.tmW[seg], &full[st], k, (s.tile - a.plan.tile0[seg]) * kTile, once);
-          }
-        }
-      };
-      auto load_x = [&](const Steps& s, int st) {
-        for (int h = 0; h < sub; ++h)
-          tma_load_2d(smem + st * stage_bytes + sub * kWBytes + h * x_bytes, &a.tmX, &full[st],
-                      (s.kb * sub + h) * kBlockK, 0);
-      };
-      Steps w, x;
-      w.at(a, blockIdx.x);
-      x.at(a, blockIdx.x);
-      // weights of the first stages before the wait, their rows after it
-      int pre = 0;
-      for (; pre < a.stages && w.more(a); ++pre, w.next(a)) load_w(w, pre, 0);
-      griddep_wait();
-      asm volatile("fence.proxy.async.global;" ::: "memory");
-      for (int i = 0; i < pre; ++i, x.next(a)) load_x(x, i);
-      bool ok = true;
-      int st = 0;
-      uint32_t ph = 1;
-      for (; ok && w.more(a); w.next(a)) {
-        ok = mbar_wait(&empty[st], ph ^ 1, &abort_flag, a.status);
-        if (!ok) break;
-        load_w(w, st, static_cast<int>(ph));
-        load_x(w, st);
-        if (++st == a.stages) {
-          st = 0;
-          ph ^= 1;
+      int seg = 0;
+      while (seg + 1 < a.nseg && s.tile >= a.plan.tile0[seg + 1]) ++seg;
+      for (int h = 0; h < sub; ++h, dst += kWBytes) {
+        const int k = (s.kb * sub + h) * kBlockK;
+        if (lora) {
+          for (int i = 0; i < a.n_lora; ++i)
+            if (issuer) tma_load_2d(dst + i * 16 * kBlockK * 2, &a.tmA[i], &full[st], k, 0);
+        } else if (issuer) {
+          tma_load_2d_hint(dst, &a.tmW[seg], &full[st], k, (s.tile - a.plan.tile0[seg]) * kTile, once);
         }
       }
-      if (!ok) {
-        volatile int never = 0;
-        for (int i = 0; i < a.stages; ++i)
-          if (armed[i] >= 0) mbar_wait(&full[i], static_cast<uint32_t>(armed[i]), &never, nullptr);
+    };
+    auto load_x = [&](const Steps& s, int st) {
+      for (int h = 0; h < sub; ++h)
+        if (issuer)
+          tma_load_2d(smem + st * stage_bytes + sub * kWBytes + h * x_bytes, &a.tmX, &full[st],
+                      (s.kb * sub + h) * kBlockK, 0);
+    };
+    Steps w, x;
+    w.at(a, blockIdx.x);
+    x.at(a, blockIdx.x);
+    // weights of the first stages before the wait, their rows after it
+    int used = 0;  // stages filled so far
+    for (; used < a.stages && w.more(a); ++used, w.next(a)) load_w(w, used);
+    griddep_wait();
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    for (int i = 0; i < used; ++i, x.next(a)) load_x(x, i);
+    bool ok = true;
+    int st = 0;
+    uint32_t ph = 1;
+    for (; w.more(a); w.next(a)) {
+      ok = mbar_wait_warp(&empty[st], ph ^ 1, &abort_flag, a.status);
+      if (!ok) break;
+      load_w(w, st);
+      load_x(w, st);
+      ++used;
+      if (++st == a.stages) {
+        st = 0;
+        ph ^= 1;
+      }
+    }
+    if (!ok) {
+      // every copy issued lands before the CTA can exit: the last use of every stage
+      volatile int never = 0;
+      for (int i = 0; i < a.stages && i < used; ++i) {
+        const int u = used - 1 - i;
+        mbar_wait(&full[u % a.stages], static_cast<uint32_t>((u / a.stages) & 1), &never, nullptr);
       }
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16_f32(kTile, a.n);
-      bool ok = true, issued = false;
-      int st = 0, it = 0;
-      uint32_t ph = 0;
-      Steps s;
-      for (s.at(a, blockIdx.x); ok && s.more(a); ++it) {
-        const int acc = it & 1;
-        if (!mbar_wait(&tempty[acc], ((it >> 1) & 1) ^ 1, &abort_flag, a.status)) {
+    // The whole warp runs the loop, one lane issues.
+    const bool issuer = elect_one();
+    const uint32_t idesc = idesc_bf16_f32(kTile, a.n);
+    bool ok = true, issued = false;
+    int st = 0, it = 0;
+    uint32_t ph = 0;
+    Steps s;
+    for (s.at(a, blockIdx.x); ok && s.more(a); ++it) {
+      const int acc = it & 1;
+      if (!mbar_wait_warp(&tempty[acc], ((it >> 1) & 1) ^ 1, &abort_flag, a.status)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const int unit = s.u, len = s.end - s.kb;
+      // accumulation group of step i: i * groups / len
+      for (int i = 0, left = 0; s.u == unit; s.next(a), i += a.groups) {
+        const int group = a.groups == 1 ? 0 : i / len;
+        const bool first = left != group + 1;
+        left = group + 1;
+        const uint32_t d = tmem + acc * a.acc_cols + group * a.n;
+        if (!mbar_wait_warp(&full[st], ph, &abort_flag, a.status)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        const int unit = s.u, len = s.end - s.kb;
-        // accumulation group of step i: i * groups / len
-        for (int i = 0, left = 0; s.u == unit; s.next(a), i += a.groups) {
-          const int group = i / len;
-          const bool first = left != group + 1;
-          left = group + 1;
-          const uint32_t d = tmem + acc * a.acc_cols + group * a.n;
-          if (!mbar_wait(&full[st], ph, &abort_flag, a.status)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t base = smem_u32(smem + st * stage_bytes);
+        const uint32_t base = smem_u32(smem + st * stage_bytes);
+        if (issuer) {
           for (int h = 0; h < sub; ++h) {
             const uint64_t wd = smem_desc(base + h * kWBytes, 16, 1024, kSwizzle128B);
             const uint64_t xd = smem_desc(base + sub * kWBytes + h * x_bytes, 16, 1024, kSwizzle128B);
@@ -207,20 +212,20 @@ __global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_cons
             for (int k = 0; k < kBlockK / 16; ++k)
               mma_bf16_ss(d, wd + 2 * k, xd + 2 * k, idesc, (!first || h > 0 || k > 0) ? 1u : 0u);
           }
-          issued = true;
           mma_commit(&empty[st]);
-          if (++st == a.stages) {
-            st = 0;
-            ph ^= 1;
-          }
         }
-        if (ok) mma_commit(&tfull[acc]);
+        issued = true;
+        if (++st == a.stages) {
+          st = 0;
+          ph ^= 1;
+        }
       }
-      if (!ok && issued) {
-        mma_commit(&drain_bar);
-        volatile int never = 0;
-        mbar_wait(&drain_bar, 0, &never, nullptr);
-      }
+      if (ok && issuer) mma_commit(&tfull[acc]);
+    }
+    if (!ok && issued && issuer) {
+      mma_commit(&drain_bar);
+      volatile int never = 0;
+      mbar_wait(&drain_bar, 0, &never, nullptr);
     }
   } else {
     // ---------------------------------------------------------------- epilogue (warps 2..5)
