@@ -44,12 +44,12 @@ struct crf_ctx {
 namespace {
 
 enum ProfKind : int {
-  kPQkv, kPO, kPGateUp, kPDown, kPAttn, kPNorm, kPEmbed, kPRope, kPCopy,
+  kPQkv, kPO, kPGateUp, kPDown, kPAttn, kPNorm, kPEmbed, kPCopy,
   kPDecode, kPLmHead, kPKl, kPDrift, kPCheck, kPNumKinds
 };
 const char* const kProfNames[kPNumKinds] = {
     "gemm_qkv_rope_paged", "gemm_o_resid", "gemm_gateup_swiglu", "gemm_down_resid",
-    "attn_prefill_paged", "rmsnorm", "embed_gather", "rope_table", "row_copy",
+    "attn_prefill_paged", "rmsnorm", "embed_gather", "row_copy",
     "tail_decode", "lm_head", "kl_reduce", "drift_gram", "page_check"};
 
 // Brackets the launches issued in its lifetime with two events on `st` when
@@ -713,18 +713,17 @@ bool device_page_check() {
   return !(e && e[0] == '1');
 }
 
-// Opens a call on `st`: clears the call's abort word and the `flag_words` ready words after it,
-// and checks every page id of the listed tables (in [0, num_pages), no page twice). Enqueued
-// work only: the host does not wait.
-crf_status open_call(crf_ctx* ctx, const PageCheck& pc, int num_pages, uint8_t* ws, size_t off_abort,
-                     size_t flag_words, size_t off_ptab, uint32_t ptab_slots, cudaStream_t st) {
-  int* abort = reinterpret_cast<int*>(ws + off_abort);
-  ProfScope ps(ctx, kPCheck, st, device_page_check() ? 1 : 0);
-  CRF_CUDA(cudaMemsetAsync(abort, 0, (1 + flag_words) * sizeof(int), st));
-  if (!device_page_check()) return CRF_OK;
-  int* table = reinterpret_cast<int*>(ws + off_ptab);
-  CRF_CUDA(cudaMemsetAsync(table, 0xff, static_cast<size_t>(ptab_slots) * sizeof(int), st));
-  CRF_CUDA(launch_validate_pages(pc, num_pages, table, ptab_slots - 1, abort, ctx->status_dev, st));
+// Opens a call on `st`: clears the call's abort word, the ready words after it and the page table
+// (one range), then checks every page id of the listed tables and forms the call's rotation angles
+// (launch_open_call). Enqueued work only: the host does not wait.
+crf_status open_call(crf_ctx* ctx, const PageCheck& pc, int num_pages, uint8_t* ws, const Plan& p, const Dims& D,
+                     float2* angles, int n_pos, const RowPositions* rows, cudaStream_t st) {
+  int* abort = reinterpret_cast<int*>(ws + p.off_abort);
+  int* table = reinterpret_cast<int*>(ws + p.off_ptab);
+  ProfScope ps(ctx, kPCheck, st, 1);
+  CRF_CUDA(cudaMemsetAsync(abort, 0, p.off_ptab - p.off_abort + static_cast<size_t>(p.ptab_slots) * sizeof(int), st));
+  CRF_CUDA(launch_open_call(pc, num_pages, table, p.ptab_slots - 1, abort, ctx->status_dev, device_page_check(), angles,
+                            n_pos, rows, D.d, D.theta, st));
   return CRF_OK;
 }
 
@@ -919,6 +918,8 @@ crf_status crf_recompute_window(crf_ctx* ctx, const crf_model* model, const crf_
   if (ws_bytes < plan.total)
     return fail(CRF_ENOMEM, "workspace %zu bytes, %zu needed", ws_bytes, plan.total);
 
+  // every kernel of the call may become resident, and set itself up, while the one before finishes
+  PdlScope pdl;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   LayerCtx c;
   c.D = &D;
@@ -939,14 +940,9 @@ crf_status crf_recompute_window(crf_ctx* ctx, const crf_model* model, const crf_
       pc.pt[i] = reqs[i].page_table;
       pc.first[i + 1] = pc.first[i] + (reqs[i].n_tokens + kPage - 1) / kPage;
     }
-    s = open_call(ctx, pc, pool->num_pages, ws, plan.off_abort, plan.flag_words, plan.off_ptab,
-                  plan.ptab_slots, st);
+    s = open_call(ctx, pc, pool->num_pages, ws, plan, D, reinterpret_cast<float2*>(ws + plan.off_rope), plan.max_n,
+                  nullptr, st);
     if (s != CRF_OK) return s;
-  }
-
-  {
-    ProfScope ps(ctx, kPRope, st);
-    CRF_CUDA(launch_rope_table(reinterpret_cast<float2*>(ws + plan.off_rope), plan.max_n, D.d, D.theta, st));
   }
 
   __nv_bfloat16* G[2] = {reinterpret_cast<__nv_bfloat16*>(ws + plan.off_g0),
@@ -1040,9 +1036,10 @@ crf_status crf_recompute_window(crf_ctx* ctx, const crf_model* model, const crf_
       ProfScope ps(ctx, kPCopy, st, copy_out ? 1 : 0);
       curp[i] = X_out + static_cast<size_t>(rt.row0[k]) * D.h;
       if (copy_out)
-        CRF_CUDA(launch_copy_bf16(static_cast<__nv_bfloat16*>(reqs[i].hidden_out[l - reqs[i].s]), curp[i],
+        CRF_CUDA(launch_copy_rows(static_cast<__nv_bfloat16*>(reqs[i].hidden_out[l - reqs[i].s]), curp[i],
                                   static_cast<size_t>(reqs[i].n_tokens) * D.h, c.abort, st));
-      if (l == reqs[i].e - 1 && reqs[i].final_hidden_out)
+      // the last row waits for its tail in the caller's checkpoint, or where there is none in a copy
+      if (l == reqs[i].e - 1 && reqs[i].final_hidden_out && !reqs[i].hidden_out)
         CRF_CUDA(cudaMemcpyAsync(dx0 + static_cast<size_t>(i) * D.h,
                                  curp[i] + static_cast<size_t>(reqs[i].n_tokens - 1) * D.h, row_bytes,
                                  cudaMemcpyDeviceToDevice, st));
@@ -1054,24 +1051,29 @@ crf_status crf_recompute_window(crf_ctx* ctx, const crf_model* model, const crf_
   for (int i = 0; i < n_req; ++i) {
     const crf_request& r = reqs[i];
     if (!r.final_hidden_out) continue;
-    __nv_bfloat16* start = dx0 + static_cast<size_t>(i) * D.h;
-    if (r.s == r.e) {
-      ProfScope ps(ctx, r.s == 0 ? kPEmbed : kPCopy, st, r.s == 0 ? 1 : 0);
-      if (r.s == 0) {
-        CRF_CUDA(launch_embed(static_cast<const __nv_bfloat16*>(model->embed), r.tokens + (r.n_tokens - 1),
-                              start, 1, D.h, D.V, ctx->status_dev, st));
-      } else {
-        CRF_CUDA(cudaMemcpyAsync(start,
-                                 static_cast<const __nv_bfloat16*>(r.hidden_in) +
-                                     static_cast<size_t>(r.n_tokens - 1) * D.h,
-                                 row_bytes, cudaMemcpyDeviceToDevice, st));
-      }
+    const size_t last = static_cast<size_t>(r.n_tokens - 1) * D.h;
+    const __nv_bfloat16* start = dx0 + static_cast<size_t>(i) * D.h;
+    const int32_t* token = nullptr;
+    if (r.s < r.e && r.hidden_out) {
+      start = static_cast<const __nv_bfloat16*>(r.hidden_out[r.e - r.s - 1]) + last;
+    } else if (r.s == r.e && r.s > 0) {
+      start = static_cast<const __nv_bfloat16*>(r.hidden_in) + last;
+    } else if (r.s == r.e) {
+      start = nullptr;
+      token = r.tokens + (r.n_tokens - 1);
     }
     if (r.e == D.N) {
       ProfScope ps(ctx, kPCopy, st, 1);
-      CRF_CUDA(launch_copy_bf16(static_cast<__nv_bfloat16*>(r.final_hidden_out), start, D.h, c.abort, st));
+      CRF_CUDA(launch_copy_rows(static_cast<__nv_bfloat16*>(r.final_hidden_out), start, D.h, c.abort, st));
     } else {
-      dec.push_back({r.e, r.n_tokens - 1, r.page_table, start, r.final_hidden_out});
+      DecodeRow d{};
+      d.e = r.e;
+      d.pos = r.n_tokens - 1;
+      d.page_table = r.page_table;
+      d.start = start;
+      d.out = r.final_hidden_out;
+      d.token = token;
+      dec.push_back(d);
     }
   }
   s = decode_rows(c, dec);
@@ -1145,14 +1147,13 @@ crf_status crf_decode_step(crf_ctx* ctx, const crf_model* model, const crf_adapt
       pc.pt[i] = rows[i].page_table;
       pc.first[i + 1] = pc.first[i] + rows[i].pos / kPage + 1;
     }
-    s = open_call(ctx, pc, pool->num_pages, ws, sp.p.off_abort, sp.p.flag_words, sp.p.off_ptab, sp.p.ptab_slots,
-                  st);
+    RowPositions rp{};
+    for (int i = 0; i < n_rows; ++i) rp.pos[i] = rows[i].pos;
+    s = open_call(ctx, pc, pool->num_pages, ws, sp.p, D, reinterpret_cast<float2*>(ws + sp.off_angles), n_rows, &rp, st);
     if (s != CRF_OK) return s;
   }
-  RowPositions rp{};
   std::vector<DecodeRow> dec;
   for (int i = 0; i < n_rows; ++i) {
-    rp.pos[i] = rows[i].pos;
     DecodeRow d{};
     d.e = 0;
     d.pos = rows[i].pos;
@@ -1161,10 +1162,6 @@ crf_status crf_decode_step(crf_ctx* ctx, const crf_model* model, const crf_adapt
     dec.push_back(d);
   }
   auto* angles = reinterpret_cast<float2*>(ws + sp.off_angles);
-  {
-    ProfScope ps(ctx, kPRope, st);
-    CRF_CUDA(launch_rope_table_rows(angles, rp, n_rows, D.d, D.theta, st));
-  }
   DecodeOpts opt;
   opt.write_kv = true;
   opt.rope_by_row = angles;

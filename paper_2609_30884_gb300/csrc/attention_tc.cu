@@ -199,7 +199,8 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
   __shared__ volatile int abort_flag;
 
   AttnWork w;
-  if (call_aborted(a.abort) || !attn_work(a, blockIdx.x, w)) return;
+  griddep_launch_dependents();
+  if (!attn_work(a, blockIdx.x, w)) return;
   const int n = a.req.len[w.req];
   const int row0 = a.req.row0[w.req];
   const int32_t* pt = a.req.page_table[w.req];
@@ -237,6 +238,11 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base_sh;
+  griddep_wait();  // q and the pages come from the kernel before
+  if (call_aborted(a.abort)) {
+    if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
+    return;
+  }
 
   if (warp < 4) {
     // setmaxnreg inside each role's branch: the softmax code is never reachable from here
@@ -523,8 +529,7 @@ cudaError_t launch_tc(const AttnTcArgs& args, cudaStream_t stream) {
     if (fa.numRegs * kThreadsAttn < kRegsNeeded) return cudaErrorInvalidConfiguration;
     once.done(dev);
   }
-  attn_tc_kernel<D><<<args.total_items, kThreadsAttn, smem, stream>>>(args);
-  return cudaGetLastError();
+  return launch_kernel(attn_tc_kernel<D>, dim3(args.total_items), dim3(kThreadsAttn), smem, stream, args);
 }
 
 }  // namespace

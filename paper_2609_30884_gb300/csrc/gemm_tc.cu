@@ -544,9 +544,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   __shared__ __align__(8) uint64_t drain_bar;
   __shared__ uint32_t tmem_base_sh;
   __shared__ volatile int abort_flag;
-  // a rejected call: every CTA of every cluster sees the same word and leaves before any set-up
-  if (call_aborted(a.abort)) return;
-
+  griddep_launch_dependents();
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);  // uniform
   const int lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
@@ -584,13 +582,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
+  griddep_wait();  // the set-up above touches nothing that the kernels before write
+  // a rejected call: every CTA of every cluster sees the same word and has no work
+  const int total_items = call_aborted(a.abort) ? 0 : a.total_items;
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (every CTA)
     // The whole warp runs the loop, one lane issues.
     const bool issuer = elect_one();
     Ring ring{0, 0u, 1, 0};
-    for (int t = unit; t < a.total_items && ring.ok; t += n_units) {
+    for (int t = unit; t < total_items && ring.ok; t += n_units) {
       const Tile tl = decode_tile(t, a);
       const int m0 = tl.m_blk * (BM * kPair) + static_cast<int>(rank) * BM;
       if (tl.xa) {
@@ -661,7 +662,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       bool issued = false;
       const uint32_t idesc = idesc_bf16_f32(BM * kPair, BN);
       const uint32_t idesc_xa = idesc_bf16_f32(BM * kPair, a.n_slots > 0 ? a.xa_n : 32);
-      for (int t = unit; t < a.total_items && ring.ok; t += n_units, ++it) {
+      for (int t = unit; t < total_items && ring.ok; t += n_units, ++it) {
         const Tile tl = decode_tile(t, a);
         const int acc = it & 1;
         const uint32_t acc_phase = (it >> 1) & 1;
@@ -735,7 +736,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     uint32_t tempty_addr[2];
     for (int i = 0; i < 2; ++i) tempty_addr[i] = mapa_shared(&tempty_bar[i], 0);
     int it = 0;
-    for (int t = unit; t < a.total_items; t += n_units, ++it) {
+    for (int t = unit; t < total_items; t += n_units, ++it) {
       const Tile tl = decode_tile(t, a);
       const int acc = it & 1;
       const uint32_t acc_phase = (it >> 1) & 1;
@@ -839,17 +840,19 @@ cudaError_t launch_impl(GemmArgs& args, int num_sms, cudaStream_t stream) {
   // before its tiles
   const int units = std::max(1, std::min(max_units, args.total_items));
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = PAIR;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3(PAIR * units);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = pdl_active() ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, args);
 }
 

@@ -43,7 +43,7 @@ constexpr int kBxCols = 64;
 // programmatic-stream-serialization attribute: such a kernel becomes resident while its
 // predecessor in the stream still runs, prefetches its weights and then waits for it
 // (griddep_wait). Every kernel launched this way calls griddep_wait before it touches memory
-// that an earlier kernel may write. The decode-row layer loop opens a scope.
+// that an earlier kernel may write. crf_recompute_window and crf_decode_step open a scope.
 class PdlScope {
  public:
   PdlScope();
@@ -136,10 +136,9 @@ struct GemmDesc {
 cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t stream);
 
 // ------------------------------------------------------------------ other kernels
-// (cos, sin) of pair i at position p at table[((i / 2) n_pos + p) 2 + i % 2]: neighbouring rows of a
-// projection read neighbouring entries.
-cudaError_t launch_rope_table(float2* table, int n_pos, int head_dim, double theta,
-                              cudaStream_t stream);
+struct RowPositions {
+  int pos[kMaxReq];
+};
 // BX rows of up to 4 modules: out[m][r, :] = 0 except columns [col_off[m], col_off[m] + 32) =
 // [B_m[r, 0:16] | B_m[r, 0:16]] (rank padded with zeros); a null B_m gives all-zero rows.
 struct BextDesc {
@@ -263,16 +262,13 @@ cudaError_t launch_swiglu_rows(const RowPart& part, int up_col, int f, const Row
 cudaError_t launch_head_rows(const __nv_bfloat16* ref, const __nv_bfloat16* cur, int n_ref, int hidden,
                              const __nv_bfloat16* g, __nv_bfloat16* xs, int terms, float* nss, cudaStream_t stream);
 // Single-query attention of `rows` decode rows (one per request) over pages [0, pos) plus own k/v.
-struct RowPositions {
-  int pos[kMaxReq];
-};
 struct DecodeAttnDesc {
   RowPart qkv;             // the q|k|v pass's output
   int col[3];              // its first columns of q, k, v
   RowUp up[3];
   RowLora lora;
   const __nv_bfloat16* bias[3];
-  const float2* rope;      // launch_rope_table's table, or [rows][head_dim / 2] with rope_by_row
+  const float2* rope;      // launch_open_call's table, or [rows][head_dim / 2] with rope_by_row
   int rope_by_row, rope_positions;
   __nv_bfloat16* kpages;
   __nv_bfloat16* vpages;
@@ -293,9 +289,6 @@ struct DecodeAttnDesc {
 cudaError_t launch_decode_attention(const DecodeAttnDesc& d, int num_pages, int num_sms, int* status,
                                     cudaStream_t stream);
 int decode_attention_splits(int max_positions);
-// (cos, sin) of the rows' positions: table [rows][head_dim / 2].
-cudaError_t launch_rope_table_rows(float2* table, const RowPositions& pos, int rows, int head_dim,
-                                   double theta, cudaStream_t stream);
 // out[r] = argmax of logits row r (lowest index among equal maxima).
 // One block whose wait on an mbarrier nothing arrives on runs out after the bounded-wait limit
 // and raises kStatusTimeout in *status (the failure path, exercised without a fault).
@@ -303,19 +296,23 @@ cudaError_t launch_wait_selftest(int* status, cudaStream_t stream);
 cudaError_t launch_argmax_rows(const float* logits, int rows, int vocab, int32_t* out,
                                cudaStream_t stream, const int* abort = nullptr);
 // dst[0 .. n) = src[0 .. n) (bf16), unless the call's abort word is set.
-cudaError_t launch_copy_bf16(__nv_bfloat16* dst, const __nv_bfloat16* src, size_t n, const int* abort,
+cudaError_t launch_copy_rows(__nv_bfloat16* dst, const __nv_bfloat16* src, size_t n, const int* abort,
                              cudaStream_t stream);
-// The page-table check that opens crf_recompute_window and crf_decode_step: every id of every
-// table in [0, num_pages) and no page twice across the tables. A failure sets *abort and raises
-// kStatusPages in *status. `table` is scratch of (mask + 1) ints, mask + 1 a power of two at
-// least twice the ids checked, filled with -1 (0xff bytes) before the launch.
+// The first kernel of crf_recompute_window and crf_decode_step. With `check`: every id of every
+// table in [0, num_pages) and no page twice across the tables; a failure sets *abort and raises
+// kStatusPages in *status. `table` is scratch of (mask + 1) ints, mask + 1 a power of two at least
+// twice the ids checked, zero before the launch. And the call's angles, (cos, sin) of rotation pair i
+// at position p: for `rows`, angles[r][head_dim / 2] of n_pos = rows positions; else of positions
+// 0 .. n_pos - 1 at angles[((i / 2) n_pos + p) 2 + i % 2], so that neighbouring rows of a projection
+// read neighbouring entries.
 struct PageCheck {
   const int32_t* pt[kMaxReq];
   int first[kMaxReq + 1];  // prefix of the tables' id counts
   int n;
 };
-cudaError_t launch_validate_pages(const PageCheck& pc, int num_pages, int* table, uint32_t mask, int* abort,
-                                  int* status, cudaStream_t stream);
+cudaError_t launch_open_call(const PageCheck& pc, int num_pages, int* table, uint32_t mask, int* abort, int* status,
+                             bool check, float2* angles, int n_pos, const RowPositions* rows, int head_dim,
+                             double theta, cudaStream_t stream);
 
 // Logits [rows, V] fp32 of rows given as terms and sums of squares (launch_head_rows, launch_add_norm_rows).
 cudaError_t launch_lm_head(const __nv_bfloat16* W, const __nv_bfloat16* xs, int terms, const float* nss, int rows,

@@ -7,28 +7,72 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
 namespace crf {
 
 namespace {
 
-// ------------------------------------------------------------------ RoPE table
-// table[((i / 2) n_pos + p) 2 + i % 2] = (cos, sin)(p * theta^(-2i/d)): the angle in turns, p * theta^(-2i/d) / (2 pi),
-// is formed in fp64 (per-frequency factors computed on the host in fp64), reduced to [0, 1)
-// and evaluated with fp32 sincospi.
-struct RopeFreqs {
+// ------------------------------------------------------------------ opening a call
+// (cos, sin)(p * theta^(-2i/d)): the angle in turns, p * theta^(-2i/d) / (2 pi), is formed in fp64
+// (per-frequency factors computed on the host in fp64), reduced to [0, 1) and evaluated with fp32
+// sincospi.
+struct RopeJob {
   double turns_per_pos[64];
+  float2* table;
+  int n, half;       // entries of the table, pairs per position
+  int by_row;        // table [rows][half] for position pos[row]; else the position-minor table
+  RowPositions pos;
 };
 
-__global__ void rope_table_kernel(float2* table, int n_pos, int half, const __grid_constant__ RopeFreqs f) {
+// Blocks [0, check_blocks): one thread per page id; an id outside [0, num_pages), or already in the
+// open-addressing table (zeros: empty; linear probing, at most mask + 1 probes), rejects the call.
+// The blocks after them: the call's rotation angles.
+__global__ void open_call_kernel(const __grid_constant__ PageCheck pc, int num_pages, int* table, uint32_t mask,
+                                 int* abort, int* status, int check_blocks, const __grid_constant__ RopeJob rope) {
+  griddep_launch_dependents();
+  griddep_wait();
+  if (static_cast<int>(blockIdx.x) >= check_blocks) {
+    const int idx = (blockIdx.x - check_blocks) * blockDim.x + threadIdx.x;
+    if (idx >= rope.n) return;
+    int p, i;
+    if (rope.by_row) {
+      p = rope.pos.pos[idx / rope.half];
+      i = idx % rope.half;
+    } else {
+      const int n_pos = rope.n / rope.half;
+      p = idx / 2 % n_pos;
+      i = idx / 2 / n_pos * 2 + idx % 2;
+    }
+    double turns = static_cast<double>(p) * rope.turns_per_pos[i];
+    turns -= floor(turns);
+    float s, c;
+    sincospif(static_cast<float>(2.0 * turns), &s, &c);
+    rope.table[idx] = make_float2(c, s);
+    return;
+  }
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n_pos * half) return;
-  const int p = idx / 2 % n_pos, i = idx / 2 / n_pos * 2 + idx % 2;
-  double turns = static_cast<double>(p) * f.turns_per_pos[i];
-  turns -= floor(turns);
-  float s, c;
-  sincospif(static_cast<float>(2.0 * turns), &s, &c);
-  table[idx] = make_float2(c, s);
+  if (idx >= pc.first[pc.n]) return;
+  int i = 0;
+  while (i + 1 < pc.n && idx >= pc.first[i + 1]) ++i;
+  const int id = pc.pt[i][idx - pc.first[i]];
+  bool bad = id < 0 || id >= num_pages;
+  if (!bad) {
+    uint32_t h = (static_cast<uint32_t>(id) * 0x9E3779B1u) & mask;
+    for (uint32_t probe = 0; probe <= mask; ++probe) {
+      const int prev = atomicCAS(table + h, 0, id + 1);
+      if (prev == 0) break;
+      if (prev == id + 1) {
+        bad = true;
+        break;
+      }
+      h = (h + 1) & mask;
+    }
+  }
+  if (bad) {
+    atomicExch(abort, 1);
+    atomicOr(status, kStatusPages);
+  }
 }
 
 // ------------------------------------------------------------------ RMSNorm (+ BX rows)
@@ -67,6 +111,8 @@ __global__ void rmsnorm_kernel(const __nv_bfloat16* __restrict__ x,
                                const __nv_bfloat16* __restrict__ g, __nv_bfloat16* __restrict__ y,
                                int rows, int hidden, float eps, const __grid_constant__ BextDesc bx,
                                int norm_blocks) {
+  griddep_launch_dependents();
+  griddep_wait();  // x comes from the kernel before, and earlier ones read y and the BX rows
   if (static_cast<int>(blockIdx.x) >= norm_blocks) {
     bext_chunk(bx, static_cast<long>(blockIdx.x - norm_blocks) * blockDim.x + threadIdx.x);
     return;
@@ -117,41 +163,17 @@ __global__ void embed_kernel(const __nv_bfloat16* __restrict__ e, const int32_t*
       reinterpret_cast<const uint4*>(e + (size_t)id * hidden)[c];
 }
 
-__global__ void copy_bf16_kernel(__nv_bfloat16* __restrict__ dst, const __nv_bfloat16* __restrict__ src,
-                                 size_t n, const int* abort) {
+// One T per thread and turn: 16 bytes, or 2 where a caller's row is not aligned to 16.
+template <typename T>
+__global__ void copy_rows_kernel(T* __restrict__ dst, const T* __restrict__ src, size_t n, const int* abort) {
+  griddep_launch_dependents();
+  griddep_wait();
   if (call_aborted(abort)) return;
   for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<size_t>(gridDim.x) * blockDim.x)
     dst[i] = src[i];
 }
 
-// One thread per page id: outside [0, num_pages), or already in the open-addressing table
-// (linear probing, at most mask + 1 probes), rejects the call.
-__global__ void validate_pages_kernel(const PageCheck pc, int num_pages, int* table, uint32_t mask,
-                                      int* abort, int* status) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= pc.first[pc.n]) return;
-  int i = 0;
-  while (i + 1 < pc.n && idx >= pc.first[i + 1]) ++i;
-  const int id = pc.pt[i][idx - pc.first[i]];
-  bool bad = id < 0 || id >= num_pages;
-  if (!bad) {
-    uint32_t h = (static_cast<uint32_t>(id) * 0x9E3779B1u) & mask;
-    for (uint32_t probe = 0; probe <= mask; ++probe) {
-      const int prev = atomicCAS(table + h, -1, id);
-      if (prev == -1) break;
-      if (prev == id) {
-        bad = true;
-        break;
-      }
-      h = (h + 1) & mask;
-    }
-  }
-  if (bad) {
-    atomicExch(abort, 1);
-    atomicOr(status, kStatusPages);
-  }
-}
 // ------------------------------------------------------------------ KL
 // Per (row, split): online (max, sum e^(z* - m), sum e^(z* - m)(z* - z)) for the
 // reference and (max, sum e^(z - m)) for the current logits.
@@ -250,17 +272,24 @@ inline int cdiv(long a, long b) { return static_cast<int>((a + b - 1) / b); }
 
 }  // namespace
 
-cudaError_t launch_rope_table(float2* table, int n_pos, int head_dim, double theta,
-                              cudaStream_t stream) {
-  const int half = head_dim / 2;
-  const int n = n_pos * half;
-  if (n == 0) return cudaSuccess;
-  if (half > 64) return cudaErrorInvalidValue;
-  RopeFreqs f;
-  for (int i = 0; i < half; ++i)
-    f.turns_per_pos[i] = std::pow(theta, -2.0 * i / head_dim) / (2.0 * 3.14159265358979323846);
-  rope_table_kernel<<<cdiv(n, 256), 256, 0, stream>>>(table, n_pos, half, f);
-  return cudaGetLastError();
+cudaError_t launch_open_call(const PageCheck& pc, int num_pages, int* table, uint32_t mask, int* abort, int* status,
+                             bool check, float2* angles, int n_pos, const RowPositions* rows, int head_dim,
+                             double theta, cudaStream_t stream) {
+  const int ids = check ? pc.first[pc.n] : 0;
+  if (static_cast<uint32_t>(ids) > (mask + 1u) / 2u) return cudaErrorInvalidValue;
+  RopeJob r{};
+  r.half = head_dim / 2;
+  if (r.half > 64 || n_pos < 0 || static_cast<long>(n_pos) * r.half > 0x7fffffffl) return cudaErrorInvalidValue;
+  r.table = angles;
+  r.n = n_pos * r.half;
+  r.by_row = rows != nullptr;
+  if (rows) r.pos = *rows;
+  for (int i = 0; i < r.half; ++i)
+    r.turns_per_pos[i] = std::pow(theta, -2.0 * i / head_dim) / (2.0 * 3.14159265358979323846);
+  const int check_blocks = cdiv(ids, 256), blocks = check_blocks + cdiv(r.n, 256);
+  if (blocks == 0) return cudaSuccess;
+  return launch_kernel(open_call_kernel, dim3(blocks), dim3(256), 0, stream, pc, num_pages, table, mask, abort, status,
+                       check_blocks, r);
 }
 
 cudaError_t launch_rmsnorm(const __nv_bfloat16* x, const __nv_bfloat16* g, __nv_bfloat16* y,
@@ -275,8 +304,7 @@ cudaError_t launch_rmsnorm(const __nv_bfloat16* x, const __nv_bfloat16* g, __nv_
   const int norm_blocks = cdiv(rows, 8);
   const int blocks = norm_blocks + static_cast<int>(cdiv(chunks, 256));
   if (blocks == 0) return cudaSuccess;
-  rmsnorm_kernel<<<blocks, 256, 0, stream>>>(x, g, y, rows, hidden, eps, d, norm_blocks);
-  return cudaGetLastError();
+  return launch_kernel(rmsnorm_kernel, dim3(blocks), dim3(256), 0, stream, x, g, y, rows, hidden, eps, d, norm_blocks);
 }
 
 cudaError_t launch_embed(const __nv_bfloat16* embed, const int32_t* tokens, __nv_bfloat16* out,
@@ -313,19 +341,6 @@ __global__ void wait_selftest_kernel(int* status) {
 cudaError_t launch_wait_selftest(int* status, cudaStream_t stream) {
   wait_selftest_kernel<<<1, 32, 0, stream>>>(status);
   return cudaGetLastError();
-}
-
-// (cos, sin) of the rows' own positions only: table[r][i] for position pos[r].
-__global__ void rope_table_rows_kernel(float2* table, int rows, int half, const RowPositions pos,
-                                       const __grid_constant__ RopeFreqs f) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= rows * half) return;
-  const int r = idx / half, i = idx % half;
-  double turns = static_cast<double>(pos.pos[r]) * f.turns_per_pos[i];
-  turns -= floor(turns);
-  float s, c;
-  sincospif(static_cast<float>(2.0 * turns), &s, &c);
-  table[idx] = make_float2(c, s);
 }
 
 // out[r] = argmax_i logits[r, i], the lowest index among equal maxima.
@@ -396,18 +411,6 @@ __global__ void argmax_rows_kernel(const float* __restrict__ logits, int vocab, 
   }
 }
 
-cudaError_t launch_rope_table_rows(float2* table, const RowPositions& pos, int rows, int head_dim,
-                                   double theta, cudaStream_t stream) {
-  const int half = head_dim / 2;
-  if (rows == 0) return cudaSuccess;
-  if (half > 64) return cudaErrorInvalidValue;
-  RopeFreqs f{};
-  for (int i = 0; i < half; ++i)
-    f.turns_per_pos[i] = std::pow(theta, -2.0 * i / head_dim) / (2.0 * 3.14159265358979323846);
-  rope_table_rows_kernel<<<cdiv(rows * half, 256), 256, 0, stream>>>(table, rows, half, pos, f);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_argmax_rows(const float* logits, int rows, int vocab, int32_t* out,
                                cudaStream_t stream, const int* abort) {
   if (rows == 0) return cudaSuccess;
@@ -415,21 +418,17 @@ cudaError_t launch_argmax_rows(const float* logits, int rows, int vocab, int32_t
   return cudaGetLastError();
 }
 
-cudaError_t launch_copy_bf16(__nv_bfloat16* dst, const __nv_bfloat16* src, size_t n, const int* abort,
+cudaError_t launch_copy_rows(__nv_bfloat16* dst, const __nv_bfloat16* src, size_t n, const int* abort,
                              cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
-  const size_t want = (n + 255) / 256;
-  copy_bf16_kernel<<<static_cast<unsigned>(want < 4096 ? want : 4096), 256, 0, stream>>>(dst, src, n, abort);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_validate_pages(const PageCheck& pc, int num_pages, int* table, uint32_t mask, int* abort,
-                                  int* status, cudaStream_t stream) {
-  const int total = pc.first[pc.n];
-  if (total == 0) return cudaSuccess;
-  if (static_cast<uint32_t>(total) > (mask + 1u) / 2u) return cudaErrorInvalidValue;
-  validate_pages_kernel<<<cdiv(total, 256), 256, 0, stream>>>(pc, num_pages, table, mask, abort, status);
-  return cudaGetLastError();
+  auto launch = [&](auto* d, const auto* f, size_t items) {
+    const size_t want = (items + 255) / 256;
+    return launch_kernel(copy_rows_kernel<std::remove_pointer_t<decltype(d)>>,
+                         dim3(static_cast<unsigned>(want < 2048 ? want : 2048)), dim3(256), 0, stream, d, f, items, abort);
+  };
+  if (n % 8 == 0 && ((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15) == 0)
+    return launch(reinterpret_cast<uint4*>(dst), reinterpret_cast<const uint4*>(src), n / 8);
+  return launch(dst, src, n);
 }
 
 cudaError_t launch_kl(const float* zref, const float* zcur, int rows, int vocab, float* out,
