@@ -133,7 +133,20 @@ __device__ __forceinline__ void split_diff(uint32_t a, uint32_t b, uint32_t& hi,
   lo = bf2_sub(bf2_sub(a, av), bf2_add(b, bv));
 }
 
-// The segment of step x, searched forward from segment s (segments are visited in order).
+// The segment that holds step x. A CTA's first one: by bisection (a walk from segment 0 took the last
+// CTAs of 392 segments several microseconds before their first copy).
+__device__ __forceinline__ int seg_find(const DriftTcArgs& a, int x) {
+  int lo = 0, hi = a.n_segs;  // seg_step0[lo] <= x < seg_step0[hi]
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (x >= a.seg_step0[mid])
+      lo = mid;
+    else
+      hi = mid;
+  }
+  return lo;
+}
+// Searched forward from segment s (segments are visited in order).
 __device__ __forceinline__ int seg_of(const DriftTcArgs& a, int s, int x) {
   while (s + 1 < a.n_segs && x >= a.seg_step0[s + 1]) ++s;
   return s;
@@ -146,7 +159,7 @@ struct ProdSeg {
 
   __device__ __forceinline__ void at(const DriftTcArgs& a, int x) {
     if (seg >= 0 && x < next0) return;
-    seg = seg_of(a, seg < 0 ? 0 : seg, x);
+    seg = seg < 0 ? seg_find(a, x) : seg_of(a, seg, x);
     side = seg & 1;
     const DriftItem& it = a.items[seg >> 1];
     len = side == 0 ? it.out_dim : it.in_dim;
@@ -515,7 +528,7 @@ __global__ void __launch_bounds__(kDtThreads, kDtCtasPerSm)
 #pragma unroll
       for (int v = 0; v < 4; ++v) acc[q][h][v] = 0.f;
 
-  int x = x0, seg = seg_of(a, 0, x0), stage = 0;  // the step, segment and stage being multiplied
+  int x = x0, seg = seg_find(a, x0), stage = 0;  // the step, segment and stage being multiplied
   uint32_t phase = 0;
   while (x < x1) {
     seg = seg_of(a, seg, x);
