@@ -311,18 +311,17 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
       bool issued = false;
       const uint32_t idesc_s = idesc_bf16_f32(kM, kN);
       const uint32_t idesc_o = idesc_bf16_f32(kM, D, false, true);
+      // descriptors of the bases; an MMA's own offset is added to the start-address field (16-byte units)
+      const uint64_t qd = smem_desc(smem_u32(sQ), 16, 1024, kSwizzle128B);
+      const uint64_t kd = smem_desc(smem_u32(sKV), 16, GROUP_BYTES, kSwizzle128B);
+      const uint64_t vd = smem_desc(smem_u32(sKV), 1024, GROUP_BYTES, kSwizzle128B);
       auto issue_s = [&](int t, int ks) {
-        const uint32_t kb = smem_u32(sKV + ks * KV_BYTES);
-        const uint32_t qb = smem_u32(sQ + t * Q_BYTES);
+        const uint64_t q = qd + static_cast<uint32_t>(t * (Q_BYTES >> 4)), k = kd + static_cast<uint32_t>(ks * (KV_BYTES >> 4));
         if (issuer) {
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint32_t in_row = (kk & 3) * 32;
-            mma_bf16_ss(tmem + t * 128,
-                        smem_desc(qb + (kk >> 2) * HALF_ROWS_BYTES + in_row, 16, 1024, kSwizzle128B),
-                        smem_desc(kb + (kk >> 2) * 1024 + in_row, 16, GROUP_BYTES, kSwizzle128B),
-                        idesc_s, kk > 0 ? 1u : 0u);
-          }
+          for (int kk = 0; kk < D / 16; ++kk)
+            mma_bf16_ss(tmem + t * 128, q + (kk >> 2) * (HALF_ROWS_BYTES >> 4) + (kk & 3) * 2,
+                        k + (kk >> 2) * 64 + (kk & 3) * 2, idesc_s, kk > 0 ? 1u : 0u);
           mma_commit(&s_full[t]);
         }
       };
@@ -335,7 +334,7 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
       // ring slot of V(j); K(j + 1) is in the one after it
       int vs = 1;
       for (int j = 0; j < J && ok; ++j) {
-        const uint32_t vb = smem_u32(sKV + vs * KV_BYTES);
+        const uint64_t v = vd + static_cast<uint32_t>(vs * (KV_BYTES >> 4));
         const int ks = vs + 1 == kSlots ? 0 : vs + 1;
         for (int t = (j < J0 ? 0 : 1); t < ntiles; ++t) {
           // phase j of p_full[t]: P_t(j) is in TMEM, and V(j) and K(j + 1) have landed
@@ -348,8 +347,7 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
 #pragma unroll
             for (int kk = 0; kk < kN / 16; ++kk) {
               // P: 16 keys = 8 packed bf16x2 columns; V: 16 key rows = two 8-key groups
-              mma_bf16_ts(tmem + 256 + t * 128, tmem + t * 128 + kk * 8,
-                          smem_desc(vb + kk * 2 * GROUP_BYTES, 1024, GROUP_BYTES, kSwizzle128B), idesc_o,
+              mma_bf16_ts(tmem + 256 + t * 128, tmem + t * 128 + kk * 8, v + kk * (2 * GROUP_BYTES >> 4), idesc_o,
                           (j > 0 || kk > 0) ? 1u : 0u);
             }
           }
