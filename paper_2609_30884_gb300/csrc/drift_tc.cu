@@ -154,12 +154,13 @@ __device__ __forceinline__ int seg_of(const DriftTcArgs& a, int s, int x) {
 
 // What the producer needs of the segment it loads, read from the arguments once per segment.
 struct ProdSeg {
+  int first;  // the CTA's first segment
   int seg = -1, side = 0, len = 0, step0 = 0, next0 = 0;
   const __nv_bfloat16 *p1 = nullptr, *p0 = nullptr;  // version 1 / version 0 of this side
 
   __device__ __forceinline__ void at(const DriftTcArgs& a, int x) {
     if (seg >= 0 && x < next0) return;
-    seg = seg < 0 ? seg_find(a, x) : seg_of(a, seg, x);
+    seg = seg_of(a, seg < 0 ? first : seg, x);
     side = seg & 1;
     const DriftItem& it = a.items[seg >> 1];
     len = side == 0 ? it.out_dim : it.in_dim;
@@ -337,11 +338,12 @@ __device__ __forceinline__ bool run_steps(int& x, int end, int& stage, uint32_t&
 // (its own or the consumers') it waits, within the same limit, for the copies it has issued, so
 // none is in flight when the CTA's shared memory goes.
 template <int R>
-__device__ __forceinline__ void produce(const DriftTcArgs& a, int x0, int x1, uint64_t* full,
+__device__ __forceinline__ void produce(const DriftTcArgs& a, int seg0, int x0, int x1, uint64_t* full,
                                         uint64_t* empty, uint32_t stage0, volatile int* abort_flag,
                                         int* status) {
   using S = DtShape<R>;
   ProdSeg ps;
+  ps.first = seg0;
   int ls = 0, issued = 0;
   bool ok = true;
   for (int lx = x0; lx < x1; ++lx) {
@@ -405,8 +407,9 @@ struct SideGram {
 // out_sq pair. Rank 4 adds the B side's two packed halves (fragment features i and i + 4).
 // `buf` is shared scratch of kCombineBytes. The slots come from other CTAs: read through L2.
 template <int R>
-__device__ void combine_item(const DriftTcArgs& a, int item, const float* __restrict__ slots,
-                             float* __restrict__ out_sq, uint8_t* buf) {
+__device__ __forceinline__ void combine_item(const DriftTcArgs& a, int item, const int (&b_lo)[2],
+                                             const int (&n_slot)[2], int out_index, const float* __restrict__ slots,
+                                             float* __restrict__ out_sq, uint8_t* buf) {
   using S = DtShape<R>;
   constexpr int RP = S::RP;
   float (*g)[S::kSlotFloats] = reinterpret_cast<float (*)[S::kSlotFloats]>(buf);
@@ -415,8 +418,6 @@ __device__ void combine_item(const DriftTcArgs& a, int item, const float* __rest
   // before any of them is added; the adds keep CTA order
   constexpr int kPer = (S::kSlotFloats + kDtConsumers - 1) / kDtConsumers;
   constexpr int kBatch = 8;
-  int b_lo[2], n_slot[2];
-  for (int side = 0; side < 2; ++side) seg_slots(a, 2 * item + side, b_lo[side], n_slot[side]);
   float v[2][kPer];
 #pragma unroll
   for (int side = 0; side < 2; ++side)
@@ -483,8 +484,8 @@ __device__ void combine_item(const DriftTcArgs& a, int item, const float* __rest
       tt += red[0][w];
       pp += red[1][w];
     }
-    out_sq[a.items[item].out_index * 2 + 0] = static_cast<float>(tt);
-    out_sq[a.items[item].out_index * 2 + 1] = static_cast<float>(pp);
+    out_sq[out_index * 2 + 0] = static_cast<float>(tt);
+    out_sq[out_index * 2 + 1] = static_cast<float>(pp);
   }
 }
 
@@ -514,9 +515,12 @@ __global__ void __launch_bounds__(kDtThreads, kDtCtasPerSm)
     *abort_flag = 0;
     fence_barrier_init();
   }
+  const int seg0 = seg_find(a, x0);
   __syncthreads();
+  // factors may come from the kernel before, and the combine kernel of an earlier call reads the slots
+  griddep_wait();
   if (warp == kDtConsumers / 32) {
-    produce<R>(a, x0, x1, full, empty, stage0, abort_flag, status);
+    produce<R>(a, seg0, x0, x1, full, empty, stage0, abort_flag, status);
     return;
   }
 
@@ -528,7 +532,7 @@ __global__ void __launch_bounds__(kDtThreads, kDtCtasPerSm)
 #pragma unroll
       for (int v = 0; v < 4; ++v) acc[q][h][v] = 0.f;
 
-  int x = x0, seg = seg_find(a, x0), stage = 0;  // the step, segment and stage being multiplied
+  int x = x0, seg = seg0, stage = 0;  // the step, segment and stage being multiplied
   uint32_t phase = 0;
   while (x < x1) {
     seg = seg_of(a, seg, x);
@@ -540,36 +544,18 @@ __global__ void __launch_bounds__(kDtThreads, kDtCtasPerSm)
     // the producer drains the copies in flight; a warp that got past a wait another warp gave
     // up on stops here too, before the flush's barriers
     if (!ok || *abort_flag) return;
-    // the warps' partial Grams summed in a fixed tree ((w0 + w4) + (w2 + w6)) + ((w1 + w5) +
-    // (w3 + w7)), then written as one slot
-#pragma unroll 1
-    for (int h = kDtConsumers / 64; h >= 1; h >>= 1) {
-      if (warp >= h && warp < 2 * h) {
+    // the warps' partial Grams summed in a fixed order, ((w0 + w4) + (w2 + w6)) + ((w1 + w5) +
+    // (w3 + w7)), into one slot: pairs of warps through the scratch, then four sums per element
+    if (warp >= 4) {
 #pragma unroll
-        for (int q = 0; q < S::kPairs; ++q)
-#pragma unroll
-          for (int hh = 0; hh < 2; ++hh)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) red[((warp - h) * S::kPairs * 8 + q * 8 + hh * 4 + v) * 32 + lane] = acc[q][hh][v];
-      }
-      consumers_sync();
-      if (warp < h) {
-#pragma unroll
-        for (int q = 0; q < S::kPairs; ++q)
-#pragma unroll
-          for (int hh = 0; hh < 2; ++hh)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) acc[q][hh][v] += red[(warp * S::kPairs * 8 + q * 8 + hh * 4 + v) * 32 + lane];
-      }
-      consumers_sync();
+      for (int q = 0; q < S::kPairs * 8; ++q)
+        red[((warp - 4) * S::kPairs * 8 + q) * 32 + lane] = acc[q >> 3][(q >> 2) & 1][q & 3];
     }
-    if (warp == 0) {
+    consumers_sync();
+    if (warp < 4) {
 #pragma unroll
-      for (int q = 0; q < S::kPairs; ++q)
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh)
-#pragma unroll
-          for (int v = 0; v < 4; ++v) red[(q * 8 + hh * 4 + v) * 32 + lane] = acc[q][hh][v];
+      for (int q = 0; q < S::kPairs * 8; ++q)
+        red[(warp * S::kPairs * 8 + q) * 32 + lane] += acc[q >> 3][(q >> 2) & 1][q & 3];
     }
     consumers_sync();
     float* out = slots + static_cast<size_t>(b + seg) * S::kSlotFloats;
@@ -577,7 +563,9 @@ __global__ void __launch_bounds__(kDtThreads, kDtCtasPerSm)
       const int q = e >> 8, rr = (e >> 4) & 15, cc = e & 15;
       const int ln = (rr & 7) * 4 + ((cc & 7) >> 1);
       const int v = (rr >> 3) * 2 + (cc & 1);
-      out[e] = red[(q * 8 + (cc >> 3) * 4 + v) * 32 + ln];
+      const float* w = red + (q * 8 + (cc >> 3) * 4 + v) * 32 + ln;
+      constexpr int kWarp = S::kPairs * 8 * 32;
+      out[e] = (w[0] + w[2 * kWarp]) + (w[kWarp] + w[3 * kWarp]);
     }
 #pragma unroll
     for (int q = 0; q < S::kPairs; ++q)
@@ -598,6 +586,10 @@ __global__ void __launch_bounds__(kDtConsumers) drift_tc_final_kernel(const __gr
                                                                       float* __restrict__ out_sq) {
   using S = DtShape<R>;
   __shared__ __align__(16) uint8_t buf[S::kCombineBytes];
+  griddep_launch_dependents();
+  int b_lo[2], n_slot[2];
+  for (int side = 0; side < 2; ++side) seg_slots(a, 2 * blockIdx.x + side, b_lo[side], n_slot[side]);
+  const int out_index = a.items[blockIdx.x].out_index;
   griddep_wait();
   if (blockIdx.x == 0 && a.zero_mask)
     for (int e = threadIdx.x; e < a.n_out; e += kDtConsumers)
@@ -605,7 +597,7 @@ __global__ void __launch_bounds__(kDtConsumers) drift_tc_final_kernel(const __gr
         out_sq[2 * e] = 0.f;
         out_sq[2 * e + 1] = 0.f;
       }
-  combine_item<R>(a, blockIdx.x, slots, out_sq, buf);
+  combine_item<R>(a, blockIdx.x, b_lo, n_slot, out_index, slots, out_sq, buf);
 }
 
 template <int R>
@@ -619,12 +611,11 @@ cudaError_t launch_rank(const DriftTcArgs& a, float* slots, float* out_sq, int* 
     if (e != cudaSuccess) return e;
     once.done(dev);
   }
-  // the Gram kernel is not dependent-launched: it overwrites the slots that the combine kernel
-  // of an earlier call on this stream reads
-  drift_tc_kernel<R><<<a.grid, kDtThreads, S::kSmem, stream>>>(a, slots, status);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  // both set themselves up (the Gram kernel's barriers and first segment, the combine's slot ranges)
+  // while the kernel before finishes
   PdlScope pdl;
+  cudaError_t e = launch_kernel(drift_tc_kernel<R>, dim3(a.grid), dim3(kDtThreads), S::kSmem, stream, a, slots, status);
+  if (e != cudaSuccess) return e;
   return launch_kernel(drift_tc_final_kernel<R>, dim3(a.n_items), dim3(kDtConsumers), 0, stream, a,
                        static_cast<const float*>(slots), out_sq);
 }
