@@ -179,9 +179,8 @@ cudaError_t launch_attention_tc(const AttnDesc& d, int num_pages, int total_rows
 constexpr int kRowsMax = 64;         // rows of one weight pass
 constexpr int kRowsMaxSeg = 3;       // projections that share an input
 constexpr int kRowsMaxSplits = 16;   // K splits of a weight tile
-constexpr int kRowsRing = 76 * 1024;       // shared-memory ring of a short pass inside a dependent chain,
-constexpr int kRowsRingLong = 150 * 1024;  // of a long one,
-constexpr int kRowsRingMax = 200 * 1024;   // and of one alone on its SMs
+constexpr int kRowsRing = 150 * 1024;     // shared-memory ring of a pass inside a dependent chain
+constexpr int kRowsRingMax = 200 * 1024;  // and of one alone on its SMs
 // fp32 rows enter a weight pass as bf16 terms: three (exact) for one or two rows, two (about 16
 // mantissa bits) from three rows on. Chosen by the rows of the whole call, so that equal rows in
 // different passes stay equal.

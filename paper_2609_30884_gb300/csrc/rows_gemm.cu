@@ -20,10 +20,11 @@
 // and the epilogue multiplies by it (nss: the sums of squares by slice).
 //
 // One CTA per SM and dependent launch: the ring's first weights are requested before the wait for the
-// kernel that makes x, so the copies run through the short kernels between two passes. A short
-// pass's ring (75 KB) fits beside decode attention's block or a long pass's ring (150 KB). Weights
-// are marked evict-first in L2, which keeps the rows' partial sums and the K/V pages there (3% of a
-// 7B generation step).
+// kernel that makes x, so the copies run through the short kernels between two passes (a ring of 75
+// KB for the short passes would fit beside decode attention's block and start earlier, but runs out
+// sooner: 7B step of one row 3.08 against 3.01 ms, of 32 rows 4.64 against 4.37; asking L2 for more
+// weights before the wait gained nothing). Weights are marked evict-first in L2, which keeps the
+// rows' partial sums and the K/V pages there (3% of a 7B generation step).
 //
 // Measured (7B shape, weights read once): LM head, 2 rows, 1.09 GB in 166 us (6.6 TB/s, 97% of the
 // copy rate); gate|up, 272 MB in 46 us (5.9 TB/s) behind the chain's prefetch. 58 rows of the 1.5B
@@ -309,12 +310,12 @@ RowsPlan rows_plan(int nseg, const int* outs, bool lora, int in_dim, int num_sms
   if (lora) ++p.tiles;
   p.ncols = p.tiles * kTile;
   const int blocks = (in_dim + kBlockK - 1) / kBlockK;
-  // From 16 blocks a CTA on, steps are two blocks (256 contiguous bytes of each weight row, asked
-  // for together) and the ring is larger: the rate is then set by how DRAM pages are visited. 7B
-  // shape: one generation step 3.69 -> 3.21 ms, LM head 184 -> 166 us; four blocks gain nothing
-  // more. Below it, one-block steps split evenly over more CTAs.
+  // From 8 blocks a CTA on, steps are two blocks (256 contiguous bytes of each weight row, asked for
+  // together): the rate is then set by how DRAM pages are visited. 7B shape: one generation step 3.69
+  // -> 3.21 ms, LM head 184 -> 166 us; four blocks gain nothing more. Below it, one-block steps split
+  // evenly over more CTAs.
   const long per_cta = (static_cast<long>(p.tiles) * blocks + num_sms - 1) / num_sms;
-  p.sub = per_cta >= 16 ? 2 : 1;
+  p.sub = per_cta >= 8 ? 2 : 1;
   p.kb = (blocks + p.sub - 1) / p.sub;
   // splits: the fewest K blocks on the busiest CTA, a unit's fixed cost counted as three blocks
   // and each split's share of the consumer's sum as a quarter
@@ -360,7 +361,7 @@ cudaError_t launch_rows_gemm(const RowsGemmDesc& d, const RowsPlan& plan, int nu
   while (a.acc_cols < a.n * a.groups) a.acc_cols *= 2;
   a.tmem_cols = std::max(32, 2 * a.acc_cols);
   const int stage = plan.sub * (kWBytes + a.n * kBlockK * 2);
-  const int ring = !pdl_active() ? kRowsRingMax : plan.sub > 1 ? kRowsRingLong : kRowsRing;
+  const int ring = pdl_active() ? kRowsRing : kRowsRingMax;
   a.stages = std::min(kMaxStages, ring / stage);
   a.y = d.y;
   a.nss = d.nss;
