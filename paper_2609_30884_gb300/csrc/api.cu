@@ -791,6 +791,8 @@ StepPlan make_step_plan(const Dims& D, const crf_decode_row* rows, int n, uint32
   long ids = 0;
   for (int i = 0; i < n; ++i) ids += rows[i].pos / kPage + 1;
   p.ptab_slots = ptab_slots_for(ids);
+  // after the abort word (and one of padding): the greedy tokens' keys (two words a row) and counts
+  p.flag_words = 1 + 3 * static_cast<size_t>(n);
   p.off_abort = take((1 + p.flag_words) * sizeof(int));
   p.off_ptab = take(static_cast<size_t>(p.ptab_slots) * sizeof(int));
   sp.total = p.total = o;
@@ -1174,11 +1176,14 @@ crf_status crf_decode_step(crf_ctx* ctx, const crf_model* model, const crf_adapt
   float* z = logits ? logits : reinterpret_cast<float*>(ws + sp.off_logits);
   {
     ProfScope ps(ctx, kPLmHead, st, 2);
+    PdlScope pdl;
     CRF_CUDA(launch_lm_head(static_cast<const __nv_bfloat16*>(model->lm_head),
                             reinterpret_cast<const __nv_bfloat16*>(base + ds.xs), rows_terms(n_rows),
                             reinterpret_cast<const float*>(base + ds.nss), n_rows, D.V, D.h, D.eps, z, ctx->num_sms,
                             ctx->status_dev, st, c.abort));
-    CRF_CUDA(launch_argmax_rows(z, n_rows, D.V, next_tokens, st, c.abort));
+    int* words = reinterpret_cast<int*>(ws + sp.p.off_abort) + 2;
+    CRF_CUDA(launch_argmax_rows(z, n_rows, D.V, reinterpret_cast<unsigned long long*>(words), words + 2 * n_rows,
+                                next_tokens, st, c.abort));
   }
   return CRF_OK;
 }
@@ -1297,6 +1302,7 @@ crf_status crf_kl(crf_ctx* ctx, const crf_model* model, const void* ref, const v
     o += align256(static_cast<size_t>(2 * n_rows) * norm_slices(hidden) * sizeof(float));
     float* logits = logits_out ? logits_out : reinterpret_cast<float*>(ws + o);
     ProfScope ps(ctx, kPLmHead, st, 1 + (2 * n_rows + kRowsMax - 1) / kRowsMax);
+    PdlScope pdl;
     CRF_CUDA(launch_head_rows(static_cast<const __nv_bfloat16*>(ref), static_cast<const __nv_bfloat16*>(cur), n_rows,
                               hidden, static_cast<const __nv_bfloat16*>(model->final_norm), xs, terms, nss, st));
     CRF_CUDA(launch_lm_head(static_cast<const __nv_bfloat16*>(model->lm_head), xs, terms, nss, 2 * n_rows, vocab, hidden,

@@ -213,6 +213,7 @@ struct RowsGemmDesc {
   float eps;
   int* status;
   const int* abort;        // per-call abort word, or null: a rejected call stores nothing
+  bool alone;              // a long pass by itself (the LM head): the largest ring
 };
 cudaError_t launch_rows_gemm(const RowsGemmDesc& d, const RowsPlan& plan, int num_sms, cudaStream_t stream);
 
@@ -288,12 +289,13 @@ struct DecodeAttnDesc {
 cudaError_t launch_decode_attention(const DecodeAttnDesc& d, int num_pages, int num_sms, int* status,
                                     cudaStream_t stream);
 int decode_attention_splits(int max_positions);
-// out[r] = argmax of logits row r (lowest index among equal maxima).
 // One block whose wait on an mbarrier nothing arrives on runs out after the bounded-wait limit
 // and raises kStatusTimeout in *status (the failure path, exercised without a fault).
 cudaError_t launch_wait_selftest(int* status, cudaStream_t stream);
-cudaError_t launch_argmax_rows(const float* logits, int rows, int vocab, int32_t* out,
-                               cudaStream_t stream, const int* abort = nullptr);
+// out[r] = argmax of logits row r (lowest index among equal maxima). key, count: one entry per row, zero
+// before the launch.
+cudaError_t launch_argmax_rows(const float* logits, int rows, int vocab, unsigned long long* key, int* count,
+                               int32_t* out, cudaStream_t stream, const int* abort);
 // dst[0 .. n) = src[0 .. n) (bf16), unless the call's abort word is set.
 cudaError_t launch_copy_rows(__nv_bfloat16* dst, const __nv_bfloat16* src, size_t n, const int* abort,
                              cudaStream_t stream);

@@ -228,6 +228,7 @@ cudaError_t launch_lm_head(const __nv_bfloat16* W, const __nv_bfloat16* xs, int 
     d.eps = eps;
     d.status = status;
     d.abort = abort;
+    d.alone = true;
     cudaError_t e = launch_rows_gemm(d, plan, num_sms, stream);
     if (e != cudaSuccess) return e;
   }

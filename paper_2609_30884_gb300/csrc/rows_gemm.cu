@@ -356,12 +356,12 @@ cudaError_t launch_rows_gemm(const RowsGemmDesc& d, const RowsPlan& plan, int nu
   a.units = plan.tiles * plan.splits;
   a.rows = d.rows;
   // exact rows keep fp32 accuracy: groups of a unit's steps accumulate apart (at least one each)
-  a.groups = d.terms == 3 ? std::min(pdl_active() ? 4 : 8, plan.kb / plan.splits) : 1;
+  a.groups = d.terms == 3 ? std::min(d.alone ? 8 : 4, plan.kb / plan.splits) : 1;
   a.acc_cols = 16;
   while (a.acc_cols < a.n * a.groups) a.acc_cols *= 2;
   a.tmem_cols = std::max(32, 2 * a.acc_cols);
   const int stage = plan.sub * (kWBytes + a.n * kBlockK * 2);
-  const int ring = pdl_active() ? kRowsRing : kRowsRingMax;
+  const int ring = d.alone ? kRowsRingMax : kRowsRing;
   a.stages = std::min(kMaxStages, ring / stage);
   a.y = d.y;
   a.nss = d.nss;

@@ -3,10 +3,12 @@
 #include "common.cuh"
 #include "kernels.h"
 
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <optional>
 #include <type_traits>
 
 namespace crf {
@@ -178,33 +180,49 @@ __global__ void copy_rows_kernel(T* __restrict__ dst, const T* __restrict__ src,
 // Per (row, split): online (max, sum e^(z* - m), sum e^(z* - m)(z* - z)) for the
 // reference and (max, sum e^(z - m)) for the current logits.
 constexpr int kKlThreads = 256;
+constexpr int kKlAhead = 8;
 
 __global__ void __launch_bounds__(kKlThreads) kl_partial_kernel(const float* __restrict__ zr,
                                                                 const float* __restrict__ zc,
                                                                 int vocab, int splits,
                                                                 float* __restrict__ part) {
+  griddep_launch_dependents();
+  griddep_wait();
   const int row = blockIdx.y, sp = blockIdx.x;
   const int per = (vocab + splits - 1) / splits;
   const int v0 = sp * per, v1 = min(vocab, v0 + per);
   const float* a = zr + (size_t)row * vocab;
   const float* b = zc + (size_t)row * vocab;
   float mr = -FLT_MAX, sr = 0.f, dr = 0.f, mc = -FLT_MAX, sc = 0.f;
-  for (int i = v0 + threadIdx.x; i < v1; i += kKlThreads) {
-    const float x = a[i], y = b[i];
-    if (x > mr) {
-      const float f = __expf(mr - x);
-      sr *= f;
-      dr *= f;
-      mr = x;
+  // the logits of eight turns in flight together, then added in order: one row pair has about two
+  // turns a thread, 29 have 54, which took a memory latency each
+  for (int i0 = v0 + threadIdx.x; i0 < v1; i0 += kKlAhead * kKlThreads) {
+    float xs[kKlAhead], ys[kKlAhead];
+#pragma unroll
+    for (int u = 0; u < kKlAhead; ++u) {
+      const int i = i0 + u * kKlThreads;
+      xs[u] = i < v1 ? a[i] : 0.f;
+      ys[u] = i < v1 ? b[i] : 0.f;
     }
-    const float e = __expf(x - mr);
-    sr += e;
-    dr += e * (x - y);
-    if (y > mc) {
-      sc *= __expf(mc - y);
-      mc = y;
+#pragma unroll
+    for (int u = 0; u < kKlAhead; ++u) {
+      if (i0 + u * kKlThreads >= v1) break;
+      const float x = xs[u], y = ys[u];
+      if (x > mr) {
+        const float f = __expf(mr - x);
+        sr *= f;
+        dr *= f;
+        mr = x;
+      }
+      const float e = __expf(x - mr);
+      sr += e;
+      dr += e * (x - y);
+      if (y > mc) {
+        sc *= __expf(mc - y);
+        mc = y;
+      }
+      sc += __expf(y - mc);
     }
-    sc += __expf(y - mc);
   }
   // block combine
   __shared__ float s_mr[kKlThreads], s_sr[kKlThreads], s_dr[kKlThreads], s_mc[kKlThreads],
@@ -244,6 +262,8 @@ __global__ void __launch_bounds__(kKlThreads) kl_partial_kernel(const float* __r
 
 // KL = D/S* + (M + log S) - (M* + log S*), combining the splits of one row (warp per row).
 __global__ void kl_final_kernel(const float* part, int splits, float* out, int rows) {
+  griddep_launch_dependents();
+  griddep_wait();
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
@@ -343,79 +363,67 @@ cudaError_t launch_wait_selftest(int* status, cudaStream_t stream) {
   return cudaGetLastError();
 }
 
-// out[r] = argmax_i logits[r, i], the lowest index among equal maxima.
-// One block per row; 16-byte loads, four in flight per thread before their compares.
-__global__ void argmax_rows_kernel(const float* __restrict__ logits, int vocab, int32_t* out,
-                                   const int* abort) {
+// out[r] = argmax_i logits[r, i], the lowest index among equal maxima; NaNs never win. Each row is cut
+// over gridDim.x blocks (one block a row pulled 608 KB through one SM, about 8 us). A logit and its
+// index make one 64-bit key that orders by value, then by the lower index; the blocks of a row meet in
+// an atomic maximum, which no order of arrival changes, and the last of them writes the token.
+constexpr int kArgmaxThreads = 256;
+constexpr int kArgmaxAhead = 8;
+__global__ void __launch_bounds__(kArgmaxThreads) argmax_rows_kernel(const float* __restrict__ logits, int vocab,
+                                                                     unsigned long long* key, int* count, int32_t* out,
+                                                                     const int* abort) {
+  griddep_launch_dependents();
+  griddep_wait();
   if (call_aborted(abort)) return;
-  const int r = blockIdx.x;
+  const int r = blockIdx.y;
   const float* z = logits + (size_t)r * vocab;
-  float best = -INFINITY;
-  int arg = 0x7fffffff;
-  auto take = [&](float v, int i) {
-    if (v > best || (v == best && i < arg)) {
-      best = v;
-      arg = i;
-    }
-  };
-  // elements before the row's first 16-byte boundary, then whole float4s, then the tail
-  const int mis = static_cast<int>(reinterpret_cast<uintptr_t>(z) & 15) / 4;
-  const int head = min(vocab, mis ? 4 - mis : 0);
-  for (int i = threadIdx.x; i < head; i += blockDim.x) take(z[i], i);
-  const int n4 = (vocab - head) / 4;
-  const float4* z4 = reinterpret_cast<const float4*>(z + head);
-  constexpr int kU = 4;
-  for (int i0 = threadIdx.x; i0 < n4; i0 += kU * blockDim.x) {
-    float4 v[kU];
+  const int per = (vocab + gridDim.x - 1) / gridDim.x;
+  const int v0 = blockIdx.x * per, v1 = min(vocab, v0 + per);
+  unsigned long long best = 0;
+  for (int i0 = v0 + threadIdx.x; i0 < v1; i0 += kArgmaxAhead * kArgmaxThreads) {
+    float v[kArgmaxAhead];
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int i = i0 + u * blockDim.x;
-      v[u] = i < n4 ? __ldg(z4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int u = 0; u < kArgmaxAhead; ++u) {
+      const int i = i0 + u * kArgmaxThreads;
+      v[u] = i < v1 ? __ldg(z + i) : NAN;
     }
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int i = i0 + u * blockDim.x;
-      if (i < n4) {
-        const int b = head + 4 * i;
-        take(v[u].x, b);
-        take(v[u].y, b + 1);
-        take(v[u].z, b + 2);
-        take(v[u].w, b + 3);
-      }
+    for (int u = 0; u < kArgmaxAhead; ++u) {
+      if (isnan(v[u])) continue;
+      const uint32_t b = __float_as_uint(v[u] == 0.f ? 0.f : v[u]);  // both zeros are equal
+      const uint32_t order = b >> 31 ? ~b : b | 0x80000000u;
+      const unsigned long long k =
+          static_cast<unsigned long long>(order) << 32 | ~static_cast<uint32_t>(i0 + u * kArgmaxThreads);
+      if (k > best) best = k;
     }
   }
-  for (int i = head + 4 * n4 + threadIdx.x; i < vocab; i += blockDim.x) take(z[i], i);
-  __shared__ float sb[32];
-  __shared__ int sa[32];
+  __shared__ unsigned long long sb[kArgmaxThreads / 32];
+#pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-    const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
-    if (ob > best || (ob == best && oa < arg)) {
-      best = ob;
-      arg = oa;
-    }
+    const unsigned long long k = __shfl_xor_sync(0xffffffffu, best, o);
+    if (k > best) best = k;
   }
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) {
-    sb[w] = best;
-    sa[w] = arg;
-  }
+  if ((threadIdx.x & 31) == 0) sb[threadIdx.x >> 5] = best;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int i = 1; i < static_cast<int>(blockDim.x >> 5); ++i)
-      if (sb[i] > best || (sb[i] == best && sa[i] < arg)) {
-        best = sb[i];
-        arg = sa[i];
-      }
-    out[r] = arg;
-  }
+  if (threadIdx.x != 0) return;
+#pragma unroll
+  for (int w = 1; w < kArgmaxThreads / 32; ++w)
+    if (sb[w] > best) best = sb[w];
+  atomicMax(key + r, best);
+  __threadfence();
+  if (atomicAdd(count + r, 1) != static_cast<int>(gridDim.x) - 1) return;
+  __threadfence();
+  best = atomicMax(key + r, 0ull);
+  out[r] = best == 0 ? 0x7fffffff : static_cast<int32_t>(~static_cast<uint32_t>(best));
 }
 
-cudaError_t launch_argmax_rows(const float* logits, int rows, int vocab, int32_t* out,
-                               cudaStream_t stream, const int* abort) {
+cudaError_t launch_argmax_rows(const float* logits, int rows, int vocab, unsigned long long* key, int* count,
+                               int32_t* out, cudaStream_t stream, const int* abort) {
   if (rows == 0) return cudaSuccess;
-  argmax_rows_kernel<<<rows, 1024, 0, stream>>>(logits, vocab, out, abort);
-  return cudaGetLastError();
+  // about two blocks per SM over all rows, at least 4096 logits each
+  const int by_rows = std::max(1, 304 / rows), by_vocab = (vocab + 4095) / 4096;
+  return launch_kernel(argmax_rows_kernel, dim3(std::min(std::min(32, by_rows), by_vocab), rows), dim3(kArgmaxThreads), 0,
+                       stream, logits, vocab, key, count, out, abort);
 }
 
 cudaError_t launch_copy_rows(__nv_bfloat16* dst, const __nv_bfloat16* src, size_t n, const int* abort,
@@ -434,9 +442,16 @@ cudaError_t launch_copy_rows(__nv_bfloat16* dst, const __nv_bfloat16* src, size_
 cudaError_t launch_kl(const float* zref, const float* zcur, int rows, int vocab, float* out,
                       float* part, int splits, cudaStream_t stream) {
   if (rows == 0) return cudaSuccess;
-  kl_partial_kernel<<<dim3(splits, rows), kKlThreads, 0, stream>>>(zref, zcur, vocab, splits, part);
-  kl_final_kernel<<<cdiv(rows, 8), 256, 0, stream>>>(part, splits, out, rows);
-  return cudaGetLastError();
+  // Launched early, one block per SM finds its SM free when the logits are done (one row pair, 7B: 168 ->
+  // 162 us with the LM head); twice as many pile up on the first SMs with room and make the rest
+  // wait (29 pairs, 1.5B: 103 -> 112 us), so those launch when the LM head has ended.
+  std::optional<PdlScope> pdl;
+  if (static_cast<long>(splits) * rows <= 152) pdl.emplace();
+  const cudaError_t e =
+      launch_kernel(kl_partial_kernel, dim3(splits, rows), dim3(kKlThreads), 0, stream, zref, zcur, vocab, splits, part);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(kl_final_kernel, dim3(cdiv(rows, 8)), dim3(256), 0, stream, static_cast<const float*>(part),
+                       splits, out, rows);
 }
 
 }  // namespace crf
