@@ -1,6 +1,6 @@
 // Persistent tcgen05 GEMM for sm_103a with the unmerged LoRA product and fused epilogues.
 //
-//   D[256 x BN] = A[256 x K] * B[BN x K]^T  (+ XA[256 x 64] * BL^T),  BN = 256 or 128
+//   D[256 x BN] = A[256 x K] * B[BN x K]^T  (+ XA[256 x 64] * BL^T),  BN = 256, 192 or 128
 //
 // A cluster of two CTAs on one TPC works on a 256 x BN tile with cta_group::2 MMAs. Each CTA
 // stages its own 128 rows of A and its own half of the B rows, so the operand bytes each SM
@@ -532,8 +532,8 @@ __device__ __noinline__ void drain_xa(const GemmArgs& a, int m_blk, uint32_t tac
 
 template <int BN, int STAGES, int EPI>
 __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_constant__ GemmArgs a) {
-  static_assert(BN == 256 || BN == 128, "CTA-pair tiles of 256 or 128 columns");
-  constexpr uint32_t TMEM_COLS = 2 * BN;
+  static_assert(BN == 256 || BN == 128 || (BN == 192 && EPI == kEpiResid), "CTA-pair tiles");
+  constexpr uint32_t TMEM_COLS = BN == 192 ? 512 : 2 * BN;  // two accumulators; a power of two
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -862,22 +862,31 @@ int group_tiles(const GemmDesc& d, int g, int bn) {
   return (d.group_cols[g] + cols - 1) / cols;
 }
 
-// 256-column tiles run the MMAs at their best rate; 128-column ones leave less of the last wave empty
-// and half the epilogue exposed at its end. Compared in K blocks of a 256-column tile: a tile's
-// hand-over costs about two, the last epilogue 10 and 5. Which one is taken changes no result: an
-// element's K order is the same.
+// 256-column tiles run the MMAs at their best rate; narrower ones leave less of the last wave empty
+// and less of the epilogue exposed at its end. Compared in K blocks of a 256-column tile: a tile's
+// hand-over costs about two, the last epilogue 10 per 256 columns, a 192-column block 0.84 and a
+// 128-column one 0.8 (its operands are half again as many bytes from L2 per FLOP: down of a 7B batch
+// of 8228 rows takes 445 us on 256 columns, 754 on 128). 192 columns only where an epilogue has no
+// heads or halves to keep together. Which one is taken changes no result: an element's K order is the
+// same.
 int tile_columns(const GemmDesc& d, int row_tiles, int num_kb, int units) {
-  // 128-column block 0.8: its operands are half again as many bytes from L2 per FLOP (down of a 7B
-  // batch of 8228 rows: 445 us on 256 columns, 754 on 128)
-  double cost[2];
-  for (int i = 0; i < 2; ++i) {
-    const int bn = i == 0 ? 256 : 128;
+  const int widths[3] = {256, 192, 128};
+  const double block[3] = {1.0, 0.84, 0.8};
+  int best = 0;
+  double best_cost = 0;
+  for (int i = 0; i < 3; ++i) {
+    const int bn = widths[i];
+    if (bn == 192 && d.epi != kEpiResid) continue;
     long tiles = 0;
     for (int g = 0; g < d.ngroups; ++g) tiles += static_cast<long>(group_tiles(d, g, bn)) * row_tiles;
     const long waves = (tiles + units - 1) / std::max(1, units);
-    cost[i] = waves * (num_kb * (i == 0 ? 1.0 : 0.8) + 2) + (i == 0 ? 10 : 5);
+    const double cost = waves * (num_kb * block[i] + 2) + 10.0 * bn / 256;
+    if (i == 0 || cost < best_cost) {
+      best = bn;
+      best_cost = cost;
+    }
   }
-  return cost[1] < cost[0] ? 128 : 256;
+  return best;
 }
 
 }  // namespace
@@ -978,6 +987,7 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t stream) {
   if (d.M == 0 || a.total_n == 0) return cudaSuccess;
   // one kernel per epilogue: each carries only its own epilogue code, which keeps the hot loops
   // of all its warps inside the SM's instruction cache
+  if (bn == 192) return launch_impl<192, 7, kEpiResid>(a, num_sms, stream);
   if (bn == 128) switch (d.epi) {
       case kEpiQkv: return launch_impl<128, 8, kEpiQkv>(a, num_sms, stream);
       case kEpiResid: return launch_impl<128, 8, kEpiResid>(a, num_sms, stream);
