@@ -207,3 +207,44 @@ def test_rows_of_a_batch_match_the_row_alone(rows, longest):
         m = ~own[:, None, :, None].expand_as(new)
         assert torch.equal(new[m], old[m])
     ctx.close()
+
+
+@pytest.mark.parametrize("vocab,rows", [(4096, 1), (4097, 2), (9001, 3), (20000, 32)])
+def test_greedy_token_over_several_blocks(vocab, rows):
+    """The greedy token where a row's logits are shared by several blocks (one at 4096, a second with
+    one logit at 4097, several with a ragged last one): equal LM head rows spread over all blocks tie for
+    the maximum and the lowest index wins; a NaN logit (a NaN in the LM head's first row) never does. With
+    every LM head row zero all logits are zeros of both signs, and token 0 wins."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2609_30884_gb300 as crf
+    cfg, lc = synth.replace(synth.TINY, vocab=vocab), synth.LORA_TINY
+    dm, ad = DeviceModel(cfg), DeviceAdapter(cfg, lc, 1)
+    pos = [5 + i for i in range(rows)]
+    P = sum(pages_needed(p + 1) for p in pos)
+    pts = split_page_tables([p + 1 for p in pos], P, seed=5)
+    pool = make_pool(cfg, P, fill="random", seed=6)
+    ctx = crf.Context(0)
+    tok = synth.token_ids(cfg, rows, device="cuda") % vocab
+
+    def step():
+        nxt = torch.empty(rows, dtype=torch.int32, device="cuda")
+        z = torch.empty(rows, vocab, device="cuda")
+        ctx.decode_step(dm.crf, ad.crf, pool, pos, pts, tok, nxt,
+                        ctx.decode_workspace(dm.crf, ad.crf, pos, pts, tok), logits=z)
+        ctx.check()
+        return to_np(nxt), to_np(z)
+
+    period = 97  # every block holds copies of every distinct row
+    dm.lm_head.copy_(dm.lm_head[:period].repeat(-(-vocab // period), 1)[:vocab].clone())
+    dm.lm_head[0, 0] = float("nan")
+    nxt, z = step()
+    for r in range(rows):
+        assert np.isnan(z[r, 0])
+        assert np.sum(z[r] == np.nanmax(z[r])) > 1
+        assert nxt[r] == np.nanargmax(z[r])
+    dm.lm_head.zero_()
+    dm.lm_head[::2].neg_()
+    nxt, z = step()
+    assert np.all(z == 0) and np.all(nxt == 0)
+    ctx.close()

@@ -84,6 +84,54 @@ def test_window_single_request(ctx, tiny, n, s, e):
     assert err <= REL_KVH, f"final hidden rel err {err:.3e}"
 
 
+@pytest.mark.parametrize("hidden,ffn,n", [(512, 688, 300), (576, 1024, 257), (1536, 688, 1025),
+                                          (1600, 1024, 1281), (2048, 688, 2003)])
+def test_window_tile_and_norm_widths(ctx, hidden, ffn, n):
+    """Widths at which the GEMM tiles and the norm change form, with one or a few rows past a 256-row tile
+    and every module adapted: rows that fill 2 pieces of a lane's registers exactly, 3 of 6 (a ragged
+    last piece), 6 exactly, and one past them (read twice); down on 128, 128, 128, 192 (64 columns in the
+    last tile) and 256 columns; gate|up on 128 (a ragged last tile at ffn 688) and, the last two, 256. One
+    layer from a restart, so the plain bar holds its two residual adds and nothing a later layer
+    amplifies."""
+    import paper_2609_30884_gb300 as crf
+    cfg = synth.replace(synth.TINY, n_layers=1, hidden=hidden, ffn=ffn)
+    lc = synth.replace(synth.LORA_TINY, modules=synth.MODULES)
+    dm, cur = DeviceModel(cfg), DeviceAdapter(cfg, lc, 1)
+    P = pages_needed(n) + 3
+    pool = make_pool(cfg, P, fill="random", seed=31)
+    pt = split_page_tables([n], P, seed=3)[0]
+    tokens = synth.token_ids(cfg, n, device="cuda")
+    h_out = [torch.empty(n, hidden, dtype=torch.bfloat16, device="cuda")]
+    before, opool = snapshot(pool), oracle_pool(pool)
+    _run(ctx, dm, cur, pool, [crf.Request(pt, 0, 1, n_tokens=n, tokens=tokens, hidden_out=h_out)])
+    oreq = C.RequestCache(to_np(tokens).astype(np.int64), pt.cpu().numpy())
+    C.recover(oracle_model(dm), oracle_adapter(cur), opool, oreq, 0, 1, restart=None)
+    _check_request(cfg, pool, before, opool, pt, n, 0, 1, h_out, oreq.hidden)
+
+
+@pytest.mark.parametrize("s,e", [(1, 4), (4, 4), (1, 3), (2, 2)])
+def test_final_hidden_out_of_any_alignment(ctx, tiny, s, e):
+    """final_hidden_out two bytes past a 16-byte boundary gets the bits of an aligned one, where it is a
+    copy of the last row (the window ends at the last layer, or there is none left) and where the
+    remaining layers run on that row; the element on either side stays."""
+    import paper_2609_30884_gb300 as crf
+    cfg, _, dm, cur, _, _ = tiny
+    n = 129
+    pool = make_pool(cfg, pages_needed(n), fill="random", seed=12)
+    pt = split_page_tables([n], pages_needed(n), seed=2)[0]
+    h_in = synth.hidden_state(cfg, n, device="cuda")
+    got = []
+    for shift in (0, 1):
+        buf = torch.full((cfg.hidden + 2,), 7.0, dtype=torch.bfloat16, device="cuda")
+        _run(ctx, dm, cur, pool, [crf.Request(pt, s, e, n_tokens=n, hidden_in=h_in,
+                                              final_hidden_out=buf[shift:shift + cfg.hidden])])
+        rest = buf.clone()
+        rest[shift:shift + cfg.hidden] = 7.0
+        assert torch.all(rest == 7.0)
+        got.append(buf[shift:shift + cfg.hidden].clone())
+    assert torch.equal(got[0], got[1])
+
+
 def test_batched_requests_shared_pool(ctx, tiny):
     cfg, lc, dm, cur, om, oa = tiny
     lengths = [100, 257, 512]
