@@ -41,10 +41,10 @@ UNIT = "layer*tokens/s"
 # and starts of complete affected suffixes (..N); full prefill is always timed. Default: 1, 2, 4.
 SWEEPS = {"1.5b-16k": ((1, 2, 4, 8), (14, 26))}
 FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
-# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu --set full
+# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
 # capture of the kernel as it now stands, at the full launch size of the 7B-shape 16K workload
 # (profiles/gemm_gateup_swiglu_7b16k.md). An entry is removed whenever its kernel changes.
-NCU_TRAFFIC_BYTES = {"gemm_gateup_swiglu": 2.921001e9 + 0.616805e9}
+NCU_TRAFFIC_BYTES = {"gemm_gateup_swiglu": 2.83e9 + 0.61476e9}
 
 
 def load_peaks():
@@ -687,7 +687,7 @@ def run_drift_case(args):
 
 
 def run_kl_only(args):
-    """crf_kl with the model's head alone (final norm + LM head GEMV + KL over --decode-rows row
+    """crf_kl with the model's head alone (final norm + LM head pass + KL over --decode-rows row
     pairs): the small profiling case of the head kernels (only the head weights on the device)."""
     import torch
     import synth

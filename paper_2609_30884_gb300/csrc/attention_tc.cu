@@ -14,7 +14,8 @@
 //               pages of 16 tokens each per tile, one 4-D copy per page)
 //               through one ring of kSlots shared-memory slots, so page
 //               gathers run two kv tiles ahead
-//   warp 1      allocates TMEM and issues tcgen05.mma from one thread:
+//   warp 1      allocates TMEM and issues tcgen05.mma (the warp runs the loop on
+//               voted waits, one elected lane issues):
 //               S_t = Q_t K^T into TMEM, then O_t += P_t V with P_t read
 //               from TMEM (A operand) and V an MN-major shared operand.
 //               The SM's MMA queue holds about two instructions, so every
@@ -29,6 +30,9 @@
 //               into TMEM as bf16 over the S columns; O rescaled in TMEM only
 //               when the running max grows by more than 2^8
 // TMEM: S0 | S1 | O0 | O1, 128 columns each. Every wait is bounded.
+// Bound by each tile's chain S -> softmax -> P V, not by the tensor pipe. One layer of the 7B shape at
+// 16384 rows: 1588 us with the producer's and issuer's loops in one lane, 1493 by whole warps, 1442
+// with the MMA descriptors formed once (1335 TFLOP/s of causal work).
 //
 // K/V slot layout: the 128 keys of a tile in 16 groups of 8 keys, group c at
 // c * HALVES * 1024 bytes, and within a group one 1 KB 128B-swizzled atom per

@@ -8,9 +8,10 @@
 // issues the MMAs; both CTAs hold 128 accumulator lanes in their own TMEM and drain them through
 // the same epilogue.
 //
-// Per CTA: warp 0 loads operands into a STAGES-deep shared-memory ring (TMA, issued by one lane),
-// warp 1 owns TMEM (two accumulators, so the epilogue of tile i overlaps the main loop of tile
-// i+1) and, in the MMA-issuing CTA, issues tcgen05.mma from one thread; warps 2..5 drain the
+// Per CTA: warp 0 loads operands into a STAGES-deep shared-memory ring (TMA: the warp runs the
+// loop on voted waits, which keeps its state in the uniform registers that TMA and MMA operands live
+// in, and one elected lane issues), warp 1 owns TMEM (two accumulators, so the epilogue of tile i overlaps the main loop of tile
+// i+1) and, in the MMA-issuing CTA, issues tcgen05.mma the same way; warps 2..5 drain the
 // accumulator (one TMEM lane = one output row per thread) through the fused epilogue. Operands
 // are bf16, K-major, staged with 128-byte swizzle; accumulation is fp32 in TMEM.
 //
@@ -31,10 +32,12 @@
 // (1.5B shape, 2003 rows: 7 of the 28 us of q|k|v, 19 of the 77 us of down). Items over a quarter of K
 // each were slower: their sums met through memory.
 //
-// Measured (us a launch: items, epilogue through shared memory and tile width together, before ->
-// now): 1.5B shape, 2003 rows: q|k|v 34 -> 28, o 33 -> 24, gate|up 99 -> 88, down 84 -> 60; 4096 rows:
-// 45 -> 39, 48 -> 35, 164 -> 150, 131 -> 108; 7B, 16384 rows: 370 -> 358, 282 -> 283, 2582 -> 2546,
-// 1288 -> 1356 (K = 18944 makes its 64 items long).
+// Measured (us a launch; first column: the XA product in each row block's first tile, 256-column tiles,
+// one row a thread in the epilogue; then: XA items, epilogue through shared memory, 128 columns; last:
+// loops run by whole warps and, for o and down, 192 columns):
+//   1.5B,  2003 rows: q|k|v  34,  28,  25   o  33,  24,  21   gate|up   99,   88,   71   down   84,   60,   45
+//   1.5B,  4096 rows:        45,  39,  34      48,  35,  29            164,  150,  126         131,  108,   80
+//   7B,   16384 rows:       370, 358, 318     282, 283, 258           2582, 2546, 2271        1288, 1356, 1255
 #include "common.cuh"
 #include "kernels.h"
 

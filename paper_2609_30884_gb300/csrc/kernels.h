@@ -41,9 +41,11 @@ constexpr int kBxCols = 64;
 // Programmatic dependent launch for chains of short kernels. While a PdlScope is alive on the
 // calling thread, the launchers below that go through launch_kernel() give their kernels the
 // programmatic-stream-serialization attribute: such a kernel becomes resident while its
-// predecessor in the stream still runs, prefetches its weights and then waits for it
-// (griddep_wait). Every kernel launched this way calls griddep_wait before it touches memory
-// that an earlier kernel may write. crf_recompute_window and crf_decode_step open a scope.
+// predecessor in the stream still runs, sets itself up (a weight pass requests its first weights) and
+// then waits for it (griddep_wait). Every kernel launched this way calls griddep_wait before it
+// touches memory that an earlier kernel may write, and before it ends, since the kernels behind it
+// count on all before it having ended. Window calls, generation steps, the KL reduction over few
+// rows and drift open a scope.
 class PdlScope {
  public:
   PdlScope();

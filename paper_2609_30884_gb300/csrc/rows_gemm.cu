@@ -9,7 +9,7 @@
 // of bf16 values are exact in fp32, accumulation is fp32. The tensor core cuts its running
 // sums off instead of rounding them, so a long sum drifts by half a unit a step (4e-6 of a logit's
 // size after 224 steps, against 1e-7 for rounded sums): where the rows are exact, a unit's steps
-// accumulate in up to eight groups of TMEM columns, which the epilogue adds.
+// accumulate in four groups of TMEM columns (eight in a pass of its own), which the epilogue adds.
 //
 // Units of work: (128-row weight tile, K split); a tile's `splits` units are spread over CTAs so
 // that a narrow projection still fills the chip, and each writes its own partial sums
@@ -26,10 +26,11 @@
 // weights before the wait gained nothing). Weights are marked evict-first in L2, which keeps the
 // rows' partial sums and the K/V pages there (3% of a 7B generation step).
 //
-// Measured (7B shape, weights read once): LM head, 2 rows, 1.09 GB in 166 us (6.6 TB/s, 97% of the
-// copy rate); gate|up, 272 MB in 46 us (5.9 TB/s) behind the chain's prefetch. 58 rows of the 1.5B
-// LM head: 92 us in one pass (a pass for every 8 rows before: 779 us); a generation step of 32 rows:
-// 18.0 -> 4.8 ms.
+// Measured with the norm before it: LM head of the 7B shape, 2 rows, 1.09 GB in 162 us (6.7 TB/s, the
+// copy rate); gate|up of one row, alone and cold, 272 MB in
+// 45 us (6.1 TB/s; 56 us before); 58 rows of the 1.5B LM head 83 us in one pass (a pass for every 8 rows before: 779 us).
+// Generation steps with all that this layout brought, CUDA-core and mma.sync passes of 8 rows before:
+// 7B 1 row 4.06 -> 2.95 ms, 32 rows 18.0 -> 4.32 ms, 1.5B 8 rows 2.35 -> 1.39 ms.
 #include "common.cuh"
 #include "kernels.h"
 #include "tma_map.h"

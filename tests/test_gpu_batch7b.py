@@ -3,9 +3,9 @@ its own window, one shared pool with a randomly permuted page table.
 
 * Batching is invisible in the window: the batched call gives bit-identical pages and refreshed
   checkpoints to running every request alone (each row is computed the same way whatever else
-  shares its tile or launch); the first-step rows agree to the per-layer 1e-2 bar (their GEMV
-  kernel depends on how many rows share a weight pass, and its rounding compounds over the layers
-  after the window).
+  shares its tile or launch); the first-step rows agree to the per-layer 1e-2 bar (how many
+  bf16 terms carry a row depends on how many rows share a weight pass, and the rounding compounds over
+  the layers after the window).
 * Against the oracle, per request, on what it computes at this size: K and V of every position of
   the request's first window layer, and that layer's output at 48 rows spread over the prefix,
   held to 1e-2 or 1.25x the distance the oracle's layer moves at the same rows when it stores its
@@ -81,9 +81,8 @@ def test_batch7b_equals_single_and_oracle(ctx):
             assert torch.equal(request_kv_t(pool.k_pages[l], pts[i], n), request_kv_t(got_k[l], pts[i], n)), (i, l)
             assert torch.equal(request_kv_t(pool.v_pages[l], pts[i], n), request_kv_t(got_v[l], pts[i], n)), (i, l)
             assert torch.equal(keep1[i][2][l - s], keep[i][2][l - s]), (i, l)
-        # the first-step row takes the tensor-core GEMV (main and adapter-down products) when >= 3
-        # rows share a weight pass and the CUDA-core one alone: both fp32-accurate, but their
-        # rounding differs and compounds over every layer the row passes after its window (26 after a
+        # the first-step row enters the weight passes as two bf16 terms when many rows share
+        # them and as three alone: the rounding differs and compounds over every layer the row passes after its window (26 after a
         # window [0, 2)), so it is held to the per-layer bar the oracle tests use
         fin_err.append(rel_frob(to_np(keep1[i][3]), to_np(keep[i][3])))
     print("first-step row, batched vs alone:", [f"{x:.2e}" for x in fin_err])
