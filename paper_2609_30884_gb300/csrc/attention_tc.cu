@@ -4,7 +4,7 @@
 // whose K/V are the cache entries of Eq. 1 (projections of Eq. S3).
 //
 // softmax(q k^T / sqrt(d) + causal mask) v over the whole prefix for every
-// query head; query head h reads kv head h / (Hq / Hkv). One CTA takes two
+// query head; query head h reads kv head h / (Hq / Hkv). One CTA (or two, below) takes two
 // consecutive 128-row query tiles of one head (rows q0 .. q0+255): both read
 // the same K/V tiles except the last, which only the second tile needs, so
 // each K/V tile is fetched once for 256 query rows whatever the group size.
@@ -33,6 +33,11 @@
 // Bound by each tile's chain S -> softmax -> P V, not by the tensor pipe. One layer of the 7B shape at
 // 16384 rows: 1588 us with the producer's and issuer's loops in one lane, 1493 by whole warps, 1442
 // with the MMA descriptors formed once (1335 TFLOP/s of causal work).
+//
+// The last pair's chain over all keys sets the time of a short prefix that leaves SMs idle (1.5B shape,
+// 2003 rows: 96 CTAs). There (splits_keys) a cluster of two shares each pair's keys and meets in
+// shared memory: prefill of 2003 rows 1.49 -> 1.43 ms, tiny window 112 -> 107 us, 387-row 7B window
+// 1.012 -> 1.007 ms. Errors of the checkpoints against 64 bits stay the same to 2e-6.
 //
 // K/V slot layout: the 128 keys of a tile in 16 groups of 8 keys, group c at
 // c * HALVES * 1024 bytes, and within a group one 1 KB 128B-swizzled atom per
@@ -78,13 +83,43 @@ struct AttnTcArgs {
 
 struct AttnWork {
   int req, qp, head, g;
+  bool split;
 };
 
-// Items: (request, 256-row query pair, head), longest (latest) query pairs first.
+// Whether the query pairs of a request of `len` rows are dealt to two CTAs each (halves of their keys):
+// where its longest pair alone runs over twice an even share of all pairs on 152 SMs. The halves cost a
+// second prologue and an exchange, which 1.5 times an even share does not repay (1.5B shape, us a
+// window of 4096 rows: 905 whole, 912 split; a prefill of 2003 rows, 2.8 times: 1490 and 1429).
+// A property of the request, not of the call: a request gives the same bits in any batch.
+constexpr int kSplitTiles = 4;  // pairs of fewer kv tiles are not split
+__host__ __device__ inline bool splits_keys(int len, int n_q_heads) {
+  const long long tiles = (len + kN - 1) / kN, nqp = (len + 2 * kM - 1) / (2 * kM);
+  const long long sum = nqp * (nqp + 1) - (tiles & 1);  // kv tiles of all pairs of a head
+  return tiles >= kSplitTiles && tiles * 152 > 2 * n_q_heads * sum;
+}
+
+// Items: (request, 256-row query pair, head), longest (latest) query pairs first. With kPair a
+// cluster of two takes one item of a request that splits, two of one that does not.
+template <bool kPair>
 __device__ __forceinline__ bool attn_work(const AttnTcArgs& a, int idx, AttnWork& w) {
+  const int rank = idx & 1;
+  if (kPair) idx >>= 1;
   for (int i = 0; i < a.req.n; ++i) {
     const int nqp = (a.req.len[i] + 2 * kM - 1) / (2 * kM);
-    const int items = nqp * a.n_q_heads;
+    int items = nqp * a.n_q_heads;
+    w.split = false;
+    if (kPair) {
+      w.split = splits_keys(a.req.len[i], a.n_q_heads);
+      if (!w.split) {
+        const int clusters = (items + 1) / 2;
+        if (idx >= clusters) {
+          idx -= clusters;
+          continue;
+        }
+        idx = 2 * idx + rank;
+        if (idx >= items) return false;
+      }
+    }
     if (idx < items) {
       w.req = i;
       w.qp = nqp - 1 - idx / a.n_q_heads;
@@ -183,8 +218,12 @@ __device__ __forceinline__ void regs_inc_softmax() {
   asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
 }
 
-template <int D>
-__global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_constant__ AttnTcArgs a) {
+__device__ __forceinline__ void st_cluster_f32(uint32_t cluster_addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
+}
+
+template <int D, bool kPair>
+__device__ __forceinline__ void attn_body(const AttnTcArgs& a) {
   constexpr int HALVES = D / 64;
   constexpr int Q_BYTES = kM * D * 2;
   constexpr int KV_BYTES = kN * D * 2;
@@ -204,15 +243,35 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
 
   AttnWork w;
   griddep_launch_dependents();
-  if (!attn_work(a, blockIdx.x, w)) return;
+  if (!attn_work<kPair>(a, blockIdx.x, w)) return;
   const int n = a.req.len[w.req];
   const int row0 = a.req.row0[w.req];
   const int32_t* pt = a.req.page_table[w.req];
   const int q0 = w.qp * 2 * kM;
   const int ntiles = q0 + kM < n ? 2 : 1;
   const int kv_end = min(q0 + ntiles * kM, n);
-  const int J = (kv_end + kN - 1) / kN;    // kv tiles of the last query tile
-  const int J0 = ntiles == 2 ? J - 1 : J;  // kv tiles of query tile 0 (its diagonal is tile J0-1)
+  int J = (kv_end + kN - 1) / kN;    // kv tiles of the last query tile
+  int J0 = ntiles == 2 ? J - 1 : J;  // kv tiles of query tile 0 (its diagonal is tile J0-1)
+  // A split pair: the even CTA takes the first half of the kv tiles, the odd one the rest with
+  // both diagonals; tiles are counted from `jb` below.
+  int jb = 0;
+  bool split = false, diagonal = true;
+  const int rank = kPair ? static_cast<int>(blockIdx.x & 1) : 0;
+  if (kPair && w.split) {
+    split = J >= kSplitTiles;
+    if (!split && rank == 1) return;
+    if (split) {
+      const int half = J / 2;
+      diagonal = rank == 1;
+      if (rank == 1) {
+        jb = half;
+        J -= half;
+        J0 -= half;
+      } else {
+        J = J0 = half;
+      }
+    }
+  }
   const int n_pages = (n + kPage - 1) / kPage;
 
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);  // uniform
@@ -269,7 +328,7 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
       uint32_t ph = 0;
       // pages past the prefix repeat the last page: finite data, masked below
       auto page_id = [&](int j) {
-        return checked_page(pt[min(j * kPagesPerTile + (lane & (kPagesPerTile - 1)), n_pages - 1)], a.req.num_pages,
+        return checked_page(pt[min((jb + j) * kPagesPerTile + (lane & (kPagesPerTile - 1)), n_pages - 1)], a.req.num_pages,
                             a.status);
       };
       int ids = page_id(0);
@@ -367,21 +426,26 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
         mbar_wait(&drain_bar, 0, &never, nullptr);
       }
     }
+    if (kPair && split) {
+      __syncwarp();
+      cluster_sync();
+      cluster_sync();
+    }
   } else {
     regs_inc_softmax();
     // ---------------------------------------------------------------- softmax + epilogue
     const int t = (warp - 4) >> 2;
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;  // query row within the tile (= TMEM lane)
+    const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
+    const uint32_t tO = tmem + lane_off + 256 + t * 128;
+    const float sl2 = 1.4426950408889634f * rsqrtf(static_cast<float>(D));
+    const int qrow = q0 + t * kM + r;
+    float m_run = -INFINITY, l_run = 0.f;  // running max in raw score units
+    bool ok = t < ntiles;
     if (t < ntiles) {
-      const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
       const uint32_t tS = tmem + lane_off + t * 128;
-      const uint32_t tO = tmem + lane_off + 256 + t * 128;
-      const float sl2 = 1.4426950408889634f * rsqrtf(static_cast<float>(D));
-      const int qrow = q0 + t * kM + r;
       const int Jt = t == 0 ? J0 : J;
-      float m_run = -INFINITY, l_run = 0.f;  // running max in raw score units
-      bool ok = true;
       for (int j = 0; j < Jt && ok; ++j) {
         // warp-uniform outcome: the TMEM accesses below are warp-collective
         ok = __all_sync(0xffffffffu, mbar_wait(&s_full[t], j & 1, &abort_flag, a.status));
@@ -394,9 +458,9 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
           mbar_arrive(&kv_empty[(2 * j) % kSlots]);
           if (j > 0) mbar_arrive(&kv_empty[(2 * j - 1) % kSlots]);
         }
-        const int k0 = j * kN;
+        const int k0 = (jb + j) * kN;
         const bool last = j == Jt - 1;
-        if (last) {
+        if (last && diagonal) {
           // keys above min(query row, prefix end - 1) are masked on the diagonal tile
           softmax_tile<D, true>(tS, tO, j == 0, min(qrow, kv_end - 1) - k0, sl2, m_run, l_run);
         } else {
@@ -436,25 +500,63 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
         if (lane == 0) mbar_arrive(&p_full[t]);
       }
       if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&o_full, 0, &abort_flag, a.status));
-      if (ok) {
+    }
+    // A split pair's halves meet in shared memory, free once every product of both CTAs is done: each
+    // CTA hands its rows of the peer's query tile over (column-major, so a warp writes whole lines)
+    // and finishes its own (tile 0 in the even CTA).
+    float* xo = reinterpret_cast<float*>(sKV);  // [D][128] of O, then 128 maxima and 128 sums
+    const bool give = kPair && split && t != rank;
+    if (kPair && split) {
+      __syncwarp();
+      cluster_sync();
+      if (give && t < ntiles) {
         tc_fence_after();
-        const float inv = l_run > 0.f ? 1.0f / l_run : 0.f;
-        const bool store = qrow < n;
-        __nv_bfloat16* dst = a.out + (size_t)(row0 + qrow) * a.ldo + w.head * D;
+        const uint32_t peer = mapa_shared(xo, rank ^ 1) + r * 4;
+#pragma unroll 1
         for (int c = 0; c < D / 32; ++c) {
           uint32_t o[32];
           tmem_ld32(tO + c * 32, o);
           tmem_ld_wait();
-          if (store) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              uint4 v;
-              v.x = pack_bf16(__uint_as_float(o[8 * i + 0]) * inv, __uint_as_float(o[8 * i + 1]) * inv);
-              v.y = pack_bf16(__uint_as_float(o[8 * i + 2]) * inv, __uint_as_float(o[8 * i + 3]) * inv);
-              v.z = pack_bf16(__uint_as_float(o[8 * i + 4]) * inv, __uint_as_float(o[8 * i + 5]) * inv);
-              v.w = pack_bf16(__uint_as_float(o[8 * i + 6]) * inv, __uint_as_float(o[8 * i + 7]) * inv);
-              reinterpret_cast<uint4*>(dst + c * 32)[i] = v;
-            }
+          for (int i = 0; i < 32; ++i) st_cluster_f32(peer + (c * 32 + i) * kM * 4, __uint_as_float(o[i]));
+        }
+        st_cluster_f32(peer + D * kM * 4, m_run);
+        st_cluster_f32(peer + (D + 1) * kM * 4, l_run);
+        tc_fence_before();
+      }
+      __syncwarp();
+      cluster_sync();
+    }
+    if (ok && !give) {
+      tc_fence_after();
+      float own = 1.f, other = 0.f;
+      if (kPair && split) {
+        const float m1 = xo[D * kM + r], l1 = xo[(D + 1) * kM + r], m = fmaxf(m_run, m1);
+        own = ex2_approx((m_run - m) * sl2);
+        other = ex2_approx((m1 - m) * sl2);
+        l_run = l_run * own + l1 * other;
+      }
+      const float inv = l_run > 0.f ? 1.0f / l_run : 0.f;
+      const bool store = qrow < n;
+      __nv_bfloat16* dst = a.out + (size_t)(row0 + qrow) * a.ldo + w.head * D;
+      for (int c = 0; c < D / 32; ++c) {
+        uint32_t o[32];
+        tmem_ld32(tO + c * 32, o);
+        tmem_ld_wait();
+        if (kPair && split) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            o[i] = __float_as_uint(__uint_as_float(o[i]) * own + xo[(c * 32 + i) * kM + r] * other);
+        }
+        if (store) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            uint4 v;
+            v.x = pack_bf16(__uint_as_float(o[8 * i + 0]) * inv, __uint_as_float(o[8 * i + 1]) * inv);
+            v.y = pack_bf16(__uint_as_float(o[8 * i + 2]) * inv, __uint_as_float(o[8 * i + 3]) * inv);
+            v.z = pack_bf16(__uint_as_float(o[8 * i + 4]) * inv, __uint_as_float(o[8 * i + 5]) * inv);
+            v.w = pack_bf16(__uint_as_float(o[8 * i + 6]) * inv, __uint_as_float(o[8 * i + 7]) * inv);
+            reinterpret_cast<uint4*>(dst + c * 32)[i] = v;
           }
         }
       }
@@ -467,6 +569,18 @@ __global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_c
     tc_fence_after();
     tmem_dealloc(tmem, TMEM_COLS);
   }
+}
+
+template <int D>
+__global__ void __launch_bounds__(kThreadsAttn, 1) attn_tc_kernel(const __grid_constant__ AttnTcArgs a) {
+  attn_body<D, false>(a);
+}
+
+// Launched where a request of the call splits its keys.
+template <int D>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsAttn, 1)
+    attn_tc_pair_kernel(const __grid_constant__ AttnTcArgs a) {
+  attn_body<D, true>(a);
 }
 
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
@@ -516,22 +630,26 @@ bool map2d(CUtensorMap* m, const void* base, long rows, int cols, int box_rows) 
 }
 
 template <int D>
-cudaError_t launch_tc(const AttnTcArgs& args, cudaStream_t stream) {
+cudaError_t launch_tc(const AttnTcArgs& args, bool pair, cudaStream_t stream) {
   constexpr int smem = 2 * kM * D * 2 + kSlots * kN * D * 2 + 1024;
+  static_assert((D + 2) * kM * 4 <= kSlots * kN * D * 2, "a split pair's exchange fits the K/V ring");
   static PerDevice once;
   int dev = 0;
   if (once.pending(&dev)) {
-    cudaError_t e = cudaFuncSetAttribute(attn_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    // setmaxnreg.inc waits until the CTA's register pool can serve it: refuse to launch a
-    // build whose per-thread launch count leaves the split short
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, attn_tc_kernel<D>);
-    if (e != cudaSuccess) return e;
-    if (fa.numRegs * kThreadsAttn < kRegsNeeded) return cudaErrorInvalidConfiguration;
+    for (auto* kern : {attn_tc_kernel<D>, attn_tc_pair_kernel<D>}) {
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (e != cudaSuccess) return e;
+      // setmaxnreg.inc waits until the CTA's register pool can serve it: refuse to launch a
+      // build whose per-thread launch count leaves the split short
+      cudaFuncAttributes fa;
+      e = cudaFuncGetAttributes(&fa, kern);
+      if (e != cudaSuccess) return e;
+      if (fa.numRegs * kThreadsAttn < kRegsNeeded) return cudaErrorInvalidConfiguration;
+    }
     once.done(dev);
   }
-  return launch_kernel(attn_tc_kernel<D>, dim3(args.total_items), dim3(kThreadsAttn), smem, stream, args);
+  return launch_kernel(pair ? attn_tc_pair_kernel<D> : attn_tc_kernel<D>, dim3(args.total_items), dim3(kThreadsAttn), smem,
+                       stream, args);
 }
 
 }  // namespace
@@ -552,12 +670,16 @@ cudaError_t launch_attention_tc(const AttnDesc& d, int num_pages, int total_rows
   a.req = d.req;
   a.status = d.status;
   a.abort = d.abort;
+  bool pair = false;
+  for (int i = 0; i < d.req.n; ++i) pair |= splits_keys(d.req.len[i], d.n_q_heads);
   a.total_items = 0;
-  for (int i = 0; i < d.req.n; ++i)
-    a.total_items += ((d.req.len[i] + 2 * kM - 1) / (2 * kM)) * d.n_q_heads;
+  for (int i = 0; i < d.req.n; ++i) {
+    const int items = ((d.req.len[i] + 2 * kM - 1) / (2 * kM)) * d.n_q_heads;
+    a.total_items += !pair ? items : splits_keys(d.req.len[i], d.n_q_heads) ? 2 * items : (items + 1) / 2 * 2;
+  }
   if (a.total_items == 0) return cudaSuccess;
-  if (D == 128) return launch_tc<128>(a, stream);
-  if (D == 64) return launch_tc<64>(a, stream);
+  if (D == 128) return launch_tc<128>(a, pair, stream);
+  if (D == 64) return launch_tc<64>(a, pair, stream);
   return cudaErrorInvalidValue;
 }
 

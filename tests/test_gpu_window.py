@@ -132,6 +132,36 @@ def test_final_hidden_out_of_any_alignment(ctx, tiny, s, e):
     assert torch.equal(got[0], got[1])
 
 
+@pytest.mark.parametrize("lengths", [(384,), (385,), (513,), (769,), (1409,), (130, 385, 1, 900, 257)])
+def test_attention_keys_split_over_two_ctas(ctx, lengths):
+    """Prefixes around the one from which a query pair's keys are dealt to two CTAs (four kv tiles: 385
+    rows), pairs of even and odd tile counts, a last pair of one query tile, and a batch that mixes
+    requests that split with ones that do not, with an odd number of (pair, head) items in those. One
+    layer from the tokens against the oracle; in the batch, each request alone gives the same bits."""
+    import paper_2609_30884_gb300 as crf
+    cfg = synth.replace(synth.TINY, n_layers=1, n_q_heads=3, n_kv_heads=1)
+    dm, cur = DeviceModel(cfg), DeviceAdapter(cfg, synth.LORA_TINY, 1)
+    P = sum(pages_needed(n) for n in lengths) + 3
+    pool = make_pool(cfg, P, fill="random", seed=41)
+    pts = split_page_tables(list(lengths), P, seed=3)
+    before, opool = snapshot(pool), oracle_pool(pool)
+    tokens = [synth.token_ids(cfg, n, request=i, device="cuda") for i, n in enumerate(lengths)]
+
+    def run(idx):
+        outs = [[torch.empty(lengths[i], cfg.hidden, dtype=torch.bfloat16, device="cuda")] for i in idx]
+        _run(ctx, dm, cur, pool, [crf.Request(pts[i], 0, 1, n_tokens=lengths[i], tokens=tokens[i], hidden_out=o)
+                                  for i, o in zip(idx, outs)])
+        return outs
+
+    outs = run(range(len(lengths)))
+    for i, n in enumerate(lengths):
+        oreq = C.RequestCache(to_np(tokens[i]).astype(np.int64), pts[i].cpu().numpy())
+        C.recover(oracle_model(dm), oracle_adapter(cur), opool, oreq, 0, 1, restart=None)
+        _check_request(cfg, pool, before, opool, pts[i], n, 0, 1, outs[i], oreq.hidden, tag=f"req{i}")
+        if len(lengths) > 1:
+            assert torch.equal(run([i])[0][0], outs[i][0])
+
+
 def test_batched_requests_shared_pool(ctx, tiny):
     cfg, lc, dm, cur, om, oa = tiny
     lengths = [100, 257, 512]
