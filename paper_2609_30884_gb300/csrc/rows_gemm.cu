@@ -7,9 +7,13 @@
 // the B operand: each fp32 row enters as bf16 terms in rows of their own (kTerms per row, 2: about
 // 16 mantissa bits, 3: the whole fp32 value), and the epilogue adds a row's term columns; products
 // of bf16 values are exact in fp32, accumulation is fp32. The tensor core cuts its running
-// sums off instead of rounding them, so a long sum drifts by half a unit a step (4e-6 of a logit's
-// size after 224 steps, against 1e-7 for rounded sums): where the rows are exact, a unit's steps
-// accumulate in four groups of TMEM columns (eight in a pass of its own), which the epilogue adds.
+// sums off instead of rounding them, so a long sum drifts by half a unit a step: where the rows are
+// exact (three terms), a unit's steps accumulate in groups of TMEM columns, and one or two rows, which
+// fill 6 of 16 columns, bring every other K block's terms 8 columns on (a box that starts 8 rows
+// early, zero-filled) into sums of their own
+// (the LM head alone: a pass in the chain has four groups). Error of the 7B LM head's logits against 64
+// bits, one pair of rows: 4.48e-7 in sums of 32 MMAs, 1.17e-7 in sums of 4; fp32 sums on CUDA cores
+// 1.22e-7. 1.5B: 2.17e-7, 1.02e-7, 1.10e-7.
 //
 // Units of work: (128-row weight tile, K split); a tile's `splits` units are spread over CTAs so
 // that a narrow projection still fills the chip, and each writes its own partial sums
@@ -26,8 +30,8 @@
 // weights before the wait gained nothing). Weights are marked evict-first in L2, which keeps the
 // rows' partial sums and the K/V pages there (3% of a 7B generation step).
 //
-// Measured with the norm before it: LM head of the 7B shape, 2 rows, 1.09 GB in 162 us (6.7 TB/s, the
-// copy rate); gate|up of one row, alone and cold, 272 MB in
+// Measured with the norm before it: LM head of the 7B shape, 2 rows, 1.09 GB in 170 us (6.4 TB/s; 162
+// with sums of 32 MMAs); gate|up of one row, alone and cold, 272 MB in
 // 45 us (6.1 TB/s; 56 us before); 58 rows of the 1.5B LM head 83 us in one pass (a pass for every 8 rows before: 779 us).
 // Generation steps with all that this layout brought, CUDA-core and mma.sync passes of 8 rows before:
 // 7B 1 row 4.06 -> 2.95 ms, 32 rows 18.0 -> 4.32 ms, 1.5B 8 rows 2.35 -> 1.39 ms.
@@ -44,6 +48,7 @@ namespace {
 
 constexpr int kTile = 128;
 constexpr int kBlockK = 64;  // one 128-byte swizzled box; a step takes plan.sub of them side by side
+constexpr int kExactGroups = 32;  // accumulation groups of a pass of its own: all of TMEM
 constexpr int kRgThreads = 192;  // producer, MMA and four epilogue warps
 constexpr int kMaxStages = 12;
 constexpr int kWBytes = kTile * kBlockK * 2;
@@ -55,6 +60,7 @@ struct RowsGemmArgs {
   RowsPlan plan;
   int nseg, n_lora, units;
   int rows, n, stages, acc_cols, groups;
+  int phases;   // 2: odd K blocks bring their rows 8 columns on, into sums of their own
   uint32_t tmem_cols;
   float* y;
   const float* nss;
@@ -80,8 +86,16 @@ struct Steps {
   __device__ __forceinline__ bool more(const RowsGemmArgs& a) const { return u < a.units; }
 };
 
-template <int kTerms>
-__global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_constant__ RowsGemmArgs a) {
+// s + e += x, the rounding error of s + x kept in e.
+__device__ __forceinline__ void two_sum(float& s, float& e, float x) {
+  const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+  e += __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+  s = t;
+}
+
+// kExact: a pass of its own over exact rows (three terms, 16 columns).
+template <int kTerms, bool kExact>
+__global__ void __launch_bounds__(kRgThreads, 1) rows_gemm_kernel(const __grid_constant__ RowsGemmArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -144,7 +158,7 @@ __global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_cons
       for (int h = 0; h < sub; ++h)
         if (issuer)
           tma_load_2d(smem + st * stage_bytes + sub * kWBytes + h * x_bytes, &a.tmX, &full[st],
-                      (s.kb * sub + h) * kBlockK, 0);
+                      (s.kb * sub + h) * kBlockK, kExact && a.phases == 2 ? -8 * ((s.kb * sub + h) & 1) : 0);
     };
     Steps w, x;
     w.at(a, blockIdx.x);
@@ -187,8 +201,8 @@ __global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_cons
     uint32_t ph = 0;
     Steps s;
     for (s.at(a, blockIdx.x); ok && s.more(a); ++it) {
-      const int acc = it & 1;
-      if (!mbar_wait_warp(&tempty[acc], ((it >> 1) & 1) ^ 1, &abort_flag, a.status)) {
+      const int acc = kExact ? 0 : it & 1, turn = kExact ? it : it >> 1;
+      if (!mbar_wait_warp(&tempty[acc], (turn & 1) ^ 1, &abort_flag, a.status)) {
         ok = false;
         break;
       }
@@ -244,24 +258,14 @@ __global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_cons
     const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
     int it = 0;
     for (int u = blockIdx.x; u < a.units; u += gridDim.x, ++it) {
-      const int acc = it & 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(&tfull[acc], (it >> 1) & 1, &abort_flag, a.status))) break;
+      const int acc = kExact ? 0 : it & 1, turn = kExact ? it : it >> 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(&tfull[acc], turn & 1, &abort_flag, a.status))) break;
       tc_fence_after();
       const int tile = u / a.plan.splits;
       const int col = tile * kTile + quarter * 32 + lane;
       float* y = a.y + static_cast<size_t>(u - tile * a.plan.splits) * a.rows * a.plan.ncols + col;
       const bool store = !skip && col < a.plan.ncols;
-      for (int c = 0; c < a.n; c += 16) {
-        float v[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = 0.f;
-        for (int k = 0; k < a.groups; ++k) {
-          uint32_t w[16];
-          tmem_ld16(tmem + lane_off + acc * a.acc_cols + k * a.n + c, w);
-          tmem_ld_wait();
-#pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] += __uint_as_float(w[i]);
-        }
+      auto put = [&](int c, const float (&v)[16]) {
 #pragma unroll
         for (int i = 0; i < 16 / kTerms; ++i) {
           const int r = c / kTerms + i;
@@ -270,10 +274,65 @@ __global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_cons
           for (int t = 1; t < kTerms; ++t) s += v[kTerms * i + t];
           if (store && r < a.rows) y[static_cast<size_t>(r) * a.plan.ncols] = s * s_inv[r];
         }
+      };
+      auto release = [&]() {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tempty[acc]);
+      };
+      const uint32_t t0 = tmem + lane_off + acc * a.acc_cols;
+      if constexpr (kExact) {
+        // Four groups as a tree, read before the accumulator is handed back; the rounding errors of the
+        // sum over the fours are carried along while the next unit's products run (before the
+        // hand-back it outlasts the ring: LM head and KL of the 7B shape 170 us).
+        float f[kExactGroups / 4][16];
+#pragma unroll
+        for (int k = 0; k < kExactGroups / 4; ++k) {
+          // groups past the last hold what an earlier launch left: read, not used
+          uint32_t w[4][16];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) tmem_ld16(t0 + (4 * k + q) * 16, w[q]);
+          tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const float g1 = 4 * k + 1 < a.groups ? __uint_as_float(w[1][i]) : 0.f;
+            const float g2 = 4 * k + 2 < a.groups ? __uint_as_float(w[2][i]) : 0.f;
+            const float g3 = 4 * k + 3 < a.groups ? __uint_as_float(w[3][i]) : 0.f;
+            f[k][i] = (__uint_as_float(w[0][i]) + g1) + (g2 + g3);
+          }
+        }
+        release();
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          float e = 0.f;
+          v[i] = f[0][i];
+#pragma unroll
+          for (int k = 1; k < kExactGroups / 4; ++k)
+            if (4 * k < a.groups) two_sum(v[i], e, f[k][i]);
+          if (isfinite(v[i])) v[i] += e;  // a sum that is not finite has no error term
+        }
+        if (a.phases == 2) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) v[i] += v[8 + i];
+        }
+        put(0, v);
+      } else {
+        for (int c = 0; c < a.n; c += 16) {
+          float v[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] = 0.f;
+          for (int k = 0; k < a.groups; ++k) {
+            uint32_t w[16];
+            tmem_ld16(t0 + k * a.n + c, w);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] += __uint_as_float(w[i]);
+          }
+          put(c, v);
+        }
+        release();
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&tempty[acc]);
     }
   }
 
@@ -285,17 +344,17 @@ __global__ void __launch_bounds__(kRgThreads) rows_gemm_kernel(const __grid_cons
   }
 }
 
-template <int kTerms>
+template <int kTerms, bool kExact>
 cudaError_t launch_terms(const RowsGemmArgs& a, int grid, int smem, cudaStream_t stream) {
   static PerDevice once;
   int dev = 0;
   if (once.pending(&dev)) {
-    cudaError_t e = cudaFuncSetAttribute(rows_gemm_kernel<kTerms>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(rows_gemm_kernel<kTerms, kExact>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kRowsRingMax + 1024);
     if (e != cudaSuccess) return e;
     once.done(dev);
   }
-  return launch_kernel(rows_gemm_kernel<kTerms>, dim3(grid), dim3(kRgThreads), smem, stream, a);
+  return launch_kernel(rows_gemm_kernel<kTerms, kExact>, dim3(grid), dim3(kRgThreads), smem, stream, a);
 }
 
 }  // namespace
@@ -356,11 +415,17 @@ cudaError_t launch_rows_gemm(const RowsGemmDesc& d, const RowsPlan& plan, int nu
   a.n_lora = d.n_lora;
   a.units = plan.tiles * plan.splits;
   a.rows = d.rows;
-  // exact rows keep fp32 accuracy: groups of a unit's steps accumulate apart (at least one each)
-  a.groups = d.terms == 3 ? std::min(d.alone ? 8 : 4, plan.kb / plan.splits) : 1;
-  a.acc_cols = 16;
+  // exact rows: groups of a unit's steps accumulate apart (at least one step each)
+  // A pass of its own fills all of TMEM with one accumulator of 32 groups, so its next unit's products
+  // wait until the epilogue has read it (LM head and KL of one 7B pair: 164 us with 8 groups in two
+  // accumulators, 168 so). A pass in the chain gains nothing from more than four: its rows meet bf16
+  // softmax weights (errors of 1e-5 and up), and 32 cost a 7B step 1.2%.
+  const bool exact = d.terms == 3 && d.alone;
+  a.phases = exact && d.rows * d.terms <= 8 ? 2 : 1;
+  a.groups = d.terms == 3 ? std::min(exact ? kExactGroups : 4, plan.kb / plan.splits) : 1;
+  a.acc_cols = exact ? 16 * kExactGroups : 16;
   while (a.acc_cols < a.n * a.groups) a.acc_cols *= 2;
-  a.tmem_cols = std::max(32, 2 * a.acc_cols);
+  a.tmem_cols = std::max(32, exact ? a.acc_cols : 2 * a.acc_cols);
   const int stage = plan.sub * (kWBytes + a.n * kBlockK * 2);
   const int ring = d.alone ? kRowsRingMax : kRowsRing;
   a.stages = std::min(kMaxStages, ring / stage);
@@ -374,7 +439,8 @@ cudaError_t launch_rows_gemm(const RowsGemmDesc& d, const RowsPlan& plan, int nu
   const int grid = std::min(num_sms, a.units);
   if (grid < 1) return cudaSuccess;
   const int smem = a.stages * stage + 1024;
-  return d.terms == 2 ? launch_terms<2>(a, grid, smem, stream) : launch_terms<3>(a, grid, smem, stream);
+  if (exact) return launch_terms<3, true>(a, grid, smem, stream);
+  return d.terms == 2 ? launch_terms<2, false>(a, grid, smem, stream) : launch_terms<3, false>(a, grid, smem, stream);
 }
 
 }  // namespace crf

@@ -60,6 +60,26 @@ def test_kl_with_model_head(ctx, cfg):
     assert np.all(to_np(out) <= bound + 1e-4)
 
 
+@pytest.mark.parametrize("hidden", [64, 192, 1536, 1600, 3584, 8192])
+def test_head_logits_of_one_pair_keep_fp32_accuracy(ctx, hidden):
+    """Logits of one row pair, from one K block to two steps a group, against 64-bit products of the same
+    fp32 rows x g / rms. A chain of c = ceil(hidden / 2048) * 4 MMAs drops at most one unit (2^-23) of its
+    running sum at each; the chains, 64 or one per 64 columns if those are fewer, err
+    independently, so that sums to at most c / sqrt(chains) units of the logits' norm, below one up to
+    here; the division of the norm, the sum's end and the rms factor round by half a unit each: two
+    units in all. (Sums of 32 MMAs measure 3.8 at 3584.)"""
+    cfg = synth.replace(synth.TINY, hidden=hidden, vocab=5000)
+    dm = DeviceModel(cfg, layers=[])
+    h = synth.hidden_state(cfg, 2, "one-pair", std=2.0, device="cuda")
+    out = torch.empty(1, dtype=torch.float32, device="cuda")
+    z = torch.empty(2, cfg.vocab, dtype=torch.float32, device="cuda")
+    ctx.kl(dm.crf, h[:1], h[1:], out, cfg.vocab, ctx.kl_workspace(1, cfg.vocab, hidden), logits_out=z)
+    ctx.check()
+    x = h.double()
+    want = (x * torch.rsqrt(x.square().mean(-1, keepdim=True) + cfg.rms_eps) * dm.final_norm.double()) @ dm.lm_head.double().T
+    assert (z.double() - want).norm() <= 2 * 2.0 ** -23 * want.norm()
+
+
 @pytest.mark.parametrize("cfg,lc", [(synth.TINY, synth.LORA_TINY), (synth.QWEN15B, synth.LORA_QWEN)],
                          ids=["tiny-r8", "1.5b-r16"])
 def test_drift_matches_oracle(ctx, cfg, lc):
