@@ -223,9 +223,11 @@ __global__ void __launch_bounds__(kThreadsStream, 1) decode_attn_stream(const __
   const uint32_t q_base = smem_u32(sQ);
   const int mi = lane >> 3, li = lane & 7;  // ldmatrix: matrix index, row within it
   const int r0 = lane >> 2, cq = 2 * (lane & 3);
-  // a pair's elements, one per thread and turn: q of the group's heads, own k, own v. Their bias
-  // and B rows are weights: the first pair's are read before the wait.
-  constexpr int kTurns = (kMaxGroup + 2) * D / kCompute;
+  // a pair's elements, one per thread and turn: q of the group's heads, own k, own v (the last turn may
+  // be part-filled: 2.5 turns of eight heads at D = 64). Their bias and B rows are weights: the first
+  // pair's are read before the wait.
+  constexpr int kTurns = ((kMaxGroup + 2) * D + kCompute - 1) / kCompute;
+  static_assert(kTurns * kCompute >= (kMaxGroup + 2) * D, "every element of the largest group has a turn");
   UpRow u[kTurns];
   float val[kTurns];
   auto element = [&](int t, int g, int& m, int& j) {

@@ -248,3 +248,56 @@ def test_greedy_token_over_several_blocks(vocab, rows):
     nxt, z = step()
     assert np.all(z == 0) and np.all(nxt == 0)
     ctx.close()
+
+
+@pytest.mark.parametrize("head_dim,hq,hkv", [(64, 7, 1), (64, 14, 2), (64, 16, 2), (128, 7, 1), (128, 16, 2)])
+def test_groups_of_seven_and_eight_heads(head_dim, hq, hkv):
+    """The largest groups of query heads a KV head has, at both head dimensions: q of the group and the
+    row's own k and v are 576 to 1280 elements of a block, whose 256 threads take them in turns. A
+    generation step of a row with an empty cache (its own key and value alone make o), one in a chunk's
+    middle and one that opens a chunk, then the first-step row of a window, against the oracle: logits,
+    the K/V slots written, the final row."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2609_30884_gb300 as crf
+    cfg = synth.replace(synth.TINY, n_layers=2, n_q_heads=hq, n_kv_heads=hkv, head_dim=head_dim, qkv_bias=True)
+    dm, ad = DeviceModel(cfg), DeviceAdapter(cfg, synth.LORA_TINY, 1)
+    om, oa = oracle_model(dm), oracle_adapter(ad)
+    pos = [0, 77, 256]
+    P = sum(pages_needed(p + 1) for p in pos) + 3
+    pts = split_page_tables([p + 1 for p in pos], P, seed=17)
+    pool = make_pool(cfg, P, fill="random", seed=18)
+    opool = oracle_pool(pool)
+    ctx = crf.Context(0)
+    tok = synth.token_ids(cfg, len(pos), device="cuda")
+    nxt = torch.empty(len(pos), dtype=torch.int32, device="cuda")
+    logits = torch.empty(len(pos), cfg.vocab, device="cuda")
+    ws = ctx.decode_workspace(dm.crf, ad.crf, pos, pts, tok)
+    ctx.decode_step(dm.crf, ad.crf, pool, pos, pts, tok, nxt, ws, logits=logits)
+    ctx.check()
+    for i, p in enumerate(pos):
+        x, pt = C.embed(om, [int(tok[i])]), pts[i].cpu().numpy()
+        page, off = int(pt[p // 16]), p % 16
+        for l in range(cfg.n_layers):
+            kh, vh = opool.read(l, pt, p)
+            x, k, v = Dec.decode_row(x, p, kh, vh, om.layers[l], oa.layers[l], om.dims)
+            assert rel_frob(to_np(pool.k_pages[l][page, :, off]), k) <= REL_KVH, (p, l, "k")
+            assert rel_frob(to_np(pool.v_pages[l][page, :, off]), v) <= REL_KVH, (p, l, "v")
+        z = C.logits(om, x[0])[0]
+        assert rel_frob(to_np(logits[i]), z) <= REL_KVH, p
+        assert int(nxt[i]) == int(torch.argmax(logits[i]))
+
+    n = 257
+    P = pages_needed(n) + 3
+    pt = split_page_tables([n], P, seed=19)[0]
+    pool = make_pool(cfg, P, fill="random", seed=20)
+    opool = oracle_pool(pool)
+    tokens = synth.token_ids(cfg, n, request=1, device="cuda")
+    fin = torch.empty(cfg.hidden, dtype=torch.bfloat16, device="cuda")
+    req = crf.Request(pt, 0, 1, tokens=tokens, final_hidden_out=fin)
+    ctx.recompute_window(dm.crf, ad.crf, pool, [req], ctx.workspace(dm.crf, ad.crf, [req]))
+    ctx.check()
+    oreq = C.RequestCache(to_np(tokens).astype(np.int64), pt.cpu().numpy())
+    _, h_last = C.recover(om, oa, opool, oreq, 0, 1)
+    assert rel_frob(to_np(fin), h_last) <= REL_KVH
+    ctx.close()
