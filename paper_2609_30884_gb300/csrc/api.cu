@@ -1302,9 +1302,11 @@ crf_status crf_kl(crf_ctx* ctx, const crf_model* model, const void* ref, const v
     o += align256(static_cast<size_t>(2 * n_rows) * norm_slices(hidden) * sizeof(float));
     float* logits = logits_out ? logits_out : reinterpret_cast<float*>(ws + o);
     ProfScope ps(ctx, kPLmHead, st, 1 + (2 * n_rows + kRowsMax - 1) / kRowsMax);
-    PdlScope pdl;
+    // An ordinary launch opens the chain: the LM head pass reads its first weights before its own wait,
+    // so whatever the caller enqueued before (it may have written the head) must have ended by then.
     CRF_CUDA(launch_head_rows(static_cast<const __nv_bfloat16*>(ref), static_cast<const __nv_bfloat16*>(cur), n_rows,
                               hidden, static_cast<const __nv_bfloat16*>(model->final_norm), xs, terms, nss, st));
+    PdlScope pdl;
     CRF_CUDA(launch_lm_head(static_cast<const __nv_bfloat16*>(model->lm_head), xs, terms, nss, 2 * n_rows, vocab, hidden,
                             model->dims.rms_eps, logits, ctx->num_sms, ctx->status_dev, st));
     zr = logits;

@@ -43,9 +43,11 @@ constexpr int kBxCols = 64;
 // programmatic-stream-serialization attribute: such a kernel becomes resident while its
 // predecessor in the stream still runs, sets itself up (a weight pass requests its first weights) and
 // then waits for it (griddep_wait). Every kernel launched this way calls griddep_wait before it
-// touches memory that an earlier kernel may write, and before it ends, since the kernels behind it
-// count on all before it having ended. Window calls, generation steps, the KL reduction over few
-// rows and drift open a scope.
+// touches memory that an earlier kernel of the call may write, and before it ends, since the kernels
+// behind it count on all before it having ended. Weights, and cached K/V pages that the call does not
+// write, may be read before that wait, so a chain with such reads opens with an ordinary launch or a
+// memset: what the caller enqueued before has then ended and is visible. Window calls, generation
+// steps, the LM head pass of a KL call, the KL reduction over few rows and drift open a scope.
 class PdlScope {
  public:
   PdlScope();

@@ -37,6 +37,66 @@ def test_kl_from_logits(ctx, rows, vocab, scale):
     assert np.all(np.abs(to_np(out)) < 1e-5)
 
 
+def _captured_edges(stream, enqueue):
+    """(number of nodes, [(from, to, programmatic)] as node indices in capture order) of what ``enqueue``
+    puts on ``stream``: captured into a graph that is never launched."""
+    import ctypes
+    import paper_2609_30884_gb300 as crf
+    rt = crf.abi.load()  # linked against the runtime: its symbols resolve through this handle
+    P, N = ctypes.c_void_p, ctypes.c_size_t
+
+    def call(name, *args):
+        fn = getattr(rt, name)
+        fn.restype = ctypes.c_int
+        assert fn(*args) == 0, name
+
+    s, graph, n = P(stream.cuda_stream), P(), N()
+    stream.synchronize()
+    call("cudaStreamBeginCapture", s, ctypes.c_int(2))  # relaxed
+    try:
+        with torch.cuda.stream(stream):
+            enqueue()
+    finally:
+        call("cudaStreamEndCapture", s, ctypes.byref(graph))
+    call("cudaGraphGetNodes", graph, None, ctypes.byref(n))
+    nodes = (P * n.value)()
+    call("cudaGraphGetNodes", graph, nodes, ctypes.byref(n))
+    at = {v: i for i, v in enumerate(nodes)}
+    call("cudaGraphGetEdges", graph, None, None, None, ctypes.byref(n))
+    src, dst, data = (P * n.value)(), (P * n.value)(), (ctypes.c_uint8 * (8 * n.value))()
+    call("cudaGraphGetEdges", graph, src, dst, data, ctypes.byref(n))
+    edges = [(at[a], at[b], data[8 * i + 2] != 0) for i, (a, b) in enumerate(zip(src, dst))]  # byte 2: the edge's type
+    call("cudaGraphDestroy", graph)
+    return len(nodes), edges
+
+
+@pytest.mark.parametrize("rows", [1, 40])
+def test_kl_with_model_head_waits_for_earlier_work(ctx, rows):
+    """The LM head pass reads its first weights before its own wait (one row pair, and two passes of
+    it): whatever the caller enqueued before the call, such as a kernel that writes the head, must have
+    ended when the call's first kernel starts. Shown on the captured graph, without running anything:
+    the edge out of the caller's kernel is a full dependency, and the later ones (the pass behind the
+    rows' kernel) are programmatic."""
+    dm = DeviceModel(synth.TINY, layers=[])
+    cfg = synth.TINY
+    h = synth.hidden_state(cfg, rows, "href", std=2.0, device="cuda")
+    out = torch.empty(rows, dtype=torch.float32, device="cuda")
+    ws = ctx.kl_workspace(rows, cfg.vocab, cfg.hidden)
+    stream = torch.cuda.Stream()
+
+    def enqueue():
+        dm.lm_head.mul_(2)
+        ctx.kl(dm.crf, h, h, out, cfg.vocab, ws, stream=stream)
+
+    n, edges = _captured_edges(stream, enqueue)
+    assert n >= 5 and len(edges) == n - 1
+    sources = {a for a, _, _ in edges} - {b for _, b, _ in edges}
+    assert len(sources) == 1
+    first = [p for a, _, p in edges if a in sources]
+    assert first == [False]
+    assert any(p for _, _, p in edges)
+
+
 @pytest.mark.parametrize("cfg", [synth.TINY, synth.QWEN15B], ids=["tiny", "1.5b"])
 def test_kl_with_model_head(ctx, cfg):
     dm = DeviceModel(cfg, layers=[])
