@@ -1035,16 +1035,18 @@ crf_status crf_recompute_window(crf_ctx* ctx, const crf_model* model, const crf_
     for (int k = 0; k < rt.n; ++k) {
       const int i = act[k];
       const bool copy_out = !single && reqs[i].hidden_out;
-      ProfScope ps(ctx, kPCopy, st, copy_out ? 1 : 0);
+      // The last row waits for its tail in the checkpoint of a call's only request. In a batch it is
+      // copied at once (requests may share one buffer for checkpoints their caller does not want), and
+      // where there is no checkpoint.
+      const bool keep_row = l == reqs[i].e - 1 && reqs[i].final_hidden_out && (n_req > 1 || !reqs[i].hidden_out);
+      ProfScope ps(ctx, kPCopy, st, (copy_out ? 1 : 0) + (keep_row ? 1 : 0));
       curp[i] = X_out + static_cast<size_t>(rt.row0[k]) * D.h;
       if (copy_out)
         CRF_CUDA(launch_copy_rows(static_cast<__nv_bfloat16*>(reqs[i].hidden_out[l - reqs[i].s]), curp[i],
                                   static_cast<size_t>(reqs[i].n_tokens) * D.h, c.abort, st));
-      // the last row waits for its tail in the caller's checkpoint, or where there is none in a copy
-      if (l == reqs[i].e - 1 && reqs[i].final_hidden_out && !reqs[i].hidden_out)
-        CRF_CUDA(cudaMemcpyAsync(dx0 + static_cast<size_t>(i) * D.h,
-                                 curp[i] + static_cast<size_t>(reqs[i].n_tokens - 1) * D.h, row_bytes,
-                                 cudaMemcpyDeviceToDevice, st));
+      if (keep_row)
+        CRF_CUDA(launch_copy_rows(dx0 + static_cast<size_t>(i) * D.h,
+                                  curp[i] + static_cast<size_t>(reqs[i].n_tokens - 1) * D.h, D.h, c.abort, st));
     }
   }
 
@@ -1056,10 +1058,16 @@ crf_status crf_recompute_window(crf_ctx* ctx, const crf_model* model, const crf_
     const size_t last = static_cast<size_t>(r.n_tokens - 1) * D.h;
     const __nv_bfloat16* start = dx0 + static_cast<size_t>(i) * D.h;
     const int32_t* token = nullptr;
-    if (r.s < r.e && r.hidden_out) {
+    if (r.s < r.e && r.hidden_out && n_req == 1) {
       start = static_cast<const __nv_bfloat16*>(r.hidden_out[r.e - r.s - 1]) + last;
     } else if (r.s == r.e && r.s > 0) {
-      start = static_cast<const __nv_bfloat16*>(r.hidden_in) + last;
+      const auto* row = static_cast<const __nv_bfloat16*>(r.hidden_in) + last;
+      if (n_req == 1) {
+        start = row;
+      } else {
+        ProfScope ps(ctx, kPCopy, st, 1);
+        CRF_CUDA(launch_copy_rows(dx0 + static_cast<size_t>(i) * D.h, row, D.h, c.abort, st));
+      }
     } else if (r.s == r.e) {
       start = nullptr;
       token = r.tokens + (r.n_tokens - 1);

@@ -195,6 +195,35 @@ def test_batched_requests_shared_pool(ctx, tiny):
         assert torch.equal(free_slots(pool.v_pages[l], free), free_slots(bv[l], free))
 
 
+def test_batch_may_share_unwanted_checkpoints(ctx, tiny):
+    """Requests of a batch whose caller wants only the first-step rows may name one buffer for all their
+    checkpoints, and one request's final row may be another's restart row: each row starts from its own
+    request's state. Windows end at different layers, one of them last, one request is direct reuse;
+    the final rows have the bits of the same batch with buffers of its own."""
+    import paper_2609_30884_gb300 as crf
+    cfg, _, dm, cur, _, _ = tiny
+    n, windows = 200, [(0, 1), (1, 3), (2, 3), (1, 4), (2, 2)]
+    P = len(windows) * pages_needed(n)
+    pts = split_page_tables([n] * len(windows), P, seed=4)
+    h_in = [synth.hidden_state(cfg, n, layer=i, device="cuda") for i in range(len(windows))]
+    finals = []
+    for shared in (False, True):
+        pool = make_pool(cfg, P, fill="random", seed=6)
+        junk = torch.empty(n, cfg.hidden, dtype=torch.bfloat16, device="cuda")
+        fin = torch.empty(len(windows), cfg.hidden, dtype=torch.bfloat16, device="cuda")
+        own = [h.clone() for h in h_in]
+        outs = [own[4][-1] if shared and i == 3 else fin[i] for i in range(len(windows))]
+        reqs = [crf.Request(pts[i], s, e, n_tokens=n, tokens=synth.token_ids(cfg, n, request=i, device="cuda"),
+                            hidden_in=own[i] if s > 0 else None,
+                            hidden_out=[junk if shared else torch.empty_like(junk) for _ in range(s, e)],
+                            final_hidden_out=outs[i]) for i, (s, e) in enumerate(windows)]
+        order = [0, 1, 2, 4, 3]  # the reuse before the request that writes its final row over the restart row
+        _run(ctx, dm, cur, pool, [reqs[i] for i in order])
+        finals.append([o.clone() for o in outs])
+    for i, (a, b) in enumerate(zip(*finals)):
+        assert torch.equal(a, b), i
+
+
 def test_identical_adapter_reproduces_stale_cache_bitexact(ctx, tiny):
     cfg, lc, dm, _, _, _ = tiny
     v0 = DeviceAdapter(cfg, lc, 0)
