@@ -14,9 +14,11 @@ namespace crf {
 enum : int { kStatusTimeout = 1, kStatusBounds = 2, kStatusPages = 4 };
 
 // The per-call abort word: set by the page-table check that opens a call when a page id is out of
-// the pool or a page appears twice. Every later kernel of the call that reads pages or writes
-// memory outside the call's workspace tests it first and returns at once, so a rejected call
-// writes nothing outside its workspace. Null where a launch has no such word.
+// the pool or a page appears twice. Every later kernel of the call that writes memory outside the call's
+// workspace tests it before it writes, and one that reads pages tests it before it uses what it read,
+// so a rejected call writes nothing outside its workspace. (Decode attention's copy warp asks for cached
+// pages before the check has ended, from ids that it clamps to the pool.) Null where a launch has no
+// such word.
 __device__ __forceinline__ bool call_aborted(const int* abort) { return abort != nullptr && *abort != 0; }
 
 #ifdef CRF_DEBUG
@@ -40,9 +42,10 @@ __device__ __forceinline__ int checked_token(int tok, int vocab, int* status) {
 // with CRF_DEBUG defined, an id outside [0, num_pages) sets kStatusBounds and
 // comes back as page 0, so the copy that uses it stays inside the pool and
 // every barrier still completes; the host reports the bit. In every build the
-// page-table check that opens the call has already rejected bad ids (the call's
-// abort word), so in the release build this check compiles away and the id is
-// returned unchanged.
+// page-table check that opens the call rejects bad ids (the call's abort word,
+// tested before the id is used: decode attention's copy warp alone does not wait for it
+// and clamps the id itself), so in the release build this check compiles away and the
+// id is returned unchanged.
 __device__ __forceinline__ int checked_page(int page, int num_pages, int* status) {
 #ifdef CRF_DEBUG
   if (page < 0 || page >= num_pages) {

@@ -199,7 +199,10 @@ __global__ void __launch_bounds__(kThreadsStream, 1) decode_attn_stream(const __
           const int32_t* pt = p.page_table[k.r];
           mbar_arrive_expect_tx(&full[st], 2 * pages * HALVES * kPage * 128);
           for (int pg = 0; pg < pages; ++pg) {
-            const int page = checked_page(pt[t0 / kPage + pg], a.num_pages, a.status);
+            // read before the page check's verdict is known: of an id outside the pool the nearest page
+            // is copied, inside the pool's rows (fewer than 2^31: they fit the GPU's memory), and the
+            // block stops at the abort word before it uses it
+            const int page = min(max(checked_page(pt[t0 / kPage + pg], a.num_pages, a.status), 0), a.num_pages - 1);
             const int row = (page * p.n_kv_heads + k.g) * kPage;
             for (int h = 0; h < HALVES; ++h) {
               const int off = h * HALF + pg * (kPage * 128);

@@ -133,6 +133,48 @@ def test_decode_step_rejects_bad_arguments():
     assert not torch.all(logits[0] == 7.0) and int(nxt[0]) >= 0
 
 
+@pytest.mark.parametrize("bad", [2 ** 31 - 1, -2 ** 31, 2 ** 27, 2 ** 26, -1, 60])
+def test_far_page_ids_of_cached_keys_are_rejected(bad):
+    """A cached page's id far outside the pool (also where its row index, id x 2 heads x 16, would leave 32
+    bits): decode attention asks for such a page before the page check has ended. The step and a direct
+    reuse write nothing and report CRF_EINVAL, and the same workspace then serves the right ids."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2609_30884_gb300 as crf
+    cfg = synth.TINY
+    dm, ad = DeviceModel(cfg), DeviceAdapter(cfg, synth.LORA_TINY, 1)
+    P, pos = 60, 700
+    pool = make_pool(cfg, P, fill="random", seed=7)
+    ctx = crf.Context(0)
+    good = torch.arange(pages_needed(pos + 1), dtype=torch.int32, device="cuda")
+    wrong = good.clone()
+    wrong[torch.tensor([3, 30], device="cuda")] = bad
+    tok = synth.token_ids(cfg, 1, device="cuda")
+    h = synth.hidden_state(cfg, pos + 1, device="cuda")
+    nxt = torch.full((1,), -5, dtype=torch.int32, device="cuda")
+    z = torch.full((1, cfg.vocab), 7.0, device="cuda")
+    fin = torch.full((cfg.hidden,), 7.0, dtype=torch.bfloat16, device="cuda")
+    ws = ctx.decode_workspace(dm.crf, ad.crf, [pos], [good], tok)
+
+    def reuse(pt):
+        req = crf.Request(pt, 2, 2, n_tokens=pos + 1, hidden_in=h, final_hidden_out=fin)
+        ctx.recompute_window(dm.crf, ad.crf, pool, [req], ctx.workspace(dm.crf, ad.crf, [req]))
+
+    before = snapshot(pool)
+    for call in (lambda: ctx.decode_step(dm.crf, ad.crf, pool, [pos], [wrong], tok, nxt, ws, logits=z), lambda: reuse(wrong)):
+        call()
+        with pytest.raises(crf.CrfError) as ei:
+            ctx.check()
+        assert ei.value.status == crf.abi.EINVAL
+    assert torch.all(z == 7.0) and int(nxt) == -5 and torch.all(fin == 7.0)
+    assert all(torch.equal(a, b) for a, b in zip(pool.k_pages + pool.v_pages, before[0] + before[1]))
+    reuse(good)
+    ctx.decode_step(dm.crf, ad.crf, pool, [pos], [good], tok, nxt, ws, logits=z)
+    ctx.check()
+    assert int(nxt) == int(z.argmax()) and torch.all(torch.isfinite(z)) and not torch.all(fin == 7.0)
+    ctx.close()
+
+
 def test_chunk_boundary_positions_do_not_stall():
     """Rows whose position opens a new 128-key chunk (it holds only the row's own key), each streamed
     by blocks of three chunks: the empty chunk reuses a stage whose copies are long consumed, and no
