@@ -179,7 +179,7 @@ struct Plan {
 
 // Scratch of the decode rows (byte offsets from its start, 256-byte aligned): the fp32 rows, their
 // slices' sums of squares, the bf16 terms entering the four passes, one pass's partial sums and the
-// attention partials.
+// attention partials. The same for every adapter: a workspace sized under one serves calls under any.
 struct DecodeScratch {
   size_t x, nss, xs, os, ms, y, part, total;
 };
@@ -214,7 +214,7 @@ DecodePasses decode_passes(const Dims& D, uint32_t mask, int num_sms) {
   return p;
 }
 
-DecodeScratch decode_scratch(const Dims& D, uint32_t mask, int rows, int attn_splits, int num_sms) {
+DecodeScratch decode_scratch(const Dims& D, int rows, int attn_splits, int num_sms) {
   DecodeScratch s;
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -223,10 +223,13 @@ DecodeScratch decode_scratch(const Dims& D, uint32_t mask, int rows, int attn_sp
     return at;
   };
   const size_t R = static_cast<size_t>(rows), T = static_cast<size_t>(rows_terms(rows));
-  const DecodePasses p = decode_passes(D, mask, num_sms);
+  // a pass without LoRA rows has a tile less and may be cut into more splits: the larger of both
   size_t y = 0;
-  for (const RowsPlan* q : {&p.qkv, &p.o, &p.gu, &p.down})
-    y = std::max(y, R * static_cast<size_t>(q->splits) * q->ncols * sizeof(float));
+  for (uint32_t mask : {0u, 0x7Fu}) {
+    const DecodePasses p = decode_passes(D, mask, num_sms);
+    for (const RowsPlan* q : {&p.qkv, &p.o, &p.gu, &p.down})
+      y = std::max(y, R * static_cast<size_t>(q->splits) * q->ncols * sizeof(float));
+  }
   s.x = take(R * D.h * sizeof(float));
   s.nss = take(R * norm_slices(D.h) * sizeof(float));
   s.xs = take(R * T * D.h * 2);
@@ -248,7 +251,7 @@ uint32_t ptab_slots_for(long ids) {
   return s;
 }
 
-Plan make_plan(const Dims& D, const crf_request* reqs, int n_req, uint32_t mask, int num_sms) {
+Plan make_plan(const Dims& D, const crf_request* reqs, int n_req, int num_sms) {
   Plan p;
   for (int l = 0; l < D.N; ++l) {
     int m = 0;
@@ -291,7 +294,7 @@ Plan make_plan(const Dims& D, const crf_request* reqs, int n_req, uint32_t mask,
   p.off_abort = take((1 + p.flag_words) * sizeof(int));
   p.off_ptab = take(static_cast<size_t>(p.ptab_slots) * sizeof(int));
   p.splits = dec_splits(p.max_n);
-  p.off_dec = take(p.dec_rows ? decode_scratch(D, mask, p.dec_rows, p.splits, num_sms).total : 0);
+  p.off_dec = take(p.dec_rows ? decode_scratch(D, p.dec_rows, p.splits, num_sms).total : 0);
   p.total = o;
   return p;
 }
@@ -582,7 +585,7 @@ crf_status decode_rows(const LayerCtx& c, std::vector<DecodeRow> rows, const Dec
   const uint32_t mask = c.ad->dims.module_mask;
   const DecodePasses passes = decode_passes(D, mask, sms);
   // the scratch was sized for p.dec_rows >= R rows: both use the term count of the rows that run
-  const DecodeScratch ds = decode_scratch(D, mask, R, p.splits, sms);
+  const DecodeScratch ds = decode_scratch(D, R, p.splits, sms);
   const int terms = rows_terms(R);
   uint8_t* base = c.ws + p.off_dec;
   float* x = reinterpret_cast<float*>(base + ds.x);
@@ -771,7 +774,7 @@ struct StepPlan {
   size_t off_angles, off_logits, total;
 };  // p.off_abort / p.off_ptab / p.ptab_slots: the page check of the rows' tables
 
-StepPlan make_step_plan(const Dims& D, const crf_decode_row* rows, int n, uint32_t mask, int num_sms) {
+StepPlan make_step_plan(const Dims& D, const crf_decode_row* rows, int n, int num_sms) {
   StepPlan sp;
   Plan& p = sp.p;
   p.dec_rows = n;
@@ -784,7 +787,7 @@ StepPlan make_step_plan(const Dims& D, const crf_decode_row* rows, int n, uint32
     o = align256(o + bytes);
     return at;
   };
-  p.off_dec = take(decode_scratch(D, mask, n, p.splits, num_sms).total);
+  p.off_dec = take(decode_scratch(D, n, p.splits, num_sms).total);
   p.off_rope = 0;
   sp.off_angles = take(static_cast<size_t>(n) * (D.d / 2) * sizeof(float2));
   sp.off_logits = take(static_cast<size_t>(n) * D.V * 4);
@@ -895,7 +898,7 @@ crf_status crf_workspace_size(crf_ctx* ctx, const crf_model* model, const crf_lo
   for (int i = 0; i < n_req; ++i)
     if (reqs[i].n_tokens < 1 || reqs[i].s < 0 || reqs[i].s > reqs[i].e || reqs[i].e > D.N)
       return fail(CRF_EINVAL, "request %d malformed", i);
-  *bytes = make_plan(D, reqs, n_req, lora->module_mask, ctx->num_sms).total;
+  *bytes = make_plan(D, reqs, n_req, ctx->num_sms).total;
   return CRF_OK;
 }
 
@@ -914,7 +917,7 @@ crf_status crf_recompute_window(crf_ctx* ctx, const crf_model* model, const crf_
   const Dims D = dims_of(model->dims);
   s = validate_requests(ctx, model, cur, pool, reqs, n_req, D);
   if (s != CRF_OK) return s;
-  const Plan plan = make_plan(D, reqs, n_req, cur->dims.module_mask, ctx->num_sms);
+  const Plan plan = make_plan(D, reqs, n_req, ctx->num_sms);
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255))
     return fail(CRF_EINVAL, "workspace null or not 256-byte aligned");
   if (ws_bytes < plan.total)
@@ -1102,7 +1105,7 @@ crf_status crf_decode_workspace_size(crf_ctx* ctx, const crf_model* model, const
   if (n_rows < 1 || n_rows > CRF_MAX_REQUESTS) return fail(CRF_EINVAL, "n_rows out of range");
   for (int i = 0; i < n_rows; ++i)
     if (rows[i].pos < 0) return fail(CRF_EINVAL, "row %d: negative position", i);
-  *bytes = make_step_plan(dims_of(model->dims), rows, n_rows, lora->module_mask, ctx->num_sms).total;
+  *bytes = make_step_plan(dims_of(model->dims), rows, n_rows, ctx->num_sms).total;
   return CRF_OK;
 }
 
@@ -1132,7 +1135,7 @@ crf_status crf_decode_step(crf_ctx* ctx, const crf_model* model, const crf_adapt
       return fail(CRF_EINVAL, "kv pool layer %d null or misaligned", l);
   s = validate_decode_rows(pool, rows, n_rows);
   if (s != CRF_OK) return s;
-  const StepPlan sp = make_step_plan(D, rows, n_rows, cur->dims.module_mask, ctx->num_sms);
+  const StepPlan sp = make_step_plan(D, rows, n_rows, ctx->num_sms);
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255))
     return fail(CRF_EINVAL, "workspace null or not 256-byte aligned");
   if (ws_bytes < sp.total) return fail(CRF_ENOMEM, "workspace %zu bytes, %zu needed", ws_bytes, sp.total);
@@ -1179,7 +1182,7 @@ crf_status crf_decode_step(crf_ctx* ctx, const crf_model* model, const crf_adapt
   s = decode_rows(c, dec, opt);
   if (s != CRF_OK) return s;
   // LM head over the final rows' terms, greedy token
-  const DecodeScratch ds = decode_scratch(D, cur->dims.module_mask, n_rows, sp.p.splits, ctx->num_sms);
+  const DecodeScratch ds = decode_scratch(D, n_rows, sp.p.splits, ctx->num_sms);
   const uint8_t* base = ws + sp.p.off_dec;
   float* z = logits ? logits : reinterpret_cast<float*>(ws + sp.off_logits);
   {

@@ -102,6 +102,27 @@ def test_variant_window_tail_kl(ctx, models, shape, rank, modules):
             assert torch.equal(pool.k_pages[l], bk[l]) and torch.equal(pool.v_pages[l], bv[l])
 
 
+@pytest.mark.parametrize("shape", list(SHAPES))
+def test_workspace_serves_any_adapter(ctx, shape):
+    """A workspace sized under one adapter takes the same call under any other: windows with a first-step
+    row and generation steps, one row and several, need the same bytes whatever the rank and modules
+    (on the 1.5B shapes the down pass without LoRA rows is cut into more splits than with them)."""
+    import paper_2609_30884_gb300 as crf
+    cfg, n, (s, e) = SHAPES[shape]
+    dims = DeviceModel(cfg, layers=[], with_head=False).crf
+    pt = torch.arange(pages_needed(n), dtype=torch.int32, device="cuda")
+    h = torch.empty(n, cfg.hidden, dtype=torch.bfloat16, device="cuda")
+    tok = torch.zeros(5, dtype=torch.int32, device="cuda")
+    sizes = set()
+    for rank, modules in VARIANTS + [(16, synth.MODULES), (4, ())]:
+        ad = crf.Adapter(rank, 2.0 * rank, modules, [None] * cfg.n_layers)
+        req = crf.Request(pt, s, e, hidden_in=h, final_hidden_out=h[0])
+        sizes.add((ctx.workspace_size(dims, ad, [req]), ctx.workspace_size(dims, ad, [req] * 5),
+                   ctx.decode_workspace(dims, ad, [n], [pt], tok).numel(),
+                   ctx.decode_workspace(dims, ad, [n] * 5, [pt] * 5, tok).numel()))
+    assert len(sizes) == 1, sizes
+
+
 @pytest.mark.parametrize("rank,modules", VARIANTS[:3], ids=["r4-all", "r8-v", "r8-q+v"])
 def test_variant_drift(ctx, rank, modules):
     cfg = SMALL128
