@@ -448,6 +448,23 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
+// x / (1 + e^-x). The divide is formed from an approximate reciprocal, whose quotient is corrected once by
+// its remainder (Markstein, IBM J. Res. Dev. 34, 1990): d >= 1, so nothing needs a range check but the
+// scale of 1/16, which keeps the reciprocal normal up to the largest finite d; where d or x is infinite
+// the remainder is NaN and the quotient already the result. Against the compiler's divide over all 2^32
+// inputs: two differ, by one unit in the last place, and the sign of silu(-0). That divide branches per
+// element (prefill of 2003 rows of the 1.5B shape: 1784 us, 1449 so, 1444 with the unrounded
+// __fdividef, which gives 0 below x = -87.3).
+__device__ __forceinline__ float silu(float x) {
+  const float d = 1.0f + __expf(-x);
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d * 0.0625f));
+  r *= 0.0625f;
+  const float q = x * r;
+  const float rem = __fmaf_rn(-q, d, x);
+  return rem == rem ? __fmaf_rn(rem, r, q) : q;
+}
+
 // ---------------------------------------------------------------- mma.sync (m16n8k16, bf16)
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2,
                                         uint32_t& r3) {

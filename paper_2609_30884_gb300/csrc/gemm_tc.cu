@@ -248,10 +248,8 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs& a, const Tile& tl,
           for (int e = 0; e < 4; ++e) {
             float v[2];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const float x = __uint_as_float(gt[8 * k + 2 * e + h]);
-              v[h] = __fdividef(x, 1.0f + __expf(-x)) * __uint_as_float(up[8 * k + 2 * e + h]);
-            }
+            for (int h = 0; h < 2; ++h)
+              v[h] = silu(__uint_as_float(gt[8 * k + 2 * e + h])) * __uint_as_float(up[8 * k + 2 * e + h]);
             p[e] = pack_bf16(v[0], v[1]);
           }
           *scratch_at(scr, lane, h2 / 8 + k) = make_uint4(p[0], p[1], p[2], p[3]);

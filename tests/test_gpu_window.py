@@ -162,6 +162,37 @@ def test_attention_keys_split_over_two_ctas(ctx, lengths):
             assert torch.equal(run([i])[0][0], outs[i][0])
 
 
+@pytest.mark.parametrize("ffn", [688, 1280])
+def test_swiglu_of_far_negative_gates(ctx, ffn):
+    """silu where 1 + e^-x lies between 2^126 and 2^128 (x from -87.4 to -88.7): a divide that flushes
+    there gives 0. Gates of one value each, ups so large that the products are of order one, and
+    a down projection that copies them: x + silu(g) u, rounded to bf16 (2^-9 of it, the product
+    another 2^-9, and the gate's exponential 2^-16)."""
+    import paper_2609_30884_gb300 as crf
+    cfg = synth.replace(synth.TINY, n_layers=1, ffn=ffn)
+    h, n, dev = cfg.hidden, 130, "cuda"
+    w = {k: torch.zeros_like(v) for k, v in synth.layer_weights(cfg, 0, 0, dev).items()}
+    gates = torch.tensor([-85.0, -87.0, -87.5, -88.0, -88.5, -1.0], device=dev).repeat(h // 6 + 1)[:h]
+    w["ln1"].fill_(1.0)
+    w["ln2"].fill_(1.0)
+    w["W_gate"][:h, 0] = gates.bfloat16()
+    silu = gates.double() / (1.0 + torch.exp(-gates.double()))
+    w["W_up"][:h, 0] = (3.0 / silu.abs()).bfloat16()
+    w["W_down"][:, :h] = torch.eye(h, device=dev).bfloat16()
+    pool = make_pool(cfg, pages_needed(n))
+    pt = split_page_tables([n], pages_needed(n), seed=2)[0]
+    out = torch.empty(n, h, dtype=torch.bfloat16, device=dev)
+    model = crf.Model(dict(n_layers=1, hidden=h, n_q_heads=cfg.n_q_heads, n_kv_heads=cfg.n_kv_heads, head_dim=cfg.head_dim,
+                           ffn=ffn, vocab=cfg.vocab, rms_eps=0.0, rope_theta=1e4, qkv_bias=False), [w], torch.ones(cfg.vocab, h, dtype=torch.bfloat16, device=dev))
+    ad = crf.Adapter(4, 8.0, (), [None])
+    req = crf.Request(pt, 0, 1, tokens=torch.zeros(n, dtype=torch.int32, device=dev), hidden_out=[out])
+    ctx.recompute_window(model, ad, pool, [req], ctx.workspace(model, ad, [req]))
+    ctx.check()
+    prod = silu * w["W_up"][:h, 0].double()
+    want = 1.0 + prod
+    assert torch.all((out.double() - want).abs() <= 2.0 ** -8 * (want.abs() + prod.abs()))
+
+
 def test_batched_requests_shared_pool(ctx, tiny):
     cfg, lc, dm, cur, om, oa = tiny
     lengths = [100, 257, 512]
