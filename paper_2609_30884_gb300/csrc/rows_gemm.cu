@@ -8,12 +8,14 @@
 // 16 mantissa bits, 3: the whole fp32 value), and the epilogue adds a row's term columns; products
 // of bf16 values are exact in fp32, accumulation is fp32. The tensor core cuts its running
 // sums off instead of rounding them, so a long sum drifts by half a unit a step: where the rows are
-// exact (three terms), a unit's steps accumulate in groups of TMEM columns, and one or two rows, which
-// fill 6 of 16 columns, bring every other K block's terms 8 columns on (a box that starts 8 rows
-// early, zero-filled) into sums of their own
-// (the LM head alone: a pass in the chain has four groups). Error of the 7B LM head's logits against 64
-// bits, one pair of rows: 4.48e-7 in sums of 32 MMAs, 1.17e-7 in sums of 4; fp32 sums on CUDA cores
-// 1.22e-7. 1.5B: 2.17e-7, 1.02e-7, 1.10e-7.
+// exact (three terms: one or two rows), a unit's steps accumulate in groups of TMEM columns, and the
+// rows, which fill at most 6 of an operand's 16 rows, change sides with every K block: an 8-row atom of
+// zeros is the other half of the operand, reached through the descriptor's stride. So every block of a
+// group has sums of its own, of four MMAs. (Boxes that start 8 rows early, zero-filled, did the same and took
+// 2.5 us a pass more: 7B step of one row 3.30 ms, 3.03 so.)
+// Error of the logits against 64 bits, sums of 4 MMAs / of 32 to 60 / fp32 on CUDA cores: the LM head alone, one
+// pair of rows, 7B 1.17e-7 / 4.48e-7 / 1.22e-7, 1.5B 1.01e-7 / 2.17e-7 / 1.10e-7; one layer and the head, one
+// row, 7B 2.9e-7 / 1.2e-6 / 3.2e-7, 1.5B 2.5e-7 / 5.1e-7 / 2.6e-7.
 //
 // Units of work: (128-row weight tile, K split); a tile's `splits` units are spread over CTAs so
 // that a narrow projection still fills the chip, and each writes its own partial sums
@@ -48,19 +50,19 @@ namespace {
 
 constexpr int kTile = 128;
 constexpr int kBlockK = 64;  // one 128-byte swizzled box; a step takes plan.sub of them side by side
-constexpr int kExactGroups = 32;  // accumulation groups of a pass of its own: all of TMEM
+constexpr int kExactGroups = 32;  // most accumulation groups of exact rows: all of TMEM
 constexpr int kRgThreads = 192;  // producer, MMA and four epilogue warps
 constexpr int kMaxStages = 12;
 constexpr int kWBytes = kTile * kBlockK * 2;
+constexpr int kAtom = 8 * kBlockK * 2;  // 8 operand rows; one of zeros on either side of the ring
 
 struct RowsGemmArgs {
   CUtensorMap tmW[kRowsMaxSeg];
   CUtensorMap tmA[kRowsMaxSeg];  // LoRA A rows, box of 16
-  CUtensorMap tmX;               // the rows' terms, box of n
+  CUtensorMap tmX;               // the rows' terms, box of 8 (exact rows) or n
   RowsPlan plan;
   int nseg, n_lora, units;
   int rows, n, stages, acc_cols, groups;
-  int phases;   // 2: odd K blocks bring their rows 8 columns on, into sums of their own
   uint32_t tmem_cols;
   float* y;
   const float* nss;
@@ -93,12 +95,19 @@ __device__ __forceinline__ void two_sum(float& s, float& e, float x) {
   s = t;
 }
 
-// kExact: a pass of its own over exact rows (three terms, 16 columns).
-template <int kTerms, bool kExact>
+// Groups of exact rows in the first of the two accumulators.
+__device__ __forceinline__ int first_half(int groups) { return (groups + 1) / 2; }
+
+// kExact: one or two rows in three terms (16 columns). A unit's steps fill both accumulators, half of
+// its groups in each, so the epilogue reads the first while the second is multiplied. Else: two terms, and
+// the accumulators take units in turn. kAlone: exact rows of a pass by itself (the LM head).
+template <bool kExact, bool kAlone>
 __global__ void __launch_bounds__(kRgThreads, 1) rows_gemm_kernel(const __grid_constant__ RowsGemmArgs a) {
+  constexpr int kTerms = kExact ? 3 : 2;
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                             ~static_cast<uintptr_t>(1023));
+  uint8_t* zero_lo = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                                ~static_cast<uintptr_t>(1023));
+  uint8_t* smem = zero_lo + kAtom;  // the ring
   __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages];
   __shared__ __align__(8) uint64_t tfull[2], tempty[2], drain_bar;
   __shared__ uint32_t tmem_base_sh;
@@ -108,8 +117,9 @@ __global__ void __launch_bounds__(kRgThreads, 1) rows_gemm_kernel(const __grid_c
   griddep_launch_dependents();
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int sub = a.plan.sub;
-  const int x_bytes = a.n * kBlockK * 2;
+  const int x_bytes = kExact ? kAtom : a.n * kBlockK * 2;
   const int stage_bytes = sub * (kWBytes + x_bytes);
+  uint8_t* zero_hi = smem + a.stages * stage_bytes;
   if (threadIdx.x == 0) {
     for (int i = 0; i < a.stages; ++i) {
       mbar_init(&full[i], 1);
@@ -126,6 +136,11 @@ __global__ void __launch_bounds__(kRgThreads, 1) rows_gemm_kernel(const __grid_c
   if (warp == 1) {
     tmem_alloc(&tmem_base_sh, a.tmem_cols);
     tmem_relinquish();
+  }
+  if (kExact && threadIdx.x < 2 * kAtom / 16) {
+    uint8_t* z = threadIdx.x < kAtom / 16 ? zero_lo : zero_hi - kAtom;
+    reinterpret_cast<uint4*>(z)[threadIdx.x] = make_uint4(0, 0, 0, 0);
+    fence_proxy_async_smem();  // before the MMAs read them
   }
   tc_fence_before();
   __syncthreads();
@@ -158,7 +173,7 @@ __global__ void __launch_bounds__(kRgThreads, 1) rows_gemm_kernel(const __grid_c
       for (int h = 0; h < sub; ++h)
         if (issuer)
           tma_load_2d(smem + st * stage_bytes + sub * kWBytes + h * x_bytes, &a.tmX, &full[st],
-                      (s.kb * sub + h) * kBlockK, kExact && a.phases == 2 ? -8 * ((s.kb * sub + h) & 1) : 0);
+                      (s.kb * sub + h) * kBlockK, 0);
     };
     Steps w, x;
     w.at(a, blockIdx.x);
@@ -201,7 +216,8 @@ __global__ void __launch_bounds__(kRgThreads, 1) rows_gemm_kernel(const __grid_c
     uint32_t ph = 0;
     Steps s;
     for (s.at(a, blockIdx.x); ok && s.more(a); ++it) {
-      const int acc = kExact ? 0 : it & 1, turn = kExact ? it : it >> 1;
+      int acc = kExact ? 0 : it & 1;
+      const int turn = kExact ? it : it >> 1;
       if (!mbar_wait_warp(&tempty[acc], (turn & 1) ^ 1, &abort_flag, a.status)) {
         ok = false;
         break;
@@ -210,9 +226,21 @@ __global__ void __launch_bounds__(kRgThreads, 1) rows_gemm_kernel(const __grid_c
       const int unit = s.u, len = s.end - s.kb;
       // accumulation group of step i: i * groups / len
       for (int i = 0, left = 0; s.u == unit; s.next(a), i += a.groups) {
-        const int group = a.groups == 1 ? 0 : i / len;
+        int group = kExact ? i / len : 0;
         const bool first = left != group + 1;
         left = group + 1;
+        if (kExact && group >= first_half(a.groups)) {
+          if (acc == 0) {
+            if (issuer) mma_commit(&tfull[0]);
+            if (!mbar_wait_warp(&tempty[1], (turn & 1) ^ 1, &abort_flag, a.status)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            acc = 1;
+          }
+          group -= first_half(a.groups);
+        }
         const uint32_t d = tmem + acc * a.acc_cols + group * a.n;
         if (!mbar_wait_warp(&full[st], ph, &abort_flag, a.status)) {
           ok = false;
@@ -223,7 +251,11 @@ __global__ void __launch_bounds__(kRgThreads, 1) rows_gemm_kernel(const __grid_c
         if (issuer) {
           for (int h = 0; h < sub; ++h) {
             const uint64_t wd = smem_desc(base + h * kWBytes, 16, 1024, kSwizzle128B);
-            const uint64_t xd = smem_desc(base + sub * kWBytes + h * x_bytes, 16, 1024, kSwizzle128B);
+            const uint32_t x = base + sub * kWBytes + h * x_bytes;
+            uint64_t xd = smem_desc(x, 16, 1024, kSwizzle128B);
+            if constexpr (kExact)  // the rows and 8 of zeros, or the other way round
+              xd = ((s.kb * sub + h) & 1) == 0 ? smem_desc(x, 16, smem_u32(zero_hi) - x, kSwizzle128B)
+                                               : smem_desc(smem_u32(zero_lo), 16, x - smem_u32(zero_lo), kSwizzle128B);
 #pragma unroll
             for (int k = 0; k < kBlockK / 16; ++k)
               mma_bf16_ss(d, wd + 2 * k, xd + 2 * k, idesc, (!first || h > 0 || k > 0) ? 1u : 0u);
@@ -257,10 +289,8 @@ __global__ void __launch_bounds__(kRgThreads, 1) rows_gemm_kernel(const __grid_c
     const int quarter = warp & 3;
     const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
     int it = 0;
-    for (int u = blockIdx.x; u < a.units; u += gridDim.x, ++it) {
-      const int acc = kExact ? 0 : it & 1, turn = kExact ? it : it >> 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(&tfull[acc], turn & 1, &abort_flag, a.status))) break;
-      tc_fence_after();
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < a.units; u += gridDim.x, ++it) {
       const int tile = u / a.plan.splits;
       const int col = tile * kTile + quarter * 32 + lane;
       float* y = a.y + static_cast<size_t>(u - tile * a.plan.splits) * a.rows * a.plan.ncols + col;
@@ -275,63 +305,71 @@ __global__ void __launch_bounds__(kRgThreads, 1) rows_gemm_kernel(const __grid_c
           if (store && r < a.rows) y[static_cast<size_t>(r) * a.plan.ncols] = s * s_inv[r];
         }
       };
-      auto release = [&]() {
+      auto take = [&](int acc, int turn) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&tfull[acc], turn & 1, &abort_flag, a.status));
+        tc_fence_after();
+        return tmem + lane_off + acc * a.acc_cols;
+      };
+      auto release = [&](int acc) {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&tempty[acc]);
       };
-      const uint32_t t0 = tmem + lane_off + acc * a.acc_cols;
       if constexpr (kExact) {
-        // Four groups as a tree, read before the accumulator is handed back; the rounding errors of the
-        // sum over the fours are carried along while the next unit's products run (before the
-        // hand-back it outlasts the ring: LM head and KL of the 7B shape 170 us).
-        float f[kExactGroups / 4][16];
+        // Four groups as a tree, the fours in order; in a pass by itself with the rounding errors of that sum
+        // carried along (7B LM head's logits: 1.23e-7 without, 1.17e-7 with them).
+        float v[16], e[16];
 #pragma unroll
-        for (int k = 0; k < kExactGroups / 4; ++k) {
-          // groups past the last hold what an earlier launch left: read, not used
-          uint32_t w[4][16];
+        for (int i = 0; i < 16; ++i) v[i] = e[i] = 0.f;
+#pragma unroll 1
+        for (int acc = 0; acc < 2; ++acc) {
+          const int ng = acc == 0 ? first_half(a.groups) : a.groups - first_half(a.groups);
+          if (ng == 0) break;
+          const uint32_t t0 = take(acc, it);
+          if (!ok) break;
+#pragma unroll 1
+          for (int k = 0; k < ng; k += 4) {
+            // groups past the last hold what an earlier launch left: read, not used
+            uint32_t w[4][16];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) tmem_ld16(t0 + (4 * k + q) * 16, w[q]);
-          tmem_ld_wait();
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float g1 = 4 * k + 1 < a.groups ? __uint_as_float(w[1][i]) : 0.f;
-            const float g2 = 4 * k + 2 < a.groups ? __uint_as_float(w[2][i]) : 0.f;
-            const float g3 = 4 * k + 3 < a.groups ? __uint_as_float(w[3][i]) : 0.f;
-            f[k][i] = (__uint_as_float(w[0][i]) + g1) + (g2 + g3);
-          }
-        }
-        release();
-        float v[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          float e = 0.f;
-          v[i] = f[0][i];
-#pragma unroll
-          for (int k = 1; k < kExactGroups / 4; ++k)
-            if (4 * k < a.groups) two_sum(v[i], e, f[k][i]);
-          if (isfinite(v[i])) v[i] += e;  // a sum that is not finite has no error term
-        }
-        if (a.phases == 2) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) v[i] += v[8 + i];
-        }
-        put(0, v);
-      } else {
-        for (int c = 0; c < a.n; c += 16) {
-          float v[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] = 0.f;
-          for (int k = 0; k < a.groups; ++k) {
-            uint32_t w[16];
-            tmem_ld16(t0 + k * a.n + c, w);
+            for (int q = 0; q < 4; ++q) tmem_ld16(t0 + (k + q) * 16, w[q]);
             tmem_ld_wait();
 #pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] += __uint_as_float(w[i]);
+            for (int i = 0; i < 16; ++i) {
+              const float g1 = k + 1 < ng ? __uint_as_float(w[1][i]) : 0.f;
+              const float g2 = k + 2 < ng ? __uint_as_float(w[2][i]) : 0.f;
+              const float g3 = k + 3 < ng ? __uint_as_float(w[3][i]) : 0.f;
+              const float f = (__uint_as_float(w[0][i]) + g1) + (g2 + g3);
+              if constexpr (kAlone)
+                two_sum(v[i], e[i], f);
+              else
+                v[i] += f;
+            }
           }
+          release(acc);
+        }
+        if (!ok) break;
+        if constexpr (kAlone) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (isfinite(v[i])) v[i] += e[i];  // a sum that is not finite has no error term
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] += v[8 + i];
+        put(0, v);
+      } else {
+        const uint32_t t0 = take(it & 1, it >> 1);
+        if (!ok) break;
+        for (int c = 0; c < a.n; c += 16) {
+          uint32_t w[16];
+          tmem_ld16(t0 + c, w);
+          tmem_ld_wait();
+          float v[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(w[i]);
           put(c, v);
         }
-        release();
+        release(it & 1);
       }
     }
   }
@@ -344,17 +382,17 @@ __global__ void __launch_bounds__(kRgThreads, 1) rows_gemm_kernel(const __grid_c
   }
 }
 
-template <int kTerms, bool kExact>
-cudaError_t launch_terms(const RowsGemmArgs& a, int grid, int smem, cudaStream_t stream) {
+template <bool kExact, bool kAlone>
+cudaError_t launch_form(const RowsGemmArgs& a, int grid, int smem, cudaStream_t stream) {
   static PerDevice once;
   int dev = 0;
   if (once.pending(&dev)) {
-    cudaError_t e = cudaFuncSetAttribute(rows_gemm_kernel<kTerms, kExact>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kRowsRingMax + 1024);
+    cudaError_t e = cudaFuncSetAttribute(rows_gemm_kernel<kExact, kAlone>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kRowsRingMax + 2 * kAtom + 1024);
     if (e != cudaSuccess) return e;
     once.done(dev);
   }
-  return launch_kernel(rows_gemm_kernel<kTerms, kExact>, dim3(grid), dim3(kRgThreads), smem, stream, a);
+  return launch_kernel(rows_gemm_kernel<kExact, kAlone>, dim3(grid), dim3(kRgThreads), smem, stream, a);
 }
 
 }  // namespace
@@ -396,7 +434,7 @@ cudaError_t launch_rows_gemm(const RowsGemmDesc& d, const RowsPlan& plan, int nu
   RowsGemmArgs a;
   std::memset(&a, 0, sizeof(a));
   if (d.rows < 1 || d.rows > kRowsMax || d.nseg < 1 || d.nseg > kRowsMaxSeg || d.n_lora < 0 || d.n_lora > kRowsMaxSeg ||
-      (d.terms != 2 && d.terms != 3) || (d.terms == 3 && d.rows > 5) || d.in_dim % 8 != 0)
+      (d.terms != 2 && d.terms != 3) || (d.terms == 3 && d.rows > 2) || d.in_dim % 8 != 0)
     return cudaErrorInvalidValue;
   for (int s = 0; s < kRowsMaxSeg; ++s) {
     const int src = s < d.nseg ? s : 0;  // unused maps alias a valid one
@@ -408,25 +446,23 @@ cudaError_t launch_rows_gemm(const RowsGemmDesc& d, const RowsPlan& plan, int nu
     }
   }
   a.n = (d.rows * d.terms + 15) / 16 * 16;
-  if (!tensor_map_rows(&a.tmX, d.x, static_cast<long>(d.rows) * d.terms, d.in_dim, a.n)) return cudaErrorInvalidValue;
+  const int x_rows = d.terms == 3 ? 8 : a.n;
+  if (!tensor_map_rows(&a.tmX, d.x, static_cast<long>(d.rows) * d.terms, d.in_dim, x_rows)) return cudaErrorInvalidValue;
   a.plan = plan;
   if (d.ncols > 0) a.plan.ncols = d.ncols;
   a.nseg = d.nseg;
   a.n_lora = d.n_lora;
   a.units = plan.tiles * plan.splits;
   a.rows = d.rows;
-  // exact rows: groups of a unit's steps accumulate apart (at least one step each)
-  // A pass of its own fills all of TMEM with one accumulator of 32 groups, so its next unit's products
-  // wait until the epilogue has read it (LM head and KL of one 7B pair: 164 us with 8 groups in two
-  // accumulators, 168 so). A pass in the chain gains nothing from more than four: its rows meet bf16
-  // softmax weights (errors of 1e-5 and up), and 32 cost a 7B step 1.2%.
-  const bool exact = d.terms == 3 && d.alone;
-  a.phases = exact && d.rows * d.terms <= 8 ? 2 : 1;
-  a.groups = d.terms == 3 ? std::min(exact ? kExactGroups : 4, plan.kb / plan.splits) : 1;
-  a.acc_cols = exact ? 16 * kExactGroups : 16;
-  while (a.acc_cols < a.n * a.groups) a.acc_cols *= 2;
-  a.tmem_cols = std::max(32, exact ? a.acc_cols : 2 * a.acc_cols);
-  const int stage = plan.sub * (kWBytes + a.n * kBlockK * 2);
+  // exact rows: a group for every two blocks of the longest unit, at least one step each, at most what TMEM
+  // holds; half of them make an accumulator
+  const bool exact = d.terms == 3;
+  const int longest = (plan.kb + plan.splits - 1) / plan.splits * plan.sub;
+  a.groups = exact ? std::min({kExactGroups, plan.kb / plan.splits, (longest + 1) / 2}) : 1;
+  a.acc_cols = exact ? 16 * kExactGroups / 2 : 16;
+  while (a.acc_cols < a.n) a.acc_cols *= 2;
+  a.tmem_cols = 2 * a.acc_cols;
+  const int stage = plan.sub * (kWBytes + x_rows * kBlockK * 2);
   const int ring = d.alone ? kRowsRingMax : kRowsRing;
   a.stages = std::min(kMaxStages, ring / stage);
   a.y = d.y;
@@ -438,9 +474,9 @@ cudaError_t launch_rows_gemm(const RowsGemmDesc& d, const RowsPlan& plan, int nu
   a.abort = d.abort;
   const int grid = std::min(num_sms, a.units);
   if (grid < 1) return cudaSuccess;
-  const int smem = a.stages * stage + 1024;
-  if (exact) return launch_terms<3, true>(a, grid, smem, stream);
-  return d.terms == 2 ? launch_terms<2, false>(a, grid, smem, stream) : launch_terms<3, false>(a, grid, smem, stream);
+  const int smem = a.stages * stage + 2 * kAtom + 1024;
+  if (!exact) return launch_form<false, false>(a, grid, smem, stream);
+  return d.alone ? launch_form<true, true>(a, grid, smem, stream) : launch_form<true, false>(a, grid, smem, stream);
 }
 
 }  // namespace crf

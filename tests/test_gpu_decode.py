@@ -343,3 +343,39 @@ def test_groups_of_seven_and_eight_heads(head_dim, hq, hkv):
     _, h_last = C.recover(om, oa, opool, oreq, 0, 1)
     assert rel_frob(to_np(fin), h_last) <= REL_KVH
     ctx.close()
+
+
+@pytest.mark.parametrize("rows", [1, 2])
+@pytest.mark.parametrize("shape,limit", [("tiny", 2.6e-7), ("odd", 2.6e-7), ("1.5b", 3.6e-7)])
+def test_one_and_two_rows_keep_fp32_sums(shape, limit, rows):
+    """One or two rows go through the weight passes at fp32 accuracy. A generation step of one layer with
+    empty caches (o is the row's own value, so no weight or key is rounded to bf16) against the oracle in
+    64 bits: relative error of the logits. fp32 sums on CUDA cores gave 1.7e-7 (tiny, at most 2.0e-7) and
+    2.6e-7 (1.5B shape, at most 2.9e-7) over 16 to 48 rows; running sums that the tensor core cuts off
+    over 60 products of 16, 4.7e-7 to 5.6e-7 on the 1.5B shape. The limits leave a fifth over the former's
+    largest. "odd": 5 K blocks, and 17 of which the last holds 8 columns, one weight tile past a whole one."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2609_30884_gb300 as crf
+    base, lc = (synth.QWEN15B, synth.LORA_QWEN) if shape == "1.5b" else (synth.TINY, synth.LORA_TINY)
+    cfg = synth.replace(base, n_layers=1, vocab=4096)
+    if shape == "odd":
+        cfg = synth.replace(cfg, hidden=320, ffn=1032, vocab=3001)
+    dm, ad = DeviceModel(cfg), DeviceAdapter(cfg, synth.replace(lc, modules=synth.MODULES), 1)
+    om, oa = oracle_model(dm), oracle_adapter(ad)
+    pool = make_pool(cfg, rows)
+    pts = [torch.tensor([i], dtype=torch.int32, device="cuda") for i in range(rows)]
+    ctx = crf.Context(0)
+    ws = ctx.decode_workspace(dm.crf, ad.crf, [0] * rows, pts, torch.zeros(rows, dtype=torch.int32, device="cuda"))
+    none = np.zeros((0, cfg.n_kv_heads, cfg.head_dim))
+    for first in (5, 901, 2777):
+        tok = torch.arange(first, first + rows, dtype=torch.int32, device="cuda")
+        nxt = torch.empty(rows, dtype=torch.int32, device="cuda")
+        z = torch.empty(rows, cfg.vocab, device="cuda")
+        ctx.decode_step(dm.crf, ad.crf, pool, [0] * rows, pts, tok, nxt, ws, logits=z)
+        ctx.check()
+        for i in range(rows):
+            x = C.embed(om, [first + i], np.float64)
+            x, _, _ = Dec.decode_row(x, 0, none, none, om.layers[0], oa.layers[0], om.dims, np.float64)
+            assert rel_frob(to_np(z[i]), C.logits(om, x[0], np.float64)[0]) <= limit, (first, i)
+    ctx.close()
