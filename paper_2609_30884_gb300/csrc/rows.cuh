@@ -56,14 +56,22 @@ __device__ __forceinline__ float up_dot(const UpRow& u, const float* xa) {
 }
 
 // v as kTerms bf16 terms (each the rounding of what the ones before leave), stored `dim` apart:
-// two keep about 16 mantissa bits, three all 24 of an fp32 value.
+// two keep about 16 mantissa bits, three all 24 of an fp32 value. An infinity or NaN is its first term
+// alone, and a value that would round to infinity is cut off instead: its terms still sum to it.
 template <int kTerms>
 __device__ __forceinline__ void store_terms(__nv_bfloat16* dst, int dim, float v) {
+  __nv_bfloat16 h = __float2bfloat16_rn(v);
+  float rest = v - __bfloat162float(h);
+  if (!isfinite(rest)) {
+    if (isfinite(v)) h = __float2bfloat16_rz(v);
+    rest = isfinite(v) ? v - __bfloat162float(h) : 0.f;
+  }
+  dst[0] = h;
 #pragma unroll
-  for (int t = 0; t < kTerms; ++t) {
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
+  for (int t = 1; t < kTerms; ++t) {
+    h = __float2bfloat16_rn(rest);
     dst[static_cast<size_t>(t) * dim] = h;
-    v -= __bfloat162float(h);
+    rest -= __bfloat162float(h);
   }
 }
 

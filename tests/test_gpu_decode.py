@@ -379,3 +379,46 @@ def test_one_and_two_rows_keep_fp32_sums(shape, limit, rows):
             x, _, _ = Dec.decode_row(x, 0, none, none, om.layers[0], oa.layers[0], om.dims, np.float64)
             assert rel_frob(to_np(z[i]), C.logits(om, x[0], np.float64)[0]) <= limit, (first, i)
     ctx.close()
+
+
+@pytest.mark.parametrize("rows", [1, 2, 3])
+def test_rows_carry_infinities_and_the_largest_values(rows):
+    """An MLP activation that overflows gives the row's outputs an infinity of its weights' signs, and one
+    between the largest bf16 and the largest fp32 value stays finite: rows enter the weight passes as
+    bf16 terms, of which none may be infinity minus infinity. Gate and up of one value, all other weights
+    zero, so the first-step row is 1 + w silu(g) u (rounded to bf16; the terms keep 2^-17)."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2609_30884_gb300 as crf
+    cfg = synth.replace(synth.TINY, n_layers=1)
+    h, dev = cfg.hidden, "cuda"
+    sign = torch.where(torch.arange(h, device=dev) % 3 == 0, -1.0, 1.0)
+    pool = make_pool(cfg, rows)
+    ctx = crf.Context(0)
+    ones = torch.ones(cfg.vocab, h, dtype=torch.bfloat16, device=dev)
+    dims = dict(n_layers=1, hidden=h, n_q_heads=cfg.n_q_heads, n_kv_heads=cfg.n_kv_heads, head_dim=cfg.head_dim,
+                ffn=cfg.ffn, vocab=cfg.vocab, rms_eps=0.0, rope_theta=1e4, qkv_bias=False)
+    ad = crf.Adapter(4, 8.0, (), [None])
+    for gate, up, down in ((2.0 ** 66, 2.0 ** 66, 1.0), (1.3125 * 2.0 ** 64, 1.5234375 * 2.0 ** 63, 2.0 ** -100)):
+        w = {k: torch.zeros_like(v) for k, v in synth.layer_weights(cfg, 0, 0, dev).items()}
+        w["ln1"].fill_(1.0)
+        w["ln2"].fill_(1.0)
+        w["W_gate"][7, 0], w["W_up"][7, 0] = gate, up
+        w["W_down"][:, 7] = (down * sign).bfloat16()
+        model = crf.Model(dims, [w], ones)
+        fin = torch.empty(rows, h, dtype=torch.bfloat16, device=dev)
+        reqs = [crf.Request(torch.tensor([i], dtype=torch.int32, device=dev), 0, 0, final_hidden_out=fin[i],
+                            tokens=torch.zeros(1, dtype=torch.int32, device=dev)) for i in range(rows)]
+        ctx.recompute_window(model, ad, pool, reqs, ctx.workspace(model, ad, reqs))
+        ctx.check()
+        with np.errstate(over="ignore"):
+            act = np.float32(gate) * np.float32(up)
+        assert np.isinf(act) == (down == 1.0)
+        want = 1.0 + sign.double() * down * float(act)
+        for i in range(rows):
+            got = fin[i].double()
+            if np.isinf(act):
+                assert torch.equal(got, want), i
+            else:
+                assert torch.all((got - want).abs() <= 2.0 ** -8 * want.abs()), i
+    ctx.close()
