@@ -466,7 +466,7 @@ crf_status run_layer(const LayerCtx& c, int l, const __nv_bfloat16* X_in, __nv_b
     a.status = c.ctx->status_dev;
     a.abort = c.abort;
     ProfScope ps(c.ctx, kPAttn, c.st);
-    CRF_CUDA(launch_attention_tc(a, c.pool->num_pages, M, c.st));
+    CRF_CUDA(launch_attention_tc(a, c.pool->num_pages, M, c.ctx->num_sms, c.st));
   }
 
   // 5-6. output projection + residual: X1 = X_in + O W_o^T (+ LoRA)
@@ -1194,7 +1194,7 @@ crf_status crf_decode_step(crf_ctx* ctx, const crf_model* model, const crf_adapt
                             ctx->status_dev, st, c.abort));
     int* words = reinterpret_cast<int*>(ws + sp.p.off_abort) + 2;
     CRF_CUDA(launch_argmax_rows(z, n_rows, D.V, reinterpret_cast<unsigned long long*>(words), words + 2 * n_rows,
-                                next_tokens, st, c.abort));
+                                next_tokens, ctx->num_sms, st, c.abort));
   }
   return CRF_OK;
 }
@@ -1325,7 +1325,7 @@ crf_status crf_kl(crf_ctx* ctx, const crf_model* model, const void* ref, const v
   }
   {
     ProfScope ps(ctx, kPKl, st, 2);
-    CRF_CUDA(launch_kl(zr, zc, n_rows, vocab, out_kl, part, sp, st));
+    CRF_CUDA(launch_kl(zr, zc, n_rows, vocab, out_kl, part, sp, ctx->num_sms, st));
   }
   return CRF_OK;
 }

@@ -75,7 +75,7 @@ struct AttnTcArgs {
   __nv_bfloat16* out;
   int ldo;
   int n_q_heads, n_kv_heads, group;
-  int total_items;
+  int total_items, num_sms;
   ReqTable req;
   int* status;
   const int* abort;
@@ -87,15 +87,15 @@ struct AttnWork {
 };
 
 // Whether the query pairs of a request of `len` rows are dealt to two CTAs each (halves of their keys):
-// where its longest pair alone runs over twice an even share of all pairs on 152 SMs. The halves cost a
+// where its longest pair alone runs over twice an even share of all pairs over the SMs. The halves cost a
 // second prologue and an exchange, which 1.5 times an even share does not repay (1.5B shape, us a
 // window of 4096 rows: 905 whole, 912 split; a prefill of 2003 rows, 2.8 times: 1490 and 1429).
-// A property of the request, not of the call: a request gives the same bits in any batch.
+// A property of the request (and the device), not of the call: a request gives the same bits in any batch.
 constexpr int kSplitTiles = 4;  // pairs of fewer kv tiles are not split
-__host__ __device__ inline bool splits_keys(int len, int n_q_heads) {
+__host__ __device__ inline bool splits_keys(int len, int n_q_heads, int num_sms) {
   const long long tiles = (len + kN - 1) / kN, nqp = (len + 2 * kM - 1) / (2 * kM);
   const long long sum = nqp * (nqp + 1) - (tiles & 1);  // kv tiles of all pairs of a head
-  return tiles >= kSplitTiles && tiles * 152 > 2 * n_q_heads * sum;
+  return tiles >= kSplitTiles && tiles * num_sms > 2 * n_q_heads * sum;
 }
 
 // Items: (request, 256-row query pair, head), longest (latest) query pairs first. With kPair a
@@ -109,7 +109,7 @@ __device__ __forceinline__ bool attn_work(const AttnTcArgs& a, int idx, AttnWork
     int items = nqp * a.n_q_heads;
     w.split = false;
     if (kPair) {
-      w.split = splits_keys(a.req.len[i], a.n_q_heads);
+      w.split = splits_keys(a.req.len[i], a.n_q_heads, a.num_sms);
       if (!w.split) {
         const int clusters = (items + 1) / 2;
         if (idx >= clusters) {
@@ -654,7 +654,7 @@ cudaError_t launch_tc(const AttnTcArgs& args, bool pair, cudaStream_t stream) {
 
 }  // namespace
 
-cudaError_t launch_attention_tc(const AttnDesc& d, int num_pages, int total_rows, cudaStream_t stream) {
+cudaError_t launch_attention_tc(const AttnDesc& d, int num_pages, int total_rows, int num_sms, cudaStream_t stream) {
   AttnTcArgs a;
   std::memset(&a, 0, sizeof(a));
   const int D = d.head_dim;
@@ -671,11 +671,12 @@ cudaError_t launch_attention_tc(const AttnDesc& d, int num_pages, int total_rows
   a.status = d.status;
   a.abort = d.abort;
   bool pair = false;
-  for (int i = 0; i < d.req.n; ++i) pair |= splits_keys(d.req.len[i], d.n_q_heads);
+  a.num_sms = num_sms;
+  for (int i = 0; i < d.req.n; ++i) pair |= splits_keys(d.req.len[i], d.n_q_heads, num_sms);
   a.total_items = 0;
   for (int i = 0; i < d.req.n; ++i) {
     const int items = ((d.req.len[i] + 2 * kM - 1) / (2 * kM)) * d.n_q_heads;
-    a.total_items += !pair ? items : splits_keys(d.req.len[i], d.n_q_heads) ? 2 * items : (items + 1) / 2 * 2;
+    a.total_items += !pair ? items : splits_keys(d.req.len[i], d.n_q_heads, num_sms) ? 2 * items : (items + 1) / 2 * 2;
   }
   if (a.total_items == 0) return cudaSuccess;
   if (D == 128) return launch_tc<128>(a, pair, stream);

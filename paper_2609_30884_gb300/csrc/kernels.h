@@ -105,8 +105,9 @@ struct GemmDesc {
   int group_cols[3];      // valid output columns per group (plain) / per segment (stacked)
   // Unmerged LoRA (Eq. S3), computed inside the same launch, which first forms XA[:, 32j .. 32j + 32) =
   // hi/lo of (alpha/r) x A_j^T for the n_slots adapted modules (LA[j] = A_j, [rank, K]) of each
-  // 256-row block and raises xa_flags[row block]; every output tile of an adapted group then adds one K block: XA[:, xa_base[g] .. + 64] against BX[i] (the module's
-  // [B | B] rows under its slot, zeros elsewhere; [B_rows[i], kBxCols], map index i like B).
+  // 256-row block and raises xa_flags[row block]; every output tile of an adapted group then adds one K
+  // block: XA[:, xa_base[g] .. + 64] against BX[i] (the module's [B | B] rows under its slot, zeros
+  // elsewhere; [B_rows[i], kBxCols], map index i like B).
   void* XA;
   int n_slots;
   const void* LA[3];
@@ -136,7 +137,7 @@ struct GemmDesc {
   const int* abort;       // per-call abort word (call_aborted), or null
 };
 
-// Launch the tcgen05 projection GEMM (CTA pairs, 256 x 256 tiles).
+// Launch the tcgen05 projection GEMM (CTA pairs; tiles of 256 rows and 256, 192 or 128 columns).
 cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t stream);
 
 // ------------------------------------------------------------------ other kernels
@@ -174,7 +175,7 @@ struct AttnDesc {
   const int* abort;
 };
 // tcgen05, S and O in TMEM: num_pages of the pool, total_rows of q (for the TMA maps).
-cudaError_t launch_attention_tc(const AttnDesc& d, int num_pages, int total_rows,
+cudaError_t launch_attention_tc(const AttnDesc& d, int num_pages, int total_rows, int num_sms,
                                 cudaStream_t stream);
 
 // ------------------------------------------------------------------ decode rows
@@ -299,7 +300,7 @@ cudaError_t launch_wait_selftest(int* status, cudaStream_t stream);
 // out[r] = argmax of logits row r (lowest index among equal maxima). key, count: one entry per row, zero
 // before the launch.
 cudaError_t launch_argmax_rows(const float* logits, int rows, int vocab, unsigned long long* key, int* count,
-                               int32_t* out, cudaStream_t stream, const int* abort);
+                               int32_t* out, int num_sms, cudaStream_t stream, const int* abort);
 // dst[0 .. n) = src[0 .. n) (bf16), unless the call's abort word is set.
 cudaError_t launch_copy_rows(__nv_bfloat16* dst, const __nv_bfloat16* src, size_t n, const int* abort,
                              cudaStream_t stream);
@@ -325,7 +326,7 @@ cudaError_t launch_lm_head(const __nv_bfloat16* W, const __nv_bfloat16* xs, int 
                            cudaStream_t stream, const int* abort = nullptr);
 // KL per row from fp32 logits; part: scratch [rows][splits][5].
 cudaError_t launch_kl(const float* zref, const float* zcur, int rows, int vocab, float* out,
-                      float* part, int splits, cudaStream_t stream);
+                      float* part, int splits, int num_sms, cudaStream_t stream);
 // Vocabulary splits per row of the KL reduction: about two blocks per SM over all rows, at least
 // 1024 logits per split, at most kKlMaxSplits. Every KL entry point uses this count, so they
 // reduce in the same order.

@@ -123,7 +123,7 @@ extern "C" crf_status crf_kl_logits_noalloc(int device, const float* z_ref, cons
     // the same split count as crf_kl, so both reduce in the same order; at most kKlMaxSplits
     const int splits = crf::kl_split_count(sms, n_rows, vocab);
     // Every (row, split) partial is written before it is read: nothing needs clearing.
-    const cudaError_t e = crf::launch_kl(z_ref, z_cur, n_rows, vocab, out_kl, part, splits,
+    const cudaError_t e = crf::launch_kl(z_ref, z_cur, n_rows, vocab, out_kl, part, splits, sms,
                                          static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) {
       crf::set_last_error(cudaGetErrorString(e));

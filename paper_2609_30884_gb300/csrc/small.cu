@@ -447,10 +447,10 @@ __global__ void __launch_bounds__(kArgmaxThreads) argmax_rows_kernel(const float
 }
 
 cudaError_t launch_argmax_rows(const float* logits, int rows, int vocab, unsigned long long* key, int* count,
-                               int32_t* out, cudaStream_t stream, const int* abort) {
+                               int32_t* out, int num_sms, cudaStream_t stream, const int* abort) {
   if (rows == 0) return cudaSuccess;
   // about two blocks per SM over all rows, at least 4096 logits each
-  const int by_rows = std::max(1, 304 / rows), by_vocab = (vocab + 4095) / 4096;
+  const int by_rows = std::max(1, 2 * num_sms / rows), by_vocab = (vocab + 4095) / 4096;
   return launch_kernel(argmax_rows_kernel, dim3(std::min(std::min(32, by_rows), by_vocab), rows), dim3(kArgmaxThreads), 0,
                        stream, logits, vocab, key, count, out, abort);
 }
@@ -469,13 +469,13 @@ cudaError_t launch_copy_rows(__nv_bfloat16* dst, const __nv_bfloat16* src, size_
 }
 
 cudaError_t launch_kl(const float* zref, const float* zcur, int rows, int vocab, float* out,
-                      float* part, int splits, cudaStream_t stream) {
+                      float* part, int splits, int num_sms, cudaStream_t stream) {
   if (rows == 0) return cudaSuccess;
   // Launched early, one block per SM finds its SM free when the logits are done (one row pair, 7B: 168 ->
   // 162 us with the LM head); twice as many pile up on the first SMs with room and make the rest
   // wait (29 pairs, 1.5B: 103 -> 112 us), so those launch when the LM head has ended.
   std::optional<PdlScope> pdl;
-  if (static_cast<long>(splits) * rows <= 152) pdl.emplace();
+  if (static_cast<long>(splits) * rows <= num_sms) pdl.emplace();
   const cudaError_t e =
       launch_kernel(kl_partial_kernel, dim3(splits, rows), dim3(kKlThreads), 0, stream, zref, zcur, vocab, splits, part);
   if (e != cudaSuccess) return e;
