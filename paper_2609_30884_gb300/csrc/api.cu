@@ -414,7 +414,6 @@ crf_status run_layer(const LayerCtx& c, int l, const __nv_bfloat16* X_in, __nv_b
     g.A = XN;
     g.M = M;
     g.K = D.h;
-    g.lda = D.h;
     g.ngroups = 3;
     g.nseg = 1;
     const int mods[3] = {CRF_MOD_Q, CRF_MOD_K, CRF_MOD_V};
@@ -424,7 +423,6 @@ crf_status run_layer(const LayerCtx& c, int l, const __nv_bfloat16* X_in, __nv_b
     for (int m = 0; m < 3; ++m) {
       g.B[m] = w.W[m];
       g.B_rows[m] = rows[m];
-      g.ldb[m] = D.h;
       g.group_cols[m] = rows[m];
       if (slot[m] >= 0) {
         g.BX[m] = BX[m];
@@ -454,7 +452,6 @@ crf_status run_layer(const LayerCtx& c, int l, const __nv_bfloat16* X_in, __nv_b
   {
     AttnDesc a;
     a.q = Q;
-    a.ldq = D.qd;
     a.kpages = static_cast<const __nv_bfloat16*>(c.pool->k_pages[l]);
     a.vpages = static_cast<const __nv_bfloat16*>(c.pool->v_pages[l]);
     a.out = O;
@@ -476,12 +473,10 @@ crf_status run_layer(const LayerCtx& c, int l, const __nv_bfloat16* X_in, __nv_b
     g.A = A;
     g.M = M;
     g.K = K;
-    g.lda = K;
     g.ngroups = 1;
     g.nseg = 1;
     g.B[0] = w.W[m];
     g.B_rows[0] = D.h;
-    g.ldb[0] = K;
     g.group_cols[0] = D.h;
     int slot[1];
     set_lora(g, &m, 1, slot);
@@ -517,7 +512,6 @@ crf_status run_layer(const LayerCtx& c, int l, const __nv_bfloat16* X_in, __nv_b
     g.A = XN;
     g.M = M;
     g.K = D.h;
-    g.lda = D.h;
     g.ngroups = 1;
     g.nseg = 2;
     const int mods[2] = {CRF_MOD_GATE, CRF_MOD_UP};
@@ -526,7 +520,6 @@ crf_status run_layer(const LayerCtx& c, int l, const __nv_bfloat16* X_in, __nv_b
     for (int s = 0; s < 2; ++s) {
       g.B[s] = w.W[mods[s]];
       g.B_rows[s] = D.f;
-      g.ldb[s] = D.h;
       g.BX[s] = BX[mods[s]];  // all-zero rows for a module without adapter
     }
     if (g.n_slots) {

@@ -47,6 +47,7 @@
 // uniform 8-row stride.
 #include "common.cuh"
 #include "kernels.h"
+#include "tma_map.h"
 
 #include <algorithm>
 #include <cfloat>
@@ -583,48 +584,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsAttn, 1)
   attn_body<D, true>(a);
 }
 
-using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
-  return fn;
-}
-
 // K or V pool of one layer, [rows = pages * Hkv * 16, D] row-major, as the 4-D view
 // {64 columns, 8 rows, D/64 halves, rows/8 groups} with strides {2D, 128, 16D} bytes; the box
 // {64, 8, D/64, 2} is one page of one kv head, written to shared memory group-major, halves
 // inside a group, each half an 8 x 128-byte swizzled atom.
 bool map_pool(CUtensorMap* m, const void* base, long rows, int D) {
-  EncodeTiledFn fn = encode();
+  TensorMapEncodeFn fn = tensor_map_encode();
   if (!fn) return false;
   cuuint64_t dims[4] = {64, 8, static_cast<cuuint64_t>(D / 64), static_cast<cuuint64_t>(rows / 8)};
   cuuint64_t strides[3] = {static_cast<cuuint64_t>(D) * 2, 128, static_cast<cuuint64_t>(D) * 16};
   cuuint32_t box[4] = {64, 8, static_cast<cuuint32_t>(D / 64), kPage / 8};
   cuuint32_t estr[4] = {1, 1, 1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box,
-            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-bool map2d(CUtensorMap* m, const void* base, long rows, int cols, int box_rows) {
-  EncodeTiledFn fn = encode();
-  if (!fn) return false;
-  cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
-  cuuint64_t strides[1] = {static_cast<cuuint64_t>(cols) * 2};
-  cuuint32_t box[2] = {64, static_cast<cuuint32_t>(box_rows)};
-  cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -658,7 +629,7 @@ cudaError_t launch_attention_tc(const AttnDesc& d, int num_pages, int total_rows
   AttnTcArgs a;
   std::memset(&a, 0, sizeof(a));
   const int D = d.head_dim;
-  if (!map2d(&a.tmQ, d.q, total_rows, d.n_q_heads * D, kM)) return cudaErrorInvalidValue;
+  if (!tensor_map_rows(&a.tmQ, d.q, total_rows, d.n_q_heads * D, kM)) return cudaErrorInvalidValue;
   const long pool_rows = static_cast<long>(num_pages) * d.n_kv_heads * kPage;
   if (!map_pool(&a.tmK, d.kpages, pool_rows, D)) return cudaErrorInvalidValue;
   if (!map_pool(&a.tmV, d.vpages, pool_rows, D)) return cudaErrorInvalidValue;

@@ -40,7 +40,7 @@ namespace crf {
 namespace {
 
 constexpr int kChunk = 128;  // positions per chunk
-constexpr int kStages = 2;   // 64 KB each at d = 128: with the next weight pass's ring on the same SM
+constexpr int kStages = 2;   // 64 KB each at d = 128
 constexpr int kComputeWarps = 8;
 constexpr int kCompute = 32 * kComputeWarps;
 constexpr int kThreadsStream = kCompute + 32;  // + one copy warp

@@ -40,10 +40,9 @@
 //   7B,   16384 rows:       370, 358, 318     282, 283, 258           2582, 2546, 2271        1288, 1356, 1255
 #include "common.cuh"
 #include "kernels.h"
+#include "tma_map.h"
 
 #include <algorithm>
-#include <cstdio>
-#include <cstdlib>
 #include <cstring>
 
 namespace crf {
@@ -769,39 +768,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
 }
 
 // ---------------------------------------------------------------- host side
-using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
-  return fn;
-}
-
-// 2-D bf16 map over rows x cols (row stride ld elements), box box_rows x box_cols.
-bool make_map(CUtensorMap* m, const void* base, int rows, int cols, int ld, int box_rows,
-              int box_cols, CUtensorMapSwizzle sw) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
-  cuuint64_t strides[1] = {static_cast<cuuint64_t>(ld) * 2};
-  cuuint32_t box[2] = {static_cast<cuuint32_t>(box_cols), static_cast<cuuint32_t>(box_rows)};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides,
-                  box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
-}
-
 template <int BN, int STAGES, int EPI>
 cudaError_t launch_impl(GemmArgs& args, int num_sms, cudaStream_t stream) {
   constexpr int PAIR = kPair;
@@ -858,7 +824,6 @@ cudaError_t launch_impl(GemmArgs& args, int num_sms, cudaStream_t stream) {
 }
 
 int group_tiles(const GemmDesc& d, int g, int bn) {
-  if (d.nseg > 1 && d.epi != kEpiSwiGLU) return 1;
   const int cols = d.nseg > 1 ? bn / d.nseg : bn;
   return (d.group_cols[g] + cols - 1) / cols;
 }
@@ -896,31 +861,27 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t stream) {
   constexpr int pair = kPair;
   GemmArgs a;
   std::memset(&a, 0, sizeof(a));
-  if (d.nseg != 1 && d.nseg != 2) return cudaErrorInvalidValue;
+  if (d.nseg != (d.epi == kEpiSwiGLU ? 2 : 1)) return cudaErrorInvalidValue;
   a.num_kb = (d.K + BK - 1) / BK;
   a.row_tiles = (d.M + BM * pair - 1) / (BM * pair);
   const int bn = tile_columns(d, a.row_tiles, a.num_kb, num_sms / pair);
   // rows of one B load: the CTA's share of the tile (plain) or one stacked segment
   const int b_box = d.nseg == 1 ? bn / pair : bn / d.nseg;
-  if (!make_map(&a.tmA, d.A, d.M, d.K, d.lda, BM, BK, CU_TENSOR_MAP_SWIZZLE_128B))
-    return cudaErrorInvalidValue;
+  if (!tensor_map_rows(&a.tmA, d.A, d.M, d.K, BM)) return cudaErrorInvalidValue;
   const int nmaps = d.ngroups + d.nseg - 1;
   for (int i = 0; i < 3; ++i) {
     const int src = i < nmaps ? i : 0;  // unused slots alias a valid map
-    if (!make_map(&a.tmB[i], d.B[src], d.B_rows[src], d.K, d.ldb[src], b_box, BK,
-                  CU_TENSOR_MAP_SWIZZLE_128B))
-      return cudaErrorInvalidValue;
+    if (!tensor_map_rows(&a.tmB[i], d.B[src], d.B_rows[src], d.K, b_box)) return cudaErrorInvalidValue;
   }
   bool any_ext = false;
   for (int g = 0; g < d.ngroups; ++g) any_ext |= d.ext_on[g] != 0;
   if (any_ext != (d.n_slots > 0) || d.n_slots < 0 || d.n_slots > 3) return cudaErrorInvalidValue;
   if (any_ext) {
     if (!d.XA || !d.xa_flags || (d.rank != 4 && d.rank != 8 && d.rank != 16)) return cudaErrorInvalidValue;
-    if (!make_map(&a.tmXA, d.XA, d.M, kXaCols, kXaCols, BM, BK, CU_TENSOR_MAP_SWIZZLE_128B))
-      return cudaErrorInvalidValue;
+    if (!tensor_map_rows(&a.tmXA, d.XA, d.M, kXaCols, BM)) return cudaErrorInvalidValue;
     for (int j = 0; j < 3; ++j) {
       const int src = j < d.n_slots ? j : 0;
-      if (!d.LA[src] || !make_map(&a.tmLA[j], d.LA[src], d.rank, d.K, d.K, 16, BK, CU_TENSOR_MAP_SWIZZLE_128B))
+      if (!d.LA[src] || !tensor_map_rows(&a.tmLA[j], d.LA[src], d.rank, d.K, 16))
         return cudaErrorInvalidValue;
     }
     for (int g = 0; g < d.ngroups; ++g) {
@@ -936,8 +897,7 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t stream) {
         for (int j = 0; j < nmaps; ++j)
           if (d.BX[j]) src = j;  // unused slots alias a valid map
       if (src < 0) return cudaErrorInvalidValue;
-      if (!make_map(&a.tmBX[i], d.BX[src], d.B_rows[src], kBxCols, kBxCols, b_box, BK, CU_TENSOR_MAP_SWIZZLE_128B))
-        return cudaErrorInvalidValue;
+      if (!tensor_map_rows(&a.tmBX[i], d.BX[src], d.B_rows[src], kBxCols, b_box)) return cudaErrorInvalidValue;
     }
     for (int g = 0; g < d.ngroups; ++g)
       for (int s = 0; s < (d.ngroups == 1 ? d.nseg : 1); ++s)

@@ -96,12 +96,11 @@ enum EpiKind : int {
 // matrix (plain mode, nseg == 1), or one group whose tiles stack `nseg` equal
 // row segments of different matrices (paired / stacked mode, ngroups == 1).
 struct GemmDesc {
-  const void* A;
-  int M, K, lda;
+  const void* A;          // [M, K]
+  int M, K;
   int ngroups, nseg;
-  const void* B[3];       // map index g + s
-  int B_rows[3];          // rows of each B matrix
-  int ldb[3];
+  const void* B[3];       // map index g + s; [B_rows, K]
+  int B_rows[3];
   int group_cols[3];      // valid output columns per group (plain) / per segment (stacked)
   // Unmerged LoRA (Eq. S3), computed inside the same launch, which first forms XA[:, 32j .. 32j + 32) =
   // hi/lo of (alpha/r) x A_j^T for the n_slots adapted modules (LA[j] = A_j, [rank, K]) of each
@@ -164,7 +163,6 @@ cudaError_t launch_embed(const __nv_bfloat16* embed, const int32_t* tokens, __nv
 // Causal GQA prefill attention over the paged cache of the current layer.
 struct AttnDesc {
   const __nv_bfloat16* q;  // [rows, Hq*d] post-RoPE
-  int ldq;
   const __nv_bfloat16* kpages;  // [P][Hkv][16][d]
   const __nv_bfloat16* vpages;
   __nv_bfloat16* out;      // [rows, Hq*d]
