@@ -113,13 +113,16 @@ def test_window_tile_and_norm_widths(ctx, hidden, ffn, n):
 def test_final_hidden_out_of_any_alignment(ctx, tiny, s, e):
     """final_hidden_out two bytes past a 16-byte boundary gets the bits of an aligned one, where it is a
     copy of the last row (the window ends at the last layer, or there is none left) and where the
-    remaining layers run on that row; the element on either side stays."""
+    remaining layers run on that row; the element on either side stays. The aligned row is the oracle's,
+    or the restart row itself where no layer is left."""
     import paper_2609_30884_gb300 as crf
-    cfg, _, dm, cur, _, _ = tiny
+    cfg, _, dm, cur, om, oa = tiny
     n = 129
     pool = make_pool(cfg, pages_needed(n), fill="random", seed=12)
     pt = split_page_tables([n], pages_needed(n), seed=2)[0]
     h_in = synth.hidden_state(cfg, n, device="cuda")
+    oreq = C.RequestCache(np.zeros(n, np.int64), pt.cpu().numpy())
+    _, want = C.recover(om, oa, oracle_pool(pool), oreq, s, e, restart=to_np(h_in))
     got = []
     for shift in (0, 1):
         buf = torch.full((cfg.hidden + 2,), 7.0, dtype=torch.bfloat16, device="cuda")
@@ -130,6 +133,9 @@ def test_final_hidden_out_of_any_alignment(ctx, tiny, s, e):
         assert torch.all(rest == 7.0)
         got.append(buf[shift:shift + cfg.hidden].clone())
     assert torch.equal(got[0], got[1])
+    assert rel_frob(to_np(got[0]), want) <= REL_KVH
+    if s == cfg.n_layers:
+        assert torch.equal(got[0], h_in[-1])
 
 
 @pytest.mark.parametrize("lengths", [(384,), (385,), (513,), (769,), (1409,), (130, 385, 1, 900, 257)])
