@@ -31,13 +31,17 @@
 //               when the running max grows by more than 2^8
 // TMEM: S0 | S1 | O0 | O1, 128 columns each. Every wait is bounded.
 // Bound by each tile's chain S -> softmax -> P V, not by the tensor pipe. One layer of the 7B shape at
-// 16384 rows: 1588 us with the producer's and issuer's loops in one lane, 1493 by whole warps, 1442
-// with the MMA descriptors formed once (1335 TFLOP/s of causal work).
+// 16384 rows, in a two-layer window: 1588 us with the producer's and issuer's loops in one lane, 1493 by
+// whole warps, 1442 with the MMA descriptors formed once (1335 TFLOP/s of causal work; 1350 in a window of
+// one layer, 1607 within the power-capped benchmark step).
 //
 // The last pair's chain over all keys sets the time of a short prefix that leaves SMs idle (1.5B shape,
 // 2003 rows: 96 CTAs). There (splits_keys) a cluster of two shares each pair's keys and meets in
-// shared memory: prefill of 2003 rows 1.49 -> 1.43 ms, tiny window 112 -> 107 us, 387-row 7B window
-// 1.012 -> 1.007 ms. Errors of the checkpoints against 64 bits stay the same to 2e-6.
+// shared memory: prefill of 2003 rows 1.526 -> 1.463 ms (attention 37.0 -> 30.7 us a layer), tiny window
+// 115.7 -> 111.1 us, 387-row 7B window 1.021 -> 1.016 ms. The halves' softmax weights are rounded against
+// other maxima, so a split request's bits differ from an unsplit one's; mean errors of the last checkpoint
+// against 64 bits are the same (tiny 2.856e-3 both; 387 rows 5.866e-3, split 5.868e-3; eight layers of 2003 rows
+// 1.2107e-2, split 1.2106e-2).
 //
 // K/V slot layout: the 128 keys of a tile in 16 groups of 8 keys, group c at
 // c * HALVES * 1024 bytes, and within a group one 1 KB 128B-swizzled atom per

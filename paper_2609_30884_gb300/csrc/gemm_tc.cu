@@ -34,10 +34,11 @@
 //
 // Measured (us a launch; first column: the XA product in each row block's first tile, 256-column tiles,
 // one row a thread in the epilogue; then: XA items, epilogue through shared memory, 128 columns; last:
-// loops run by whole warps and, for o and down, 192 columns):
-//   1.5B,  2003 rows: q|k|v  34,  28,  25   o  33,  24,  21   gate|up   99,   88,   71   down   84,   60,   45
-//   1.5B,  4096 rows:        45,  39,  34      48,  35,  29            164,  150,  126         131,  108,   80
-//   7B,   16384 rows:       370, 358, 318     282, 283, 258           2582, 2546, 2271        1288, 1356, 1255
+// loops run by whole warps, for o and down 192 columns, and silu() for the divide of SwiGLU):
+//   1.5B,  2003 rows: q|k|v  34,  28,  25   o  33,  24,  20   gate|up   99,   88,   73   down   84,   60,   45
+//   1.5B,  4096 rows:        45,  39,  33      48,  35,  29            164,  150,  127         131,  108,   81
+//   7B,   16384 rows:       370, 358, 311     282, 283, 252           2582, 2546, 2289        1288, 1356, 1249
+// (the last row in a one-layer window; in longer runs the power cap adds 4-7%)
 #include "common.cuh"
 #include "kernels.h"
 #include "tma_map.h"
@@ -829,7 +830,8 @@ int group_tiles(const GemmDesc& d, int g, int bn) {
 }
 
 // 256-column tiles run the MMAs at their best rate; narrower ones leave less of the last wave empty
-// and less of the epilogue exposed at its end. Compared in K blocks of a 256-column tile: a tile's
+// and less of the epilogue exposed at its end. Compared in K blocks of a 256-column tile, with factors
+// from launches of the 1.5B and 7B shapes' widths (others were not timed): a tile's
 // hand-over costs about two, the last epilogue 10 per 256 columns, a 192-column block 0.84 and a
 // 128-column one 0.8 (its operands are half again as many bytes from L2 per FLOP: down of a 7B batch
 // of 8228 rows takes 445 us on 256 columns, 754 on 128). 192 columns only where an epilogue has no

@@ -11,7 +11,7 @@
 // exact (three terms: one or two rows), a unit's steps accumulate in groups of TMEM columns, and the
 // rows, which fill at most 6 of an operand's 16 rows, change sides with every K block: an 8-row atom of
 // zeros is the other half of the operand, reached through the descriptor's stride. So every block of a
-// group has sums of its own, of four MMAs. (Boxes that start 8 rows early, zero-filled, did the same and took
+// group has sums of its own, of four MMAs. (An infinite weight makes its output NaN: infinity meets zeros. Boxes that start 8 rows early, zero-filled, did the same and took
 // 2.5 us a pass more: 7B step of one row 3.30 ms, 3.03 so.)
 // Error of the logits against 64 bits, sums of 4 MMAs / of 32 to 60 / fp32 on CUDA cores: the LM head alone, one
 // pair of rows, 7B 1.17e-7 / 4.48e-7 / 1.22e-7, 1.5B 1.01e-7 / 2.17e-7 / 1.10e-7; one layer and the head, one
@@ -28,15 +28,14 @@
 // One CTA per SM and dependent launch: the ring's first weights are requested before the wait for the
 // kernel that makes x, so the copies run through the short kernels between two passes (a ring of 75
 // KB for the short passes would fit beside decode attention's block and start earlier, but runs out
-// sooner: 7B step of one row 3.08 against 3.01 ms, of 32 rows 4.64 against 4.37; asking L2 for more
-// weights before the wait gained nothing). Weights are marked evict-first in L2, which keeps the
+// sooner: 7B step of one row 3.08 against 3.01 ms, of 32 rows 4.64 against 4.37, before sums of four MMAs;
+// asking L2 for more weights before the wait gained nothing). Weights are marked evict-first in L2, which keeps the
 // rows' partial sums and the K/V pages there (3% of a 7B generation step).
 //
-// Measured with the norm before it: LM head of the 7B shape, 2 rows, 1.09 GB in 170 us (6.4 TB/s; 162
-// with sums of 32 MMAs); gate|up of one row, alone and cold, 272 MB in
-// 45 us (6.1 TB/s; 56 us before); 58 rows of the 1.5B LM head 83 us in one pass (a pass for every 8 rows before: 779 us).
-// Generation steps with all that this layout brought, CUDA-core and mma.sync passes of 8 rows before:
-// 7B 1 row 4.06 -> 2.95 ms, 32 rows 18.0 -> 4.32 ms, 1.5B 8 rows 2.35 -> 1.39 ms.
+// Measured alone and cold: LM head of the 7B shape, 2 rows, 1.09 GB in 164 us (6.6 TB/s); gate|up of one
+// row, 272 MB in 46 us (5.9 TB/s; 56 us before); 58 rows of the 1.5B LM head 79 us in one pass (a pass
+// for every 8 rows before: 779 us). Generation steps with all that this layout brought, CUDA-core and
+// mma.sync passes of 8 rows before: 7B 1 row 4.06 -> 3.03 ms, 32 rows 18.2 -> 4.28 ms, 1.5B 8 rows 2.36 -> 1.35 ms.
 #include "common.cuh"
 #include "kernels.h"
 #include "tma_map.h"
