@@ -11,12 +11,14 @@
 // exact (three terms: one or two rows), a unit's steps accumulate in groups of TMEM columns, and the
 // rows, which fill at most 6 of an operand's 16 rows, change sides with every K block: an 8-row atom of
 // zeros is the other half of the operand, reached through the descriptor's stride. So every block of a
-// group has sums of its own, of four MMAs. (An infinite weight makes its output NaN: infinity meets zeros. Boxes that start 8 rows early, zero-filled, did the same and took
-// 2.5 us a pass more: 7B step of one row 3.30 ms, 3.03 so.)
+// group has sums of its own, of four MMAs. (Boxes that start 8 rows early, zero-filled, did the same and
+// took 2.5 us a pass more: 7B step of one row 3.30 ms, 3.03 so. An infinite weight makes its output NaN:
+// infinity meets zeros.)
 // Error of the logits against 64 bits, sums of 4 MMAs / of 32 to 60 / fp32 on CUDA cores: the LM head alone, one
 // pair of rows, 7B 1.17e-7 / 4.48e-7 / 1.22e-7, 1.5B 1.01e-7 / 2.17e-7 / 1.10e-7; one layer and the head, one
 // row, 7B 2.9e-7 / 1.2e-6 / 3.2e-7, 1.5B 2.5e-7 / 5.1e-7 / 2.6e-7.
-// (From 4096 columns a unit on, a sum holds eight: hidden 8192, ffn 28672, 3.4e-7 against 3.8e-7 on CUDA cores.)
+// (Beyond 4096 columns a unit a sum holds up to eight: hidden 8192, ffn 28672, 3.4e-7 against 3.8e-7 on
+// CUDA cores.)
 //
 // Units of work: (128-row weight tile, K split); a tile's `splits` units are spread over CTAs so
 // that a narrow projection still fills the chip, and each writes its own partial sums
